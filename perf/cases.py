@@ -106,8 +106,7 @@ def _geometry(c):
     return (c["H"], c["W"]), (c["K"],) * 2, torch.channels_last
 
 
-def prepare(case, seed):
-    c = case
+def _inputs(c, seed):
     geo, kgeo, fmt = _geometry(c)
     dtype = _DTYPES[c["dtype"]]
     gen = torch.Generator(device="cuda").manual_seed(seed)
@@ -129,7 +128,12 @@ def prepare(case, seed):
     s["dY"] = normal((c["B"], c["Cout"]) + geo, scale=0.1)
     if c["op"] in ("train", "first", "backward"):
         s["W"] = normal((c["Cout"], c["Cin"]) + kgeo, scale=(2.0 / (c["Cin"] * math.prod(kgeo))) ** 0.5)
-    if c["op"] == "backward":
+    return s
+
+
+def prepare(case, seed):
+    s = _inputs(case, seed)
+    if case["op"] == "backward":
         s["S"] = xb.xconv_sketch(s.pop("X"), s["Z"])       # kept since the forward pass, in the place of X
     return s
 
@@ -151,6 +155,74 @@ def run(state):
     out["dW"] = xb.xconv_wgrad(S, s["dY"], s["Z"], kernel_size=K, kernel_depth=KD)
     if op in ("train", "backward"):
         out["dX"] = xb.xconv_dgrad(s["dY"], s["W"])
+    return out
+
+
+def _signs(seed, count, device="cuda"):
+    """The first `count` entries (a multiple of 128) of the Rademacher stream that include/xconv.h defines: entry e is
+    bit e mod 128 of Philox-4x32-10 block e div 128."""
+    blk = torch.arange(count // 128, dtype=torch.int64, device=device)
+    m32 = 0xFFFFFFFF
+    c0, c1, c2, c3 = blk & m32, blk >> 32, torch.zeros_like(blk), torch.zeros_like(blk)
+    k0, k1 = seed & m32, seed >> 32
+    for _ in range(10):
+        p0, p1 = c0 * 0xD2511F53, c2 * 0xCD9E8D57           # 64-bit products; the shift below masks off the sign
+        c0, c1, c2, c3 = ((p1 >> 32) & m32) ^ c1 ^ k0, p1 & m32, ((p0 >> 32) & m32) ^ c3 ^ k1, p0 & m32
+        k0, k1 = (k0 + 0x9E3779B9) & m32, (k1 + 0xBB67AE85) & m32
+    bit = torch.arange(32, dtype=torch.int64, device=device)
+    words = torch.stack((c0, c1, c2, c3), dim=1).reshape(-1, 1)
+    return (1 - 2 * ((words >> bit) & 1).to(torch.int8)).reshape(-1)
+
+
+def _shifted(t, off):
+    """t[:, z + dz, y + dy, x + dx, :] with zeros outside (t: [n, D, H, W, C])."""
+    out = torch.zeros_like(t)
+    src, dst = [slice(None)], [slice(None)]
+    for d, n in zip(off, t.shape[1:4]):
+        dst.append(slice(max(0, -d), max(0, min(n, n - d))))
+        src.append(slice(max(0, d), max(0, min(n, n + d))))
+    out[dst] = t[src]
+    return out
+
+
+def exact(case, seed):
+    """What run returns, in 64 bits: the definitions in include/xconv.h, one kernel offset at a time."""
+    c = case
+    geo, kgeo, fmt = _geometry(c)
+    s = _inputs(c, seed)
+    shape = (c["D"], c["H"], c["W"])
+    offsets = [(z, y, x) for z in range(kgeo[0] if c["D"] > 1 else 1) for y in range(c["K"]) for x in range(c["K"])]
+    pads = ((kgeo[0] - 1) // 2 if c["D"] > 1 else 0, (c["K"] - 1) // 2, (c["K"] - 1) // 2)
+    offsets = [tuple(k - p for k, p in zip(o, pads)) for o in offsets]
+
+    def rows(t):                                             # [n, D, H, W, C] in 64 bits
+        return t.movedim(1, -1).reshape(t.shape[0], *shape, t.shape[1]).double()
+
+    def back(t):                                             # ... and back to (n, C, [D,] H, W)
+        return t.reshape(t.shape[0], *geo, t.shape[-1]).movedim(-1, 1)
+
+    X, dY = rows(s["X"]), rows(s["dY"])
+    if c["op"] == "seeded":
+        n = X[0].numel() * c["r"]
+        Z = _signs(s["seed"], (n + 127) // 128 * 128)[:n].double().reshape(c["r"], *X.shape[1:])
+    else:
+        Z = rows(s["Z"])
+    S = Z.flatten(1) @ X.flatten(1).T
+    out = {} if c["op"] == "backward" else {"S": S}
+    if c["op"] in ("train", "first"):
+        Wt = s["W"].double().flatten(2)                      # [Cout, Cin, offset]
+        out["Y"] = back(sum(_shifted(X, o) @ Wt[:, :, t].T for t, o in enumerate(offsets)))
+    if c["r"] > c["B"]:
+        P, Q = dY, (S.T @ Z.flatten(1)).reshape(c["B"], *Z.shape[1:])
+    else:
+        P, Q = (S @ dY.flatten(1)).reshape(c["r"], *dY.shape[1:]), Z
+    P = P.flatten(0, 3).T / c["r"]
+    dW = torch.stack([P @ _shifted(Q, o).flatten(0, 3) for o in offsets], dim=-1)
+    out["dW"] = dW.reshape(c["Cout"], c["Cin"], *kgeo)
+    del P, Q, Z, X
+    if c["op"] in ("train", "backward"):
+        Wt = s["W"].double().flatten(2)
+        out["dX"] = back(sum(_shifted(dY, tuple(-d for d in o)) @ Wt[:, :, t] for t, o in enumerate(offsets)))
     return out
 
 
@@ -181,6 +253,6 @@ def work(case):
 
 
 def tolerance(case):
-    """Relative errors against the float64 oracle on these layers: float storage up to 1.3e-6 (sums of up to a few
+    """Relative errors against 64 bits on these layers: float storage up to 1.3e-6 (sums of up to a few
     million products), bfloat16 1.7e-3 and float16 2.1e-4 (each two independent roundings to the storage type)."""
     return {"rel": {"f32": 5e-6, "bf16": 7e-3, "f16": 9e-4}[case["dtype"]]}
