@@ -79,8 +79,7 @@ static xconv_desc flat(const xconv_desc* d) {
   f.zero_blocks = nullptr;
   return f;
 }
-// The tensor-core contraction and convolution work plane by plane: D times the probes for the contraction,
-// D times the batch for the convolutions.  A planar kernel on a volume treats every plane as an image of its
+// The tensor-core contraction works plane by plane, on D times the probes.  A planar kernel on a volume treats every plane as an image of its
 // own (D = 1 from there on); a 3 x 3 x 3 kernel keeps D, so that the kernels know where a volume ends.
 static xconv_desc planes_ct(const xconv_desc* d) {
   xconv_desc f = *d;
@@ -89,12 +88,6 @@ static xconv_desc planes_ct(const xconv_desc* d) {
     f.D = 1; f.KD = 1; f.pad_d = 0;
     if (depth(d) > 1) f.zero_blocks = nullptr;      // the mask is per probe, and r now counts planes
   }
-  return f;
-}
-static xconv_desc planes_cv(const xconv_desc* d) {
-  xconv_desc f = *d;
-  f.B = d->B * depth(d);
-  if (kdepth(d) == 1) { f.D = 1; f.KD = 1; f.pad_d = 0; }
   return f;
 }
 static inline bool volumetric(const xconv_desc* d) { return kdepth(d) == 3; }
@@ -453,19 +446,10 @@ static xconv_status run_conv_simt(const xconv_desc* d, bool dgrad, const void* i
   return check_launch();
 }
 
-// Scratch of the convolution calls: the header, and for the tensor-core dgrad the transposed weights.
-static size_t conv_ws_bytes(const xconv_desc* d, bool dgrad) {
-  TcConvPlan t;
-  const xconv_desc c = planes_cv(d);
-  if (tc_plan_conv(&c, dgrad, &t)) return WS_HEADER + align_up(t.wt_bytes, 256);
-  return WS_HEADER;
-}
-
 static xconv_status run_conv(const xconv_desc* d, bool dgrad, const void* in, const void* Wt, void* out,
                              char* ws, cudaStream_t st) {
   TcConvPlan t;
-  const xconv_desc c = planes_cv(d);
-  if (tc_plan_conv(&c, dgrad, &t)) return tc_run_conv(&c, t, dgrad, in, Wt, out, ws, ws + WS_HEADER, st);
+  if (tc_plan_conv(d, dgrad, &t)) return tc_run_conv(d, t, dgrad, in, Wt, out, ws, st);
   return d->dtype == XCONV_F32 ? run_conv_simt<float>(d, dgrad, in, Wt, out, st)
          : d->dtype == XCONV_F16 ? run_conv_simt<f16>(d, dgrad, in, Wt, out, st)
                                  : run_conv_simt<bf16>(d, dgrad, in, Wt, out, st);
@@ -644,7 +628,7 @@ size_t xconv_workspace_bytes(const xconv_desc* desc, int op) {
     case XCONV_OP_WGRAD:
     case XCONV_OP_BACKPROBE:
     case XCONV_OP_CONTRACT: return plan_wgrad(desc).bytes;
-    case XCONV_OP_DGRAD: return conv_ws_bytes(desc, true);
+    case XCONV_OP_DGRAD: return WS_HEADER;      // the convolutions need the status header only
     case XCONV_OP_WGRAD_INDEPENDENT: return validate_indep(desc) == XCONV_OK ? plan_indep(desc).bytes : 0;
     default: return 0;
   }
@@ -661,8 +645,7 @@ int xconv_engine_for(const xconv_desc* desc, int op) {
     case XCONV_OP_FORWARD:
     case XCONV_OP_DGRAD: {
       TcConvPlan t;
-      const xconv_desc c = planes_cv(desc);
-      return tc_plan_conv(&c, op == XCONV_OP_DGRAD, &t) ? tc : XCONV_ENGINE_SIMT_F32;
+      return tc_plan_conv(desc, op == XCONV_OP_DGRAD, &t) ? tc : XCONV_ENGINE_SIMT_F32;
     }
     default: return XCONV_ENGINE_NONE;
   }
@@ -890,7 +873,7 @@ xconv_status xconv_dgrad(const xconv_desc* desc, const void* dY, const void* W, 
   if (s != XCONV_OK) return s;
   if (!dY || !W || !dX) return XCONV_ERR_INVALID_ARG;
   if (!aligned16(dY) || !aligned16(W) || !aligned16(dX)) return XCONV_ERR_ALIGNMENT;
-  if (!ws || ws_bytes < conv_ws_bytes(desc, true)) return XCONV_ERR_WORKSPACE;
+  if (!ws || ws_bytes < WS_HEADER) return XCONV_ERR_WORKSPACE;
   if (!aligned16(ws)) return XCONV_ERR_ALIGNMENT;
   new_call();
   return run_conv(desc, true, dY, W, dX, static_cast<char*>(ws), static_cast<cudaStream_t>(cuda_stream));

@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 #include <stddef.h>
+#include <stdint.h>
 
 #include "../../include/xconv.h"
 
@@ -36,10 +37,15 @@ struct TcWgradPlan {
 };
 
 struct TcConvPlan {
-  int tile_n, tiles_n, stages, patch_w, patch_h, patches_x, patches_y;
-  int m_sub;           // 2 = a work unit covers the same patch of two images, which share the weight tile
-  int cw;              // input channels per stage: 64 (128-byte tile rows) or 32 (64-byte rows, more stages)
-  size_t wt_bytes;     // dgrad only: transposed, flipped copy of the weights
+  int patch_w, patch_h;      // output pixels of one 128-row MMA tile
+  int tile_n, tiles_n;       // channels out per column tile
+  int m_sub, acc_bufs;       // patches that share each weight tile; accumulator sets in tensor memory
+  int cw, nbw, ocw;          // channels per input tile row, per MN-major weight block (dX), per staging tile
+  int resident, w_slots, a_slots;   // all weights in shared memory, or a ring of w_slots tiles; input boxes
+  uint32_t a_sub_bytes;      // shared memory of one patch's box
+  int groups;                // of epilogue warps: two where a patch is over quickly, one beside long mainloops, whose issue
+                             // slots the second would only take
+  long patches;
 };
 
 // Fill the plan and say whether the tcgen05 kernels cover this layer.  tc_plan_wgrad returns a mask:
@@ -49,7 +55,7 @@ int tc_plan_wgrad(const xconv_desc* d, TcWgradPlan* p);
 
 bool tc_plan_conv(const xconv_desc* d, bool dgrad, TcConvPlan* p);
 xconv_status tc_run_conv(const xconv_desc* d, const TcConvPlan& p, bool dgrad, const void* in, const void* W,
-                         void* out, char* ws_head, char* wt, cudaStream_t st);
+                         void* out, char* ws_head, cudaStream_t st);
 
 // `seed` != nullptr: Z is not read; its tiles are redrawn inside the kernel from the Philox stream of *seed
 // (Rademacher entries; see xconv_probes_from_seed).  Only for layers tc_sketch_can_redraw accepts.

@@ -1,5 +1,7 @@
 // tcgen05 / TMEM / TMA kernels for bfloat16 storage (sm_100a).
 //
+// (the exact convolutions have a kernel of their own, conv_tc.cu)
+//
 // One kernel template, three problem shapes, all dense contractions with float accumulation in
 // tensor memory:
 //   SKETCH    S = Z^T X       (Algorithm 1 forward step 3)  D[row,col] = sum_k A[row,k] Bm[col,k],
@@ -11,10 +13,6 @@
 //             reduction runs over image patches, and the offset is added to the patch coordinates of
 //             the TMA box of Z -- out-of-image rows are zero-filled by the TMA unit, which is exactly
 //             the zero padding of the convolution.  No shifted or im2col copy of Z is ever made.
-//   CONV      Y = conv(X, w)  (forward step 1, Eq. 5) and, with transposed and flipped weights, the exact
-//             dX: D[pixel, co] = sum_{offset, ci} In[pixel + offset, ci] W[co, offset, ci] for one image
-//             patch per work unit; both tiles K-major (channels contiguous), the reduction runs over
-//             (offset, 64-channel block), and the offset again moves the TMA box of the input.
 //
 // Structure of a CTA (192 or 320 threads): warp 0 = TMA producer, warp 1 = MMA issuer and TMEM owner,
 // warps 2..5 (2..9) = epilogue, one (two) per TMEM lane quadrant; two share the columns of a tile.  A ring of shared-memory stages is handed
@@ -23,16 +21,12 @@
 // its outstanding copies (bounded again), frees its tensor memory and returns.
 #include "tc_api.h"
 
-#include <cuda.h>
-#include <cudaTypedefs.h>
-
-#include <algorithm>
-
 #include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace xconv {
 
-enum : int { MODE_SKETCH = 0, MODE_BACKPROBE = 1, MODE_CONTRACT = 2, MODE_CONV = 3 };
+enum : int { MODE_SKETCH = 0, MODE_BACKPROBE = 1, MODE_CONTRACT = 2 };
 
 struct TcParams {
   int mode;
@@ -88,11 +82,10 @@ struct TcParams {
   long rows, cols;         // valid MMA rows / columns of the whole problem
   // outputs
   float* part;             // SKETCH: [split][rows][cols]; CONTRACT: [split][Cout][T][Cin]
-  bf16* L;                 // BACKPROBE: [r][Q]; CONV: output [B][H][W][Co]
+  bf16* L;                 // BACKPROBE: [r][Q]
   long Q;
-  int T, Cin;              // CONTRACT output indexing; CONV: offsets and input channels
-  int H, W, cgroups;       // CONV: image size and input-channel blocks of 64
-  int nimg;                // CONV: images; with m_sub = 2 a unit covers the same patch of images img and img + 1
+  int T, Cin;              // CONTRACT output indexing
+  int H;                   // CONTRACT: rows of the image
   // Probing vectors redrawn inside the kernel (Algorithm 1 keeps the seed, not Z): the tile of Z is not copied
   // from global memory; the epilogue warps write it into the stage from the Philox stream of the seed.
   int seeded;              // 0: Z is read from memory
@@ -100,7 +93,7 @@ struct TcParams {
   int z_is_a;              // SKETCH: Z is the A operand (probes on the MMA rows) instead of the B operand
   long z_row_len;          // entries of one probing vector, H*W*Cin
   long rows_z;             // probing vectors (rows of Z)
-  // Volumes: the planes (probe x depth for CONTRACT, image x depth for CONV) are the outermost tensor axis; a
+  // Volumes: the planes (probe x depth) are the outermost tensor axis; a
   // kernel offset with a depth component dz reads plane + dz, and where that leaves the volume the box is
   // sent to row H of the plane instead, which lies outside the image: the copy engine fills it with zeros.
   // CONTRACT in halves with block-sparse probes (Eq. 7) whose all-zero 64-channel blocks the caller has named.  Row tn of
@@ -118,130 +111,6 @@ struct TcParams {
   unsigned int tag;        // tag of this call
 };
 
-// ------------------------------------------------------------------------------------ PTX wrappers
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.b32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-// Bounded wait: about one second after a short spin.  Returns false (and records the tag) on expiry.
-__device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, unsigned int* status, unsigned int tag,
-                                            unsigned long long limit_ns = 1000000000ull) {
-  for (int i = 0; i < 4096; ++i)
-    if (mbar_try_wait(bar, parity)) return true;
-  const unsigned long long t0 = global_ns();
-  for (;;) {
-    for (int i = 0; i < 256; ++i)
-      if (mbar_try_wait(bar, parity)) return true;
-    if (global_ns() - t0 > limit_ns) {
-      atomicExch(status, tag);
-      return false;
-    }
-  }
-}
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, unsigned int* status, unsigned int tag) {
-  if (mbar_try_wait(bar, parity)) return true;       // the common case costs one instruction
-  return mbar_wait_slow(bar, parity, status, tag);
-}
-
-// The same operations on a 32-bit shared-memory address the caller keeps in a register.
-__device__ __forceinline__ bool mbar_try_wait_a(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.b32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ void umma_commit_a(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3, int c4,
-                                            uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], [%7];"
-      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4),
-        "r"(smem_u32(bar)) : "memory");
-}
-// Tensor store shared -> global (bulk async-group completion) and its bookkeeping.
-__device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, uint32_t src, int c0, int c1, int c2) {
-  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];"
-               ::"l"(reinterpret_cast<uint64_t>(map)), "r"(src), "r"(c0), "r"(c1), "r"(c2) : "memory");
-}
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// all earlier bulk stores of this thread have finished READING shared memory / have completed
-template <int N>
-__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory"); }
-// at most `pending` (1, 3 or 7) of this thread's bulk stores may still be reading shared memory
-__device__ __forceinline__ void bulk_wait_read_upto(int pending) {
-  if (pending >= 7) bulk_wait_read<7>();
-  else if (pending >= 3) bulk_wait_read<3>();
-  else if (pending >= 1) bulk_wait_read<1>();
-  else bulk_wait_read<0>();
-}
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-__device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
-  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
-}
-
-__device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t ncols) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(ncols)
-               : "memory");
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// D[tmem] (+)= A[smem] * B[smem], 16-bit inputs (bfloat16 or float16, per the instruction descriptor), float
-// accumulate; issued by one thread.  The two
-// shared-memory descriptors come as 32-bit halves: only the low half (start address) changes between
-// k-steps, so the issuing thread -- whose own instruction stream is the critical path of the CTA when
-// the tiles are small -- spends one 32-bit add per operand and k-step.
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
-                                          uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-      "mov.b64 da, {%1, %2};\n\t"
-      "mov.b64 db, {%3, %4};\n\t"
-      "setp.ne.b32 p, %6, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");
-}
 // All MMAs of one stage, fully unrolled.  The issuing thread runs alone in its warp, so every instruction
 // it executes costs a full dependent-issue slot (~6 cycles): a 128x64x16 MMA occupies the tensor pipe for
 // 32 cycles, i.e. about five instructions.  KS k-steps, TWO = two 128-row tiles share the B tile.
@@ -278,35 +147,6 @@ __device__ __forceinline__ void umma_stage_taps(uint32_t d, uint32_t unit_cols, 
     a_lo += a_step;
     b_lo += b_step;
   }
-}
-
-// mbarrier arrive once every MMA issued so far by this thread has finished.
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
-}
-
-// 32 lanes x 32 consecutive 32-bit columns: thread t of the warp receives lane (quadrant*32 + t).
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-        "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-        "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-      : "r"(taddr) : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-      : "r"(taddr) : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
 // The 64 sign bits of entries e0 .. e0+63 of Z (e0 a multiple of 64): entry e takes bit (e mod 128) of the
@@ -403,14 +243,6 @@ __device__ __forceinline__ bool umma_halves_items(int nkb, int& s, uint32_t& par
   return true;
 }
 
-// Two floats rounded to the 16-bit storage type, packed (first in the low half).
-__device__ __forceinline__ uint32_t pack2(uint32_t a, uint32_t b, bool f16) {
-  if (f16) { __half2 h = __floats2half2_rn(__uint_as_float(a), __uint_as_float(b)); return *reinterpret_cast<uint32_t*>(&h); }
-  __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(a), __uint_as_float(b));
-  return *reinterpret_cast<uint32_t*>(&h);
-}
-
-constexpr int TILE_M = 128;
 constexpr int MAX_STAGES = 8;
 constexpr int ZLIST_SMEM = 128;      // list entries of a unit held in shared memory (the rest are read from global memory)
 // Epilogue warps per tensor-memory lane quadrant: one, or two where a tile's epilogue outlasts its mainloop (the
@@ -419,11 +251,7 @@ constexpr int ZLIST_SMEM = 128;      // list entries of a unit held in shared me
 constexpr int MAX_EPI_GROUPS = 2;
 constexpr int TC_THREADS = 64 + 128 * MAX_EPI_GROUPS;     // launch bound; a launch has 64 + 128 * epi_groups threads
 
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-struct Unit { int tm, tn, tap; long split, kb0; int nkb; int px, py, img; int blk0, nblk; };
+struct Unit { int tm, tn, tap; long split, kb0; int nkb; int blk0, nblk; };
 
 // Work unit u -> tile, offset, k-split.  32-bit divisions throughout (a launch has far fewer than 2^31 units):
 // every role of a CTA decodes each of its units on its own critical path, one instruction per ~6 clocks, and a
@@ -431,17 +259,8 @@ struct Unit { int tm, tn, tap; long split, kb0; int nkb; int px, py, img; int bl
 __device__ __forceinline__ Unit decode_unit(const TcParams& p, long u_) {
   Unit w;
   const uint32_t u = (uint32_t)u_;
-  w.px = w.py = w.img = 0;
   w.blk0 = w.nblk = 0;
-  if (p.mode == MODE_CONV) {                 // channel tiles innermost, then patches of one image
-    uint32_t q = u;
-    const uint32_t tn = (uint32_t)p.tiles_n, px = (uint32_t)p.patches_x, py = (uint32_t)p.patches_y;
-    w.tn = (int)(q % tn); q /= tn;
-    w.px = (int)(q % px); q /= px;
-    w.py = (int)(q % py); q /= py;
-    w.img = (int)q * p.m_sub;
-    w.tm = 0; w.tap = 0; w.split = 0;
-  } else if (p.mode == MODE_BACKPROBE) {     // probe tiles innermost: the dY tile is re-read while hot in L2
+  if (p.mode == MODE_BACKPROBE) {            // probe tiles innermost: the dY tile is re-read while hot in L2
     const uint32_t tm = (uint32_t)p.tiles_m;
     w.tm = tm == 1 ? 0 : (int)(u % tm);
     w.tn = tm == 1 ? (int)u : (int)(u / tm);
@@ -751,11 +570,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         int kc = 0, px = 0, py = 0, pj = 0, dx = 0, dy = 0, dz = 0, pz = 0;
         if (p.mode == MODE_SKETCH) kc = (int)((p.k_weave ? w.split : w.kb0) * 64 * p.kgroup);
         else if (p.mode == MODE_BACKPROBE) kc = (int)w.kb0 * p.ksteps * 16;
-        else if (p.mode == MODE_CONV) {      // pj counts channel blocks, kc = offset * Cin; w.img is a plane
-          dx = dy = -p.pad;
-          dz = -p.pad_d;
-          pz = w.img % p.depth;
-        } else {
+        else {
           uint32_t q = (uint32_t)w.kb0;
           px = (int)(q % (uint32_t)p.patches_x); q /= (uint32_t)p.patches_x;
           py = (int)(q % (uint32_t)p.patches_y); q /= (uint32_t)p.patches_y;
@@ -797,17 +612,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
               for (int b = 0; b < w.nblk; ++b)
                 tma_load_3d(b_dst + (uint32_t)b * p.b_box_bytes, &map_b, 0, kc, w.blk0 + b, &full_bar[s]);
             kc += p.ksteps * 16;
-          } else if (p.mode == MODE_CONV) {
-            // input patch moved by the kernel offset (zero fill outside the image) and the matching
-            // [tile_n output channels x 64 input channels] block of the weights
-            const bool inside = (unsigned)(pz + dz) < (unsigned)p.depth;
-            tma_load_5d(a_dst, &map_a, 0, w.px * p.patch_w + dx, inside ? w.py * p.patch_h + dy : p.H, pj, w.img + dz,
-                        &full_bar[s]);
-            tma_load_2d(b_dst, &map_b, kc + (pj << p.cw_shift), col0, &full_bar[s]);
-            if (++pj == p.cgroups) {
-              pj = 0; kc += p.Cin;
-              if (++dx > p.pad) { dx = -p.pad; if (++dy > p.pad) { dy = -p.pad; ++dz; } }
-            }
           } else {
             // one 5-d box per operand: (64 channels, patch x, patch y, channel groups of 64, probe)
             const int x0 = px * p.patch_w, y0 = py * p.patch_h;
@@ -1149,10 +953,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
       } else
       for (int mt = 0; mt < p.m_sub; ++mt) {
-        // first row of this warp; CONV: rows are the pixels of the patch, the row tile picks the image
-        const long row_w = (p.mode == MODE_CONV ? 0L : ((long)w.tm * p.m_sub + mt) * TILE_M) + quad * 32;
+        const long row_w = ((long)w.tm * p.m_sub + mt) * TILE_M + quad * 32;   // first row of this warp
         if (row_w >= p.rows) continue;                                         // warp-uniform
-        if (p.mode == MODE_CONV && w.img + mt >= p.nimg) continue;
         const long row = row_w + lane;
         for (int cu = eg * 32; cu < unit_cols; cu += 32 * p.epi_groups) {
           // several offsets per unit (CONTRACT): tile_n is then a multiple of 32 and a chunk lies in one offset
@@ -1169,42 +971,19 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           }
           const int nc = min(32, p.tile_n - c);
           if (row >= p.rows) continue;
-          if (p.mode == MODE_CONV) {
-            // D[pixel of the patch, co] -> out[img][y][x][co]: 32 consecutive channels per thread
-            const int pr = (int)row / p.patch_w, pc = (int)row % p.patch_w;
-            const int y = w.py * p.patch_h + pr, x = w.px * p.patch_w + pc;
-            if (y < p.H && x < p.W) {
-              bf16* dst = p.L + (((long)(w.img + mt) * p.H + y) * p.W + x) * p.cols + col0 + c;
-              if (nc == 32 && col0 + c + 32 <= p.cols) {
+          // SKETCH / CONTRACT: partial tile in the order the accumulator comes out of tensor memory:
+          // block(split, offset, tile) [128-row tile][32-column chunk][4-column group][row][4 floats],
+          // so that the 32 lanes of every store write 512 contiguous bytes.  The reduce kernels undo it.
+          const int chunks = (p.tile_n + 31) >> 5, qn = p.tile_n < 32 ? p.tile_n >> 2 : 8;   // 4-column groups per chunk
+          float* blk = p.part + ((((long)w.split * p.taps + w.tap + tap_l) * p.tiles_m + w.tm) * p.tiles_n + w.tn) *
+                                    ((long)p.m_sub * TILE_M * chunks * qn * 4);
+          float* dst = blk + ((long)(mt * chunks + (c >> 5)) * qn * TILE_M + quad * 32 + lane) * 4;
 #pragma unroll
-                for (int i = 0; i < 32; i += 8) {
-                  uint4 o;
-                  o.x = pack2(v[i + 0], v[i + 1], F16); o.y = pack2(v[i + 2], v[i + 3], F16);
-                  o.z = pack2(v[i + 4], v[i + 5], F16); o.w = pack2(v[i + 6], v[i + 7], F16);
-                  *reinterpret_cast<uint4*>(dst + i) = o;
-                }
-              } else {
-#pragma unroll
-                for (int i = 0; i < 32; ++i)
-                  if (i < nc && col0 + c + i < p.cols)
-                    reinterpret_cast<unsigned short*>(dst)[i] = (unsigned short)(pack2(v[i], v[i], F16) & 0xFFFFu);
-              }
-            }
-          } else {
-            // SKETCH / CONTRACT: partial tile in the order the accumulator comes out of tensor memory:
-            // block(split, offset, tile) [128-row tile][32-column chunk][4-column group][row][4 floats],
-            // so that the 32 lanes of every store write 512 contiguous bytes.  The reduce kernels undo it.
-            const int chunks = (p.tile_n + 31) >> 5, qn = p.tile_n < 32 ? p.tile_n >> 2 : 8;   // 4-column groups per chunk
-            float* blk = p.part + ((((long)w.split * p.taps + w.tap + tap_l) * p.tiles_m + w.tm) * p.tiles_n + w.tn) *
-                                      ((long)p.m_sub * TILE_M * chunks * qn * 4);
-            float* dst = blk + ((long)(mt * chunks + (c >> 5)) * qn * TILE_M + quad * 32 + lane) * 4;
-#pragma unroll
-            for (int i = 0; i < 32; i += 4) {
-              if (i >= nc) break;
-              *reinterpret_cast<float4*>(dst + (long)(i >> 2) * TILE_M * 4) =
-                  make_float4(__uint_as_float(v[i]), __uint_as_float(v[i + 1]), __uint_as_float(v[i + 2]),
-                              __uint_as_float(v[i + 3]));
-            }
+          for (int i = 0; i < 32; i += 4) {
+            if (i >= nc) break;
+            *reinterpret_cast<float4*>(dst + (long)(i >> 2) * TILE_M * 4) =
+                make_float4(__uint_as_float(v[i]), __uint_as_float(v[i + 1]), __uint_as_float(v[i + 2]),
+                            __uint_as_float(v[i + 3]));
           }
         }
       }
@@ -1326,46 +1105,9 @@ __global__ void __launch_bounds__(256) reduce_contract_partials(const float* __r
 
 // ------------------------------------------------------------------------------------ host side
 
-static inline long cdivl(long a, long b) { return (a + b - 1) / b; }
-static inline int round_up(int v, int a) { return (v + a - 1) / a * a; }
-static const int SMEM_LIMIT = 227 * 1024;
-static const int STATIC_SMEM_SLACK = 2048;     // barriers + alignment slack
-static const int NUM_SMS = 148;
 static const int BP_SLOT_BYTES = 4 * 32 * 128;      // back-probe output staging: per slot and epilogue group, 4 warps x 32 rows x 64 positions
-
-static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  if (!fn) {
-    void* ptr = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(ptr);
-  }
-  return fn;
-}
-
-// Tensor map over 16-bit elements (bfloat16, or float16 if `f16`), 128-byte swizzle unless told otherwise;
-// dims/strides innermost first, strides in bytes for dims 1..rank-1.
-static bool make_map(CUtensorMap* m, const void* base, int rank, const uint64_t* dims, const uint64_t* strides,
-                     const uint32_t* box, bool f16, CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B) {
-  PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
-  if (!fn) return false;
-  cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-  cuuint64_t d[5], st[4];
-  cuuint32_t bx[5];
-  for (int i = 0; i < rank; ++i) { d[i] = dims[i]; bx[i] = box[i]; }
-  for (int i = 0; i + 1 < rank; ++i) st[i] = strides[i];
-  CUresult r = fn(m, f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), d, st, bx, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS;
-}
-
 // Columns a partial tile occupies in its stored (accumulator-order) layout.
 static int tile_cols_stored(int tile_n) { return tile_n < 32 ? tile_n : (tile_n + 31) / 32 * 32; }
-
-static int pow2_cols(int n) { int c = 32; while (c < n) c *= 2; return c; }
 
 static int pick_stages(uint32_t stage_bytes, int want_ctas_per_sm) {
   const int budget = SMEM_LIMIT / want_ctas_per_sm - STATIC_SMEM_SLACK;
@@ -1900,129 +1642,6 @@ xconv_status tc_run_wait_selftest(char* ws_head, unsigned long long limit_ns, cu
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { set_cuda_error((int)e); return XCONV_ERR_CUDA; }
   return XCONV_OK;
-}
-
-// ---- exact convolution and input gradient -----------------------------------------------------
-
-// Wd[n][T-1-t][m] = W[m][t][n]: the weights of the transposed convolution, laid out like W.
-__global__ void __launch_bounds__(256) flip_transpose_weights(const bf16* __restrict__ W, bf16* __restrict__ Wd,
-                                                              int Cout, int Cin, int T) {
-  pdl_trigger();
-  pdl_wait();
-  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long count = (long)Cout * T * Cin;
-  if (i >= count) return;
-  const int m = (int)(i % Cout);
-  const int t = (int)((i / Cout) % T);
-  const int n = (int)(i / ((long)Cout * T));
-  Wd[i] = W[((long)m * T + (T - 1 - t)) * Cin + n];
-}
-
-static void pick_patch_conv(int H, int W, int* pw, int* ph) {
-  // patch of at most 128 pixels (the MMA rows) covering the image with the least work per pixel:
-  // overhang and unused MMA rows both count
-  double best = 1e30; int bw = 1, bh = 1;
-  for (int w = 1; w <= std::min(W, 128); ++w)
-    for (int h = 1; h * w <= 128 && h <= H; ++h) {
-      const double cost = (double)cdivl(W, w) * (double)cdivl(H, h) * 128.0 / ((double)W * H);
-      if (cost < best - 1e-9 || (cost < best + 1e-9 && w > bw)) { best = cost; bw = w; bh = h; }
-    }
-  *pw = bw; *ph = bh;
-}
-
-bool tc_plan_conv(const xconv_desc* d, bool dgrad, TcConvPlan* p) {
-  if (d->dtype != XCONV_BF16 && d->dtype != XCONV_F16) return false;
-  const int Ci = dgrad ? d->Cout : d->Cin, Co = dgrad ? d->Cin : d->Cout;
-  if (Ci % 32 != 0 || Co % 8 != 0 || Co < 16 || d->circular) return false;   // circular padding: FP32-FMA kernels
-  p->tile_n = std::min(256, round_up(Co, 16));
-  p->tiles_n = (int)cdivl(Co, p->tile_n);
-  pick_patch_conv(d->H, d->W, &p->patch_w, &p->patch_h);
-  p->patches_x = (int)cdivl(d->W, p->patch_w);
-  p->patches_y = (int)cdivl(d->H, p->patch_h);
-  // Two images share each weight tile when the patch is a whole number of 8-row swizzle groups (the
-  // second image's rows then start on a group boundary): the traffic into the SM per MMA cycle falls
-  // from 94 to 62.5 bytes, which is what bounded the convolution.
-  const int px = p->patch_w * p->patch_h;
-  // (a kernel with a depth component shifts every plane on its own: one plane per unit then)
-  p->m_sub = (px % 8 == 0 && d->B >= 2 && d->KD <= 1) ? 2 : 1;
-  // Input channels go by 64 per stage (128-byte tile rows); layers whose channel count is a multiple of 32
-  // only take 32 per stage (64-byte rows, 64-byte swizzle).  (32 per stage everywhere, for more and smaller
-  // stages, was slower: 557 against 485 us on the 256-channel layer.)
-  const uint32_t rows = (uint32_t)(p->m_sub == 2 ? px + TILE_M : TILE_M) + (uint32_t)p->tile_n;
-  p->cw = Ci % 64 == 0 ? 64 : 32;
-  p->stages = pick_stages(rows * 2 * (uint32_t)p->cw, 1);
-  p->wt_bytes = dgrad ? (size_t)d->Cout * d->KH * d->KW * (d->KD > 1 ? d->KD : 1) * d->Cin * 2 : 0;
-  return true;
-}
-
-xconv_status tc_run_conv(const xconv_desc* d, const TcConvPlan& pl, bool dgrad, const void* in, const void* W,
-                         void* out, char* ws_head, char* wt, cudaStream_t st) {
-  const int T = d->KH * d->KW * (d->KD > 1 ? d->KD : 1);
-  const int Ci = dgrad ? d->Cout : d->Cin, Co = dgrad ? d->Cin : d->Cout;
-  const bool f16 = d->dtype == XCONV_F16;
-  const void* Wk = W;
-  if (dgrad) {
-    const long count = (long)d->Cout * T * d->Cin;
-    cudaError_t e = launch_pdl(flip_transpose_weights, dim3((unsigned)cdivl(count, 256)), dim3(256), 0, st,
-                               static_cast<const bf16*>(W), reinterpret_cast<bf16*>(wt), d->Cout, d->Cin, T);
-    count_launch();
-    if (e != cudaSuccess) { set_cuda_error((int)e); return XCONV_ERR_CUDA; }
-    Wk = wt;
-  }
-  CUtensorMap ma, mb;
-  // input as (cw channels, x, y, channel blocks of cw, image); weights as [Co][T*Ci]; cw = 64 or 32
-  const uint32_t cw = (uint32_t)pl.cw, rb = 2 * cw;                      // channels and bytes per tile row
-  const CUtensorMapSwizzle swz = cw == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
-  const uint64_t da[5] = {cw, (uint64_t)d->W, (uint64_t)d->H, (uint64_t)(Ci / cw), (uint64_t)d->B};
-  const uint64_t sa[4] = {(uint64_t)Ci * 2, (uint64_t)d->W * Ci * 2, rb, (uint64_t)d->H * d->W * Ci * 2};
-  const uint32_t box_a[5] = {cw, (uint32_t)pl.patch_w, (uint32_t)pl.patch_h, 1, (uint32_t)pl.m_sub};
-  const uint64_t db[2] = {(uint64_t)T * Ci, (uint64_t)Co};
-  const uint64_t sb[1] = {(uint64_t)T * Ci * 2};
-  const uint32_t box_b[2] = {cw, (uint32_t)pl.tile_n};
-  if (!make_map(&ma, in, 5, da, sa, box_a, f16, swz) || !make_map(&mb, Wk, 2, db, sb, box_b, f16, swz)) return XCONV_ERR_CUDA;
-  TcParams p{};
-  p.f16 = f16 ? 1 : 0;
-  p.mode = MODE_CONV;
-  p.tile_n = pl.tile_n;
-  const uint32_t px = (uint32_t)(pl.patch_w * pl.patch_h);
-  p.m_sub = pl.m_sub;
-  p.acc_bufs = (2 * pl.m_sub * pl.tile_n <= 512) ? 2 : 1;
-  p.tmem_cols = pow2_cols(p.acc_bufs * pl.m_sub * pl.tile_n);
-  p.stages = pl.stages;
-  p.ksteps = (int)cw / 16;
-  p.a_boxes = p.b_boxes = 1;
-  // one image: the patch fills the first px rows of a 128-row tile.  Two images: the second image's px
-  // rows follow the first's directly and its MMA tile starts there; 128 rows behind that start belong to the stage.
-  p.a_sub_bytes = (pl.m_sub == 2 ? px : (uint32_t)TILE_M) * rb;
-  p.a_stage_bytes = (pl.m_sub == 2 ? px + TILE_M : (uint32_t)TILE_M) * rb;
-  p.b_stage_bytes = (uint32_t)pl.tile_n * rb;
-  p.tx_bytes = (uint32_t)pl.m_sub * px * rb + p.b_stage_bytes;
-  if (cw == 32) { p.layout = 4; p.sbo = 8 * rb; p.mn_step = 16 * rb; p.cw_shift = 5; }   // 64-byte swizzle
-  p.a_mn_major = p.b_mn_major = 0;
-  p.tiles_m = 1;
-  p.tiles_n = pl.tiles_n;
-  p.taps = 1;
-  p.kblocks = (long)T * (Ci / cw);
-  p.kblocks_per_split = p.kblocks;
-  p.units = cdivl(d->B, pl.m_sub) * pl.patches_y * pl.patches_x * pl.tiles_n;
-  p.nimg = d->B;
-  p.patch_w = pl.patch_w;
-  p.patch_h = pl.patch_h;
-  p.patches_x = pl.patches_x;
-  p.patches_y = pl.patches_y;
-  p.pad = (d->KH - 1) / 2;
-  p.depth = d->D > 1 ? d->D : 1;
-  p.pad_d = d->KD > 1 ? (d->KD - 1) / 2 : 0;
-  p.rows = (long)pl.patch_w * pl.patch_h;
-  p.cols = Co;
-  p.L = static_cast<bf16*>(out);
-  p.T = T;
-  p.Cin = Ci;
-  p.H = d->H;
-  p.W = d->W;
-  p.cgroups = Ci / cw;
-  p.status = reinterpret_cast<unsigned int*>(ws_head);
-  return launch(ma, mb, p, (unsigned)std::min<long>(p.units, NUM_SMS), st);
 }
 
 }  // namespace xconv
