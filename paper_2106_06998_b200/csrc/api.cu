@@ -130,8 +130,45 @@ static SketchPlan plan_sketch(const xconv_desc* d_, bool seeded = false) {
   return p;
 }
 
+// 16-bit tensors whose channel count is not a multiple of 8 have rows the copy engine cannot step through (16-byte rule).
+// The tensor-core kernels then get a copy in the workspace with the channels padded by zeros to the next multiple of 8.
+static inline int pad8(int c) { return (c + 7) / 8 * 8; }
+static size_t padded_bytes(long rows, int c) { return c % 8 ? align_up((size_t)rows * pad8(c) * 2, 256) : 0; }
+
+template <typename T>
+__global__ void __launch_bounds__(256) pad_channels_kernel(const T* __restrict__ in, T* __restrict__ out, long pieces, int C,
+                                                           int per_row) {
+  pdl_trigger();
+  pdl_wait();
+  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;      // one 16-byte piece of the padded tensor
+  if (i >= pieces) return;
+  const long row = i / per_row;
+  const int c0 = (int)(i - row * per_row) * 8;
+  uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    if (c0 + k < C) w[k >> 1] |= (uint32_t)in[row * C + c0 + k] << (16 * (k & 1));
+  *reinterpret_cast<uint4*>(out + i * 8) = make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// `t` itself, or its padded copy at *ws (which then moves on behind it).
+static xconv_status pad_channels(const void*& t, long rows, int C, char*& ws, cudaStream_t st) {
+  if (C % 8 == 0) return XCONV_OK;
+  const long pieces = rows * (pad8(C) / 8);
+  const cudaError_t e = launch_pdl(pad_channels_kernel<unsigned short>, dim3((unsigned)cdiv(pieces, 256)), dim3(256), 0, st,
+                                   static_cast<const unsigned short*>(t), reinterpret_cast<unsigned short*>(ws), pieces, C, pad8(C) / 8);
+  ++g_launches;
+  if (e != cudaSuccess) { g_last_cuda_error = (int)e; return XCONV_ERR_CUDA; }
+  t = ws;
+  ws += padded_bytes(rows, C);
+  return XCONV_OK;
+}
+
 struct WgradPlan {
   bool tc_bp, tc_ct;
+  bool halo;                           // contraction of few channels (contract_tc.cu) instead of the one of tc_kernels.cu
+  TcHaloPlan h;                        // ... on the layer with its channels padded to multiples of 8
+  size_t ct_bytes;                     // scratch of the contraction: partial sums, padded copies
   int splits; long items_per_split;    // simt contraction
   TcWgradPlan t;                       // tcgen05: contraction fields (planned on the per-plane layer)
   TcWgradPlan tb;                      // tcgen05: back-probe fields (planned on the flattened layer)
@@ -150,8 +187,27 @@ static WgradPlan plan_wgrad_core(const xconv_desc* d) {
   p.tc_bp = (tc_plan_wgrad(&f, &p.tb) & 1) != 0;
   const xconv_desc c = planes_ct(d);    // the tensor-core contraction works plane by plane
   p.tc_ct = (tc_plan_wgrad(&c, &p.t) & 2) != 0;
+  // The contraction for few channels: wherever the other one does not go, and where that one leaves MMA rows empty or copies
+  // Z once per offset.  Measured, other -> this, us: 3 x 3, 32 -> 32 channels, 64 probes of 64 x 64: 27.6 -> 17.0, 128 -> 32
+  // channels out 35 -> 22 (but 32 -> 256 31 -> 37, 128 -> 128 35 -> 41, 64 -> 64 20.8 -> 20.7); 5 x 5, 32 channels 58 -> 20,
+  // 128: 36.4 -> 36.5; pointwise, 64 channels 12.6 -> 9.9, 128: 14.7 -> 19.4; 3 x 3 x 3, 32 -> 64 73 -> 30, 128 -> 128 38 -> 28,
+  // 96 -> 96, a quarter of it padding, 43 -> 47.  (A list of zero blocks is only read by the other one.)
+  xconv_desc e = *d;
+  e.Cin = pad8(d->Cin); e.Cout = pad8(d->Cout);
+  const int most = std::max(d->Cin, d->Cout);
+  const bool whole = (d->Cin == 32 || d->Cin % 64 == 0) && (d->Cout == 32 || d->Cout % 64 == 0);
+  const bool few = volumetric(d) ? most <= 128 && whole : d->KH == 3 ? d->Cout <= 32 : most <= 64;
+  const bool other = p.tc_ct && (p.t.ct_masked || !few);
+  if (!other && tc_plan_halo(&e, &p.h)) {
+    p.halo = true;
+    const long px = (long)depth(d) * d->H * d->W * d->r;
+    p.ct_bytes = align_up(p.h.part_bytes, 256) + padded_bytes(px, d->Cin) + padded_bytes(px, d->Cout);
+    p.bytes = p.part_off + p.ct_bytes;
+    return p;
+  }
   if (p.tc_ct) {
-    p.bytes = p.part_off + align_up(p.t.part_bytes, 256);
+    p.ct_bytes = align_up(p.t.part_bytes, 256);
+    p.bytes = p.part_off + p.ct_bytes;
     return p;
   }
   const long items = (long)d->r * depth(d) * d->H * cdiv(d->W, 32);
@@ -162,7 +218,8 @@ static WgradPlan plan_wgrad_core(const xconv_desc* d) {
   splits = std::min(splits, 4096L);
   p.items_per_split = cdiv(items, splits);
   p.splits = (int)cdiv(items, p.items_per_split);
-  p.bytes = p.part_off + align_up((size_t)p.splits * d->Cout * T * d->Cin * sizeof(float), 256);
+  p.ct_bytes = align_up((size_t)p.splits * d->Cout * T * d->Cin * sizeof(float), 256);
+  p.bytes = p.part_off + p.ct_bytes;
   return p;
 }
 
@@ -191,13 +248,11 @@ static SwappedWgrad plan_wgrad_swapped(const xconv_desc* d) {
   w.p1 = plan_wgrad_core(&w.d1);
   w.p2 = plan_wgrad_core(&w.d2);
   const size_t es = d->dtype == XCONV_F32 ? 4 : 2;
-  const int T = kdepth(d) * d->KH * d->KW;
   w.x_off = WS_HEADER;
   w.st_off = w.x_off + align_up((size_t)d->B * depth(d) * d->H * d->W * d->Cin * es, 256);
   w.sb_off = w.st_off + align_up((size_t)d->r * d->B * 4, 256);
   w.part_off = w.sb_off + align_up((size_t)d->r * d->B * 2, 256);
-  const size_t part = w.p2.tc_ct ? w.p2.t.part_bytes : (size_t)w.p2.splits * d->Cout * T * d->Cin * sizeof(float);
-  w.bytes = w.part_off + align_up(part, 256);
+  w.bytes = w.part_off + w.p2.ct_bytes;
   return w;
 }
 
@@ -446,10 +501,34 @@ static xconv_status run_conv_simt(const xconv_desc* d, bool dgrad, const void* i
   return check_launch();
 }
 
+// The convolution with its input channels padded (see pad8) and the scratch its copies take behind the header; the output
+// channels have to be a multiple of 8 themselves.
+static xconv_desc conv_padded(const xconv_desc* d) {
+  xconv_desc e = *d;
+  e.Cin = pad8(d->Cin);
+  return e;
+}
+static size_t conv_ws_bytes(const xconv_desc* d, bool dgrad) {
+  const xconv_desc e = conv_padded(d);
+  TcConvPlan t;
+  if (dgrad || d->Cin % 8 == 0 || !tc_plan_conv(&e, dgrad, &t)) return WS_HEADER;
+  return WS_HEADER + padded_bytes((long)d->B * depth(d) * d->H * d->W, d->Cin) +
+         padded_bytes((long)d->Cout * kdepth(d) * d->KH * d->KW, d->Cin);
+}
+
 static xconv_status run_conv(const xconv_desc* d, bool dgrad, const void* in, const void* Wt, void* out,
                              char* ws, cudaStream_t st) {
   TcConvPlan t;
-  if (tc_plan_conv(d, dgrad, &t)) return tc_run_conv(d, t, dgrad, in, Wt, out, ws, st);
+  const xconv_desc e = conv_padded(d);
+  if ((!dgrad || d->Cin % 8 == 0) && tc_plan_conv(&e, dgrad, &t)) {
+    char* copies = ws + WS_HEADER;
+    if (!dgrad) {
+      xconv_status s = pad_channels(in, (long)d->B * depth(d) * d->H * d->W, d->Cin, copies, st);
+      if (s == XCONV_OK) s = pad_channels(Wt, (long)d->Cout * kdepth(d) * d->KH * d->KW, d->Cin, copies, st);
+      if (s != XCONV_OK) return s;
+    }
+    return tc_run_conv(&e, t, dgrad, in, Wt, out, ws, st);
+  }
   return d->dtype == XCONV_F32 ? run_conv_simt<float>(d, dgrad, in, Wt, out, st)
          : d->dtype == XCONV_F16 ? run_conv_simt<f16>(d, dgrad, in, Wt, out, st)
                                  : run_conv_simt<bf16>(d, dgrad, in, Wt, out, st);
@@ -475,6 +554,16 @@ static xconv_status run_backprobe(const xconv_desc* d, const WgradPlan& p, const
 
 static xconv_status run_contract(const xconv_desc* d, const WgradPlan& p, const void* L, const void* Z,
                                  float* dW, float alpha, char* part, char* w, cudaStream_t st) {
+  if (p.halo) {
+    xconv_desc e = *d;
+    e.Cin = pad8(d->Cin); e.Cout = pad8(d->Cout);
+    const long px = (long)depth(d) * d->H * d->W * d->r;
+    char* copies = part + align_up(p.h.part_bytes, 256);
+    xconv_status s = pad_channels(Z, px, d->Cin, copies, st);
+    if (s == XCONV_OK) s = pad_channels(L, px, d->Cout, copies, st);
+    if (s != XCONV_OK) return s;
+    return tc_run_halo(&e, p.h, L, Z, d->Cout, d->Cin, dW, alpha, w, part, st);
+  }
   if (p.tc_ct) {
     const xconv_desc c = planes_ct(d);
     return tc_run_contract(&c, p.t, L, Z, dW, alpha, w, part, st);
@@ -572,11 +661,9 @@ static IndepPlan plan_indep(const xconv_desc* d) {
   ip.d2.zero_blocks = nullptr;
   ip.p2 = plan_wgrad_core(&ip.d2);
   const size_t es = d->dtype == XCONV_F32 ? 4 : 2;
-  const int T = kdepth(d) * d->KH * d->KW;
   ip.x_off = WS_HEADER;
   ip.part_off = ip.x_off + align_up((size_t)d->B * depth(d) * d->H * d->W * d->Cin * es, 256);
-  const size_t part = ip.p2.tc_ct ? ip.p2.t.part_bytes : (size_t)ip.p2.splits * d->Cout * T * d->Cin * sizeof(float);
-  ip.bytes = ip.part_off + align_up(part, 256);
+  ip.bytes = ip.part_off + ip.p2.ct_bytes;
   return ip;
 }
 
@@ -616,7 +703,7 @@ extern "C" {
 size_t xconv_workspace_bytes(const xconv_desc* desc, int op) {
   if (validate(desc) != XCONV_OK) return 0;
   switch (op) {
-    case XCONV_OP_FORWARD:
+    case XCONV_OP_FORWARD: return std::max(plan_sketch(desc).bytes, conv_ws_bytes(desc, false));
     case XCONV_OP_SKETCH: return plan_sketch(desc).bytes;
     case XCONV_OP_WGRAD_SEEDED: return plan_wgrad(desc).bytes + (wgrad_redraws(desc) ? 0 : probes_bytes(desc));
     case XCONV_OP_SKETCH_SEEDED: {
@@ -640,12 +727,16 @@ int xconv_engine_for(const xconv_desc* desc, int op) {
   switch (op) {
     case XCONV_OP_SKETCH: return plan_sketch(desc).tc ? tc : XCONV_ENGINE_SIMT_F32;
     case XCONV_OP_WGRAD:
-    case XCONV_OP_CONTRACT: return plan_wgrad(desc).tc_ct ? tc : XCONV_ENGINE_SIMT_F32;
+    case XCONV_OP_CONTRACT: {
+      const WgradPlan p = plan_wgrad(desc);
+      return p.halo || p.tc_ct ? tc : XCONV_ENGINE_SIMT_F32;
+    }
     case XCONV_OP_BACKPROBE: return plan_wgrad(desc).tc_bp ? tc : XCONV_ENGINE_SIMT_F32;
     case XCONV_OP_FORWARD:
     case XCONV_OP_DGRAD: {
       TcConvPlan t;
-      return tc_plan_conv(desc, op == XCONV_OP_DGRAD, &t) ? tc : XCONV_ENGINE_SIMT_F32;
+      const xconv_desc e = conv_padded(desc);
+      return (op == XCONV_OP_FORWARD || desc->Cin % 8 == 0) && tc_plan_conv(&e, op == XCONV_OP_DGRAD, &t) ? tc : XCONV_ENGINE_SIMT_F32;
     }
     default: return XCONV_ENGINE_NONE;
   }
@@ -811,8 +902,7 @@ xconv_status xconv_forward(const xconv_desc* desc, const void* X, const void* W,
   if (!X || !W || !Z || !Y || !sketch) return XCONV_ERR_INVALID_ARG;
   if (!aligned16(X) || !aligned16(W) || !aligned16(Z) || !aligned16(Y) || !aligned16(sketch))
     return XCONV_ERR_ALIGNMENT;
-  const SketchPlan p = plan_sketch(desc);
-  if (!ws || ws_bytes < p.bytes) return XCONV_ERR_WORKSPACE;
+  if (!ws || ws_bytes < std::max(plan_sketch(desc).bytes, conv_ws_bytes(desc, false))) return XCONV_ERR_WORKSPACE;
   if (!aligned16(ws)) return XCONV_ERR_ALIGNMENT;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   new_call();

@@ -48,6 +48,16 @@ struct TcConvPlan {
   long patches;
 };
 
+struct TcHaloPlan {            // contraction of layers with few channels (contract_tc.cu)
+  int pw, ph, stages;         // patch; stages of the ring
+  int cwa, cwb;               // channels per block of L and of Z
+  int rows_on_a;              // L moved by image rows on the MMA rows, else one dy per work unit
+  int mt, mg_n, dy_n, dz_n, dz_per, ng_n, ng_per, a_blocks, cols;
+  uint32_t a_blk, b_blk;      // shared memory of a channel block
+  long patches, splits, units;
+  size_t part_bytes;
+};
+
 // Fill the plan and say whether the tcgen05 kernels cover this layer.  tc_plan_wgrad returns a mask:
 // bit 0 = back-probe covered, bit 1 = contraction covered.
 bool tc_plan_sketch(const xconv_desc* d, TcSketchPlan* p, bool redraw = false);   // redraw: plan for a seeded call
@@ -68,6 +78,11 @@ xconv_status tc_run_backprobe(const xconv_desc* d, const TcWgradPlan& p, const v
                               void* L, char* ws_head, cudaStream_t st, const unsigned long long* seed = nullptr);
 xconv_status tc_run_contract(const xconv_desc* d, const TcWgradPlan& p, const void* L, const void* Z, float* dW,
                              float alpha, char* ws_head, char* part, cudaStream_t st);
+
+bool tc_plan_halo(const xconv_desc* d, TcHaloPlan* p);
+// `cout_out`, `cin_out`: the channels of dW where d->Cout and d->Cin count padded ones.
+xconv_status tc_run_halo(const xconv_desc* d, const TcHaloPlan& p, const void* L, const void* Z, int cout_out, int cin_out, float* dW,
+                         float alpha, char* ws_head, char* part, cudaStream_t st);
 
 xconv_status tc_run_wait_selftest(char* ws_head, unsigned long long limit_ns, cudaStream_t st);
 

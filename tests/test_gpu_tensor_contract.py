@@ -1,0 +1,62 @@
+"""The offset contraction for few channels at the edges of its tiles: patches that overhang the image, channel counts that are
+not whole blocks or not multiples of 8 (padded copies), every way the offsets are spread over the two sides of the MMA.
+Fed with an L already rounded to storage: the bar is the one of the contraction alone in test_gpu_parity.py (products of
+16-bit values are exact in float, the sums are float)."""
+import numpy as np
+import pytest
+import torch
+
+import __graft_entry__ as entry
+from oracle import xconv_oracle as O
+from paper_2106_06998_b200 import binding as xb
+from paper_2106_06998_b200 import inputs
+from tests._util import check, host
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    entry.build()
+    torch.cuda.set_device(0)
+
+
+@pytest.mark.parametrize("dtype,r,Cin,Cout,D,H,W,K,KD", [
+    ("bf16", 3, 3, 5, 1, 4, 4, 3, 1),          # one patch mostly outside the image; both channel counts padded
+    ("f16", 2, 1, 64, 1, 17, 35, 3, 1),        # one input channel; two row tiles, the second half empty
+    ("bf16", 5, 32, 32, 1, 33, 130, 3, 1),     # one MMA for nine offsets
+    ("f16", 3, 16, 32, 1, 12, 19, 5, 1),       # 25 offsets, the fifth row shift in a row tile of its own
+    ("f16", 2, 48, 24, 1, 9, 30, 5, 1),        # 320 columns: two pieces, one dy per unit, the single L block read four times
+    ("bf16", 2, 128, 128, 1, 10, 28, 3, 1),    # one dy per unit, two channel blocks on each side
+    ("f16", 4, 96, 120, 1, 7, 16, 3, 1),       # last channel blocks partly padding
+    ("bf16", 2, 16, 24, 1, 11, 21, 1, 1),      # pointwise with the rows of one shift
+    ("bf16", 2, 32, 16, 5, 6, 20, 3, 3),       # 27 offsets in one unit
+    ("f16", 2, 64, 64, 3, 8, 18, 3, 3),        # one dz per unit
+    ("bf16", 3, 24, 48, 4, 9, 9, 3, 1),        # planar kernel on the planes of a volume
+])
+def test_contraction(dtype, r, Cin, Cout, D, H, W, K, KD):
+    g = np.random.Generator(np.random.PCG64([r, Cin, Cout, H, W, K]))
+    geo = (D, H, W) if D > 1 else (H, W)
+    L, Z = (inputs.round_to_storage(g.standard_normal((r, c) + geo).astype(np.float32), dtype) for c in (Cout, Cin))
+    Ld, Zd = xb.to_device(L, dtype), xb.to_device(Z, dtype)
+    desc = xb.make_desc(8, Cin, Cout, H, W, r, Zd.dtype, K, D=D, KD=KD)
+    assert xb.engine_for(desc, xb.OP_CONTRACT) == "tcgen05_" + dtype
+    want = (O.wgrad_contract3d(L, Z, (KD, K, K)) if D > 1 else O.wgrad_contract(L, Z, K, K))
+    dW = xb.xconv_contract(Ld, Zd, kernel_size=K, kernel_depth=KD)
+    again = xb.xconv_contract(Ld, Zd, kernel_size=K, kernel_depth=KD)
+    torch.cuda.synchronize()
+    check("dW", host(dW), want, 1e-4)
+    assert torch.equal(dW, again)
+    # nothing is written behind dW, and the scale per input channel is applied to the channels it belongs to
+    scale = torch.from_numpy(g.uniform(0.5, 2.0, Cin).astype(np.float32)).cuda()
+    buf = torch.full((dW.numel() + 64,), 7.0, device="cuda")
+    ws = xb.workspace(xb.workspace_bytes(desc, xb.OP_CONTRACT), "cuda")
+    desc.chan_scale = scale.data_ptr()
+    status = xb.lib().xconv_contract(xb.ctypes.byref(desc), Ld.data_ptr(), Zd.data_ptr(), buf.data_ptr(), ws.data_ptr(), ws.numel(),
+                                     torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    assert status == 0 and bool((buf[dW.numel():] == 7.0).all())
+    taps = KD * K * K
+    got = host(buf[:dW.numel()].reshape(Cout, taps, Cin))
+    flat = want.reshape(Cout, Cin, taps).transpose(0, 2, 1) * r
+    check("dW with chan_scale", got, flat * host(scale), 1e-4)
