@@ -83,7 +83,8 @@ typedef enum { XCONV_OP_FORWARD = 0, XCONV_OP_WGRAD = 1, XCONV_OP_DGRAD = 2, XCO
                XCONV_OP_WGRAD_SEEDED = 7, XCONV_OP_WGRAD_INDEPENDENT = 8,
                XCONV_OP_SKETCH_SEEDED_GAUSSIAN = 9, XCONV_OP_WGRAD_SEEDED_GAUSSIAN = 10 } xconv_op;
 
-/* Which arithmetic engine a call will use for its dominant kernel. */
+/* Which arithmetic engine a call will use for its dominant kernel: FP32 multiply-adds or the tensor cores (by tcgen05, or
+ * by mma.sync in the kernels that stream few samples or few probes through registers), per storage type. */
 typedef enum { XCONV_ENGINE_NONE = 0, XCONV_ENGINE_SIMT_F32 = 1, XCONV_ENGINE_TCGEN05_BF16 = 2,
                XCONV_ENGINE_TCGEN05_F16 = 3 } xconv_engine;
 

@@ -100,6 +100,7 @@ static const size_t WS_HEADER = 256;   // word 0: status left by pipelined kerne
 
 struct SketchPlan {
   bool tc;
+  bool stream; StreamSketchPlan s;     // few samples or few probes (stream_tc.cu)
   int splits; long k_per_split;        // simt
   TcSketchPlan t;                      // tcgen05
   size_t part_off, bytes;
@@ -111,6 +112,11 @@ static SketchPlan plan_sketch(const xconv_desc* d_, bool seeded = false) {
   SketchPlan p{};
   const long K = (long)d->H * d->W * d->Cin;
   p.part_off = WS_HEADER;
+  p.stream = tc_plan_sketch_stream(d, seeded, &p.s);
+  if (p.stream) {
+    p.bytes = p.part_off + align_up(p.s.part_bytes, 256);
+    return p;
+  }
   p.tc = tc_plan_sketch(d, &p.t, seeded && tc_sketch_can_redraw(d));
   if (p.tc) {
     p.bytes = p.part_off + align_up(p.t.part_bytes, 256);
@@ -166,6 +172,7 @@ static xconv_status pad_channels(const void*& t, long rows, int C, char*& ws, cu
 
 struct WgradPlan {
   bool tc_bp, tc_ct;
+  bool stream_bp;                      // back-probe of few rows (stream_tc.cu)
   bool halo;                           // contraction of few channels (contract_tc.cu) instead of the one of tc_kernels.cu
   TcHaloPlan h;                        // ... on the layer with its channels padded to multiples of 8
   size_t ct_bytes;                     // scratch of the contraction: partial sums, padded copies
@@ -185,6 +192,7 @@ static WgradPlan plan_wgrad_core(const xconv_desc* d) {
   p.part_off = p.sb_off + align_up((size_t)d->r * d->B * 2, 256);
   const xconv_desc f = flat(d);
   p.tc_bp = (tc_plan_wgrad(&f, &p.tb) & 1) != 0;
+  p.stream_bp = tc_backprobe_streams(&f, p.tc_bp);
   const xconv_desc c = planes_ct(d);    // the tensor-core contraction works plane by plane
   p.tc_ct = (tc_plan_wgrad(&c, &p.t) & 2) != 0;
   // The contraction for few channels: wherever the other one does not go, and where that one leaves MMA rows empty or copies
@@ -377,6 +385,15 @@ static size_t probes_bytes(const xconv_desc* d) {
 
 // ----------------------------------------------------------------------------------- launchers
 
+static xconv_status run_reduce(const float* part, float* out, long count, int splits, float alpha, const float* chan_scale,
+                               int period, cudaStream_t st) {
+  const cudaError_t e = launch_pdl(reduce_partials, dim3((unsigned)cdiv(count, RP_OUT)), dim3(RP_OUT * RP_LANES), 0, st, part, out,
+                                   count, splits, alpha, chan_scale, period);
+  ++g_launches;
+  if (e != cudaSuccess) { g_last_cuda_error = (int)e; return XCONV_ERR_CUDA; }
+  return XCONV_OK;
+}
+
 template <typename T>
 static xconv_status run_sketch_simt(const xconv_desc* d, const SketchPlan& p, const void* X, const void* Z,
                                     float* S, char* ws, cudaStream_t st) {
@@ -395,16 +412,14 @@ static xconv_status run_sketch_simt(const xconv_desc* d, const SketchPlan& p, co
   }
   xconv_status s = check_launch();
   if (s != XCONV_OK) return s;
-  const long count = (long)d->r * d->B;
-  reduce_partials<<<(unsigned)cdiv(count, RP_OUT), RP_OUT * RP_LANES, 0, st>>>(part, S, count, p.splits, 1.0f, nullptr, 1);
-  return check_launch();
+  return run_reduce(part, S, (long)d->r * d->B, p.splits, 1.0f, nullptr, 1, st);
 }
 
 // Whether the sketch kernel of this layer redraws Z itself; otherwise the seeded call first writes Z
 // into the workspace (behind the regular scratch) and runs the regular kernels on it.
 static bool sketch_redraws(const xconv_desc* d, const SketchPlan& p) {
   const xconv_desc fl = flat(d);
-  return p.tc && tc_sketch_can_redraw(&fl);
+  return p.stream || (p.tc && tc_sketch_can_redraw(&fl));
 }
 
 static xconv_status run_sketch(const xconv_desc* d_, const void* X, const void* Z, float* S, void* ws,
@@ -421,6 +436,11 @@ static xconv_status run_sketch(const xconv_desc* d_, const void* X, const void* 
     xconv_status s = run_probes_from_seed(d, *seed, w + p.bytes, st);
     if (s != XCONV_OK) return s;
     Z = w + p.bytes;
+  }
+  if (p.stream) {
+    float* part = reinterpret_cast<float*>(w + p.part_off);
+    xconv_status s = tc_run_sketch_stream(d, p.s, X, Z, part, st, redraw ? seed : nullptr);
+    return s == XCONV_OK ? run_reduce(part, S, (long)d->r * d->B, p.s.splits, 1.0f, nullptr, 1, st) : s;
   }
   if (p.tc) return tc_run_sketch(d, p.t, X, Z, S, w, w + p.part_off, st, redraw ? seed : nullptr);
   return d->dtype == XCONV_F32 ? run_sketch_simt<float>(d, p, X, Z, S, w, st)
@@ -475,9 +495,7 @@ static xconv_status run_contract_simt(const xconv_desc* d, const WgradPlan& p, c
 #undef XC_CONTRACT
   xconv_status s = check_launch();
   if (s != XCONV_OK) return s;
-  const long count = (long)d->Cout * T9 * d->Cin;
-  reduce_partials<<<(unsigned)cdiv(count, RP_OUT), RP_OUT * RP_LANES, 0, st>>>(part, dW, count, p.splits, alpha, d->chan_scale, d->Cin);
-  return check_launch();
+  return run_reduce(part, dW, (long)d->Cout * T9 * d->Cin, p.splits, alpha, d->chan_scale, d->Cin, st);
 }
 
 template <typename T>
@@ -537,6 +555,10 @@ static xconv_status run_conv(const xconv_desc* d, bool dgrad, const void* in, co
 // L = S dY^T into `L`; `Sb` receives the bfloat16 copy of S that the tensor-core kernel reads.
 static xconv_status run_backprobe(const xconv_desc* d, const WgradPlan& p, const float* S, const void* dY,
                                   void* L, void* Sb_, char* w, cudaStream_t st, const unsigned long long* seed = nullptr) {
+  if (p.stream_bp) {
+    const xconv_desc f = flat(d);
+    return tc_run_backprobe_stream(&f, S, d->B, 1, dY, L, !p.tc_bp, st, nullptr);
+  }
   if (p.tc_bp) {
     const long n = (long)d->r * d->B;
     cudaError_t e = d->dtype == XCONV_F16
@@ -585,7 +607,7 @@ static xconv_status check_ws(void* ws, size_t ws_bytes, size_t need) {
 // probes first, r > B, with that step on the tensor cores) instead of writing them to the workspace first.
 static bool wgrad_redraws(const xconv_desc* d) {
   const SwappedWgrad sw = plan_wgrad_swapped(d);
-  return sw.on && sw.p1.tc_bp;
+  return sw.on && (sw.p1.stream_bp ? ((long)depth(d) * d->H * d->W * d->Cin) % 64 == 0 : sw.p1.tc_bp);
 }
 
 // `seed` != nullptr (only where wgrad_redraws holds): Z is not read.
@@ -600,12 +622,17 @@ static xconv_status run_wgrad(const xconv_desc* d, const float* S, const void* d
   if (sw.on) {
     // Xr = S^T Z, then the offset contraction over the batch (see plan_wgrad_swapped)
     if ((s = validate(&sw.d1)) != XCONV_OK || (s = validate(&sw.d2)) != XCONV_OK) return s;
-    float* St = reinterpret_cast<float*>(w + sw.st_off);
-    const long n = (long)d->r * d->B;
-    transpose_f32<<<(unsigned)cdiv(n, 256), 256, 0, st>>>(S, St, d->r, d->B);
-    s = check_launch();
-    if (s != XCONV_OK) return s;
-    s = run_backprobe(&sw.d1, sw.p1, St, Z, w + sw.x_off, w + sw.sb_off, w, st, seed);
+    if (sw.p1.stream_bp) {                 // reads S by its columns itself
+      const xconv_desc f = flat(&sw.d1);
+      s = tc_run_backprobe_stream(&f, S, 1, d->B, Z, w + sw.x_off, !sw.p1.tc_bp, st, seed);
+    } else {
+      float* St = reinterpret_cast<float*>(w + sw.st_off);
+      const long n = (long)d->r * d->B;
+      transpose_f32<<<(unsigned)cdiv(n, 256), 256, 0, st>>>(S, St, d->r, d->B);
+      s = check_launch();
+      if (s != XCONV_OK) return s;
+      s = run_backprobe(&sw.d1, sw.p1, St, Z, w + sw.x_off, w + sw.sb_off, w, st, seed);
+    }
     if (s != XCONV_OK) return s;
     return run_contract(&sw.d2, sw.p2, dY, w + sw.x_off, dW, alpha, w + sw.part_off, w, st);
   }
@@ -725,13 +752,19 @@ int xconv_engine_for(const xconv_desc* desc, int op) {
   if (validate(desc) != XCONV_OK) return XCONV_ENGINE_NONE;
   const int tc = desc->dtype == XCONV_F16 ? XCONV_ENGINE_TCGEN05_F16 : XCONV_ENGINE_TCGEN05_BF16;
   switch (op) {
-    case XCONV_OP_SKETCH: return plan_sketch(desc).tc ? tc : XCONV_ENGINE_SIMT_F32;
+    case XCONV_OP_SKETCH: {
+      const SketchPlan p = plan_sketch(desc);
+      return p.stream || p.tc ? tc : XCONV_ENGINE_SIMT_F32;
+    }
     case XCONV_OP_WGRAD:
     case XCONV_OP_CONTRACT: {
       const WgradPlan p = plan_wgrad(desc);
       return p.halo || p.tc_ct ? tc : XCONV_ENGINE_SIMT_F32;
     }
-    case XCONV_OP_BACKPROBE: return plan_wgrad(desc).tc_bp ? tc : XCONV_ENGINE_SIMT_F32;
+    case XCONV_OP_BACKPROBE: {
+      const WgradPlan p = plan_wgrad(desc);
+      return p.stream_bp || p.tc_bp ? tc : XCONV_ENGINE_SIMT_F32;
+    }
     case XCONV_OP_FORWARD:
     case XCONV_OP_DGRAD: {
       TcConvPlan t;

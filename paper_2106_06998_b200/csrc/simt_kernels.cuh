@@ -178,6 +178,8 @@ static __global__ void __launch_bounds__(RP_OUT * RP_LANES)
 reduce_partials(const float* __restrict__ part, float* __restrict__ out, long count, int splits, float alpha,
                 const float* __restrict__ chan_scale, int period) {
   __shared__ float acc[RP_LANES][RP_OUT];
+  pdl_trigger();
+  pdl_wait();
   const int o = threadIdx.x % RP_OUT, g = threadIdx.x / RP_OUT;
   const long i = (long)blockIdx.x * RP_OUT + o;
   float s = 0.f;

@@ -1,0 +1,489 @@
+// Sketch and back-probe of layers with few samples or few probes, 16-bit storage: kernels that stream one large operand
+// from memory through registers.
+//
+// A row of the small side (16 samples, say) leaves the tcgen05 kernels one narrow MMA per 128-byte row piece, and their
+// time goes with the hand-shakes of a CTA's roles per tile, a multiple of the time the bytes take.  These kernels have no
+// roles, no stages and no barriers: every warp loads its operands straight into the fragments of mma.sync (16 x 8 x 16, float
+// accumulators), whose rate -- far below tcgen05's, far above what is needed at 16 multiply-adds per byte -- is not
+// what bounds them.  Two facts make the fragments free:
+//  - the order of the reduction index is ours, as long as both operands use the same: a thread's fragments of two k-steps
+//    are then 16 consecutive bytes of a row (sketch);
+//  - the order of the columns is ours too: a thread that holds 8 neighbouring columns of two rows pairs them into the B
+//    fragments of 8 column tiles with one byte permutation each, and its accumulators are 16 neighbouring columns of the
+//    result (back-probe).
+// Probing vectors redrawn from a seed are drawn into the fragments: a fragment register is two sign bits of a Philox word
+// moved to bits 15 and 31, two instructions.
+#include "common.cuh"
+#include "tc_api.h"
+
+#include <algorithm>
+
+namespace xconv {
+
+template <bool F16>
+__device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  if (F16)
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+  else
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint4 ldg_stream(const void* p) {
+  uint4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint32_t word(const uint4& v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
+template <bool F16>
+__device__ __forceinline__ unsigned short to16(float v) {
+  if (F16) { const __half h = __float2half_rn(v); return *reinterpret_cast<const unsigned short*>(&h); }
+  const __nv_bfloat16 h = __float2bfloat16_rn(v);
+  return *reinterpret_cast<const unsigned short*>(&h);
+}
+template <bool F16>
+__device__ __forceinline__ float from16(unsigned short v) {
+  if (F16) return __half2float(__ushort_as_half(v));
+  return __uint_as_float((uint32_t)v << 16);
+}
+template <bool F16>
+__device__ __forceinline__ uint32_t pack16(float a, float b) { return (uint32_t)to16<F16>(a) | ((uint32_t)to16<F16>(b) << 16); }
+
+// The 128 sign bits of entries e0 .. e0+127 of Z (e0 a multiple of 64, `whole`: of 128).
+__device__ __forceinline__ uint4 sign_bits128(unsigned long long e0, bool whole, uint32_t k0, uint32_t k1) {
+  const unsigned long long b = e0 >> 7;
+  uint4 w = philox4x32_10((uint32_t)b, (uint32_t)(b >> 32), k0, k1);
+  if (!whole && (e0 & 64)) {                          // the second half of this block, the first of the next
+    const uint4 v = philox4x32_10((uint32_t)(b + 1), (uint32_t)((b + 1) >> 32), k0, k1);
+    w = make_uint4(w.z, w.w, v.x, v.y);
+  }
+  return w;
+}
+
+// ------------------------------------------------------------------------------------ sketch
+
+// part[split][m][n] (or [n][m] if `swap`) = sum over this block's k of A[m,k] Bm[n,k]: 16 MT rows of A per block, up to
+// 8 NT rows of Bm.  The blocks take the pieces of the k axis in turn and the eight warps the k-steps of a piece, so that at
+// any time the GPU reads neighbouring bytes of every row; the warps' tiles are added in warp order.
+struct SketchStream {
+  const uint16_t *A, *Bm;
+  float* part;
+  int M, N, swap;
+  long K;
+  uint32_t seed_lo, seed_hi;
+};
+
+template <bool F16, int MT, int NT, bool SEEDED>
+__global__ void __launch_bounds__(256, 2) sketch_stream_kernel(const SketchStream p) {
+  __shared__ float red[8][16 * 8 + 1];
+  __shared__ uint4 bits[SEEDED ? 8 : 1][SEEDED ? 16 * MT : 1];
+  pdl_trigger();
+  pdl_wait();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int m0 = blockIdx.y * 16 * MT;
+  float acc[MT][NT][4];
+#pragma unroll
+  for (int i = 0; i < MT; ++i)
+#pragma unroll
+    for (int j = 0; j < NT; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.f;
+  const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+
+  if (!SEEDED) {
+    // k-step of 32: thread (g, t) holds k = 8t .. 8t+7 of its rows, the pairs in order
+    constexpr int U = MT * 2 + NT <= 3 ? 4 : MT * 2 + NT <= 6 ? 2 : 1;       // k-steps whose loads are in flight together
+    const uint16_t* arow = p.A + (long)(m0 + g) * p.K + 8 * t;
+    const uint16_t* brow = p.Bm + (long)g * p.K + 8 * t;
+    for (long k0 = (long)blockIdx.x * 256 * U + warp * 32; k0 < p.K; k0 += (long)gridDim.x * 256 * U) {
+      uint4 a[U][MT][2], b[U][NT];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const long k = k0 + 256 * u;
+        const bool in = k + 8 * t < p.K;                                    // (K is a multiple of 8)
+#pragma unroll
+        for (int i = 0; i < MT; ++i)
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            a[u][i][h] = in && m0 + 16 * i + 8 * h + g < p.M ? ldg_stream(arow + (long)(16 * i + 8 * h) * p.K + k) : zero;
+#pragma unroll
+        for (int j = 0; j < NT; ++j) b[u][j] = in && 8 * j + g < p.N ? ldg_stream(brow + (long)(8 * j) * p.K + k) : zero;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int i = 0; i < MT; ++i) {
+          const uint4 lo = a[u][i][0], hi = a[u][i][1];
+          const uint32_t f0[4] = {lo.x, hi.x, lo.y, hi.y}, f1[4] = {lo.z, hi.z, lo.w, hi.w};
+#pragma unroll
+          for (int j = 0; j < NT; ++j) {
+            mma16816<F16>(acc[i][j], f0, b[u][j].x, b[u][j].y);
+            mma16816<F16>(acc[i][j], f1, b[u][j].z, b[u][j].w);
+          }
+        }
+    }
+  } else {
+    // A = the signs of the seed.  128 k at a time: each lane draws one row's 128 signs (MT / 2 of them), the rows' words go
+    // through shared memory.  In a step of 32 k (one word) the pairs are (s, s + 16), s = 4t .. 4t+3.
+    const uint32_t ones = F16 ? 0x3C003C00u : 0x3F803F80u;
+    const bool whole = (p.K & 127) == 0;
+    const uint16_t* brow = p.Bm + (long)g * p.K + 4 * t;
+    for (long k0 = (long)blockIdx.x * 1024 + warp * 128; k0 < p.K; k0 += (long)gridDim.x * 1024) {
+      uint2 x[4][NT][2];
+#pragma unroll
+      for (int w = 0; w < 4; ++w)
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            x[w][j][h] = k0 + 32 * w < p.K && 8 * j + g < p.N                // (K is a multiple of 64)
+                             ? *reinterpret_cast<const uint2*>(brow + (long)(8 * j) * p.K + k0 + 32 * w + 16 * h) : make_uint2(0u, 0u);
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < (16 * MT + 31) / 32; ++i) {
+        const int row = 32 * i + lane;
+        if (row < 16 * MT)
+          bits[warp][row] = sign_bits128((unsigned long long)(m0 + row) * (unsigned long long)p.K + (unsigned long long)k0, whole,
+                                         p.seed_lo, p.seed_hi);
+      }
+      __syncwarp();
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        uint32_t b[NT][4];
+#pragma unroll
+        for (int j = 0; j < NT; ++j) {
+          const uint2 lo = x[w][j][0], hi = x[w][j][1];
+          b[j][0] = __byte_perm(lo.x, hi.x, 0x5410); b[j][1] = __byte_perm(lo.x, hi.x, 0x7632);
+          b[j][2] = __byte_perm(lo.y, hi.y, 0x5410); b[j][3] = __byte_perm(lo.y, hi.y, 0x7632);
+        }
+#pragma unroll
+        for (int i = 0; i < MT; ++i) {
+          const uint32_t w0 = reinterpret_cast<const uint32_t*>(&bits[warp][16 * i + g])[w] << (12 - 4 * t);
+          const uint32_t w1 = reinterpret_cast<const uint32_t*>(&bits[warp][16 * i + 8 + g])[w] << (12 - 4 * t);
+          const uint32_t f0[4] = {((w0 << 3) & 0x80008000u) ^ ones, ((w1 << 3) & 0x80008000u) ^ ones,
+                                  ((w0 << 2) & 0x80008000u) ^ ones, ((w1 << 2) & 0x80008000u) ^ ones};
+          const uint32_t f1[4] = {((w0 << 1) & 0x80008000u) ^ ones, ((w1 << 1) & 0x80008000u) ^ ones,
+                                  (w0 & 0x80008000u) ^ ones, (w1 & 0x80008000u) ^ ones};
+#pragma unroll
+          for (int j = 0; j < NT; ++j) {
+            mma16816<F16>(acc[i][j], f0, b[j][0], b[j][1]);
+            mma16816<F16>(acc[i][j], f1, b[j][2], b[j][3]);
+          }
+        }
+      }
+    }
+  }
+  // the warps' tiles, 16 x 8 at a time
+  float* out = p.part + (long)blockIdx.x * p.M * p.N;
+#pragma unroll
+  for (int i = 0; i < MT; ++i)
+#pragma unroll
+    for (int j = 0; j < NT; ++j) {
+      __syncthreads();
+#pragma unroll
+      for (int e = 0; e < 4; ++e) red[warp][(g + 8 * (e >> 1)) * 8 + 2 * t + (e & 1)] = acc[i][j][e];
+      __syncthreads();
+      if (threadIdx.x < 128) {
+        float s = red[0][threadIdx.x];
+#pragma unroll
+        for (int w = 1; w < 8; ++w) s += red[w][threadIdx.x];
+        const int m = m0 + 16 * i + (int)threadIdx.x / 8, n = 8 * j + (int)threadIdx.x % 8;
+        if (m < p.M && n < p.N) out[p.swap ? (long)n * p.M + m : (long)m * p.N + n] = s;
+      }
+    }
+}
+
+// ------------------------------------------------------------------------------------ back-probe
+
+// L[row][q] = sum over k of S(row, k) * Y[k][q], rounded to storage: up to 16 MT rows, a warp owns 64 columns.  S(row, k) =
+// S[row * s_row + k * s_k] (float, rounded to storage in shared memory, so that neither a transposed nor a 16-bit copy of it
+// is written).  SEEDED: Y = the signs of the seed.
+struct BackprobeStream {
+  const float* S;
+  long s_row, s_k;
+  const uint16_t* Y;
+  uint16_t* L;
+  int rows, K, K16, ld;                               // K16: K rounded up to 64; ld: row pitch of S in shared memory
+  long Q, groups;                                     // groups of 64 columns
+  uint32_t seed_lo, seed_hi;
+};
+
+// SPLIT: S as the sum of two 16-bit values (16 bits of it in bfloat16; 22 in float16, where every row is scaled by a power of two
+// into the range first), multiplied one after the other: for the layers whose sums used the float S all along (what it is
+// rounded to shows in the result: relative error against 64 bits 1.7e-3 with the float S or with two values, 2.4e-3 with one).
+// KC: k-steps of 16 that are loaded together.  ALL: they are the whole reduction; a warp then takes 4 / KC groups of
+// columns at a time, so that as many bytes are in flight as with a long reduction.  Otherwise the loads of the next
+// KC k-steps (of the next group behind the last) are under way while these are multiplied.
+template <bool F16, int MT, bool SEEDED, int KC, bool ALL, bool SPLIT>
+__global__ void __launch_bounds__(256, MT >= 4 ? 1 : 2) backprobe_stream_kernel(const BackprobeStream p) {
+  extern __shared__ __align__(16) uint16_t s16[];     // [16 MT][ld], then (SEEDED) 8 warps x 32 rows x 8 bytes of signs
+  pdl_trigger();
+  pdl_wait();
+  __shared__ float unscale[SPLIT ? 16 * MT : 1];      // SPLIT: what the row's sums are multiplied by
+  uint16_t* s16lo = s16 + 16 * MT * p.ld;             // SPLIT: the second values
+  if (SPLIT) {
+    for (int row = threadIdx.x >> 5; row < 16 * MT; row += 8) {
+      const bool live = row < p.rows;
+      float up = 1.0f, down = 1.0f;
+      if (F16) {
+        float most = 0.f;
+        if (live)
+          for (int k = threadIdx.x & 31; k < p.K; k += 32) {
+            const float a = fabsf(p.S[row * p.s_row + k * p.s_k]);
+            if (a < __int_as_float(0x7F800000)) most = fmaxf(most, a);
+          }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, o));
+        const int e = most > 0.f ? min(126, max(-126, 14 - ilogbf(most))) : 0;
+        up = __int_as_float((127 + e) << 23);
+        down = __int_as_float((127 - e) << 23);
+      }
+      for (int k = threadIdx.x & 31; k < p.K16; k += 32) {
+        const float v = live && k < p.K ? p.S[row * p.s_row + k * p.s_k] * up : 0.f;
+        const uint16_t hi = to16<F16>(v);
+        const float h = from16<F16>(hi);
+        s16[row * p.ld + k] = hi;
+        s16lo[row * p.ld + k] = fabsf(h) < __int_as_float(0x7F800000) ? to16<F16>(v - h) : (uint16_t)0;
+      }
+      if ((threadIdx.x & 31) == 0) unscale[row] = down;
+    }
+  } else {
+    for (int i = threadIdx.x; i < 16 * MT * p.K16; i += 256) {
+      const int row = p.s_k == 1 ? i / p.K16 : i % (16 * MT), k = p.s_k == 1 ? i % p.K16 : i / (16 * MT);
+      s16[row * p.ld + k] = row < p.rows && k < p.K ? to16<F16>(p.S[row * p.s_row + k * p.s_k]) : (uint16_t)0;
+    }
+  }
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const uint32_t ones = F16 ? 0x3C003C00u : 0x3F803F80u;
+  uint2* bits = reinterpret_cast<uint2*>(s16 + (SPLIT ? 2 : 1) * 16 * MT * p.ld) + warp * 32;
+  constexpr int GB = ALL ? 4 / KC : 1, VB = ALL ? GB : 2;
+  const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+  float acc[MT][8][4];
+  uint4 v[VB][KC][4];
+  auto fetch = [&](int gb, long grp, int k0) {        // rows 2t, 2t+1, 2t+8, 2t+9 of every k-step, 8 columns of each
+    const long q = grp * 64 + 8 * g;
+#pragma unroll
+    for (int u = 0; u < KC; ++u)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int k = k0 + 16 * u + 2 * t + (r & 1) + 8 * (r >> 1);
+        v[gb][u][r] = k < p.K && q < p.Q ? ldg_stream(p.Y + (long)k * p.Q + q) : zero;
+      }
+  };
+  auto draw = [&](long grp, int k0) {                 // the signs of 32 rows, one row's 64 bits per lane (half a Philox block)
+    __syncwarp();
+    const unsigned long long e0 = (unsigned long long)(k0 + lane) * (unsigned long long)p.Q + (unsigned long long)(grp * 64);
+    const unsigned long long blk = e0 >> 7;
+    const uint4 w = philox4x32_10((uint32_t)blk, (uint32_t)(blk >> 32), p.seed_lo, p.seed_hi);
+    bits[lane] = (e0 & 64) ? make_uint2(w.z, w.w) : make_uint2(w.x, w.y);
+    __syncwarp();
+  };
+  auto multiply = [&](int gb, int k0) {
+#pragma unroll
+    for (int u = 0; u < KC; ++u) {
+      uint32_t a[SPLIT ? 2 * MT : MT][4];
+#pragma unroll
+      for (int i = 0; i < (SPLIT ? 2 * MT : MT); ++i) {
+        const uint16_t* s = s16 + (16 * i + g) * p.ld + k0 + 16 * u + 2 * t;      // (the second values follow the first)
+        a[i][0] = *reinterpret_cast<const uint32_t*>(s);
+        a[i][1] = *reinterpret_cast<const uint32_t*>(s + 8 * p.ld);
+        a[i][2] = *reinterpret_cast<const uint32_t*>(s + 8);
+        a[i][3] = *reinterpret_cast<const uint32_t*>(s + 8 * p.ld + 8);
+      }
+      uint32_t x0 = 0, x1 = 0;                        // SEEDED: eight signs of the two rows of a pair, at bits 0 and 16
+      if (SEEDED) {
+        const uint8_t* sb = reinterpret_cast<const uint8_t*>(bits) + (16 * u + 2 * t) * 8 + g;
+        x0 = (uint32_t)sb[0] | ((uint32_t)sb[8] << 16);
+        x1 = (uint32_t)sb[64] | ((uint32_t)sb[72] << 16);
+      }
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {                   // column 8 g + c is column g of tile c
+        uint32_t b0, b1;
+        if (SEEDED) {
+          b0 = ((x0 << (15 - c)) & 0x80008000u) ^ ones;
+          b1 = ((x1 << (15 - c)) & 0x80008000u) ^ ones;
+        } else {
+          b0 = __byte_perm(word(v[gb][u][0], c >> 1), word(v[gb][u][1], c >> 1), (c & 1) ? 0x7632 : 0x5410);
+          b1 = __byte_perm(word(v[gb][u][2], c >> 1), word(v[gb][u][3], c >> 1), (c & 1) ? 0x7632 : 0x5410);
+        }
+#pragma unroll
+        for (int i = 0; i < MT; ++i) {
+          mma16816<F16>(acc[i][c], a[i], b0, b1);
+          if (SPLIT) mma16816<F16>(acc[i][c], a[MT + i], b0, b1);
+        }
+      }
+    }
+  };
+  if (!ALL && !SEEDED) fetch(0, (long)blockIdx.x * 8 + warp, 0);
+  for (long grp0 = ((long)blockIdx.x * 8 + warp) * GB; grp0 < p.groups; grp0 += (long)gridDim.x * 8 * GB) {
+    if (ALL && !SEEDED)
+#pragma unroll
+      for (int gb = 0; gb < GB; ++gb) fetch(gb, grp0 + gb, 0);
+#pragma unroll
+    for (int gb = 0; gb < GB; ++gb) {
+      const long grp = grp0 + gb;
+      if (grp >= p.groups) break;
+#pragma unroll
+      for (int i = 0; i < MT; ++i)
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) acc[i][c][e] = 0.f;
+      if (ALL) {
+        multiply(gb, 0);
+      } else {
+        for (int k0 = 0; k0 < p.K16; k0 += 32 * KC) {       // (K16 is a multiple of 64)
+          if (SEEDED) draw(grp, k0);
+          else fetch(1, grp, k0 + 16 * KC);
+          multiply(0, k0);
+          const bool last = k0 + 32 * KC >= p.K16;
+          if (SEEDED) draw(grp, k0 + 16 * KC);
+          else fetch(0, last ? grp + (long)gridDim.x * 8 : grp, last ? 0 : k0 + 32 * KC);
+          multiply(1, k0 + 16 * KC);
+        }
+      }
+      // accumulator columns 2t and 2t+1 of tile c are the columns 16 t + c and 16 t + 8 + c
+      const long qo = grp * 64 + 16 * t;
+#pragma unroll
+      for (int i = 0; i < MT; ++i)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int row = 16 * i + 8 * h + g;
+          if (row >= p.rows) continue;
+          if (SPLIT && F16) {
+            const float d = unscale[row];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) { acc[i][c][2 * h] *= d; acc[i][c][2 * h + 1] *= d; }
+          }
+#pragma unroll
+          for (int s = 0; s < 2; ++s) {
+            if (qo + 8 * s >= p.Q) continue;
+            uint4 o;
+            o.x = pack16<F16>(acc[i][0][2 * h + s], acc[i][1][2 * h + s]); o.y = pack16<F16>(acc[i][2][2 * h + s], acc[i][3][2 * h + s]);
+            o.z = pack16<F16>(acc[i][4][2 * h + s], acc[i][5][2 * h + s]); o.w = pack16<F16>(acc[i][6][2 * h + s], acc[i][7][2 * h + s]);
+            *reinterpret_cast<uint4*>(p.L + (long)row * p.Q + qo + 8 * s) = o;
+          }
+        }
+    }
+  }
+}
+
+// ------------------------------------------------------------------------------------ host side
+
+static long cdiv_(long a, long b) { return (a + b - 1) / b; }
+
+// Measured against the tcgen05 sketch, other -> this, us: 8 x 4 (probes x samples), 3.5 M terms 178 -> 22; 16 x 64, 200704
+// terms 13.3 -> 11.5; 512 x 8, 65536 terms 14.5 -> 10.0; 128 x 16, 262144 terms 16.3 -> 15.8; but 64 x 16, 2.1 M terms 76 -> 113
+// (a load instruction touches eight rows, and many rows far apart cost it more than the bytes do): more than 32 rows only
+// up to 131072 terms.  Redrawn from the seed only the few samples are read: 64 x 16 64 -> 31, 256 x 16 190 -> 90.
+bool tc_plan_sketch_stream(const xconv_desc* d, bool seeded, StreamSketchPlan* p) {
+  if (d->dtype != XCONV_BF16 && d->dtype != XCONV_F16) return false;
+  const long K = (long)d->H * d->W * d->Cin;
+  if (K % 8 != 0 || K < 2048 || std::min(d->r, d->B) > 16) return false;
+  if (seeded && (d->B > 16 || K % 64 != 0)) return false;            // the signs are drawn on the row side
+  p->swap = d->B <= d->r || seeded ? 0 : 1;                          // 0: rows = probes
+  if (!p->swap && d->B > 16) return false;
+  const int M = p->swap ? d->B : d->r, N = p->swap ? d->r : d->B;
+  if (!seeded && M > 32 && K > 131072) return false;
+  p->mt = seeded || M > 32 ? 4 : M > 16 ? 2 : 1;
+  p->nt = N > 8 ? 2 : 1;
+  p->tiles_m = (int)cdiv_(M, 16 * p->mt);
+  // two blocks per SM, and at least one k-step of 32 per warp and block
+  const long splits = std::max(1L, std::min(cdiv_(2L * 148, p->tiles_m), cdiv_(K, seeded ? 1024 : 256)));
+  p->splits = (int)splits;
+  p->part_bytes = (size_t)p->splits * d->r * d->B * sizeof(float);
+  return true;
+}
+
+template <bool F16>
+static cudaError_t launch_sketch_stream(const StreamSketchPlan& pl, bool seeded, const SketchStream& q, cudaStream_t st) {
+  const dim3 grid((unsigned)pl.splits, (unsigned)pl.tiles_m), block(256);
+  if (seeded) return pl.nt == 2 ? launch_pdl(sketch_stream_kernel<F16, 4, 2, true>, grid, block, 0, st, q)
+                                : launch_pdl(sketch_stream_kernel<F16, 4, 1, true>, grid, block, 0, st, q);
+  if (pl.mt == 4) return pl.nt == 2 ? launch_pdl(sketch_stream_kernel<F16, 4, 2, false>, grid, block, 0, st, q)
+                                    : launch_pdl(sketch_stream_kernel<F16, 4, 1, false>, grid, block, 0, st, q);
+  if (pl.mt == 2) return pl.nt == 2 ? launch_pdl(sketch_stream_kernel<F16, 2, 2, false>, grid, block, 0, st, q)
+                                    : launch_pdl(sketch_stream_kernel<F16, 2, 1, false>, grid, block, 0, st, q);
+  return pl.nt == 2 ? launch_pdl(sketch_stream_kernel<F16, 1, 2, false>, grid, block, 0, st, q)
+                    : launch_pdl(sketch_stream_kernel<F16, 1, 1, false>, grid, block, 0, st, q);
+}
+
+xconv_status tc_run_sketch_stream(const xconv_desc* d, const StreamSketchPlan& pl, const void* X, const void* Z, float* part,
+                                  cudaStream_t st, const unsigned long long* seed) {
+  SketchStream q{};
+  q.A = static_cast<const uint16_t*>(pl.swap ? X : Z);
+  q.Bm = static_cast<const uint16_t*>(pl.swap ? Z : X);
+  q.part = part;
+  q.M = pl.swap ? d->B : d->r;
+  q.N = pl.swap ? d->r : d->B;
+  q.swap = pl.swap;
+  q.K = (long)d->H * d->W * d->Cin;
+  if (seed) { q.seed_lo = (uint32_t)(*seed & 0xFFFFFFFFull); q.seed_hi = (uint32_t)(*seed >> 32); }
+  const cudaError_t e = d->dtype == XCONV_F16 ? launch_sketch_stream<true>(pl, seed != nullptr, q, st)
+                                              : launch_sketch_stream<false>(pl, seed != nullptr, q, st);
+  count_launch();
+  if (e != cudaSuccess) { set_cuda_error((int)e); return XCONV_ERR_CUDA; }
+  return XCONV_OK;
+}
+
+static int stream_k(int K) { return (int)(cdiv_(K, 64) * 64); }
+static size_t stream_smem(int mt, int K, bool seeded, bool split) {
+  return (size_t)(16 * mt) * (stream_k(K) + 8) * (split ? 4 : 2) + (seeded ? 8 * 32 * 8 : 0);
+}
+
+// `other`: the tcgen05 back-probe serves the layer.  Up to 16 rows this one is faster where every warp has two groups of columns
+// or the reduction is short; measured, other -> this, us: 4 rows, 8 terms, 3.5 M columns 76 -> 21; 16 rows, 64 terms, 2.1 M
+// columns 76 -> 62, 256 terms 269 -> 192; but 8 rows, 512 terms, 65536 columns 14.5 -> 24; 32 rows, 128 terms, 200704 columns
+// 15 -> 20; 64 rows, 128 terms, 802816 columns 56 -> 88 (mma.sync holds its pipe for some 20 clocks or more, whatever feeds it).
+// Where the choice is between this and the FP32-FMA kernel: 50 rows, 50 terms, 153760 columns 61 -> 16.
+bool tc_backprobe_streams(const xconv_desc* d, bool other) {
+  if (d->dtype != XCONV_BF16 && d->dtype != XCONV_F16) return false;
+  const long Q = (long)d->H * d->W * d->Cout;
+  if (Q % 8 != 0 || Q < 2048 || d->r > 64 || stream_smem(d->r > 32 ? 4 : d->r > 16 ? 2 : 1, d->B, true, !other) > 96 * 1024) return false;
+  return !other || (d->r <= 16 && (d->B <= 64 || Q >= 2L * 64 * 16 * 148));
+}
+
+template <bool F16, int MT>
+static cudaError_t launch_backprobe_stream(const BackprobeStream& q, bool seeded, bool split, unsigned grid, size_t smem, cudaStream_t st) {
+  constexpr int KC = MT == 1 ? 2 : 1;
+  void (*kernel)(BackprobeStream);
+  if (split) kernel = seeded ? backprobe_stream_kernel<F16, MT, true, 2, false, true> : backprobe_stream_kernel<F16, MT, false, KC, false, true>;
+  else if (MT > 1) return cudaErrorInvalidValue;      // (one value per entry of S: up to 16 rows only)
+  else
+    kernel = seeded ? backprobe_stream_kernel<F16, 1, true, 2, false, false>
+             : q.K <= 16 ? backprobe_stream_kernel<F16, 1, false, 1, true, false>
+             : q.K <= 32 ? backprobe_stream_kernel<F16, 1, false, 2, true, false>
+             : q.K <= 64 ? backprobe_stream_kernel<F16, 1, false, 4, true, false> : backprobe_stream_kernel<F16, 1, false, 2, false, false>;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+  return e != cudaSuccess ? e : launch_pdl(kernel, dim3(grid), dim3(256), smem, st, q);
+}
+
+xconv_status tc_run_backprobe_stream(const xconv_desc* d, const float* S, long s_row, long s_k, const void* dY, void* L,
+                                     bool split, cudaStream_t st, const unsigned long long* seed) {
+  BackprobeStream q{};
+  q.S = S; q.s_row = s_row; q.s_k = s_k;
+  q.Y = static_cast<const uint16_t*>(dY);
+  q.L = static_cast<uint16_t*>(L);
+  q.rows = d->r; q.K = d->B; q.K16 = stream_k(d->B); q.ld = q.K16 + 8;
+  q.Q = (long)d->H * d->W * d->Cout;
+  q.groups = cdiv_(q.Q, 64);
+  if (seed) { q.seed_lo = (uint32_t)(*seed & 0xFFFFFFFFull); q.seed_hi = (uint32_t)(*seed >> 32); }
+  const int mt = d->r > 32 ? 4 : d->r > 16 ? 2 : 1;
+  const unsigned grid = (unsigned)std::min<long>(cdiv_(q.groups, 8), 148L * (mt == 4 ? 1 : 2));
+  const size_t smem = stream_smem(mt, d->B, seed != nullptr, split);
+  cudaError_t e;
+  if (d->dtype == XCONV_F16)
+    e = mt == 4 ? launch_backprobe_stream<true, 4>(q, seed != nullptr, split, grid, smem, st)
+        : mt == 2 ? launch_backprobe_stream<true, 2>(q, seed != nullptr, split, grid, smem, st)
+                  : launch_backprobe_stream<true, 1>(q, seed != nullptr, split, grid, smem, st);
+  else
+    e = mt == 4 ? launch_backprobe_stream<false, 4>(q, seed != nullptr, split, grid, smem, st)
+        : mt == 2 ? launch_backprobe_stream<false, 2>(q, seed != nullptr, split, grid, smem, st)
+                  : launch_backprobe_stream<false, 1>(q, seed != nullptr, split, grid, smem, st);
+  count_launch();
+  if (e != cudaSuccess) { set_cuda_error((int)e); return XCONV_ERR_CUDA; }
+  return XCONV_OK;
+}
+
+}  // namespace xconv

@@ -58,6 +58,12 @@ struct TcHaloPlan {            // contraction of layers with few channels (contr
   size_t part_bytes;
 };
 
+struct StreamSketchPlan {      // sketch with at most 16 samples or 16 probes (stream_tc.cu)
+  int swap;                   // 0: MMA rows = probes, columns = samples; 1: rows = samples
+  int mt, nt, tiles_m, splits;
+  size_t part_bytes;          // [split][r][B] float
+};
+
 // Fill the plan and say whether the tcgen05 kernels cover this layer.  tc_plan_wgrad returns a mask:
 // bit 0 = back-probe covered, bit 1 = contraction covered.
 bool tc_plan_sketch(const xconv_desc* d, TcSketchPlan* p, bool redraw = false);   // redraw: plan for a seeded call
@@ -83,6 +89,17 @@ bool tc_plan_halo(const xconv_desc* d, TcHaloPlan* p);
 // `cout_out`, `cin_out`: the channels of dW where d->Cout and d->Cin count padded ones.
 xconv_status tc_run_halo(const xconv_desc* d, const TcHaloPlan& p, const void* L, const void* Z, int cout_out, int cin_out, float* dW,
                          float alpha, char* ws_head, char* part, cudaStream_t st);
+
+// The streaming kernels for few samples or few probes.  The sketch leaves its partial sums in `part`; the back-probe takes
+// S(row, k) = S[row * s_row + k * s_k], rows = d->r, reduction = d->B, and redraws its streamed operand if `seed` is given
+// (H*W*Cout a multiple of 64 then).
+bool tc_plan_sketch_stream(const xconv_desc* d, bool seeded, StreamSketchPlan* p);
+xconv_status tc_run_sketch_stream(const xconv_desc* d, const StreamSketchPlan& p, const void* X, const void* Z, float* part,
+                                  cudaStream_t st, const unsigned long long* seed);
+bool tc_backprobe_streams(const xconv_desc* d, bool other);
+// (`split`: S with more than its 16-bit rounding, see the kernel.)
+xconv_status tc_run_backprobe_stream(const xconv_desc* d, const float* S, long s_row, long s_k, const void* dY, void* L,
+                                     bool split, cudaStream_t st, const unsigned long long* seed);
 
 xconv_status tc_run_wait_selftest(char* ws_head, unsigned long long limit_ns, cudaStream_t st);
 
