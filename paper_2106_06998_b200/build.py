@@ -8,7 +8,7 @@ import subprocess
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libxconv.so")
-SOURCES = ["api.cu", "tc_kernels.cu", "conv_tc.cu", "contract_tc.cu", "stream_tc.cu", "static_scratch.cu"]
+SOURCES = ["api.cu", "tc_kernels.cu", "conv_tc.cu", "contract_tc.cu", "stream_tc.cu", "conv_fma.cu", "static_scratch.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "--use_fast_math=false", "-Xcompiler", "-fPIC,-O2", "-cudart", "static"]
 
@@ -33,15 +33,18 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     ``extra_flags`` go to nvcc."""
     if not force and not _stale():
         return LIB
-    objs = []
+    objs, jobs = [], []
     for src in SOURCES:
         obj = os.path.join(CSRC, src.replace(".cu", ".o"))
         cmd = [_nvcc(), *[f for f in NVCC_FLAGS if f != "--use_fast_math=false"], *extra_flags, "-c",
                os.path.join(CSRC, src), "-o", obj]
         if verbose:
             cmd.insert(1, "-Xptxas=-v")
-        subprocess.run(cmd, check=True)
+        jobs.append((cmd, subprocess.Popen(cmd)))
         objs.append(obj)
+    for cmd, job in jobs:                       # the sources compile side by side
+        if job.wait() != 0:
+            raise subprocess.CalledProcessError(job.returncode, cmd)
     subprocess.run([_nvcc(), "-shared", "-cudart", "static", "-o", LIB, *objs, "-ldl"], check=True)
     return LIB
 

@@ -9,6 +9,7 @@
 
 #include "common.cuh"
 #include "simt_kernels.cuh"
+#include "conv_fma.h"
 #include "tc_api.h"
 #include <type_traits>
 
@@ -503,6 +504,10 @@ static xconv_status run_conv_simt(const xconv_desc* d, bool dgrad, const void* i
                                   cudaStream_t st) {
   const int Ci = dgrad ? d->Cout : d->Cin, Co = dgrad ? d->Cin : d->Cout;
   const int D = depth(d), planes = d->B * D;
+  ConvFma g;
+  if constexpr (std::is_same<T, float>::value)
+    if (plan_conv_fma(d, dgrad, &g))
+      return run_conv_fma(d, g, dgrad, static_cast<const float*>(in), static_cast<const float*>(Wt), static_cast<float*>(out), st);
   dim3 grid((unsigned)((long)planes * d->H * cdiv(d->W, 32)), (unsigned)cdiv(Co, 64));
   const T* i_ = static_cast<const T*>(in);
   const T* w_ = static_cast<const T*>(Wt);
