@@ -184,7 +184,8 @@ def _like(shape_head, geo, dim, **kw):
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    # torch.cuda.current_stream() builds a Stream object around this number: 4 us a call, a fifth of a small layer's call
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 _ws_cache: dict = {}
