@@ -440,7 +440,7 @@ static xconv_status run_sketch(const xconv_desc* d_, const void* X, const void* 
   }
   if (p.stream) {
     float* part = reinterpret_cast<float*>(w + p.part_off);
-    xconv_status s = tc_run_sketch_stream(d, p.s, X, Z, part, st, redraw ? seed : nullptr);
+    xconv_status s = tc_run_sketch_stream(d, p.s, X, Z, part, w, st, redraw ? seed : nullptr);
     return s == XCONV_OK ? run_reduce(part, S, (long)d->r * d->B, p.s.splits, 1.0f, nullptr, 1, st) : s;
   }
   if (p.tc) return tc_run_sketch(d, p.t, X, Z, S, w, w + p.part_off, st, redraw ? seed : nullptr);
@@ -562,7 +562,7 @@ static xconv_status run_backprobe(const xconv_desc* d, const WgradPlan& p, const
                                   void* L, void* Sb_, char* w, cudaStream_t st, const unsigned long long* seed = nullptr) {
   if (p.stream_bp) {
     const xconv_desc f = flat(d);
-    return tc_run_backprobe_stream(&f, S, d->B, 1, dY, L, !p.tc_bp, st, nullptr);
+    return tc_run_backprobe_stream(&f, S, d->B, 1, dY, L, !p.tc_bp, w, st, nullptr);
   }
   if (p.tc_bp) {
     const long n = (long)d->r * d->B;
@@ -629,7 +629,7 @@ static xconv_status run_wgrad(const xconv_desc* d, const float* S, const void* d
     if ((s = validate(&sw.d1)) != XCONV_OK || (s = validate(&sw.d2)) != XCONV_OK) return s;
     if (sw.p1.stream_bp) {                 // reads S by its columns itself
       const xconv_desc f = flat(&sw.d1);
-      s = tc_run_backprobe_stream(&f, S, 1, d->B, Z, w + sw.x_off, !sw.p1.tc_bp, st, seed);
+      s = tc_run_backprobe_stream(&f, S, 1, d->B, Z, w + sw.x_off, !sw.p1.tc_bp, w, st, seed);
     } else {
       float* St = reinterpret_cast<float*>(w + sw.st_off);
       const long n = (long)d->r * d->B;

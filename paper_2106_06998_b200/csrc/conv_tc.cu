@@ -417,7 +417,7 @@ static int block_width(int c) { return c > 32 ? 64 : c > 16 ? 32 : 16; }
 struct ConvGeo { long W, H, D, B; };
 static ConvGeo conv_geo(const xconv_desc* d) {
   const long depth = d->D > 1 ? d->D : 1, kd = d->KD > 1 ? d->KD : 1;
-  if (kd == 1 && d->KH == 1 && (long)d->B * depth * d->H * d->W < (1L << 31)) return {(long)d->B * depth * d->H * d->W, 1, 1, 1};
+  if (kd == 1 && d->KH == 1 && (long)d->B * depth * d->H * d->W < (1L << 31) - 256) return {(long)d->B * depth * d->H * d->W, 1, 1, 1};
   if (kd == 1) return {d->W, d->H, 1, (long)d->B * depth};        // a planar kernel takes every plane as an image
   return {d->W, d->H, depth, d->B};
 }

@@ -71,6 +71,7 @@ struct SketchStream {
   int M, N, swap;
   long K;
   uint32_t seed_lo, seed_hi;
+  unsigned int *status, tag;                          // workspace header: this call is the last to use it
 };
 
 template <bool F16, int MT, int NT, bool SEEDED>
@@ -79,6 +80,7 @@ __global__ void __launch_bounds__(256, 2) sketch_stream_kernel(const SketchStrea
   __shared__ uint4 bits[SEEDED ? 8 : 1][SEEDED ? 16 * MT : 1];
   pdl_trigger();
   pdl_wait();
+  if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) p.status[1] = p.tag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int m0 = blockIdx.y * 16 * MT;
   float acc[MT][NT][4];
@@ -206,6 +208,7 @@ struct BackprobeStream {
   int rows, K, K16, ld;                               // K16: K rounded up to 64; ld: row pitch of S in shared memory
   long Q, groups;                                     // groups of 64 columns
   uint32_t seed_lo, seed_hi;
+  unsigned int *status, tag;
 };
 
 // SPLIT: S as the sum of two 16-bit values (16 bits of it in bfloat16; 22 in float16, where every row is scaled by a power of two
@@ -219,6 +222,7 @@ __global__ void __launch_bounds__(256, MT >= 4 ? 1 : 2) backprobe_stream_kernel(
   extern __shared__ __align__(16) uint16_t s16[];     // [16 MT][ld], then (SEEDED) 8 warps x 32 rows x 8 bytes of signs
   pdl_trigger();
   pdl_wait();
+  if (threadIdx.x == 0 && blockIdx.x == 0) p.status[1] = p.tag;
   __shared__ float unscale[SPLIT ? 16 * MT : 1];      // SPLIT: what the row's sums are multiplied by
   uint16_t* s16lo = s16 + 16 * MT * p.ld;             // SPLIT: the second values
   if (SPLIT) {
@@ -410,8 +414,10 @@ static cudaError_t launch_sketch_stream(const StreamSketchPlan& pl, bool seeded,
 }
 
 xconv_status tc_run_sketch_stream(const xconv_desc* d, const StreamSketchPlan& pl, const void* X, const void* Z, float* part,
-                                  cudaStream_t st, const unsigned long long* seed) {
+                                  char* ws_head, cudaStream_t st, const unsigned long long* seed) {
   SketchStream q{};
+  q.status = reinterpret_cast<unsigned int*>(ws_head);
+  q.tag = call_tag();
   q.A = static_cast<const uint16_t*>(pl.swap ? X : Z);
   q.Bm = static_cast<const uint16_t*>(pl.swap ? Z : X);
   q.part = part;
@@ -460,8 +466,10 @@ static cudaError_t launch_backprobe_stream(const BackprobeStream& q, bool seeded
 }
 
 xconv_status tc_run_backprobe_stream(const xconv_desc* d, const float* S, long s_row, long s_k, const void* dY, void* L,
-                                     bool split, cudaStream_t st, const unsigned long long* seed) {
+                                     bool split, char* ws_head, cudaStream_t st, const unsigned long long* seed) {
   BackprobeStream q{};
+  q.status = reinterpret_cast<unsigned int*>(ws_head);
+  q.tag = call_tag();
   q.S = S; q.s_row = s_row; q.s_k = s_k;
   q.Y = static_cast<const uint16_t*>(dY);
   q.L = static_cast<uint16_t*>(L);

@@ -95,11 +95,11 @@ xconv_status tc_run_halo(const xconv_desc* d, const TcHaloPlan& p, const void* L
 // (H*W*Cout a multiple of 64 then).
 bool tc_plan_sketch_stream(const xconv_desc* d, bool seeded, StreamSketchPlan* p);
 xconv_status tc_run_sketch_stream(const xconv_desc* d, const StreamSketchPlan& p, const void* X, const void* Z, float* part,
-                                  cudaStream_t st, const unsigned long long* seed);
+                                  char* ws_head, cudaStream_t st, const unsigned long long* seed);
 bool tc_backprobe_streams(const xconv_desc* d, bool other);
 // (`split`: S with more than its 16-bit rounding, see the kernel.)
 xconv_status tc_run_backprobe_stream(const xconv_desc* d, const float* S, long s_row, long s_k, const void* dY, void* L,
-                                     bool split, cudaStream_t st, const unsigned long long* seed);
+                                     bool split, char* ws_head, cudaStream_t st, const unsigned long long* seed);
 
 xconv_status tc_run_wait_selftest(char* ws_head, unsigned long long limit_ns, cudaStream_t st);
 

@@ -1,6 +1,6 @@
-// tcgen05 / TMEM / TMA kernels for bfloat16 storage (sm_100a).
-//
-// (the exact convolutions have a kernel of their own, conv_tc.cu)
+// tcgen05 / TMEM / TMA kernels of the sketch, the back-probe and the contraction of wide layers for 16-bit storage (sm_100a).
+// (The exact convolutions are in conv_tc.cu, the contraction of few channels in contract_tc.cu, the sketch and the back-probe
+// of few samples or few probes in stream_tc.cu.)
 //
 // One kernel template, three problem shapes, all dense contractions with float accumulation in
 // tensor memory:
