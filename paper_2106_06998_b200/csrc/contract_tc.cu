@@ -109,8 +109,7 @@ contract_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
     prefetch_tmap(&map_a);
     prefetch_tmap(&map_b);
   }
-  if (warp == 1) tmem_alloc(&tmem_slot, (uint32_t)p.tmem_cols);
-  pdl_trigger();
+  if (warp == 1) tmem_alloc_then_trigger(&tmem_slot, (uint32_t)p.tmem_cols);
   pdl_wait();
   if (threadIdx.x == 0) {
     go = (*reinterpret_cast<volatile unsigned int*>(p.status) != p.tag) ? 1 : 0;

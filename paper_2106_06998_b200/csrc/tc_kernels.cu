@@ -346,8 +346,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       const uint4 o = z_pack8(i, F16 ? 0x3C003C00u : 0x3F803F80u);
       asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(z_lut + (i << 4)), "r"(o.x), "r"(o.y), "r"(o.z), "r"(o.w) : "memory");
     }
-  if (warp == 1) tmem_alloc(&tmem_slot, (uint32_t)p.tmem_cols);
-  pdl_trigger();
+  if (warp == 1) tmem_alloc_then_trigger(&tmem_slot, (uint32_t)p.tmem_cols);
   pdl_wait();                              // from here on the previous kernel's results are visible
   // Block-sparse probes (one unit per CTA): the unit's stretch of its tile's list, zl_len entries (and the entry behind
   // the last, which the producer may fetch but never uses), goes to shared memory.

@@ -117,6 +117,13 @@ __device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t ncols) {
                : "memory");
   asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
+// The go-ahead for the next kernel of the stream comes from the allocating warp, once the CTA has its tensor memory.  Given
+// by the other warps at once, it let that kernel's CTAs onto the SM while this allocation still waited for the CTA before
+// it: they could take the columns first and then wait for this kernel to end.  (One warp's go-ahead counts for the CTA.)
+__device__ __forceinline__ void tmem_alloc_then_trigger(uint32_t* slot, uint32_t ncols) {
+  tmem_alloc(slot, ncols);
+  pdl_trigger();
+}
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }

@@ -60,3 +60,30 @@ def test_contraction(dtype, r, Cin, Cout, D, H, W, K, KD):
     got = host(buf[:dW.numel()].reshape(Cout, taps, Cin))
     flat = want.reshape(Cout, Cin, taps).transpose(0, 2, 1) * r
     check("dW with chan_scale", got, flat * host(scale), 1e-4)
+
+
+def test_calls_in_a_row_on_layers_that_fill_tensor_memory():
+    """Several CTAs of these layers fit one SM beside each other and each takes all of its tensor memory (25 offsets, 320
+    columns), so a call's kernel starts while its columns are still held by the call before it.  The allocations have to be
+    served in the order of the stream; a hundred calls on each of two streams, interleaved with convolutions."""
+    g = np.random.Generator(np.random.PCG64(11))
+    B, C, H, W, r = 40, 32, 4, 16, 40
+    L, Z, X = (inputs.round_to_storage(g.standard_normal((n, C, H, W)).astype(np.float32), "bf16") for n in (r, r, B))
+    Wt = inputs.round_to_storage((0.05 * g.standard_normal((C, C, 5, 5))).astype(np.float32), "bf16")
+    Ld, Zd, Xd, Wd = (xb.to_device(v, "bf16") for v in (L, Z, X, Wt))
+    desc = xb.make_desc(B, C, C, H, W, r, Zd.dtype, 5)
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    like = dict(device="cuda", memory_format=torch.channels_last)
+    out = [(torch.empty((C, C, 5, 5), dtype=torch.float32, **like), torch.empty((B, C, H, W), dtype=torch.bfloat16, **like),
+            torch.empty(xb.workspace_bytes(desc, xb.OP_CONTRACT), dtype=torch.uint8, device="cuda")) for _ in streams]
+    torch.cuda.synchronize()
+    for _ in range(100):
+        for s, (dW, dX, ws) in zip(streams, out):
+            with torch.cuda.stream(s):
+                xb.contract_into(desc, Ld, Zd, dW, ws)
+                xb.dgrad_into(desc, Xd, Wd, dX, ws)
+    torch.cuda.synchronize()
+    for dW, dX, ws in out:
+        check("dW", host(dW), O.wgrad_contract(L, Z, 5, 5), 1e-4)
+        check("dX", host(dX), O.dx_exact(X, Wt), 1e-2)
+        assert xb.workspace_status(ws) == 0

@@ -143,3 +143,22 @@ def test_planning_survives_random_descriptors(lib):
         assert all(0 < s < (1 << 46) for s in sizes), (B, Cin, Cout, H, W, r, K, D, KD, sizes)
         assert all(xb.engine_for(d, op) != "none" for op in ops[:4])
         assert xb.zero_blocks_used(d) in (False, True)
+
+
+def test_kernels_that_take_tensor_memory_let_the_next_kernel_start_only_afterwards():
+    """A CTA that gives the go-ahead for the next kernel while its own allocation still waits can lose its columns to that
+    kernel, which then waits for it: neither ends.  No run can be asked to show that, so the sources are: tensor memory is
+    taken through the one function that gives the go-ahead behind the allocation, and nothing else gives it there."""
+    csrc = os.path.join(ROOT, "paper_2106_06998_b200", "csrc")
+    holders = 0
+    for name in sorted(os.listdir(csrc)):
+        if not name.endswith((".cu", ".cuh")):
+            continue
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(csrc, name)).read())
+        for kernel in re.split(r"__global__", text)[1:]:
+            body = kernel.split("\n}\n")[0]
+            if "tmem_alloc" in body:
+                holders += 1
+                assert body.count("tmem_alloc_then_trigger(") == 1 and "tmem_alloc(" not in body, name
+                assert "pdl_trigger(" not in body, name
+    assert holders == 3
