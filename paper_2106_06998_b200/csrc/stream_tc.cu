@@ -49,6 +49,17 @@ __device__ __forceinline__ float from16(unsigned short v) {
 template <bool F16>
 __device__ __forceinline__ uint32_t pack16(float a, float b) { return (uint32_t)to16<F16>(a) | ((uint32_t)to16<F16>(b) << 16); }
 
+// Two packed values with infinities and NaN replaced by zeros.
+template <bool F16>
+__device__ __forceinline__ uint32_t finite16(uint32_t v) {
+  if (F16) {
+    const __half2 h = *reinterpret_cast<const __half2*>(&v);
+    return v & __hlt2_mask(__habs2(h), __half2(__ushort_as_half(0x7C00), __ushort_as_half(0x7C00)));
+  }
+  const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(&v);
+  return v & __hlt2_mask(__habs2(h), __nv_bfloat162(__ushort_as_bfloat16(0x7F80), __ushort_as_bfloat16(0x7F80)));
+}
+
 // The 128 sign bits of entries e0 .. e0+127 of Z (e0 a multiple of 64, `whole`: of 128).
 __device__ __forceinline__ uint4 sign_bits128(unsigned long long e0, bool whole, uint32_t k0, uint32_t k1) {
   const unsigned long long b = e0 >> 7;
@@ -214,6 +225,8 @@ struct BackprobeStream {
 // SPLIT: S as the sum of two 16-bit values (16 bits of it in bfloat16; 22 in float16, where every row is scaled by a power of two
 // into the range first), multiplied one after the other: for the layers whose sums used the float S all along (what it is
 // rounded to shows in the result: relative error against 64 bits 1.7e-3 with the float S or with two values, 2.4e-3 with one).
+// Y's infinities and NaN count once, with the first value: the second is zero or of either sign, and its product with an
+// infinity would make a NaN of the sum.  So an entry of S that is not zero has a first value that is not zero either.
 // KC: k-steps of 16 that are loaded together.  ALL: they are the whole reduction; a warp then takes 4 / KC groups of
 // columns at a time, so that as many bytes are in flight as with a long reduction.  Otherwise the loads of the next
 // KC k-steps (of the next group behind the last) are under way while these are multiplied.
@@ -244,7 +257,8 @@ __global__ void __launch_bounds__(256, MT >= 4 ? 1 : 2) backprobe_stream_kernel(
       }
       for (int k = threadIdx.x & 31; k < p.K16; k += 32) {
         const float v = live && k < p.K ? p.S[row * p.s_row + k * p.s_k] * up : 0.f;
-        const uint16_t hi = to16<F16>(v);
+        uint16_t hi = to16<F16>(v);
+        if (v != 0.f && (hi & 0x7FFFu) == 0) hi |= 1u;
         const float h = from16<F16>(hi);
         s16[row * p.ld + k] = hi;
         s16lo[row * p.ld + k] = fabsf(h) < __int_as_float(0x7F800000) ? to16<F16>(v - h) : (uint16_t)0;
@@ -312,9 +326,11 @@ __global__ void __launch_bounds__(256, MT >= 4 ? 1 : 2) backprobe_stream_kernel(
           b1 = __byte_perm(word(v[gb][u][2], c >> 1), word(v[gb][u][3], c >> 1), (c & 1) ? 0x7632 : 0x5410);
         }
 #pragma unroll
-        for (int i = 0; i < MT; ++i) {
-          mma16816<F16>(acc[i][c], a[i], b0, b1);
-          if (SPLIT) mma16816<F16>(acc[i][c], a[MT + i], b0, b1);
+        for (int i = 0; i < MT; ++i) mma16816<F16>(acc[i][c], a[i], b0, b1);
+        if (SPLIT) {
+          if (!SEEDED) { b0 = finite16<F16>(b0); b1 = finite16<F16>(b1); }
+#pragma unroll
+          for (int i = 0; i < MT; ++i) mma16816<F16>(acc[i][c], a[MT + i], b0, b1);
         }
       }
     }
