@@ -131,6 +131,8 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) conv_fma(const float* 
   }
 }
 
+static const int FMA_SMEM_MAX = 227 * 1024;           // (the largest plan takes 126 KB)
+
 static long cd(long a, long b) { return (a + b - 1) / b; }
 
 // Threads of a block, patch and channel tile by the time of the busiest SM: outputs computed there (padding counts), more per
@@ -176,7 +178,8 @@ static cudaError_t launch_one(const xconv_desc* d, const ConvFma& g, const float
   const size_t smem = ((size_t)KS * KS * KD * conv_fma_ck<KS, KD>() * 8 * TN + (size_t)conv_fma_ck<KS, KD>() * g.plane +
                        (size_t)2 * g.NI * KD * (g.RH + KS - 1) * (8 * g.SW + KS - 1)) * 4;
   auto kern = conv_fma<KS, KD, DGRAD, TN, THREADS>;
-  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // (the limit belongs to the kernel, not to this launch: the same for every patch, so that no other thread finds it lowered)
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, FMA_SMEM_MAX);
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)(cd(d->W, 8L * g.SW) * cd(d->H, g.RH) * cd(planes, g.NI)), (unsigned)cd(Co, 8 * TN));
   kern<<<grid, THREADS, smem, st>>>(in, Wt, out, planes, D, d->H, d->W, Ci, Co, d->Cin, d->circular, g);

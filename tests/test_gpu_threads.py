@@ -1,0 +1,67 @@
+"""Calls from several host threads at once."""
+import threading
+
+import pytest
+import torch
+
+import __graft_entry__ as entry
+from paper_2106_06998_b200 import binding as xb
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    entry.build()
+    torch.cuda.set_device(0)
+
+
+def _layer(seed, B, Cin, Cout, geo, r, dtype, K=3):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    fmt = torch.channels_last if len(geo) == 2 else torch.channels_last_3d
+    rnd = lambda *s: torch.randn(s, generator=g, device="cuda").to(dtype).contiguous(memory_format=fmt)
+    return dict(X=rnd(B, Cin, *geo), dY=rnd(B, Cout, *geo), Z=rnd(r, Cin, *geo), W=rnd(Cout, Cin, *([K] * len(geo))),
+                K=K, KD=K if len(geo) == 3 else 1)
+
+
+def _run_threads(jobs):
+    errors = []
+
+    def guarded(job):
+        try:
+            job()
+        except Exception as e:          # an assertion of a thread is the test's
+            errors.append(e)
+
+    threads = [threading.Thread(target=guarded, args=(j,)) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors[:3]
+
+
+@pytest.mark.parametrize("one,two", [
+    # both layers of a pair run the same kernel with another amount of shared memory: 53 and 89 KB, 35 and 60 KB
+    ((3, 8, 64, (4, 40, 34), 3), (17, 3, 64, (10, 13, 32), 3)),
+    ((22, 3, 64, (29, 40), 5), (39, 16, 64, (29, 29), 5)),
+])
+def test_float_layers_of_different_geometry_from_two_host_threads(one, two):
+    def job(shape, seed):
+        B, Cin, Cout, geo, K = shape
+        d = _layer(seed, B, Cin, Cout, geo, 1, torch.float32, K)
+        s = torch.cuda.Stream()
+        with torch.cuda.stream(s):
+            ws = torch.empty(1 << 24, dtype=torch.uint8, device="cuda")
+            D = geo[0] if len(geo) == 3 else 1
+            desc = xb.make_desc(B, Cin, Cout, geo[-2], geo[-1], 1, torch.float32, K, D=D, KD=d["KD"])
+            Y = torch.empty_like(d["dY"])
+            S = torch.empty((1, B), device="cuda")
+            for i in range(1500):
+                xb.forward_into(desc, d["X"], d["W"], d["Z"], Y, S, ws)
+                if i % 100 == 0:
+                    s.synchronize()
+            s.synchronize()
+
+    torch.cuda.synchronize()
+    _run_threads([lambda: job(one, 1), lambda: job(two, 2)])
