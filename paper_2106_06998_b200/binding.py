@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import threading
 from ctypes import POINTER, Structure, c_char_p, c_float, c_int, c_int32, c_size_t, c_void_p
 
 import torch
@@ -188,16 +189,32 @@ def _stream() -> int:
     return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
-_ws_cache: dict = {}
+def _capturing() -> bool:
+    return torch._C._cuda_isCurrentStreamCapturing()
+
+
+# Calls on different streams or from different host threads may overlap, so each of them has a scratch buffer of its own: per
+# host thread (which gives them back when it ends), those of the streams it came to last.
+_ws_cache = threading.local()
+_WS_STREAMS = 8
 
 
 def workspace(nbytes: int, device) -> torch.Tensor:
-    """A cached scratch buffer of at least ``nbytes`` on ``device`` (grown on demand)."""
-    key = str(device)
-    buf = _ws_cache.get(key)
+    """A scratch buffer of at least ``nbytes`` on ``device`` for calls on the current stream: cached per host thread and
+    stream, grown on demand.  While the stream is captured into a graph it is a new buffer, whose memory is the graph's."""
+    if _capturing():
+        return torch.empty(max(nbytes, 256), dtype=torch.uint8, device=device)
+    key = (device, _stream())
+    try:
+        buffers = _ws_cache.buffers
+    except AttributeError:
+        buffers = _ws_cache.buffers = {}
+    buf = buffers.get(key)
     if buf is None or buf.numel() < nbytes:
-        buf = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=device)
-        _ws_cache[key] = buf
+        buffers.pop(key, None)
+        while len(buffers) >= _WS_STREAMS:
+            del buffers[next(iter(buffers))]
+        buf = buffers[key] = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=device)
     return buf
 
 

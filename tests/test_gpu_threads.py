@@ -1,4 +1,4 @@
-"""Calls from several host threads at once."""
+"""Calls from several host threads and on several streams at once: the same bits as one call after the other."""
 import threading
 
 import pytest
@@ -22,6 +22,12 @@ def _layer(seed, B, Cin, Cout, geo, r, dtype, K=3):
     rnd = lambda *s: torch.randn(s, generator=g, device="cuda").to(dtype).contiguous(memory_format=fmt)
     return dict(X=rnd(B, Cin, *geo), dY=rnd(B, Cout, *geo), Z=rnd(r, Cin, *geo), W=rnd(Cout, Cin, *([K] * len(geo))),
                 K=K, KD=K if len(geo) == 3 else 1)
+
+
+def _step(d):
+    Y, S = xb.xconv_forward(d["X"], d["W"], d["Z"])
+    dW = xb.xconv_wgrad(S, d["dY"], d["Z"], kernel_size=d["K"], kernel_depth=d["KD"])
+    return Y, S, dW, xb.xconv_dgrad(d["dY"], d["W"])
 
 
 def _run_threads(jobs):
@@ -65,3 +71,34 @@ def test_float_layers_of_different_geometry_from_two_host_threads(one, two):
 
     torch.cuda.synchronize()
     _run_threads([lambda: job(one, 1), lambda: job(two, 2)])
+
+
+@pytest.mark.parametrize("threads", [False, True])
+def test_layers_on_two_streams_at_once(threads):
+    """Layers whose channels are padded in the scratch memory, and one that keeps much in it, each on a stream of its own; the
+    streams of one thread, and of a thread each."""
+    layers = [_layer(1, 64, 3, 64, (56, 56), 32, torch.bfloat16), _layer(2, 64, 5, 32, (60, 52), 80, torch.float16),
+              _layer(3, 16, 32, 32, (64, 64), 64, torch.bfloat16)]
+    want = []
+    for d in layers:
+        want.append([t.clone() for t in _step(d)])
+        torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in layers]
+    got = [[] for _ in layers]
+
+    def one(i, times):
+        with torch.cuda.stream(streams[i]):
+            for _ in range(times):
+                got[i].append(_step(layers[i]))
+
+    if threads:
+        _run_threads([lambda i=i: one(i, 30) for i in range(len(layers))])
+    else:
+        for _ in range(30):
+            for i in range(len(layers)):
+                one(i, 1)
+    torch.cuda.synchronize()
+    for w, g in zip(want, got):
+        assert len(g) == 30
+        for out in g:
+            assert all(torch.equal(a, b) for a, b in zip(w, out))
