@@ -393,9 +393,10 @@ xconv_status tc_run_halo(const xconv_desc* d, const TcHaloPlan& pl, const void* 
   if (!map(&ma, L, d->Cout, pl.cwa, pl.pw, a_rows, 1) || !map(&mb, Z, d->Cin, pl.cwb, PB, pl.ph, pl.dz_per)) return XCONV_ERR_CUDA;
   const size_t smem = 1024 + (size_t)p.stages * p.stage_bytes;
   if (smem > (size_t)(SMEM_LIMIT - 1024)) return XCONV_ERR_UNSUPPORTED;
+  const unsigned grid = (unsigned)(pl.units * pl.splits);
   void (*kernel)(CUtensorMap, CUtensorMap, HaloParams) = f16 ? contract_halo_kernel<true> : contract_halo_kernel<false>;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT - 1024);
-  if (e == cudaSuccess) e = launch_pdl(kernel, dim3((unsigned)(pl.units * pl.splits)), dim3(CH_THREADS), smem, st, ma, mb, p);
+  if (e == cudaSuccess) e = launch_pdl(kernel, dim3(grid), dim3(CH_THREADS), smem_of_grid(smem, grid), st, ma, mb, p);
   count_launch();
   if (e != cudaSuccess) { set_cuda_error((int)e); return XCONV_ERR_CUDA; }
   const uint32_t groups = (uint32_t)(pl.units * pl.mt * (pl.cols / 4) * TILE_M);

@@ -543,13 +543,14 @@ xconv_status tc_run_conv(const xconv_desc* d, const TcConvPlan& pl, bool dgrad, 
     return XCONV_ERR_CUDA;
   const size_t smem = 1024 + (size_t)p.o_off + 2 * (size_t)p.o_bytes;
   if (smem > (size_t)(SMEM_LIMIT - 1024)) return XCONV_ERR_UNSUPPORTED;
+  const unsigned grid = std::min<uint32_t>(p.items, NUM_SMS);
   void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, ConvParams) =
       K == 3 ? (f16 ? conv_tc_kernel<true, 3> : conv_tc_kernel<false, 3>)
       : K == 5 ? (f16 ? conv_tc_kernel<true, 5> : conv_tc_kernel<false, 5>)
                : (f16 ? conv_tc_kernel<true, 1> : conv_tc_kernel<false, 1>);
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT - 1024);
   if (e == cudaSuccess)
-    e = launch_pdl(kernel, dim3((unsigned)std::min<uint32_t>(p.items, NUM_SMS)), dim3(128 + 128 * p.groups), smem, st, mi, mw, mo, p);
+    e = launch_pdl(kernel, dim3(grid), dim3(128 + 128 * p.groups), smem_of_grid(smem, grid), st, mi, mw, mo, p);
   count_launch();
   if (e != cudaSuccess) { set_cuda_error((int)e); return XCONV_ERR_CUDA; }
   return XCONV_OK;

@@ -1130,7 +1130,7 @@ static xconv_status launch(const CUtensorMap& ma, const CUtensorMap& mb, const T
   if (q.layout == 0) { q.sbo = 1024; q.mn_step = 2048; q.layout = 2; q.cw_shift = 6; }
   if (q.depth < 1) q.depth = 1;
   if (q.epi_groups < 1) q.epi_groups = 1;
-  e = launch_pdl(kernel, dim3(grid), dim3(64 + 128 * q.epi_groups), smem, st, ma, mb, mc ? *mc : ma, q);
+  e = launch_pdl(kernel, dim3(grid), dim3(64 + 128 * q.epi_groups), smem_of_grid(smem, grid), st, ma, mb, mc ? *mc : ma, q);
   count_launch();
   if (e != cudaSuccess) { set_cuda_error((int)e); return XCONV_ERR_CUDA; }
   return XCONV_OK;

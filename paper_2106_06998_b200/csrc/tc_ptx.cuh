@@ -219,6 +219,15 @@ static const int SMEM_LIMIT = 227 * 1024;
 static const int STATIC_SMEM_SLACK = 2048;     // barriers + alignment slack
 static const int NUM_SMS = 148;
 
+// Shared memory of a launch whose CTAs are meant to have an SM each.  Launched while the kernel before it still runs, two small
+// CTAs are otherwise placed on an SM that is free already, and the grid takes twice its time (us a call, before -> after:
+// contraction 160 -> 192 channels of 57 images of 26 x 26 after a streaming back-probe 184 -> 110; 96 -> 128 channels, 64 probes of
+// 183 x 106 1690 -> 878; the padded first layer's convolution, 32 images of 112 x 112, 55 -> 44 with its sketch).  Grids
+// beyond one wave keep what they need.
+static inline size_t smem_of_grid(size_t bytes, unsigned grid) {
+  return grid <= (unsigned)NUM_SMS ? std::max(bytes, (size_t)115 * 1024) : bytes;
+}
+
 static inline int pow2_cols(int n) { int c = 32; while (c < n) c *= 2; return c; }
 
 static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
