@@ -393,6 +393,13 @@ __global__ void __launch_bounds__(256, MT >= 4 ? 1 : 2) backprobe_stream_kernel(
 
 static long cdiv_(long a, long b) { return (a + b - 1) / b; }
 
+// Whether a launch that reads so many bytes may start while the kernel before it still runs.  An SM that holds a CTA of that
+// kernel keeps its split of L1 and shared memory, for the tensor-core kernels nearly all shared memory, as long as it is not
+// empty, and the loads in flight of these kernels live in L1.  Sketch of 4 volumes of 48^3 behind the convolution 85 -> 65 us for
+// both, back-probe of 16 samples x 64 probes of 256 x 256 x 32 with the contraction 105 -> 97; a sketch of 1 MB x 70 MB behind
+// another sketch 18.5 -> 20.7, behind the convolution 30 -> 26.  Few bytes are read before that matters.
+static bool starts_early(long bytes) { return bytes < (16L << 20); }
+
 // Measured against the tcgen05 sketch, other -> this, us: 8 x 4 (probes x samples), 3.5 M terms 178 -> 22; 16 x 64, 200704
 // terms 13.3 -> 11.5; 512 x 8, 65536 terms 14.5 -> 10.0; 128 x 16, 262144 terms 16.3 -> 15.8; but 64 x 16, 2.1 M terms 76 -> 113
 // (a load instruction touches eight rows, and many rows far apart cost it more than the bytes do): more than 32 rows only
@@ -419,14 +426,15 @@ bool tc_plan_sketch_stream(const xconv_desc* d, bool seeded, StreamSketchPlan* p
 template <bool F16>
 static cudaError_t launch_sketch_stream(const StreamSketchPlan& pl, bool seeded, const SketchStream& q, cudaStream_t st) {
   const dim3 grid((unsigned)pl.splits, (unsigned)pl.tiles_m), block(256);
-  if (seeded) return pl.nt == 2 ? launch_pdl(sketch_stream_kernel<F16, 4, 2, true>, grid, block, 0, st, q)
-                                : launch_pdl(sketch_stream_kernel<F16, 4, 1, true>, grid, block, 0, st, q);
-  if (pl.mt == 4) return pl.nt == 2 ? launch_pdl(sketch_stream_kernel<F16, 4, 2, false>, grid, block, 0, st, q)
-                                    : launch_pdl(sketch_stream_kernel<F16, 4, 1, false>, grid, block, 0, st, q);
-  if (pl.mt == 2) return pl.nt == 2 ? launch_pdl(sketch_stream_kernel<F16, 2, 2, false>, grid, block, 0, st, q)
-                                    : launch_pdl(sketch_stream_kernel<F16, 2, 1, false>, grid, block, 0, st, q);
-  return pl.nt == 2 ? launch_pdl(sketch_stream_kernel<F16, 1, 2, false>, grid, block, 0, st, q)
-                    : launch_pdl(sketch_stream_kernel<F16, 1, 1, false>, grid, block, 0, st, q);
+  const bool early = starts_early(2 * q.K * (seeded ? q.N : q.M + q.N));
+  if (seeded) return pl.nt == 2 ? launch_when(early, sketch_stream_kernel<F16, 4, 2, true>, grid, block, 0, st, q)
+                                : launch_when(early, sketch_stream_kernel<F16, 4, 1, true>, grid, block, 0, st, q);
+  if (pl.mt == 4) return pl.nt == 2 ? launch_when(early, sketch_stream_kernel<F16, 4, 2, false>, grid, block, 0, st, q)
+                                    : launch_when(early, sketch_stream_kernel<F16, 4, 1, false>, grid, block, 0, st, q);
+  if (pl.mt == 2) return pl.nt == 2 ? launch_when(early, sketch_stream_kernel<F16, 2, 2, false>, grid, block, 0, st, q)
+                                    : launch_when(early, sketch_stream_kernel<F16, 2, 1, false>, grid, block, 0, st, q);
+  return pl.nt == 2 ? launch_when(early, sketch_stream_kernel<F16, 1, 2, false>, grid, block, 0, st, q)
+                    : launch_when(early, sketch_stream_kernel<F16, 1, 1, false>, grid, block, 0, st, q);
 }
 
 xconv_status tc_run_sketch_stream(const xconv_desc* d, const StreamSketchPlan& pl, const void* X, const void* Z, float* part,
@@ -478,7 +486,8 @@ static cudaError_t launch_backprobe_stream(const BackprobeStream& q, bool seeded
              : q.K <= 32 ? backprobe_stream_kernel<F16, 1, false, 2, true, false>
              : q.K <= 64 ? backprobe_stream_kernel<F16, 1, false, 4, true, false> : backprobe_stream_kernel<F16, 1, false, 2, false, false>;
   const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
-  return e != cudaSuccess ? e : launch_pdl(kernel, dim3(grid), dim3(256), smem, st, q);
+  const bool early = starts_early(2 * q.Q * (seeded ? q.rows : q.K));      // (redrawn: what it writes)
+  return e != cudaSuccess ? e : launch_when(early, kernel, dim3(grid), dim3(256), smem, st, q);
 }
 
 xconv_status tc_run_backprobe_stream(const xconv_desc* d, const float* S, long s_row, long s_k, const void* dY, void* L,
