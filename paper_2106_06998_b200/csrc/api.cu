@@ -386,10 +386,19 @@ static size_t probes_bytes(const xconv_desc* d) {
 
 // ----------------------------------------------------------------------------------- launchers
 
+// Every block of a dependent launch pays for its go-ahead and its wait: 51200 blocks (5 x 5, 128 -> 512 channels) 34 us without,
+// 54 with; 36000 blocks 26 and 38.  A launch of one wave (eight blocks per SM) is done sooner with them.
+static const unsigned REDUCE_PDL_BLOCKS = 8 * 148;
 static xconv_status run_reduce(const float* part, float* out, long count, int splits, float alpha, const float* chan_scale,
                                int period, cudaStream_t st) {
-  const cudaError_t e = launch_pdl(reduce_partials, dim3((unsigned)cdiv(count, RP_OUT)), dim3(RP_OUT * RP_LANES), 0, st, part, out,
-                                   count, splits, alpha, chan_scale, period);
+  const dim3 grid((unsigned)cdiv(count, RP_OUT)), block(RP_OUT * RP_LANES);
+  cudaError_t e;
+  if (grid.x <= REDUCE_PDL_BLOCKS) {
+    e = launch_pdl(reduce_partials<true>, grid, block, 0, st, part, out, count, splits, alpha, chan_scale, period);
+  } else {
+    reduce_partials<false><<<grid, block, 0, st>>>(part, out, count, splits, alpha, chan_scale, period);
+    e = cudaGetLastError();
+  }
   ++g_launches;
   if (e != cudaSuccess) { g_last_cuda_error = (int)e; return XCONV_ERR_CUDA; }
   return XCONV_OK;

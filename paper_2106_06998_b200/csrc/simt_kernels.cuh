@@ -174,12 +174,15 @@ static __global__ void __launch_bounds__(256) gemm_tn_simt_async(const float* __
 // fixed order, so results are reproducible.  scale(i) = chan_scale[i % period] if chan_scale else alpha.
 // Launch with 256 threads: 32 outputs per block.
 constexpr int RP_OUT = 32, RP_LANES = 8;
+template <bool PDL>
 static __global__ void __launch_bounds__(RP_OUT * RP_LANES)
 reduce_partials(const float* __restrict__ part, float* __restrict__ out, long count, int splits, float alpha,
                 const float* __restrict__ chan_scale, int period) {
   __shared__ float acc[RP_LANES][RP_OUT];
-  pdl_trigger();
-  pdl_wait();
+  if (PDL) {
+    pdl_trigger();
+    pdl_wait();
+  }
   const int o = threadIdx.x % RP_OUT, g = threadIdx.x / RP_OUT;
   const long i = (long)blockIdx.x * RP_OUT + o;
   float s = 0.f;
