@@ -416,10 +416,13 @@ static long cdiv_(long a, long b) { return (a + b - 1) / b; }
 // another sketch 18.5 -> 20.7, behind the convolution 30 -> 26.  Few bytes are read before that matters.
 static bool starts_early(long bytes) { return bytes < (16L << 20); }
 
-// Measured against the tcgen05 sketch, other -> this, us: 8 x 4 (probes x samples), 3.5 M terms 178 -> 22; 16 x 64, 200704
-// terms 13.3 -> 11.5; 512 x 8, 65536 terms 14.5 -> 10.0; 128 x 16, 262144 terms 16.3 -> 15.8; but 64 x 16, 2.1 M terms 76 -> 113
-// (a load instruction touches eight rows, and many rows far apart cost it more than the bytes do): more than 32 rows only
-// up to 131072 terms.  Redrawn from the seed only the few samples are read: 64 x 16 64 -> 31, 256 x 16 190 -> 90.
+// Measured against the tcgen05 sketch, other -> this, us: 8 x 4 (probes x samples), 3.5 M terms 178 -> 22; 512 x 8, 65536 terms
+// 14.5 -> 10.0; 256 x 16, 25600 terms 10.0 -> 8.0; 164 x 16, 93312 terms 13.7 -> 10.8; but 64 x 16, 2.1 M terms 76 -> 113 (a load
+// instruction touches eight rows, and many rows far apart cost it more than the bytes do): more than 32 rows only up to
+// 131072 terms.  With a second column tile the rows' loads are fewer in flight: 380 x 13, 91200 terms 17.0 -> 18.8, 512 x 15,
+// 92160 terms 20.1 -> 22.6, so there up to 32 M values only (512 x 8, 97344 terms 21.6 -> 19.2).  (Left out by the limit: 64 x
+// 16, 200704 terms 13.3 -> 11.5; 128 x 16, 262144 terms 16.3 -> 15.8.)  Redrawn from the seed only the few samples are read: 64 x
+// 16 64 -> 31, 256 x 16 190 -> 90.
 bool tc_plan_sketch_stream(const xconv_desc* d, bool seeded, StreamSketchPlan* p) {
   if (d->dtype != XCONV_BF16 && d->dtype != XCONV_F16) return false;
   const long K = (long)d->H * d->W * d->Cin;
@@ -428,7 +431,7 @@ bool tc_plan_sketch_stream(const xconv_desc* d, bool seeded, StreamSketchPlan* p
   p->swap = d->B <= d->r || seeded ? 0 : 1;                          // 0: rows = probes
   if (!p->swap && d->B > 16) return false;
   const int M = p->swap ? d->B : d->r, N = p->swap ? d->r : d->B;
-  if (!seeded && M > 32 && K > 131072) return false;
+  if (!seeded && M > 32 && (K > 131072 || (N > 8 && (long)M * K > 32000000))) return false;
   p->mt = seeded || M > 32 ? 4 : M > 16 ? 2 : 1;
   p->nt = N > 8 ? 2 : 1;
   p->tiles_m = (int)cdiv_(M, 16 * p->mt);
