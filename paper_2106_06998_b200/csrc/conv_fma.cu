@@ -138,13 +138,16 @@ static long cd(long a, long b) { return (a + b - 1) / b; }
 // Threads of a block, patch and channel tile by the time of the busiest SM: outputs computed there (padding counts), more per
 // output where few warps share the SM, where a block or the channel tile is small (more loads per multiply-add: on the
 // 64 -> 64 layer blocks of 256, 128 and 64 threads take 234, 240 and 275 us) and for the halo.
-// False where conv_simt, which takes about 2.4 times as long per output but has blocks of 2048, would be done sooner, or
-// where the pixel indexes of a block would not fit 32 bits.
+// False where conv_simt, which takes about 2.4 times as long per output (2.1 in pointwise layers: with 2.4 four layers of
+// one wave and 160 to 200 channels took 20.6 -> 22.6, 26.7 -> 29.1 us) but has blocks of 2048, would be done sooner, or where
+// the pixel indexes of a block would not fit 32 bits.  The least a plan below can cost is one block of 128 threads per SM, so
+// small layers are told apart without the search (1 us of a 5 us call).
 bool plan_conv_fma(const xconv_desc* d, bool dgrad, ConvFma* g) {
   const int K = d->KH, KD = d->KD > 1 ? d->KD : 1, Co = dgrad ? d->Cin : d->Cout;
   const long planes = (long)d->B * (d->D > 1 ? d->D : 1);
   if (d->dtype != XCONV_F32 || (long)d->H * d->W * 64 > 2000000000L) return false;
-  double best = 2.4 * 2048.0 * (double)cd(planes * d->H * cd(d->W, 32) * cd(Co, 64), 148);
+  double best = (K == 1 ? 2.1 : 2.4) * 2048.0 * (double)cd(planes * d->H * cd(d->W, 32) * cd(Co, 64), 148);
+  if (best <= 64.0 * 128 * 2.0 * 1.08) return false;
   bool found = false;
   for (int threads = 256; threads >= 64; threads /= 2)
     for (int t = 8; t >= 2; t /= 2) {
