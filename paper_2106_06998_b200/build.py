@@ -42,9 +42,10 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
             cmd.insert(1, "-Xptxas=-v")
         jobs.append((cmd, subprocess.Popen(cmd)))
         objs.append(obj)
-    for cmd, job in jobs:                       # the sources compile side by side
-        if job.wait() != 0:
-            raise subprocess.CalledProcessError(job.returncode, cmd)
+    codes = [job.wait() for _, job in jobs]     # the sources compile side by side; none is left running behind an error
+    for (cmd, _), code in zip(jobs, codes):
+        if code != 0:
+            raise subprocess.CalledProcessError(code, cmd)
     subprocess.run([_nvcc(), "-shared", "-cudart", "static", "-o", LIB, *objs, "-ldl"], check=True)
     return LIB
 
