@@ -387,8 +387,8 @@ static size_t probes_bytes(const xconv_desc* d) {
 // ----------------------------------------------------------------------------------- launchers
 
 // Every block of a dependent launch pays for its go-ahead and its wait: 51200 blocks (5 x 5, 128 -> 512 channels) 34 us without,
-// 54 with; 36000 blocks 26 and 38.  A launch of one wave (eight blocks per SM) is done sooner with them.
-static const unsigned REDUCE_PDL_BLOCKS = 8 * 148;
+// 54 with; 36000 blocks 26 and 38; 18000 14 and 20.  It saves 2 us of launch (1280 blocks 22.6 without, 20.3 with).
+static const unsigned REDUCE_PDL_BLOCKS = 6000;
 static xconv_status run_reduce(const float* part, float* out, long count, int splits, float alpha, const float* chan_scale,
                                int period, cudaStream_t st) {
   const dim3 grid((unsigned)cdiv(count, RP_OUT)), block(RP_OUT * RP_LANES);
@@ -540,12 +540,12 @@ static xconv_desc conv_padded(const xconv_desc* d) {
   e.Cin = pad8(d->Cin);
   return e;
 }
-// Pointwise layers of few input channels whose blocks of conv_simt (32 pixels of a row x 64 channels) all run at once are done
+// Pointwise layers of few input channels with one block of conv_simt (32 pixels of a row x 64 channels) per SM at most are done
 // there before conv_tc has its tensor maps and its tensor memory: 17 pixels, 8 -> 384 channels 5.7 against 7.2 us a call, 48
-// pixels, 24 -> 384 5.8 against 8.2, 2809 pixels, 8 -> 160 5.3 against 5.9.
+// pixels, 24 -> 384 5.8 against 8.2, 96 blocks, 8 -> 200 4.7 against 6.8; but 270 blocks, 24 -> 72 6.2 against 5.2.
 static bool conv_tiny(const xconv_desc* d, bool dgrad) {
   const int Ci = dgrad ? d->Cout : d->Cin, Co = dgrad ? d->Cin : d->Cout;
-  return d->KH == 1 && kdepth(d) == 1 && Ci <= 24 && (long)d->B * depth(d) * d->H * cdiv(d->W, 32) * cdiv(Co, 64) <= 4 * 148;
+  return d->KH == 1 && kdepth(d) == 1 && Ci <= 24 && (long)d->B * depth(d) * d->H * cdiv(d->W, 32) * cdiv(Co, 64) <= 148;
 }
 // The tensor-core convolution of this layer, if it goes there.
 static bool plan_conv(const xconv_desc* d, bool dgrad, xconv_desc* e, TcConvPlan* t) {
