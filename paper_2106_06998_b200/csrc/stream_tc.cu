@@ -316,6 +316,7 @@ __global__ void __launch_bounds__(256, MT >= 4 ? 1 : 2) backprobe_stream_kernel(
   auto multiply = [&](int gb, int k0) {
 #pragma unroll
     for (int u = 0; u < KC; ++u) {
+      if (SPLIT && k0 + 16 * u >= p.K) break;         // (padding of the reduction: zeros)
       uint32_t a[SPLIT ? 2 * MT : MT][4];
 #pragma unroll
       for (int i = 0; i < (SPLIT ? 2 * MT : MT); ++i) {
