@@ -23,10 +23,9 @@ enum : unsigned int { WS_OK = 0u };
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// (`early` false: an ordinary launch, after the kernel before it has ended; the kernel's go-ahead still lets the next one start.)
 template <typename... KArgs, typename... Args>
-static inline cudaError_t launch_when(bool early, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                                      cudaStream_t st, Args&&... args) {
+static inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                     Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -36,13 +35,8 @@ static inline cudaError_t launch_when(bool early, void (*kernel)(KArgs...), dim3
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = early ? 1 : 0;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
-}
-template <typename... KArgs, typename... Args>
-static inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                                     Args&&... args) {
-  return launch_when(true, kernel, grid, block, smem, st, args...);
 }
 
 __device__ __forceinline__ float to_f(float v) { return v; }

@@ -410,12 +410,15 @@ __global__ void __launch_bounds__(256, MT >= 4 ? 1 : 2) backprobe_stream_kernel(
 
 static long cdiv_(long a, long b) { return (a + b - 1) / b; }
 
-// Whether a launch that reads so many bytes may start while the kernel before it still runs.  An SM that holds a CTA of that
-// kernel keeps its split of L1 and shared memory, for the tensor-core kernels nearly all shared memory, as long as it is not
-// empty, and the loads in flight of these kernels live in L1.  Sketch of 4 volumes of 48^3 behind the convolution 85 -> 65 us for
-// both, back-probe of 16 samples x 64 probes of 256 x 256 x 32 with the contraction 105 -> 97; a sketch of 1 MB x 70 MB behind
-// another sketch 18.5 -> 20.7, behind the convolution 30 -> 26.  Few bytes are read before that matters.
-static bool starts_early(long bytes) { return bytes < (16L << 20); }
+// These kernels want their SM's memory as L1, where their loads in flight live.  Without the wish they were placed on SMs still
+// split for the kernel before them (nearly all shared memory, for a tensor-core kernel) and kept that split as long as its CTAs
+// and theirs overlapped: sketch of 4 volumes of 48^3 behind the convolution 85 -> 65 us for both, back-probe of 16 samples x 64
+// probes of 256 x 256 x 32 with the contraction 105 -> 96, of 16 probes x 256 samples 116 -> 91.  (An ordinary launch, behind the end of
+// the kernel before, gives the same and costs 2 us.)  The rest is shared memory for two blocks.
+static cudaError_t want_l1(const void* kernel, size_t smem) {
+  const int share = (int)std::min<size_t>(100, std::max<size_t>(30, 2 * (smem + 2048) * 100 / (228 * 1024) + 1));
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, share);
+}
 
 // Measured against the tcgen05 sketch, other -> this, us: 8 x 4 (probes x samples), 3.5 M terms 178 -> 22; 512 x 8, 65536 terms
 // 14.5 -> 10.0; 256 x 16, 25600 terms 10.0 -> 8.0; 164 x 16, 93312 terms 13.7 -> 10.8; but 64 x 16, 2.1 M terms 76 -> 113 (a load
@@ -446,15 +449,13 @@ bool tc_plan_sketch_stream(const xconv_desc* d, bool seeded, StreamSketchPlan* p
 template <bool F16>
 static cudaError_t launch_sketch_stream(const StreamSketchPlan& pl, bool seeded, const SketchStream& q, cudaStream_t st) {
   const dim3 grid((unsigned)pl.splits, (unsigned)pl.tiles_m), block(256);
-  const bool early = starts_early(2 * q.K * (seeded ? q.N : q.M + q.N));
-  if (seeded) return pl.nt == 2 ? launch_when(early, sketch_stream_kernel<F16, 4, 2, true>, grid, block, 0, st, q)
-                                : launch_when(early, sketch_stream_kernel<F16, 4, 1, true>, grid, block, 0, st, q);
-  if (pl.mt == 4) return pl.nt == 2 ? launch_when(early, sketch_stream_kernel<F16, 4, 2, false>, grid, block, 0, st, q)
-                                    : launch_when(early, sketch_stream_kernel<F16, 4, 1, false>, grid, block, 0, st, q);
-  if (pl.mt == 2) return pl.nt == 2 ? launch_when(early, sketch_stream_kernel<F16, 2, 2, false>, grid, block, 0, st, q)
-                                    : launch_when(early, sketch_stream_kernel<F16, 2, 1, false>, grid, block, 0, st, q);
-  return pl.nt == 2 ? launch_when(early, sketch_stream_kernel<F16, 1, 2, false>, grid, block, 0, st, q)
-                    : launch_when(early, sketch_stream_kernel<F16, 1, 1, false>, grid, block, 0, st, q);
+  void (*kernel)(SketchStream) =
+      seeded ? (pl.nt == 2 ? sketch_stream_kernel<F16, 4, 2, true> : sketch_stream_kernel<F16, 4, 1, true>)
+      : pl.mt == 4 ? (pl.nt == 2 ? sketch_stream_kernel<F16, 4, 2, false> : sketch_stream_kernel<F16, 4, 1, false>)
+      : pl.mt == 2 ? (pl.nt == 2 ? sketch_stream_kernel<F16, 2, 2, false> : sketch_stream_kernel<F16, 2, 1, false>)
+                   : (pl.nt == 2 ? sketch_stream_kernel<F16, 1, 2, false> : sketch_stream_kernel<F16, 1, 1, false>);
+  const cudaError_t e = want_l1(reinterpret_cast<const void*>(kernel), 12 * 1024);      // (static shared memory)
+  return e != cudaSuccess ? e : launch_pdl(kernel, grid, block, 0, st, q);
 }
 
 xconv_status tc_run_sketch_stream(const xconv_desc* d, const StreamSketchPlan& pl, const void* X, const void* Z, float* part,
@@ -505,9 +506,9 @@ static cudaError_t launch_backprobe_stream(const BackprobeStream& q, bool seeded
              : q.K <= 16 ? backprobe_stream_kernel<F16, 1, false, 1, true, false>
              : q.K <= 32 ? backprobe_stream_kernel<F16, 1, false, 2, true, false>
              : q.K <= 64 ? backprobe_stream_kernel<F16, 1, false, 4, true, false> : backprobe_stream_kernel<F16, 1, false, 2, false, false>;
-  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
-  const bool early = starts_early(2 * q.Q * (seeded ? q.rows : q.K));      // (redrawn: what it writes)
-  return e != cudaSuccess ? e : launch_when(early, kernel, dim3(grid), dim3(256), smem, st, q);
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+  if (e == cudaSuccess) e = want_l1(reinterpret_cast<const void*>(kernel), smem);
+  return e != cudaSuccess ? e : launch_pdl(kernel, dim3(grid), dim3(256), smem, st, q);
 }
 
 xconv_status tc_run_backprobe_stream(const xconv_desc* d, const float* S, long s_row, long s_k, const void* dY, void* L,
