@@ -196,8 +196,8 @@ static WgradPlan plan_wgrad_core(const xconv_desc* d) {
   p.stream_bp = tc_backprobe_streams(&f, p.tc_bp);
   const xconv_desc c = planes_ct(d);    // the tensor-core contraction works plane by plane
   p.tc_ct = (tc_plan_wgrad(&c, &p.t) & 2) != 0;
-  // The contraction for few channels: wherever the other one does not go, and where that one leaves MMA rows empty or copies
-  // Z once per offset.  Measured, other -> this, us: 3 x 3, 32 -> 32 channels, 64 probes of 64 x 64: 27.6 -> 17.0, 128 -> 32
+  // The contraction for few channels: where the other one does not go (drained; if its channel blocks are not mostly padding, see
+  // halo_channels), and where that one leaves MMA rows empty or copies Z once per offset.  Measured, other -> this, us: 3 x 3, 32 -> 32 channels, 64 probes of 64 x 64: 27.6 -> 17.0, 128 -> 32
   // channels out 35 -> 22 (but 32 -> 256 31 -> 37, 128 -> 128 35 -> 41, 64 -> 64 20.8 -> 20.7); 5 x 5, 32 channels 58 -> 20,
   // 128: 36.4 -> 36.5; pointwise, 64 channels 12.6 -> 9.9, 128: 14.7 -> 19.4; 3 x 3 x 3, 32 -> 64 73 -> 30, 128 -> 128 38 -> 28,
   // 96 -> 96, a quarter of it padding, 43 -> 47.  (A list of zero blocks is only read by the other one.)
@@ -207,7 +207,7 @@ static WgradPlan plan_wgrad_core(const xconv_desc* d) {
   const bool whole = (d->Cin == 32 || d->Cin % 64 == 0) && (d->Cout == 32 || d->Cout % 64 == 0);
   const bool few = volumetric(d) ? most <= 128 && whole : d->KH == 3 ? d->Cout <= 32 : most <= 64;
   const bool other = p.tc_ct && (p.t.ct_masked || !few);
-  if (!other && tc_plan_halo(&e, &p.h)) {
+  if (!other && tc_plan_halo(&e, !p.tc_ct, &p.h)) {
     p.halo = true;
     const long px = (long)depth(d) * d->H * d->W * d->r;
     p.ct_bytes = align_up(p.h.part_bytes, 256) + padded_bytes(px, d->Cin) + padded_bytes(px, d->Cout);

@@ -52,7 +52,8 @@ struct TcHaloPlan {            // contraction of layers with few channels (contr
   int pw, ph, stages;         // patch; stages of the ring
   int cwa, cwb;               // channels per block of L and of Z
   int rows_on_a;              // L moved by image rows on the MMA rows, else one dy per work unit
-  int mt, mg_n, dy_n, dz_n, dz_per, ng_n, ng_per, a_blocks, cols;
+  int mt, mg_n, dy_n, dz_n, dz_per, ng_n, ng_per, j_n, j_per, a_blocks, cols;
+  int drain;                  // accumulators added up in registers every few k-steps
   uint32_t a_blk, b_blk;      // shared memory of a channel block
   long patches, splits, units;
   size_t part_bytes;
@@ -85,7 +86,7 @@ xconv_status tc_run_backprobe(const xconv_desc* d, const TcWgradPlan& p, const v
 xconv_status tc_run_contract(const xconv_desc* d, const TcWgradPlan& p, const void* L, const void* Z, float* dW,
                              float alpha, char* ws_head, char* part, cudaStream_t st);
 
-bool tc_plan_halo(const xconv_desc* d, TcHaloPlan* p);
+bool tc_plan_halo(const xconv_desc* d, bool drain, TcHaloPlan* p);
 // `cout_out`, `cin_out`: the channels of dW where d->Cout and d->Cin count padded ones.
 xconv_status tc_run_halo(const xconv_desc* d, const TcHaloPlan& p, const void* L, const void* Z, int cout_out, int cin_out, float* dW,
                          float alpha, char* ws_head, char* part, cudaStream_t st);

@@ -62,6 +62,33 @@ def test_contraction(dtype, r, Cin, Cout, D, H, W, K, KD):
     check("dW with chan_scale", got, flat * host(scale), 1e-4)
 
 
+@pytest.mark.parametrize("dtype,r,Cin,Cout,D,H,W,K,KD", [
+    ("bf16", 24, 16, 24, 1, 200, 210, 3, 1),   # long sums, one row tile; some rows of a patch per accumulator set
+    ("f16", 8, 3, 48, 1, 190, 200, 3, 1),      # two row tiles in one unit; padded input channels
+    ("bf16", 16, 48, 48, 1, 100, 100, 3, 1),   # the two row tiles as units
+    ("f16", 5, 16, 48, 1, 30, 45, 5, 1),       # three row tiles as units
+    ("bf16", 6, 48, 24, 1, 60, 77, 5, 1),      # pixel shifts in two units, the second with fewer
+    ("f16", 3, 24, 24, 12, 40, 44, 3, 3),      # one dz per unit
+    ("bf16", 60, 8, 16, 1, 5, 4, 3, 1),        # several patches per accumulator set, the last set with fewer
+    ("f16", 7, 200, 104, 1, 33, 40, 1, 1),     # pointwise, four channel blocks of columns
+    ("bf16", 2, 24, 104, 1, 33, 40, 1, 1),     # one 32-column chunk for two warps a quadrant
+])
+def test_drained_contraction_adds_up_like_float(dtype, r, Cin, Cout, D, H, W, K, KD):
+    """Channels off the multiples of 32.  An accumulator of the tensor cores holds 16 k-steps and loses less than a unit in its
+    last place, 2^-23, in each; the rest of the sum is float: 16 * 2^-23."""
+    g = np.random.Generator(np.random.PCG64([r, Cin, Cout, H, W, K, 3]))
+    geo = (D, H, W) if D > 1 else (H, W)
+    L, Z = (inputs.round_to_storage(g.standard_normal((r, c) + geo).astype(np.float32), dtype) for c in (Cout, Cin))
+    Ld, Zd = xb.to_device(L, dtype), xb.to_device(Z, dtype)
+    desc = xb.make_desc(8, Cin, Cout, H, W, r, Zd.dtype, K, D=D, KD=KD)
+    assert (Cin % 32 or Cout % 32) and xb.engine_for(desc, xb.OP_CONTRACT) == "tcgen05_" + dtype
+    dW, again = (xb.xconv_contract(Ld, Zd, kernel_size=K, kernel_depth=KD) for _ in range(2))
+    torch.cuda.synchronize()
+    want = O.wgrad_contract3d(L, Z, (KD, K, K)) if D > 1 else O.wgrad_contract(L, Z, K, K)
+    assert O.rel_fro(host(dW), want) < 16 * 2.0 ** -23
+    assert torch.equal(dW, again)
+
+
 def test_calls_in_a_row_on_layers_that_fill_tensor_memory():
     """Several CTAs of these layers fit one SM beside each other and each takes all of its tensor memory (25 offsets, 320
     columns), so a call's kernel starts while its columns are still held by the call before it.  The allocations have to be
