@@ -61,11 +61,11 @@ def test_seeded_sketch_and_estimate(dtype, r, B, C, H, W):
 
 @pytest.mark.parametrize("dtype,r,B,C,H,W", [
     ("bf16", 1, 1, 8, 16, 16),       # one row, one term
-    ("f16", 4, 8, 8, 17, 19),        # one k-step, columns that end inside a group
-    ("bf16", 16, 31, 64, 9, 9),      # two k-steps in one go
-    ("f16", 9, 64, 8, 24, 24),       # four
-    ("bf16", 12, 70, 128, 50, 50),   # a loop over the terms, the second round mostly padding; two groups per warp
-    ("bf16", 20, 21, 24, 11, 13),    # rows and terms the tcgen05 kernel does not take
+    ("f16", 4, 8, 8, 17, 19),        # columns that end inside a group
+    ("bf16", 16, 31, 64, 9, 9),      # 16 rows
+    ("f16", 9, 64, 8, 24, 24),       # (a multiple of 8 terms, of 64 columns: S rounded once)
+    ("bf16", 12, 70, 128, 50, 50),   # the second round of terms mostly padding; two groups per warp
+    ("bf16", 20, 21, 24, 11, 13),    # 32 rows
     ("f16", 50, 130, 40, 9, 11),
     ("bf16", 64, 3, 8, 31, 33),
 ])
@@ -80,6 +80,41 @@ def test_backprobe(dtype, r, B, C, H, W):
     torch.cuda.synchronize()
     check("L", host(L), O.backprobe(S, dY), TOL[dtype])
     assert torch.equal(L, L2)
+
+
+# Half a unit in the last place of the storage type: what the rounding of the result alone leaves, as a relative 2-norm.
+ROUNDING = {"bf16": 2.0 ** -9, "f16": 2.0 ** -12}
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f16"])
+@pytest.mark.parametrize("r,B,C,H,W,rounded", [
+    (4, 8, 16, 17, 20, True),        # one k-step in one go, half of it padding
+    (16, 16, 64, 5, 7, True),        # one whole k-step
+    (9, 24, 64, 9, 9, True),         # two, the second half padding
+    (16, 32, 8, 24, 24, True),       # two whole ones
+    (3, 40, 64, 9, 9, True),         # four, the last one padding
+    (16, 64, 8, 24, 24, True),
+    (12, 72, 128, 50, 52, True),     # a loop over the terms, two groups per warp
+    (16, 200, 64, 72, 72, True),
+    (16, 9, 64, 5, 7, False),        # 16 rows, S as two values
+    (12, 70, 128, 50, 52, False),
+    (17, 33, 24, 11, 13, False),     # 32 rows
+    (64, 65, 8, 17, 16, False),      # 64 rows
+])
+def test_backprobe_by_the_rounding_of_the_sketch(dtype, r, B, C, H, W, rounded):
+    """Which kernel a layer reaches shows in what is multiplied: S rounded to storage where the tcgen05 back-probe serves the
+    layer too (terms a multiple of 8, columns of 64), the float S elsewhere.  The entries of S lie a quarter of a unit off a
+    16-bit value, in one direction: against the wrong one of the two L is off by that (2^-9, 2^-12) and its rounding."""
+    assert rounded == (B % 8 == 0 and (C * H * W) % 64 == 0)
+    g = np.random.Generator(np.random.PCG64([r, B, C, H, W, 1]))
+    dY = inputs.round_to_storage((0.1 * g.standard_normal((B, C, H, W))).astype(np.float32), dtype)
+    unit = 2.0 ** -7 if dtype == "bf16" else 2.0 ** -10
+    S16 = inputs.round_to_storage((g.choice([-1.0, 1.0], (r, B)) * g.uniform(1.0, 1.99, (r, B))).astype(np.float32), dtype)
+    S = (S16 * (1.0 + 0.25 * unit)).astype(np.float32)
+    assert np.array_equal(inputs.round_to_storage(S, dtype), S16)
+    want, other = (O.backprobe(S16 if q else S, dY) for q in (rounded, not rounded))
+    L = host(xb.xconv_backprobe(torch.from_numpy(S).cuda(), xb.to_device(dY, dtype)))
+    assert O.rel_fro(L, want) < ROUNDING[dtype] < O.rel_fro(L, other)
 
 
 @pytest.mark.parametrize("dtype,bar", [("bf16", 2.0 ** -9), ("f16", 2.0 ** -12)])
@@ -98,3 +133,18 @@ def test_backprobe_keeps_the_float_sketch_where_the_tcgen05_kernel_does_not_go(d
     for j in range(2 if dtype == "f16" else 0, r):                  # (the smallest float16 rows are subnormal)
         if np.abs(want[j]).max() < 6e4 or dtype == "bf16":
             assert O.rel_fro(L[j], want[j]) < bar, j
+
+
+def test_a_call_of_streaming_kernels_alone_reports_its_own_outcome():
+    """On scratch memory whose header a timed-out call has written, through every streaming kernel by itself."""
+    lay = inputs.make_custom(4, 64, 64, 9, 9, 8, dtype="bf16", seed=3, z="gaussian", x="normal")
+    X, Z, dY = (xb.to_device(lay[k], "bf16") for k in ("X", "Z", "dY"))
+    desc = xb.make_desc(4, 64, 64, 9, 9, 8, torch.bfloat16)
+    ws = torch.zeros(max(xb.workspace_bytes(desc, o) for o in (xb.OP_SKETCH, xb.OP_SKETCH_SEEDED, xb.OP_WGRAD)), dtype=torch.uint8, device="cuda")
+    S, L = torch.empty((8, 4), device="cuda"), torch.empty((8, 64, 9, 9), dtype=torch.bfloat16, device="cuda", memory_format=torch.channels_last)
+    for call in (lambda: xb.sketch_into(desc, X, Z, S, ws), lambda: xb.sketch_seeded_into(desc, X, 7, S, ws),
+                 lambda: xb.backprobe_into(desc, S, dY, L, ws)):
+        assert xb.lib().xconv_selftest_wait_limit(ws.data_ptr(), ws.numel(), 5, torch.cuda.current_stream().cuda_stream) == 0
+        assert xb.workspace_status(ws) == 6                      # XCONV_ERR_TIMEOUT
+        call()
+        assert xb.workspace_status(ws) == 0
