@@ -9,8 +9,9 @@
 // loads): 64 KS multiply-adds for 3 + 2 KS loads, all of them broadcasts or conflict-free.  Of a block's THREADS threads TN
 // stand side by side in the channels (8 TN channels), the THREADS / TN groups on strips of a patch of SW strips x RH rows x NI
 // planes (NI > 1 for images smaller than a patch).  Input channels go by CK through shared memory, transposed so that the
-// pixels of a row are consecutive; where the pixels of the patch lie in memory is worked out once (`tab`).  At least two
-// blocks per SM: one loads while the other multiplies.
+// pixels of a row are consecutive; where the pixels of the patch lie in memory is worked out once (`tab`).  Two blocks of
+// 256 threads per SM, so that one loads while the other multiplies, except where their shared memory allows only one (3 x 3 x 3
+// layers with few channels out: up to 126 KB; the plan's cost does not know that).
 // The sums are taken in the order of conv_simt (same bits).  64 -> 64 channels, 32 x 32 images, batch 128: 560 -> 236 us (41
 // of the 68 TFLOP/s that register-only chains reach; three quarters of the rest is the last wave of blocks, then the
 // loads); 3 -> 64 channels of 112 x 112 images 457 -> 102 us; 5 x 5, 32 channels 891 -> 155 us.
