@@ -190,7 +190,7 @@ def _stream() -> int:
 
 
 def _capturing() -> bool:
-    return torch._C._cuda_isCurrentStreamCapturing()
+    return torch.cuda.is_current_stream_capturing()
 
 
 # Calls on different streams or from different host threads may overlap, so each of them has a scratch buffer of its own: per
