@@ -202,9 +202,10 @@ _WS_STREAMS = 8
 def workspace(nbytes: int, device) -> torch.Tensor:
     """A scratch buffer of at least ``nbytes`` on ``device`` for calls on the current stream: cached per host thread and
     stream, grown on demand.  While the stream is captured into a graph it is a new buffer, whose memory is the graph's."""
-    if _capturing():
+    stream = _stream()
+    if stream and _capturing():                 # (the default stream, 0, cannot be captured; asking takes as long as the rest)
         return torch.empty(max(nbytes, 256), dtype=torch.uint8, device=device)
-    key = (device, _stream())
+    key = (device, stream)
     try:
         buffers = _ws_cache.buffers
     except AttributeError:

@@ -102,3 +102,24 @@ def test_layers_on_two_streams_at_once(threads):
         assert len(g) == 30
         for out in g:
             assert all(torch.equal(a, b) for a, b in zip(w, out))
+
+
+def test_a_captured_step_has_scratch_memory_of_its_own():
+    """The public calls captured on a stream that has run them before: eager calls on that stream between the replays, of a layer
+    that needs more scratch, touch nothing that the graph uses."""
+    d, other = _layer(4, 8, 3, 48, (20, 24), 4, torch.float16), _layer(5, 32, 5, 64, (56, 56), 48, torch.float16)
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        want = [t.clone() for t in _step(d)]
+        graph = torch.cuda.CUDAGraph()
+        side.synchronize()
+        with torch.cuda.graph(graph, stream=side):
+            out = _step(d)
+        for _ in range(3):
+            for t in out:
+                t.zero_()
+            _step(other)
+            graph.replay()
+            _step(other)
+            side.synchronize()
+            assert all(torch.equal(a, b) for a, b in zip(want, out))
