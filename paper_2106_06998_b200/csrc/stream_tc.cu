@@ -317,7 +317,6 @@ __global__ void __launch_bounds__(256, MT >= 4 ? 1 : 2) backprobe_stream_kernel(
   auto multiply = [&](int gb, int k0) {
 #pragma unroll
     for (int u = 0; u < KC; ++u) {
-      if (SPLIT && k0 + 16 * u >= p.K) break;         // (padding of the reduction: zeros)
       uint32_t a[SPLIT ? 2 * MT : MT][4];
 #pragma unroll
       for (int i = 0; i < (SPLIT ? 2 * MT : MT); ++i) {
@@ -378,7 +377,8 @@ __global__ void __launch_bounds__(256, MT >= 4 ? 1 : 2) backprobe_stream_kernel(
           const bool last = k0 + 32 * KC >= p.K16;
           if (SEEDED) draw(grp, k0 + 16 * KC);
           else fetch(0, last ? grp + (long)gridDim.x * 8 : grp, last ? 0 : k0 + 32 * KC);
-          multiply(1, k0 + 16 * KC);
+          // (padding of the reduction: zeros; left out by halves, a test per k-step keeps the loads from running ahead)
+          if (!SPLIT || k0 + 16 * KC < p.K) multiply(1, k0 + 16 * KC);
         }
       }
       // accumulator columns 2t and 2t+1 of tile c are the columns 16 t + c and 16 t + 8 + c
