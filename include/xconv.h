@@ -87,9 +87,10 @@ typedef enum { XCONV_OP_FORWARD = 0, XCONV_OP_WGRAD = 1, XCONV_OP_DGRAD = 2, XCO
                XCONV_OP_SKETCH_SEEDED_GAUSSIAN = 9, XCONV_OP_WGRAD_SEEDED_GAUSSIAN = 10 } xconv_op;
 
 /* Which arithmetic engine a call will use for its dominant kernel: FP32 multiply-adds or the tensor cores (by tcgen05, or
- * by mma.sync in the kernels that stream few samples or few probes through registers), per storage type. */
+ * by mma.sync in the kernels that stream few samples or few probes through registers), per storage type.  (F32: float values
+ * as three bfloat16 parts each, summed as precisely as by FP32 multiply-adds.) */
 typedef enum { XCONV_ENGINE_NONE = 0, XCONV_ENGINE_SIMT_F32 = 1, XCONV_ENGINE_TCGEN05_BF16 = 2,
-               XCONV_ENGINE_TCGEN05_F16 = 3 } xconv_engine;
+               XCONV_ENGINE_TCGEN05_F16 = 3, XCONV_ENGINE_TCGEN05_F32 = 4 } xconv_engine;
 
 /* One convolutional layer: stride 1, dilation 1, one group, no bias, "same" output size
  * (2*pad_h = KH-1, 2*pad_w = KW-1; KH = KW in {1, 3, 5}).

@@ -20,7 +20,7 @@ LIB_PATH = os.path.join(_HERE, "libxconv.so")
 XCONV_F32, XCONV_BF16, XCONV_F16 = 0, 1, 2
 OP_FORWARD, OP_WGRAD, OP_DGRAD, OP_SKETCH, OP_BACKPROBE, OP_CONTRACT, OP_SKETCH_SEEDED, OP_WGRAD_SEEDED, OP_WGRAD_INDEPENDENT = 0, 1, 2, 3, 4, 5, 6, 7, 8
 OP_SKETCH_SEEDED_GAUSSIAN, OP_WGRAD_SEEDED_GAUSSIAN = 9, 10
-ENGINE_NAMES = {0: "none", 1: "simt_f32", 2: "tcgen05_bf16", 3: "tcgen05_f16"}
+ENGINE_NAMES = {0: "none", 1: "simt_f32", 2: "tcgen05_bf16", 3: "tcgen05_f16", 4: "tcgen05_f32"}
 STATUS_OK = 0
 
 # every symbol include/xconv.h declares

@@ -10,6 +10,7 @@
 #include "common.cuh"
 #include "simt_kernels.cuh"
 #include "conv_fma.h"
+#include "conv_split.h"
 #include "tc_api.h"
 #include <type_traits>
 
@@ -190,8 +191,8 @@ static WgradPlan plan_wgrad_core(const xconv_desc* d) {
   const size_t lsz = d->dtype == XCONV_F32 ? 4 : 2;
   p.l_off = WS_HEADER;
   p.sb_off = p.l_off + align_up((size_t)d->r * Q * lsz, 256);
-  p.part_off = p.sb_off + align_up((size_t)d->r * d->B * 2, 256);
   const xconv_desc f = flat(d);
+  p.part_off = p.sb_off + align_up((size_t)d->r * d->B * 2, 256);
   p.tc_bp = (tc_plan_wgrad(&f, &p.tb) & 1) != 0;
   p.stream_bp = tc_backprobe_streams(&f, p.tc_bp);
   const xconv_desc c = planes_ct(d);    // the tensor-core contraction works plane by plane
@@ -265,10 +266,11 @@ static SwappedWgrad plan_wgrad_swapped(const xconv_desc* d) {
   return w;
 }
 
-static WgradPlan plan_wgrad(const xconv_desc* d) {
+static WgradPlan plan_wgrad(const xconv_desc* d, SwappedWgrad* swapped = nullptr) {
   WgradPlan p = plan_wgrad_core(d);
   const SwappedWgrad w = plan_wgrad_swapped(d);
   if (w.on) p.bytes = std::max(p.bytes, w.bytes);
+  if (swapped) *swapped = w;
   return p;
 }
 
@@ -533,6 +535,19 @@ static xconv_status run_conv_simt(const xconv_desc* d, bool dgrad, const void* i
   return check_launch();
 }
 
+// Float layers whose convolution goes to the tensor cores (conv_split.cu): all but the smallest.  The call alone is faster from a
+// microsecond of multiply-adds on (us, multiply-adds -> this, 160 layers: 8 x 16 -> 16 channels of 32 x 32 12.5 -> 8.6, 4 x 192 -> 48, 37 x 37,
+// 1 x 1 14.5 -> 8.9, larger ones 236 -> 57; but 9 x 1 -> 128 channels of 13 x 13, 1 x 1, with the copies before it 15.5 -> 18.6), but it
+// is a launch more: a training step of the first of these, host and all, 57.4 -> 61.4.  3000: two of 75 multiply-adds a clock and SM.
+static bool plan_conv_f32(const xconv_desc* d, bool dgrad, ConvSplitPlan* p) {
+  const double macs = (double)d->B * depth(d) * d->H * d->W * d->Cin * d->Cout * kdepth(d) * d->KH * d->KW;
+  if (d->dtype != XCONV_F32 || macs <= 3000.0 * 148 * 75) return false;
+  // Image channels: a block of 16 is nearly all padding.  3 x 3, 1 or 3 -> 64 to 256 channels 376 -> 257, 69 -> 48, 38 -> 31 us, but 3 -> 16
+  // 142 -> 290, 1 -> 32 55 -> 72, 5 x 5 3 -> 32 388 -> 889, 3 x 3 x 3 3 -> 64 109 -> 145.
+  if ((dgrad ? d->Cout : d->Cin) < 8 && ((dgrad ? d->Cin : d->Cout) < 64 || d->KH == 5 || kdepth(d) == 3)) return false;
+  return plan_conv_split(d, dgrad, p);
+}
+
 // The convolution with its input channels padded (see pad8) and the scratch its copies take behind the header; the output
 // channels have to be a multiple of 8 themselves.
 static xconv_desc conv_padded(const xconv_desc* d) {
@@ -552,6 +567,11 @@ static bool plan_conv(const xconv_desc* d, bool dgrad, xconv_desc* e, TcConvPlan
   *e = conv_padded(d);
   return (!dgrad || d->Cin % 8 == 0) && !conv_tiny(d, dgrad) && tc_plan_conv(e, dgrad, t);
 }
+// (Scratch that a call cannot do without; a float layer with less than `conv_ws_wish` stays on multiply-adds.)
+static size_t conv_ws_wish(const xconv_desc* d, bool dgrad) {
+  ConvSplitPlan p;
+  return plan_conv_f32(d, dgrad, &p) ? WS_HEADER + p.bytes : WS_HEADER;
+}
 static size_t conv_ws_bytes(const xconv_desc* d, bool dgrad) {
   xconv_desc e;
   TcConvPlan t;
@@ -561,7 +581,11 @@ static size_t conv_ws_bytes(const xconv_desc* d, bool dgrad) {
 }
 
 static xconv_status run_conv(const xconv_desc* d, bool dgrad, const void* in, const void* Wt, void* out,
-                             char* ws, cudaStream_t st) {
+                             char* ws, size_t ws_bytes, cudaStream_t st) {
+  ConvSplitPlan f;
+  if (plan_conv_f32(d, dgrad, &f) && ws_bytes >= WS_HEADER + f.bytes)
+    return run_conv_split(d, f, dgrad, static_cast<const float*>(in), static_cast<const float*>(Wt), static_cast<float*>(out), ws,
+                          ws + WS_HEADER, st);
   TcConvPlan t;
   xconv_desc e;
   if (plan_conv(d, dgrad, &e, &t)) {
@@ -639,12 +663,12 @@ static bool wgrad_redraws(const xconv_desc* d) {
 // `seed` != nullptr (only where wgrad_redraws holds): Z is not read.
 static xconv_status run_wgrad(const xconv_desc* d, const float* S, const void* dY, const void* Z, float* dW,
                               void* ws, size_t ws_bytes, cudaStream_t st, const unsigned long long* seed = nullptr) {
-  const WgradPlan p = plan_wgrad(d);
+  SwappedWgrad sw;
+  const WgradPlan p = plan_wgrad(d, &sw);
   xconv_status s = check_ws(ws, ws_bytes, p.bytes);
   if (s != XCONV_OK) return s;
   char* w = static_cast<char*>(ws);
   const float alpha = 1.0f / (float)d->r;
-  const SwappedWgrad sw = plan_wgrad_swapped(d);
   if (sw.on) {
     // Xr = S^T Z, then the offset contraction over the batch (see plan_wgrad_swapped)
     if ((s = validate(&sw.d1)) != XCONV_OK || (s = validate(&sw.d2)) != XCONV_OK) return s;
@@ -756,7 +780,7 @@ extern "C" {
 size_t xconv_workspace_bytes(const xconv_desc* desc, int op) {
   if (validate(desc) != XCONV_OK) return 0;
   switch (op) {
-    case XCONV_OP_FORWARD: return std::max(plan_sketch(desc).bytes, conv_ws_bytes(desc, false));
+    case XCONV_OP_FORWARD: return std::max({plan_sketch(desc).bytes, conv_ws_bytes(desc, false), conv_ws_wish(desc, false)});
     case XCONV_OP_SKETCH: return plan_sketch(desc).bytes;
     case XCONV_OP_WGRAD_SEEDED: return plan_wgrad(desc).bytes + (wgrad_redraws(desc) ? 0 : probes_bytes(desc));
     case XCONV_OP_SKETCH_SEEDED: {
@@ -768,7 +792,7 @@ size_t xconv_workspace_bytes(const xconv_desc* desc, int op) {
     case XCONV_OP_WGRAD:
     case XCONV_OP_BACKPROBE:
     case XCONV_OP_CONTRACT: return plan_wgrad(desc).bytes;
-    case XCONV_OP_DGRAD: return WS_HEADER;      // the convolutions need the status header only
+    case XCONV_OP_DGRAD: return conv_ws_wish(desc, true);
     case XCONV_OP_WGRAD_INDEPENDENT: return validate_indep(desc) == XCONV_OK ? plan_indep(desc).bytes : 0;
     default: return 0;
   }
@@ -777,6 +801,7 @@ size_t xconv_workspace_bytes(const xconv_desc* desc, int op) {
 int xconv_engine_for(const xconv_desc* desc, int op) {
   if (validate(desc) != XCONV_OK) return XCONV_ENGINE_NONE;
   const int tc = desc->dtype == XCONV_F16 ? XCONV_ENGINE_TCGEN05_F16 : XCONV_ENGINE_TCGEN05_BF16;
+  const int f32 = XCONV_ENGINE_TCGEN05_F32;
   switch (op) {
     case XCONV_OP_SKETCH: {
       const SketchPlan p = plan_sketch(desc);
@@ -795,6 +820,8 @@ int xconv_engine_for(const xconv_desc* desc, int op) {
     case XCONV_OP_DGRAD: {
       TcConvPlan t;
       xconv_desc e;
+      ConvSplitPlan f;
+      if (plan_conv_f32(desc, op == XCONV_OP_DGRAD, &f)) return f32;
       return plan_conv(desc, op == XCONV_OP_DGRAD, &e, &t) ? tc : XCONV_ENGINE_SIMT_F32;
     }
     default: return XCONV_ENGINE_NONE;
@@ -965,7 +992,7 @@ xconv_status xconv_forward(const xconv_desc* desc, const void* X, const void* W,
   if (!aligned16(ws)) return XCONV_ERR_ALIGNMENT;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   new_call();
-  s = run_conv(desc, false, X, W, Y, static_cast<char*>(ws), st);
+  s = run_conv(desc, false, X, W, Y, static_cast<char*>(ws), ws_bytes, st);
   if (s != XCONV_OK) return s;
   return run_sketch(desc, X, Z, sketch, ws, ws_bytes, st);
 }
@@ -1025,7 +1052,7 @@ xconv_status xconv_dgrad(const xconv_desc* desc, const void* dY, const void* W, 
   if (!ws || ws_bytes < WS_HEADER) return XCONV_ERR_WORKSPACE;
   if (!aligned16(ws)) return XCONV_ERR_ALIGNMENT;
   new_call();
-  return run_conv(desc, true, dY, W, dX, static_cast<char*>(ws), static_cast<cudaStream_t>(cuda_stream));
+  return run_conv(desc, true, dY, W, dX, static_cast<char*>(ws), ws_bytes, static_cast<cudaStream_t>(cuda_stream));
 }
 
 // Arena layout of the host-buffer entry point: X | dY | Z | S | dW | workspace, each 256-aligned.

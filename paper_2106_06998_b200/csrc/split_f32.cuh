@@ -1,0 +1,159 @@
+// Float operands for the tensor cores: every float as the sum of three bfloat16 values,
+//
+//   x = h + m + l,   h = rn(x), m = rn(x - h), l = rn(x - h - m)      (8 + 8 + 8 significand bits: exact)
+//
+// and a product of two floats as the six products hh, hm, mh, hl, mm, lh of their parts (each exact in a float; the three
+// left out are below 2^-25 of the product together).  What keeps the sums as precise as FP32 multiply-adds is where they are
+// taken: the accumulators of the tensor cores are not rounded to nearest and lose about 2e-8 of their value with every MMA,
+// so the products hh are summed apart from the small ones, or behind them, in chains of a few MMAs, and the chains are added in
+// float registers (see the kernels for the errors measured).
+//
+// A value that no part can hold as such -- an infinity, NaN, a finite one that rounds up to an infinity -- leaves NaN in one of
+// its parts, so every sum it enters becomes NaN, and no other one: the kernels take sums that are not finite again by plain
+// multiply-adds.  (Below 2^-110 the last part runs out of exponents: what is lost there is 2^-134 in itself.)
+#pragma once
+
+#include "common.cuh"
+#include "tc_ptx.cuh"
+
+namespace xconv {
+
+// The parts of four neighbouring floats, packed in pairs.
+struct Split4 { uint2 h, m, l; };
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+__device__ __forceinline__ float low_f(uint32_t v) { return __uint_as_float(v << 16); }
+__device__ __forceinline__ float high_f(uint32_t v) { return __uint_as_float(v & 0xFFFF0000u); }
+__device__ __forceinline__ Split4 split4(float4 v) {
+  Split4 s;
+  s.h.x = pack_bf16(v.x, v.y); s.h.y = pack_bf16(v.z, v.w);
+  v.x -= low_f(s.h.x); v.y -= high_f(s.h.x); v.z -= low_f(s.h.y); v.w -= high_f(s.h.y);
+  s.m.x = pack_bf16(v.x, v.y); s.m.y = pack_bf16(v.z, v.w);
+  v.x -= low_f(s.m.x); v.y -= high_f(s.m.x); v.z -= low_f(s.m.y); v.w -= high_f(s.m.y);
+  s.l.x = pack_bf16(v.x, v.y); s.l.y = pack_bf16(v.z, v.w);
+  return s;
+}
+__device__ __forceinline__ void st_shared_v2(uint32_t addr, uint2 v) {
+  asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(v.x), "r"(v.y) : "memory");
+}
+// Byte offset of byte `b` of tile row `row` (2^rbs bytes a row, swizzled as the copy engine and the MMA descriptors have it).
+__device__ __forceinline__ uint32_t swizzled(int rbs, uint32_t row, uint32_t b) {
+  return (row << rbs) + (b ^ (((row >> (7 - rbs)) & ((1u << (rbs - 4)) - 1u)) << 4));
+}
+
+// Loads of 16 columns each, and the wait for them (the registers pass through it, so that nothing reads them before).
+__device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t (&v)[16]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+               "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]),
+                 "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]) : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&v)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]), "+r"(v[8]), "+r"(v[9]),
+                 "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]) :: "memory");
+}
+
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+}
+
+// The roles of a block's 24 warps (80 registers a thread): 0 copies operands that were split before, 1 and 2 issue MMAs -- the chains of
+// accumulator set 0 and those of set 1, since one warp's instructions (some 40 clocks an MMA, and the waits between) do not keep the
+// tensor pipe busy beside the other warps -- 3 copies the floats, 4..11 add chains up, two per quarter of the MMA rows, 12..23 convert.
+constexpr int SP_THREADS = 768, SP_LOAD = 3, SP_EPILOGUE = 4, SP_CONVERT = 12, SP_CONVERTERS = 384;
+constexpr int SP_MAX_N = 64;                         // columns of a group (two groups of 16 per epilogue warp)
+constexpr int SP_FLOATS = 4;                         // float boxes under way at most
+
+// A box of floats as the copy engine left it at `src` (2^QSHIFT pieces of four per position, one position behind the other), converted to
+// three tiles of 2^RBS bytes a row in blocks `block` bytes apart, the parts `plane` bytes apart.  Position i goes to row i, or with PITCH to
+// row i + (KS - 1) floor(i / width): `gap` = KS - 1, `inv` = ceil(2^20 / width).  By the twelve conversion warps; some 40 instructions for four
+// values (with copies of single pieces by the threads, their addresses and bounds, it was 100, and the conversion bounded every kernel).
+template <int RBS, int QSHIFT, bool PITCH>
+__device__ __forceinline__ void split_box(uint32_t src, int positions, uint32_t dst, uint32_t plane, uint32_t block, uint32_t gap, uint32_t inv) {
+  constexpr int U = 4;
+  const int tid = threadIdx.x - SP_CONVERT * 32, items = positions << QSHIFT;
+  const uint32_t q = (uint32_t)tid & ((1u << QSHIFT) - 1u), byte = (q & ((1u << (RBS - 3)) - 1u)) * 8;
+  const uint32_t to = dst + (QSHIFT > RBS - 3 ? (q >> (RBS - 3)) * block : 0u);
+  src += (uint32_t)tid * 16;
+  for (int i = tid; i < items; i += U * SP_CONVERTERS, src += U * SP_CONVERTERS * 16) {
+    float4 v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (u == 0 || i + u * SP_CONVERTERS < items)
+        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[u].x), "=f"(v[u].y), "=f"(v[u].z), "=f"(v[u].w)
+                     : "r"(src + u * SP_CONVERTERS * 16) : "memory");
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (u > 0 && i + u * SP_CONVERTERS >= items) break;
+      uint32_t row = (uint32_t)(i + u * SP_CONVERTERS) >> QSHIFT;
+      if (PITCH) row += ((row * inv) >> 20) * gap;
+      const Split4 s = split4(v[u]);
+      const uint32_t at = to + swizzled(RBS, row, byte);
+      st_shared_v2(at, s.h);
+      st_shared_v2(at + plane, s.m);
+      st_shared_v2(at + 2 * plane, s.l);
+    }
+  }
+}
+// What the converters do when a stage's tiles are written and its floats read.
+__device__ __forceinline__ void split_stage_done(uint64_t* full, uint64_t* floats_empty) {
+  fence_async_smem();
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) { mbar_arrive(full); mbar_arrive(floats_empty); }
+}
+__device__ __forceinline__ bool split_wait(uint64_t* bar, uint32_t parity, unsigned int* status, unsigned int tag) {
+  bool ok = true;
+  if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, status, tag);
+  return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+}
+__device__ __forceinline__ void split_zero(uint32_t base, uint32_t bytes) {
+  for (uint32_t i = threadIdx.x * 16; i < bytes; i += SP_THREADS * 16)
+    asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(base + i), "r"(0) : "memory");
+  fence_async_smem();
+}
+// An accumulator set's three groups of n columns added to the sums of an epilogue warp's column groups (`half`, `half` + 2 of 16).
+__device__ __forceinline__ void split_add_set(uint32_t set, uint32_t n, int half, float (&sum)[2][16]) {
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const uint32_t c = (uint32_t)(half + 2 * k) * 16;
+    if (c >= n) break;
+    uint32_t x[16], y[16];
+    tmem_ld16_issue(set + n + c, x);
+    tmem_ld16_issue(set + 2 * n + c, y);
+    tmem_ld_wait(x); tmem_ld_wait(y);
+    float small[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) small[e] = __uint_as_float(x[e]) + __uint_as_float(y[e]);
+    tmem_ld16_issue(set + c, x);
+    tmem_ld_wait(x);
+#pragma unroll
+    for (int e = 0; e < 16; ++e) sum[k][e] += __uint_as_float(x[e]) + small[e];
+  }
+}
+
+static inline uint32_t up1k(uint32_t v) { return (v + 1023u) & ~1023u; }
+// Clocks of the three MMAs of a k-step with n columns per group: the tensor pipe's half clock per column, or shared memory's 128 bytes a clock.
+static inline long split_kstep_clocks(int n) {
+  long c = 0;
+  for (int g = 1; g <= 3; ++g) c += std::max(g * n / 2, 32 + g * n / 4);
+  return c;
+}
+
+// A tensor map over floats.
+static inline bool make_map_f32(CUtensorMap* m, const void* base, int rank, const uint64_t* dims, const uint64_t* strides, const uint32_t* box,
+                         CUtensorMapSwizzle swizzle) {
+  PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
+  if (!fn) return false;
+  cuuint32_t estr[5] = {1, 1, 1, 1, 1}, bx[5];
+  cuuint64_t d[5], st[4];
+  for (int i = 0; i < rank; ++i) { d[i] = dims[i]; bx[i] = box[i]; }
+  for (int i = 0; i + 1 < rank; ++i) st[i] = strides[i];
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, (cuuint32_t)rank, const_cast<void*>(base), d, st, bx, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+}  // namespace xconv
