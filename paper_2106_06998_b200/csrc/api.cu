@@ -11,6 +11,7 @@
 #include "simt_kernels.cuh"
 #include "conv_fma.h"
 #include "conv_split.h"
+#include "contract_split.h"
 #include "tc_api.h"
 #include <type_traits>
 
@@ -177,12 +178,21 @@ struct WgradPlan {
   bool stream_bp;                      // back-probe of few rows (stream_tc.cu)
   bool halo;                           // contraction of few channels (contract_tc.cu) instead of the one of tc_kernels.cu
   TcHaloPlan h;                        // ... on the layer with its channels padded to multiples of 8
+  bool split; ContractSplitPlan c;     // contraction of float layers on the tensor cores (contract_split.cu)
   size_t ct_bytes;                     // scratch of the contraction: partial sums, padded copies
   int splits; long items_per_split;    // simt contraction
   TcWgradPlan t;                       // tcgen05: contraction fields (planned on the per-plane layer)
   TcWgradPlan tb;                      // tcgen05: back-probe fields (planned on the flattened layer)
   size_t l_off, sb_off, part_off, bytes;
 };
+
+// Float layers whose contraction goes to the tensor cores (contract_split.cu).  It was faster on every one of 160 layers (us: 84 -> 72 to
+// 2680 -> 520, two thirds of them more than threefold), by a few microseconds only where the multiply-adds (70 a clock and SM on
+// tiles of 64 x 32 channels and 32 pixels) take less than eight: those layers keep the kernel that they are known by.
+static bool plan_contract_f32(const xconv_desc* d, ContractSplitPlan* p) {
+  const double macs = (double)d->r * depth(d) * d->H * cdiv(d->W, 32) * 32 * kdepth(d) * d->KH * d->KW * align_up(d->Cin, 64) * align_up(d->Cout, 32);
+  return d->dtype == XCONV_F32 && macs > 15000.0 * 148 * 70 && plan_contract_split(d, p);
+}
 
 static WgradPlan plan_wgrad_core(const xconv_desc* d) {
   WgradPlan p{};
@@ -217,6 +227,12 @@ static WgradPlan plan_wgrad_core(const xconv_desc* d) {
   }
   if (p.tc_ct) {
     p.ct_bytes = align_up(p.t.part_bytes, 256);
+    p.bytes = p.part_off + p.ct_bytes;
+    return p;
+  }
+  if (plan_contract_f32(d, &p.c)) {
+    p.split = true;
+    p.ct_bytes = align_up(p.c.bytes, 256);
     p.bytes = p.part_off + p.ct_bytes;
     return p;
   }
@@ -636,6 +652,8 @@ static xconv_status run_contract(const xconv_desc* d, const WgradPlan& p, const 
     if (s != XCONV_OK) return s;
     return tc_run_halo(&e, p.h, L, Z, d->Cout, d->Cin, dW, alpha, w, part, st);
   }
+  if (p.split)
+    return run_contract_split(d, p.c, static_cast<const float*>(L), static_cast<const float*>(Z), dW, alpha, w, part, st);
   if (p.tc_ct) {
     const xconv_desc c = planes_ct(d);
     return tc_run_contract(&c, p.t, L, Z, dW, alpha, w, part, st);
@@ -810,7 +828,7 @@ int xconv_engine_for(const xconv_desc* desc, int op) {
     case XCONV_OP_WGRAD:
     case XCONV_OP_CONTRACT: {
       const WgradPlan p = plan_wgrad(desc);
-      return p.halo || p.tc_ct ? tc : XCONV_ENGINE_SIMT_F32;
+      return p.split ? f32 : p.halo || p.tc_ct ? tc : XCONV_ENGINE_SIMT_F32;
     }
     case XCONV_OP_BACKPROBE: {
       const WgradPlan p = plan_wgrad(desc);

@@ -54,3 +54,24 @@ def test_convolution(B, Cin, Cout, D, H, W, K, KD):
     small, dX2 = torch.empty(256, dtype=torch.uint8, device="cuda"), torch.empty_like(dX)
     xb.dgrad_into(desc, d["dY"], d["W"], dX2, small)
     check("dX without scratch", host(dX2), dXo, 1e-5)
+
+
+@pytest.mark.parametrize("r,Cin,Cout,D,H,W,K,KD", [
+    (40, 64, 64, 1, 31, 33, 3, 1),       # L moved by rows
+    (50, 33, 130, 1, 14, 30, 3, 1),      # one dy per unit, padded copies, channels behind whole tiles
+    (300, 3, 64, 1, 7, 7, 3, 1),         # images narrower than a k-step
+    (20, 24, 48, 1, 40, 29, 5, 1),       # pixel shifts in two units, two row tiles
+    (120, 72, 40, 1, 40, 40, 1, 1),      # pointwise, two blocks of columns
+    (120, 40, 200, 1, 40, 41, 1, 1),     # ... and two row tiles
+    (6, 20, 36, 9, 12, 17, 3, 3),
+])
+def test_contraction(r, Cin, Cout, D, H, W, K, KD):
+    geo = (D, H, W) if D > 1 else (H, W)
+    L, Z = _n((r, Cout) + geo, 4), _n((r, Cin) + geo, 5)
+    desc = xb.make_desc(1, Cin, Cout, H, W, r, torch.float32, K, D=D, KD=KD)
+    assert xb.engine_for(desc, xb.OP_CONTRACT) == "tcgen05_f32"
+    scale = torch.rand(Cin, device="cuda") + 0.5
+    dW = xb.xconv_contract(xb.to_device(L, "f32"), xb.to_device(Z, "f32"), kernel_size=K, kernel_depth=KD, chan_scale=scale)
+    want = O.wgrad_contract3d(L, Z, (KD, K, K)) if D > 1 else O.wgrad_contract(L, Z, K, K)
+    want = want * r * host(scale).reshape((1, -1) + (1,) * (want.ndim - 2))
+    check("dW", host(dW), want, TOL)
