@@ -12,6 +12,7 @@
 #include "conv_fma.h"
 #include "conv_split.h"
 #include "contract_split.h"
+#include "gemm_split.h"
 #include "tc_api.h"
 #include <type_traits>
 
@@ -104,10 +105,28 @@ static const size_t WS_HEADER = 256;   // word 0: status left by pipelined kerne
 struct SketchPlan {
   bool tc;
   bool stream; StreamSketchPlan s;     // few samples or few probes (stream_tc.cu)
+  bool split; GemmSplitPlan g;         // float rows on the tensor cores (gemm_split.cu)
   int splits; long k_per_split;        // simt
   TcSketchPlan t;                      // tcgen05
   size_t part_off, bytes;
 };
+
+// Float layers whose sketch and back-probe go to the tensor cores (gemm_split.cu): where their clocks, at the part of the rates they were
+// measured at and with 5000 more for launches and first copies, are below those of the multiply-adds.  Those take 70 a clock
+// and SM on tiles of 64 x 64 (sketch), and in the back-probe 310 clocks a term of a wave of blocks, or the bytes at 16 a clock and SM.
+// On 160 layers this picks within 1.5 % (sketch) and 1 % (back-probe) of the faster kernel of each; us, multiply-adds -> this:
+// sketch 128 x 64 rows, 65536 terms 39 -> 26, 512 x 4, 1.6 M terms 3500 -> 1300, but 86 x 128 rows, 4624 terms 10.4 -> 14.2; back-probe
+// 16 rows, 512 terms 84 -> 17, 256 rows, 64 terms, 48672 positions 57 -> 41, but 16 rows, 4 terms, 3.3 M positions 66 -> 308.
+static bool plan_sketch_f32(const xconv_desc* d, GemmSplitPlan* p) {
+  const double macs = (double)align_up(d->r, 64) * align_up(d->B, 64) * depth(d) * d->H * d->W * d->Cin;
+  return d->dtype == XCONV_F32 && plan_sketch_split(d, p) && 1.8 * p->clocks + 5000.0 < macs / (148.0 * 70.0);
+}
+static bool plan_backprobe_f32(const xconv_desc* d, GemmSplitPlan* p) {
+  if (d->dtype != XCONV_F32 || !plan_backprobe_split(d, p)) return false;
+  const double Q = (double)depth(d) * d->H * d->W * d->Cout;
+  const double waves = (double)cdiv(cdiv((long)Q, 1024) * cdiv(d->r, 16), 296);
+  return 1.5 * p->clocks + 5000.0 < std::max(waves * d->B * 310.0, ((double)d->B + d->r) * 4.0 * Q / (148.0 * 16.0));
+}
 
 static SketchPlan plan_sketch(const xconv_desc* d_, bool seeded = false) {
   const xconv_desc fl = flat(d_);
@@ -123,6 +142,11 @@ static SketchPlan plan_sketch(const xconv_desc* d_, bool seeded = false) {
   p.tc = tc_plan_sketch(d, &p.t, seeded && tc_sketch_can_redraw(d));
   if (p.tc) {
     p.bytes = p.part_off + align_up(p.t.part_bytes, 256);
+    return p;
+  }
+  if (plan_sketch_f32(d, &p.g)) {
+    p.split = true;
+    p.bytes = p.part_off + align_up(p.g.bytes, 256);
     return p;
   }
   const long tiles = cdiv(d->r, 64) * cdiv(d->B, 64);
@@ -175,6 +199,7 @@ static xconv_status pad_channels(const void*& t, long rows, int C, char*& ws, cu
 
 struct WgradPlan {
   bool tc_bp, tc_ct;
+  bool split_bp; GemmSplitPlan g;      // back-probe of float layers on the tensor cores (gemm_split.cu)
   bool stream_bp;                      // back-probe of few rows (stream_tc.cu)
   bool halo;                           // contraction of few channels (contract_tc.cu) instead of the one of tc_kernels.cu
   TcHaloPlan h;                        // ... on the layer with its channels padded to multiples of 8
@@ -202,7 +227,8 @@ static WgradPlan plan_wgrad_core(const xconv_desc* d) {
   p.l_off = WS_HEADER;
   p.sb_off = p.l_off + align_up((size_t)d->r * Q * lsz, 256);
   const xconv_desc f = flat(d);
-  p.part_off = p.sb_off + align_up((size_t)d->r * d->B * 2, 256);
+  p.split_bp = plan_backprobe_f32(&f, &p.g);
+  p.part_off = p.sb_off + align_up(p.split_bp ? p.g.bytes : (size_t)d->r * d->B * 2, 256);
   p.tc_bp = (tc_plan_wgrad(&f, &p.tb) & 1) != 0;
   p.stream_bp = tc_backprobe_streams(&f, p.tc_bp);
   const xconv_desc c = planes_ct(d);    // the tensor-core contraction works plane by plane
@@ -277,7 +303,7 @@ static SwappedWgrad plan_wgrad_swapped(const xconv_desc* d) {
   w.x_off = WS_HEADER;
   w.st_off = w.x_off + align_up((size_t)d->B * depth(d) * d->H * d->W * d->Cin * es, 256);
   w.sb_off = w.st_off + align_up((size_t)d->r * d->B * 4, 256);
-  w.part_off = w.sb_off + align_up((size_t)d->r * d->B * 2, 256);
+  w.part_off = w.sb_off + align_up(w.p1.split_bp ? w.p1.g.bytes : (size_t)d->r * d->B * 2, 256);
   w.bytes = w.part_off + w.p2.ct_bytes;
   return w;
 }
@@ -471,6 +497,11 @@ static xconv_status run_sketch(const xconv_desc* d_, const void* X, const void* 
     return s == XCONV_OK ? run_reduce(part, S, (long)d->r * d->B, p.s.splits, 1.0f, nullptr, 1, st) : s;
   }
   if (p.tc) return tc_run_sketch(d, p.t, X, Z, S, w, w + p.part_off, st, redraw ? seed : nullptr);
+  if (p.split) {
+    float* part = reinterpret_cast<float*>(w + p.part_off);
+    xconv_status s = run_sketch_split(d, p.g, static_cast<const float*>(X), static_cast<const float*>(Z), part, w, st);
+    return s == XCONV_OK ? run_reduce(part, S, (long)d->r * d->B, (int)p.g.splits, 1.0f, nullptr, 1, st) : s;
+  }
   return d->dtype == XCONV_F32 ? run_sketch_simt<float>(d, p, X, Z, S, w, st)
          : d->dtype == XCONV_F16 ? run_sketch_simt<f16>(d, p, X, Z, S, w, st)
                                  : run_sketch_simt<bf16>(d, p, X, Z, S, w, st);
@@ -621,6 +652,10 @@ static xconv_status run_conv(const xconv_desc* d, bool dgrad, const void* in, co
 // L = S dY^T into `L`; `Sb` receives the bfloat16 copy of S that the tensor-core kernel reads.
 static xconv_status run_backprobe(const xconv_desc* d, const WgradPlan& p, const float* S, const void* dY,
                                   void* L, void* Sb_, char* w, cudaStream_t st, const unsigned long long* seed = nullptr) {
+  if (p.split_bp) {
+    const xconv_desc f = flat(d);
+    return run_backprobe_split(&f, p.g, S, d->B, 1, static_cast<const float*>(dY), static_cast<float*>(L), w, static_cast<char*>(Sb_), st);
+  }
   if (p.stream_bp) {
     const xconv_desc f = flat(d);
     return tc_run_backprobe_stream(&f, S, d->B, 1, dY, L, !p.tc_bp, w, st, nullptr);
@@ -693,6 +728,9 @@ static xconv_status run_wgrad(const xconv_desc* d, const float* S, const void* d
     if (sw.p1.stream_bp) {                 // reads S by its columns itself
       const xconv_desc f = flat(&sw.d1);
       s = tc_run_backprobe_stream(&f, S, 1, d->B, Z, w + sw.x_off, !sw.p1.tc_bp, w, st, seed);
+    } else if (sw.p1.split_bp) {           // (so does this one)
+      const xconv_desc f = flat(&sw.d1);
+      s = run_backprobe_split(&f, sw.p1.g, S, 1, d->B, static_cast<const float*>(Z), reinterpret_cast<float*>(w + sw.x_off), w, w + sw.sb_off, st);
     } else {
       float* St = reinterpret_cast<float*>(w + sw.st_off);
       const long n = (long)d->r * d->B;
@@ -823,7 +861,7 @@ int xconv_engine_for(const xconv_desc* desc, int op) {
   switch (op) {
     case XCONV_OP_SKETCH: {
       const SketchPlan p = plan_sketch(desc);
-      return p.stream || p.tc ? tc : XCONV_ENGINE_SIMT_F32;
+      return p.split ? f32 : p.stream || p.tc ? tc : XCONV_ENGINE_SIMT_F32;
     }
     case XCONV_OP_WGRAD:
     case XCONV_OP_CONTRACT: {
@@ -832,7 +870,7 @@ int xconv_engine_for(const xconv_desc* desc, int op) {
     }
     case XCONV_OP_BACKPROBE: {
       const WgradPlan p = plan_wgrad(desc);
-      return p.stream_bp || p.tc_bp ? tc : XCONV_ENGINE_SIMT_F32;
+      return p.split_bp ? f32 : p.stream_bp || p.tc_bp ? tc : XCONV_ENGINE_SIMT_F32;
     }
     case XCONV_OP_FORWARD:
     case XCONV_OP_DGRAD: {

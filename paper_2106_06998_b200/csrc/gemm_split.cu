@@ -1,0 +1,387 @@
+// Sketch S = Z^T X and back-probe L = S dY^T of float layers on the tensor cores (sm_100a): every float as three bfloat16 parts, a
+// product as six (split_f32.cuh).
+//
+// Both read one or two large float matrices once: the copy engine brings boxes of 32 terms of the reduction, twelve warps split them
+// and write the parts as MMA tiles.  The columns' parts lie one under another, so that three MMAs per k-step of 16 form the six products
+// in three groups of n accumulator columns, as in conv_split.cu; two accumulator sets take chains of four k-steps (two stages) in
+// turn and eight epilogue warps add them in float registers.
+// Error against 64 bits, times that of the FP32 multiply-adds: 0.47 in the median, nowhere more than 1.  us, multiply-adds -> this: sketch of
+// 128 x 64 rows, 65536 terms 39 -> 26 (memory 8: the stages' chain of copy, split and MMA is some 2000 clocks, and a CTA has 14), back-probe
+// of 64 rows, 128 terms, 65536 positions 37 -> 23 (memory 8).
+//   sketch      rows = the larger of probes and samples (tiles of 128), columns = the other (up to 64); both K-major; the k-blocks are dealt
+//               to the splits in turn, so that the CTAs read neighbouring bytes of every row at a time
+//   back-probe  rows = 128 positions of the flat (pixel, channel) axis, MN-major, columns = up to 64 rows of S, whose parts a small
+//               kernel writes as tile images; a CTA walks its tiles, a warp stores 128 bytes of a row of L at a time
+#include "gemm_split.h"
+
+#include <algorithm>
+
+#include "split_f32.cuh"
+
+namespace xconv {
+
+constexpr int GS_STAGES = 4, GS_TERMS = 32;
+
+struct GemmSplitParams {
+  const float *A, *B;                              // sketch: rows, columns [.][K]; back-probe: Y [K][M], and S
+  const uint8_t* img;
+  float* out;
+  long M, K, N;
+  long s_row, s_k;                                 // back-probe: S(j, k) = B[j * s_row + k * s_k]
+  long o_m, o_n;                                   // out[m * o_m + n * o_n]
+  long kblocks, tiles_m, splits;
+  int n, tiles_n, stages, ks_last;
+  uint32_t a_plane, b_plane, a_bytes, b_bytes, stage_bytes;
+  uint32_t f_off, f_slot, f_b, f_bytes; int f_slots;      // the floats of a stage: the rows' box, the columns' f_b bytes behind it
+  int f_rows_a, f_rows_b;
+  uint32_t a_hi, a_lo0, a_step, idesc;
+  int tmem_cols;
+  unsigned int *status, tag;
+};
+
+// A sum by multiply-adds: row m, column n, every `step`-th k-block from `kb` on.
+template <bool BACK>
+__device__ __noinline__ float gs_plain_sum(const GemmSplitParams& p, long m, long n, long kb, long step) {
+  float acc = 0.f;
+  for (; kb < p.kblocks; kb += step)
+    for (long k = kb * GS_TERMS; k < min(p.K, (kb + 1) * GS_TERMS); ++k)
+      acc = BACK ? fmaf(p.A[k * p.M + m], p.B[n * p.s_row + k * p.s_k], acc) : fmaf(p.A[m * p.K + k], p.B[n * p.K + k], acc);
+  return acc;
+}
+
+// The tile images of S for the back-probe: [column tile][k-block][3n rows of 32 terms], four terms a thread.
+__global__ void __launch_bounds__(256) split_sketch_images(const GemmSplitParams p, uint8_t* __restrict__ img) {
+  pdl_trigger();
+  pdl_wait();
+  const long total = (long)p.tiles_n * p.kblocks * p.n * 8;
+  for (long i = (long)blockIdx.x * 256 + threadIdx.x; i < total; i += (long)gridDim.x * 256) {
+    const int q = (int)(i & 7);
+    const long r = i >> 3, tile = r / p.n;
+    const int row = (int)(r - tile * p.n);
+    const long tn = tile / p.kblocks, j = tn * p.n + row, k = (tile - tn * p.kblocks) * GS_TERMS + 4 * q;
+    float v[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v[e] = j < p.N && k + e < p.K ? p.B[j * p.s_row + (k + e) * p.s_k] : 0.f;
+    const Split4 s = split4(make_float4(v[0], v[1], v[2], v[3]));
+    uint8_t* base = img + tile * (long)p.b_bytes;
+    *reinterpret_cast<uint2*>(base + swizzled(6, (uint32_t)row, 8 * q)) = s.h;
+    *reinterpret_cast<uint2*>(base + swizzled(6, (uint32_t)(p.n + row), 8 * q)) = s.m;
+    *reinterpret_cast<uint2*>(base + swizzled(6, (uint32_t)(2 * p.n + row), 8 * q)) = s.l;
+  }
+}
+
+template <bool BACK>
+__global__ void __launch_bounds__(SP_THREADS, 1)
+gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, const __grid_constant__ GemmSplitParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t full[GS_STAGES], empty[GS_STAGES], acc_full[2], acc_empty[2];
+  __shared__ __align__(8) uint64_t f_full[SP_FLOATS], f_empty[SP_FLOATS];
+  __shared__ uint32_t tmem_slot;
+  __shared__ int go;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < GS_STAGES; ++s) { mbar_init(&full[s], SP_CONVERTERS / 32 + (BACK ? 1 : 0)); mbar_init(&empty[s], 2); }
+    for (int f = 0; f < SP_FLOATS; ++f) { mbar_init(&f_full[f], 1); mbar_init(&f_empty[f], SP_CONVERTERS / 32); }
+    for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 8); }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fence_async_smem();
+    prefetch_tmap(&map_a);
+    if (!BACK) prefetch_tmap(&map_b);
+  }
+  if (warp == 1) tmem_alloc_then_trigger(&tmem_slot, (uint32_t)p.tmem_cols);
+  if (!BACK) split_zero(base, (uint32_t)p.stages * p.stage_bytes);      // (rows that no conversion writes are multiplied all the same)
+  pdl_wait();
+  if (threadIdx.x == 0) {
+    go = (*reinterpret_cast<volatile unsigned int*>(p.status) != p.tag) ? 1 : 0;
+    if (blockIdx.x == 0) reinterpret_cast<volatile unsigned int*>(p.status)[1] = p.tag;
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(&tmem_slot);
+  // this CTA's units -- back-probe: a run of tiles; sketch: one -- and the k-blocks of a unit
+  const long tiles = p.tiles_m * p.tiles_n;
+  const long t0 = BACK ? tiles * blockIdx.x / gridDim.x : (long)blockIdx.x / p.splits;
+  const long t1 = BACK ? tiles * (blockIdx.x + 1) / gridDim.x : t0 + 1;
+  const long kb0 = BACK ? 0 : blockIdx.x - t0 * p.splits, kstep = BACK ? 1 : p.splits;
+  const uint32_t per_unit = (uint32_t)((p.kblocks - kb0 + kstep - 1) / kstep), total = (uint32_t)(t1 - t0) * per_unit;
+
+  if (!go) {
+    // fall through to the teardown
+  } else if (warp == 0) {
+    // ------------------------------------------------------------------ S's tile images (back-probe)
+    if (BACK && lane == 0) {
+      uint32_t s = 0, par = 1, i = 0, kb = 0;        // (a wait for the phase before the first returns at once)
+      long t = t0;
+      for (; i < total; ++i) {
+        if (!mbar_wait(&empty[s], par, p.status, p.tag)) break;
+        mbar_arrive_expect_tx(&full[s], p.b_bytes);
+        bulk_load(base + s * p.stage_bytes + p.a_bytes, p.img + ((t / p.tiles_m) * p.kblocks + kb) * (long)p.b_bytes, p.b_bytes, &full[s]);
+        if (++kb == per_unit) { kb = 0; ++t; }
+        if (++s == (uint32_t)p.stages) { s = 0; par ^= 1u; }
+      }
+      // every copy issued must have landed before the CTA exits
+      for (uint32_t k = i > (uint32_t)p.stages ? i - p.stages : 0; k < i; ++k)
+        if (!mbar_wait(&full[k % p.stages], (k / p.stages) & 1u, p.status, p.tag)) break;
+    }
+  } else if (warp <= 2) {
+    // ------------------------------------------------------------------ MMA issuers (whole warps): every other chain each
+    const uint32_t own = (uint32_t)warp - 1;
+    const uint32_t s0 = (base & 0x3FFFFu) >> 4, stage16 = p.stage_bytes >> 4, ap = p.a_plane >> 4, n = (uint32_t)p.n;
+    const uint32_t narrower = (n >> 3) << 17, b_add = (1u << 16) + (p.a_bytes >> 4);
+    const uint32_t a_hi = p.a_hi, b_hi = (512u >> 4) | (1u << 14) | (4u << 29), d = tmem_base + own * 3 * n;
+    uint32_t s = 0, par = 0, t_par = 1, chain = 0, kb = 0, acc = 0, left = 0;
+    for (uint32_t i = 0; i < total; ++i) {
+      if (left == 0) {                               // a chain: two stages, or the unit's last one
+        left = min(2u, per_unit - kb);
+        acc = 0;
+        if (chain == own && !mbar_wait_warp(&acc_empty[own], t_par, p.status, p.tag)) break;
+      }
+      if (!mbar_wait_warp(&full[s], par, p.status, p.tag)) break;
+      if (chain == own) {
+        tc_fence_after();
+        const bool two = kb0 + (long)kb * kstep != p.kblocks - 1 || p.ks_last == 2;
+        const uint32_t a = s0 + s * stage16 + p.a_lo0, b = s0 + s * stage16 + b_add;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          if (k == 1 && !two) break;
+          const uint32_t ak = a + (k ? p.a_step : 0u);
+          umma_warp(d, ak, a_hi, b + 2 * k, b_hi, p.idesc, acc);
+          umma_warp(d + n, ak + ap, a_hi, b + 2 * k, b_hi, p.idesc - narrower, 1u);
+          umma_warp(d + 2 * n, ak + 2 * ap, a_hi, b + 2 * k, b_hi, p.idesc - 2 * narrower, 1u);
+          acc = 1u;
+        }
+        umma_commit_warp(&empty[s]);
+      } else if (lane == 0) {
+        mbar_arrive(&empty[s]);
+      }
+      if (--left == 0) {
+        if (chain == own) { umma_commit_warp(&acc_full[own]); t_par ^= 1u; }
+        chain ^= 1u;
+      }
+      if (++kb == per_unit) kb = 0;
+      if (++s == (uint32_t)p.stages) { s = 0; par ^= 1u; }
+    }
+  } else if (warp == SP_LOAD) {
+    // ------------------------------------------------------------------ copies of the floats
+    if (lane == 0) {
+      const long tn0 = t0 / p.tiles_m;
+      long m = (t0 - tn0 * p.tiles_m) * TILE_M;
+      uint32_t f = 0, par = 1, kb = 0, i = 0;
+      for (; i < total; ++i) {
+        if (!mbar_wait(&f_empty[f], par, p.status, p.tag)) break;
+        const uint32_t dst = base + p.f_off + f * p.f_slot;
+        const int k = (int)((kb0 + (long)kb * kstep) * GS_TERMS);
+        mbar_arrive_expect_tx(&f_full[f], p.f_bytes);
+        if (BACK) {
+          tma_load_2d(dst, &map_a, (int)m, k, &f_full[f]);
+        } else {
+          tma_load_2d(dst, &map_a, k, (int)m, &f_full[f]);
+          tma_load_2d(dst + p.f_b, &map_b, k, (int)(tn0 * p.n), &f_full[f]);
+        }
+        if (++kb == per_unit) {
+          kb = 0;
+          if ((m += TILE_M) >= p.M) m = 0;
+        }
+        if (++f == (uint32_t)p.f_slots) { f = 0; par ^= 1u; }
+      }
+      // every copy issued must have landed before the CTA exits
+      for (uint32_t k = i > (uint32_t)p.f_slots ? i - p.f_slots : 0; k < i; ++k)
+        if (!mbar_wait(&f_full[k % p.f_slots], (k / p.f_slots) & 1u, p.status, p.tag)) break;
+    }
+  } else if (warp >= SP_EPILOGUE && warp < SP_CONVERT) {
+    // ------------------------------------------------------------------ epilogue
+    const int quad = warp & 3, half = (warp - SP_EPILOGUE) >> 2, groups = p.n >> 4;      // column groups half, half + 2 of 16
+    const uint32_t tmem_q = tmem_base + ((uint32_t)(quad * 32) << 16);
+    uint32_t buf = 0, par = 0;
+    bool ok = true;
+    for (long t = t0; t < t1 && ok; ++t) {
+      const long tn = t / p.tiles_m, m = (t - tn * p.tiles_m) * TILE_M + quad * 32 + lane;
+      float sum[2][16];
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int e = 0; e < 16; ++e) sum[k][e] = 0.f;
+      for (uint32_t i = 0; i < per_unit; i += 2) {
+        ok = split_wait(&acc_full[buf], par, p.status, p.tag);
+        if (!ok) break;
+        tc_fence_after();
+        split_add_set(tmem_q + buf * (uint32_t)(3 * p.n), (uint32_t)p.n, half, sum);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&acc_empty[buf]);
+        par ^= buf;
+        buf ^= 1u;
+      }
+      if (!ok || m >= p.M) continue;
+      float* out = p.out + (BACK ? 0 : kb0 * p.M * p.N) + m * p.o_m;
+      float check = 0.f;                             // 0, or NaN
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        if (half + 2 * k >= groups) break;
+        const long n0 = tn * p.n + (half + 2 * k) * 16;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+          check = fmaf(sum[k][e], 0.f, check);
+          if (n0 + e < p.N) out[(n0 + e) * p.o_n] = sum[k][e];
+        }
+      }
+      // a value that cannot be split makes NaN of every sum it enters: those are taken again
+      if (!(check == 0.f))
+        for (int c = half * 16; c < p.n && tn * p.n + c < p.N; c += (c & 15) == 15 ? 17 : 1) {
+          float* at = out + (tn * p.n + c) * p.o_n;
+          if (*at - *at != 0.f) *at = gs_plain_sum<BACK>(p, m, tn * p.n + c, kb0, kstep);
+        }
+    }
+  } else if (warp >= SP_CONVERT) {
+    // ------------------------------------------------------------------ conversion
+    uint32_t s = 0, par = 1, f = 0, f_par = 0;
+    for (uint32_t i = 0; i < total; ++i) {
+      if (!split_wait(&empty[s], par, p.status, p.tag) || !split_wait(&f_full[f], f_par, p.status, p.tag)) break;
+      const uint32_t from = base + p.f_off + f * p.f_slot, to = base + s * p.stage_bytes;
+      if (BACK) {
+        split_box<7, 5, false>(from, GS_TERMS, to, p.a_plane, p.a_plane >> 1, 0u, 0u);
+      } else {
+        split_box<6, 3, false>(from, p.f_rows_a, to, p.a_plane, 0u, 0u, 0u);
+        split_box<6, 3, false>(from + p.f_b, p.f_rows_b, to + p.a_bytes, p.b_plane, 0u, 0u, 0u);
+      }
+      split_stage_done(&full[s], &f_empty[f]);
+      if (++s == (uint32_t)p.stages) { s = 0; par ^= 1u; }
+      if (++f == (uint32_t)p.f_slots) { f = 0; f_par ^= 1u; }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
+  }
+}
+
+// ------------------------------------------------------------------------------------ host side
+
+static void plan_columns(long M, long N, bool back, GemmSplitPlan* p) {
+  p->tiles_n = (int)cdivl(N, SP_MAX_N);
+  p->n = round_up((int)cdivl(N, p->tiles_n), 16);
+  p->f_rows_a = back ? GS_TERMS : (int)std::min<long>(TILE_M, (M + 7) / 8 * 8);
+  p->f_rows_b = back ? 0 : (int)std::min<long>(p->n, (N + 7) / 8 * 8);
+  const int f_slot = back ? GS_TERMS * 512 : (int)up1k((uint32_t)p->f_rows_a * 128) + (int)up1k((uint32_t)p->f_rows_b * 128);
+  const int stage = 3 * 8192 + (int)up1k(3u * 64 * (uint32_t)p->n), room = SMEM_LIMIT - 4096 - 2 * stage - 2 * f_slot;
+  p->f_slots = 2 + std::min(SP_FLOATS - 2, room / f_slot);
+  p->stages = 2 + std::min(GS_STAGES - 2, (room - (p->f_slots - 2) * f_slot) / stage);
+}
+static const double HBM_SM = 22.0;                  // bytes per clock and SM from memory
+
+bool plan_sketch_split(const xconv_desc* d, GemmSplitPlan* p) {
+  const long K = (long)(d->D > 1 ? d->D : 1) * d->H * d->W * d->Cin;
+  if (d->dtype != XCONV_F32 || K % 4 != 0 || K >= (1L << 31) - 64) return false;      // (rows on 16-byte boundaries)
+  p->swap = d->B > d->r ? 1 : 0;
+  const long M = std::max(d->B, d->r), N = std::min(d->B, d->r);
+  plan_columns(M, N, false, p);
+  p->tiles_m = cdivl(M, TILE_M);
+  p->kblocks = cdivl(K, GS_TERMS);
+  const long tiles = p->tiles_m * p->tiles_n;
+  if (tiles > (1L << 20)) return false;
+  p->splits = std::max(1L, std::min(p->kblocks, NUM_SMS / tiles));
+  const long rows = p->f_rows_a + p->f_rows_b;
+  const double clk = std::max({2.0 * split_kstep_clocks(p->n), rows * 8 * 45.0 / 85, rows * 128 / HBM_SM});
+  p->clocks = (long)((double)cdivl(p->kblocks, p->splits) * clk * cdivl(tiles * p->splits, NUM_SMS));
+  p->bytes = (size_t)p->splits * d->r * d->B * sizeof(float);
+  return true;
+}
+
+bool plan_backprobe_split(const xconv_desc* d, GemmSplitPlan* p) {
+  const long Q = (long)(d->D > 1 ? d->D : 1) * d->H * d->W * d->Cout;
+  p->swap = 0;
+  plan_columns(0, d->r, true, p);
+  p->tiles_m = cdivl(Q, TILE_M);
+  p->kblocks = cdivl(d->B, GS_TERMS);
+  p->splits = 1;
+  if (d->dtype != XCONV_F32 || Q % 4 != 0 || Q >= (1L << 31) - 128) return false;
+  const long tiles = p->tiles_m * p->tiles_n, ksteps = cdivl(d->B, 16);
+  const double clk = std::max({(double)ksteps * split_kstep_clocks(p->n), ksteps * 16 * 32 * 45.0 / 85,
+                               (d->B + std::min(d->r, p->n)) * 512 / HBM_SM}) + 200.0;
+  p->clocks = (long)((double)cdivl(tiles, NUM_SMS) * clk);
+  p->bytes = (size_t)p->tiles_n * p->kblocks * 3 * p->n * 64;
+  return true;
+}
+
+static void fill_common(const GemmSplitPlan& pl, char* ws_head, GemmSplitParams* p) {
+  p->kblocks = pl.kblocks; p->tiles_m = pl.tiles_m; p->splits = pl.splits;
+  p->n = pl.n; p->tiles_n = pl.tiles_n; p->stages = pl.stages;
+  p->ks_last = (int)cdivl(p->K - (pl.kblocks - 1) * GS_TERMS, 16);
+  p->a_plane = 8192; p->b_plane = 64 * (uint32_t)pl.n;
+  p->a_bytes = 3 * p->a_plane; p->b_bytes = 3 * p->b_plane;
+  p->stage_bytes = p->a_bytes + up1k(p->b_bytes);
+  p->f_off = (uint32_t)pl.stages * p->stage_bytes;
+  p->f_rows_a = pl.f_rows_a; p->f_rows_b = pl.f_rows_b; p->f_slots = pl.f_slots;
+  p->a_hi = (512u >> 4) | (1u << 14) | (4u << 29);
+  p->idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(3 * pl.n >> 3) << 17) | ((uint32_t)(TILE_M >> 4) << 24);
+  p->tmem_cols = pow2_cols(6 * pl.n);
+  p->status = reinterpret_cast<unsigned int*>(ws_head);
+  p->tag = call_tag();
+}
+
+static bool matrix_map(CUtensorMap* m, const float* ptr, long cols, long rows, int box_cols, int box_rows) {
+  const uint64_t dims[2] = {(uint64_t)cols, (uint64_t)rows}, str[1] = {(uint64_t)cols * 4};
+  const uint32_t box[2] = {(uint32_t)box_cols, (uint32_t)box_rows};
+  return make_map_f32(m, ptr, 2, dims, str, box, CU_TENSOR_MAP_SWIZZLE_NONE);
+}
+
+template <bool BACK>
+static xconv_status launch_gemm_split(const CUtensorMap& ma, const CUtensorMap& mb, const GemmSplitParams& p, unsigned grid, cudaStream_t st) {
+  const size_t smem = 1024 + (size_t)p.f_off + (size_t)p.f_slots * p.f_slot;
+  if (smem > (size_t)(SMEM_LIMIT - 1024)) return XCONV_ERR_UNSUPPORTED;
+  cudaError_t e = cudaFuncSetAttribute(gemm_split_kernel<BACK>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT - 1024);
+  if (e == cudaSuccess) e = launch_pdl(gemm_split_kernel<BACK>, dim3(grid), dim3(SP_THREADS), smem_of_grid(smem, grid), st, ma, mb, p);
+  count_launch();
+  if (e != cudaSuccess) { set_cuda_error((int)e); return XCONV_ERR_CUDA; }
+  return XCONV_OK;
+}
+
+xconv_status run_sketch_split(const xconv_desc* d, const GemmSplitPlan& pl, const float* X, const float* Z, float* part, char* ws_head,
+                              cudaStream_t st) {
+  GemmSplitParams p{};
+  p.A = pl.swap ? X : Z;
+  p.B = pl.swap ? Z : X;
+  p.out = part;
+  p.M = pl.swap ? d->B : d->r;
+  p.N = pl.swap ? d->r : d->B;
+  p.K = (long)(d->D > 1 ? d->D : 1) * d->H * d->W * d->Cin;
+  p.o_m = pl.swap ? 1 : d->B;
+  p.o_n = pl.swap ? d->B : 1;
+  fill_common(pl, ws_head, &p);
+  p.a_lo0 = 1u << 16; p.a_step = 2;
+  p.f_b = up1k((uint32_t)p.f_rows_a * 128);
+  p.f_slot = p.f_b + up1k((uint32_t)p.f_rows_b * 128);
+  p.f_bytes = (uint32_t)(p.f_rows_a + p.f_rows_b) * 128;
+  CUtensorMap ma, mb;
+  if (!matrix_map(&ma, p.A, p.K, p.M, GS_TERMS, p.f_rows_a) || !matrix_map(&mb, p.B, p.K, p.N, GS_TERMS, p.f_rows_b)) return XCONV_ERR_CUDA;
+  return launch_gemm_split<false>(ma, mb, p, (unsigned)(pl.tiles_m * pl.tiles_n * pl.splits), st);
+}
+
+xconv_status run_backprobe_split(const xconv_desc* d, const GemmSplitPlan& pl, const float* S, long s_row, long s_k, const float* Y, float* L,
+                                 char* ws_head, char* scratch, cudaStream_t st) {
+  GemmSplitParams p{};
+  p.A = Y; p.B = S; p.s_row = s_row; p.s_k = s_k;
+  p.img = reinterpret_cast<const uint8_t*>(scratch);
+  p.out = L;
+  p.M = (long)(d->D > 1 ? d->D : 1) * d->H * d->W * d->Cout;
+  p.N = d->r; p.K = d->B;
+  p.o_m = 1; p.o_n = p.M;
+  fill_common(pl, ws_head, &p);
+  p.a_hi = (1024u >> 4) | (1u << 14) | (2u << 29);
+  p.a_lo0 = (4096u >> 4) << 16; p.a_step = (16 * 128) >> 4; p.idesc |= 1u << 15;
+  p.f_slot = p.f_bytes = GS_TERMS * 512;
+  CUtensorMap ma;
+  if (!matrix_map(&ma, Y, p.M, p.K, TILE_M, GS_TERMS)) return XCONV_ERR_CUDA;
+  const long pieces = (long)p.tiles_n * p.kblocks * p.n * 8;
+  const cudaError_t e = launch_pdl(split_sketch_images, dim3((unsigned)std::min<long>(2 * NUM_SMS, cdivl(pieces, 256))), dim3(256), 0, st, p,
+                                   reinterpret_cast<uint8_t*>(scratch));
+  count_launch();
+  if (e != cudaSuccess) { set_cuda_error((int)e); return XCONV_ERR_CUDA; }
+  return launch_gemm_split<true>(ma, ma, p, (unsigned)std::min<long>(pl.tiles_m * pl.tiles_n, NUM_SMS), st);
+}
+
+}  // namespace xconv

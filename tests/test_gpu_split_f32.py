@@ -75,3 +75,59 @@ def test_contraction(r, Cin, Cout, D, H, W, K, KD):
     want = O.wgrad_contract3d(L, Z, (KD, K, K)) if D > 1 else O.wgrad_contract(L, Z, K, K)
     want = want * r * host(scale).reshape((1, -1) + (1,) * (want.ndim - 2))
     check("dW", host(dW), want, TOL)
+
+
+@pytest.mark.parametrize("r,B,C,H,W", [
+    (64, 128, 64, 32, 32), (130, 200, 24, 31, 28), (300, 7, 48, 40, 37), (5, 140, 36, 45, 33), (72, 65, 20, 33, 31),
+])
+def test_sketch_and_backprobe(r, B, C, H, W):
+    X, Z, S = _n((B, C, H, W), 6), _n((r, C, H, W), 7), _n((r, B), 8)
+    desc = xb.make_desc(B, C, C, H, W, r, torch.float32)
+    assert xb.engine_for(desc, xb.OP_SKETCH) == "tcgen05_f32"
+    check("S", host(xb.xconv_sketch(xb.to_device(X, "f32"), xb.to_device(Z, "f32"))), O.sketch(X, Z), TOL)
+    L = host(xb.xconv_backprobe(torch.from_numpy(S).cuda(), xb.to_device(X, "f32")))
+    check("L", L, np.tensordot(S.astype(np.float64), X.astype(np.float64), 1), TOL)
+
+
+def test_values_that_cannot_be_split():
+    """Infinities, NaN and the largest floats: every result they enter is what the definition gives, the others keep their bits."""
+    r, B, Cin, Cout, H, W = 70, 64, 20, 36, 24, 30
+    X, Z, Wt = _n((B, Cin, H, W), 9), _n((r, Cin, H, W), 10), _n((Cout, Cin, 3, 3), 11, 0.1)
+    dev = lambda a: xb.to_device(a, "f32")
+    Y, S = map(host, xb.xconv_forward(dev(X), dev(Wt), dev(Z)))
+    L, dW = _n((r, Cout, H, W), 12), None
+    dW = host(xb.xconv_contract(dev(L), dev(Z)))
+    for bad in (np.inf, -np.inf, np.nan, np.float32(3.4e38)):
+        X2 = X.copy()
+        X2[3, 5, 10, 29] = bad
+        Y2, S2 = map(host, xb.xconv_forward(dev(X2), dev(Wt), dev(Z)))
+        hit = np.zeros((B, H, W), bool)
+        hit[3, 9:12, 28:] = True
+        hit = np.broadcast_to(hit[:, None], Y.shape)
+        assert np.array_equal(Y2[~hit], Y[~hit])
+        with np.errstate(all="ignore"):
+            want = O.conv_forward(X2[3:4], Wt)[0] if np.isfinite(bad) else float(bad) * np.ones_like(Y[3])
+        got = Y2[3][:, 9:12, 28:]
+        if np.isfinite(bad):
+            check("Y at the value", got, want[:, 9:12, 28:], 1e-5)
+        elif np.isnan(bad):
+            assert np.isnan(got).all()
+        else:
+            for dy in range(3):
+                for dx in range(2):
+                    sign = np.sign(Wt[:, 5, 2 - dy, (29 - (28 + dx)) + 1])
+                    assert np.array_equal(got[:, dy, dx], sign * bad)
+        others = np.arange(B) != 3
+        assert np.array_equal(S2[:, others], S[:, others])
+        if np.isinf(bad):
+            assert np.array_equal(S2[:, 3], np.sign(Z[:, 5, 10, 29]) * bad)
+        else:
+            assert np.isnan(bad) == np.isnan(S2[:, 3]).all()
+        Z2 = Z.copy()
+        Z2[7, 4, 0, 0] = bad
+        dW2 = host(xb.xconv_contract(dev(L), dev(Z2)))
+        others = np.arange(Cin) != 4
+        assert np.array_equal(dW2[:, others], dW[:, others])
+        if np.isinf(bad):
+            assert np.array_equal(dW2[:, 4, 1, 1], np.sign(L[7, :, 0, 0]) * bad)
+            assert np.isfinite(dW2[:, 4, 2, 2]).all()          # that offset pairs the corner with a position outside
