@@ -79,7 +79,9 @@ __host__ __device__ __forceinline__ HaloUnit halo_unit(const HaloParams& p, uint
   return u;
 }
 
-// The MMAs of `rows` image rows of a patch.  FORM 1 and 2: as many row tiles and one piece; 0: any number of both.
+// The MMAs of `rows` image rows of a patch.  FORM 1 and 2: as many row tiles and one piece; 12 and 13: one row tile, two or three
+// pieces; 0: any number of both.  (With the pieces known to the compiler a k-step is straight-line code; in a loop that looks them up it
+// took 135 clocks an MMA of 56: volumes of 48^3, 32 channels 49 -> 34 us.)
 template <int FORM>
 __device__ __forceinline__ void halo_mmas(const HaloParams& p, int rows, uint32_t tmem, uint32_t a0, uint32_t b0, uint32_t& acc,
                                           uint32_t id0) {
@@ -88,7 +90,11 @@ __device__ __forceinline__ void halo_mmas(const HaloParams& p, int rows, uint32_
   for (int y = 0; y < rows; ++y) {
     uint32_t a = a0, b = b0;
     for (int x = 0; x < kx; ++x) {
-      if (FORM > 0) {
+      if (FORM > 10) {
+#pragma unroll
+        for (int i = 0; i < FORM - 10; ++i)
+          umma_warp(tmem + p.piece_col[i], a, p.a_hi, b + p.piece_off[i], p.b_hi, p.piece_idesc[i], acc);
+      } else if (FORM > 0) {
         umma_warp(tmem, a, p.a_hi, b, p.b_hi, id0, acc);
         if (FORM == 2) umma_warp(tmem + (uint32_t)p.cols, a + p.a_mt16, p.a_hi, b, p.b_hi, id0, acc);
       } else {
@@ -224,6 +230,8 @@ contract_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
       const uint32_t id0 = p.piece_idesc[0] - ((uint32_t)(fewer >> 3) << 17);
       if (one) halo_issue_drained<1>(p, bar, n, tmem_base, b0, a_add, b_add, id0);
       else if (p.mt == 2 && p.pieces == 1) halo_issue_drained<2>(p, bar, n, tmem_base, b0, a_add, b_add, id0);
+      else if (p.mt == 1 && p.pieces == 2) halo_issue_drained<12>(p, bar, n, tmem_base, b0, a_add, b_add, id0);
+      else if (p.mt == 1 && p.pieces == 3) halo_issue_drained<13>(p, bar, n, tmem_base, b0, a_add, b_add, id0);
       else halo_issue_drained<0>(p, bar, n, tmem_base, b0, a_add, b_add, id0);
     } else {
       uint32_t s = 0, par = 0, acc = 0, st = b0;
@@ -234,6 +242,9 @@ contract_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
         tc_fence_after();
         const uint32_t a = p.a_lo0 | st, b = p.b_lo0 | (st + a_bytes16);
         if (one) halo_mmas<1>(p, p.ph, tmem_base, a, b, acc, p.piece_idesc[0]);
+        else if (p.mt == 2 && p.pieces == 1) halo_mmas<2>(p, p.ph, tmem_base, a, b, acc, p.piece_idesc[0]);
+        else if (p.mt == 1 && p.pieces == 2) halo_mmas<12>(p, p.ph, tmem_base, a, b, acc, 0u);
+        else if (p.mt == 1 && p.pieces == 3) halo_mmas<13>(p, p.ph, tmem_base, a, b, acc, 0u);
         else halo_mmas<0>(p, p.ph, tmem_base, a, b, acc, 0u);
         umma_commit_warp(&empty[s]);
         st += stage16;
