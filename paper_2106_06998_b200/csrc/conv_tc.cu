@@ -42,6 +42,7 @@ struct ConvParams {
   uint32_t patches, items;                        // patches of the layer; items = patches x column tiles
   uint32_t plane_rows;                            // tile rows of one plane of the box
   int m_sub, acc_bufs, groups, tile_n, tmem_cols; // groups: of epilogue warps
+  int o_per;                                      // staging tiles per group of epilogue warps
   int nb, cw, ks_full, ks_last;                   // channel blocks; MMA k-steps of a block and of the last one
   uint32_t rb;                                    // bytes of an input tile row
   uint32_t a_sub_bytes, a_tx; int a_slots;        // one patch's box in shared memory; bytes copied for it
@@ -137,7 +138,7 @@ __device__ __forceinline__ void cv_issue_one_block(const ConvParams& p, const Cv
 template <bool F16, int KS>
 __global__ void __launch_bounds__(CV_THREADS, 1)
 conv_tc_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ CUtensorMap map_w,
-               const __grid_constant__ CUtensorMap map_out, const ConvParams p) {
+               const __grid_constant__ CUtensorMap map_out, const __grid_constant__ ConvParams p) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t a_full[CV_A_SLOTS], a_empty[CV_A_SLOTS];
   __shared__ __align__(8) uint64_t w_full[CV_W_SLOTS], w_empty[CV_W_SLOTS];
@@ -308,7 +309,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
     const uint32_t orb = (uint32_t)p.ocw * 2;
     const uint32_t swz = p.ocw == 64 ? (uint32_t)v & 7u : p.ocw == 32 ? ((uint32_t)v >> 1) & 3u : ((uint32_t)v >> 2) & 1u;
     const bool leader = quad == 0 && lane == 0;
-    uint32_t lu = 0, ob = (uint32_t)group;                                // ob: staging tile (one group alone uses both)
+    uint32_t lu = 0, ob = 0;                                              // ob: which of the group's staging tiles
     for (CvWalk w(p, i0, i1); w.it < i1; ++lu) {
       const int n = w.unit(p);
       const uint32_t buf = p.acc_bufs == 2 ? lu & 1u : 0u, use = p.acc_bufs == 2 ? lu >> 1 : lu;
@@ -326,8 +327,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
       for (int sub = 0; sub < n; ++sub, w.step(p)) {
         if (share && sub != group) continue;
         for (int c = 0; c < cols; c += p.ocw) {
-          const uint32_t tile = base + p.o_off + ob * p.o_bytes, row = tile + (uint32_t)v * orb;
-          if (leader) { if (p.groups == 2) bulk_wait_read<0>(); else bulk_wait_read<1>(); }    // its last store has read the tile
+          const uint32_t tile = base + p.o_off + ((uint32_t)(group * p.o_per) + ob) * p.o_bytes, row = tile + (uint32_t)v * orb;
+          if (leader) { if (p.o_per == 1) bulk_wait_read<0>(); else bulk_wait_read<1>(); }     // the tile's last store has read it
           epi_sync(group);
           for (int h = 0; h < p.ocw && c + h < p.tile_n; h += 32) {
             uint32_t r[32];
@@ -356,7 +357,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
             tma_store_5d(&map_out, tile, n0 + c, w.x, w.y, w.z, w.b);
             bulk_commit();
           }
-          if (p.groups == 1) ob ^= 1u;
+          if (p.o_per == 2) ob ^= 1u;
         }
       }
       if (last >= n) {                                                    // one accumulator set, a unit of one patch
@@ -435,9 +436,14 @@ bool tc_plan_conv(const xconv_desc* d, bool dgrad, TcConvPlan* p) {
         p->cw = cw; p->m_sub = m_sub; p->tile_n = tile_n; p->tiles_n = tiles_n; p->acc_bufs = acc_bufs;
         p->patch_w = pw; p->patch_h = ph; p->resident = resident ? 1 : 0; p->groups = resident || acc_bufs == 1 ? 2 : 1; p->nbw = nbw; p->ocw = ocw;
         p->patches = patches;
+        p->o_per = p->groups == 1 ? 2 : 1;
         if (resident) {
+          // Two more staging tiles where they fit beside four input boxes: with one, a group waits for its last store to have read it
+          // before every tile (1 x 1, 64 -> 256 channels, 64 images of 56 x 56 28.5 -> 25.6 us, 24 -> 160, 3 x 3 122 -> 105 with the
+          // sketch; in the place of boxes 256 -> 192 channels, 1 x 1 53.4 -> 55.9).
           p->w_slots = 0;
-          p->a_slots = (int)std::min<uint32_t>(CV_A_SLOTS, 2 + (room - w_all) / a_slot);
+          if (room - w_all >= 2 * o_bytes + 2 * a_slot) p->o_per = 2;
+          p->a_slots = (int)std::min<uint32_t>(CV_A_SLOTS, 2 + (room - w_all - (p->o_per == 2 ? 2 * o_bytes : 0)) / a_slot);
         } else {
           p->a_slots = room >= a_slot + 4 * w_tile ? 3 : 2;
           p->w_slots = (int)std::min<uint32_t>(CV_W_SLOTS, (budget - (uint32_t)p->a_slots * a_slot - 2 * o_bytes) / w_tile);
@@ -462,6 +468,7 @@ xconv_status tc_run_conv(const xconv_desc* d, const TcConvPlan& pl, bool dgrad, 
   p.patches = (uint32_t)pl.patches; p.items = (uint32_t)(pl.patches * pl.tiles_n);
   p.plane_rows = (uint32_t)(p.P * (p.ph + K - 1));
   p.m_sub = pl.m_sub; p.acc_bufs = pl.acc_bufs; p.groups = pl.groups; p.tile_n = pl.tile_n;
+  p.o_per = pl.o_per;
   p.tmem_cols = pow2_cols(pl.acc_bufs * pl.m_sub * pl.tile_n);
   p.cw = pl.cw; p.nb = (int)cdivl(Ci, pl.cw); p.ks_full = pl.cw / 16; p.ks_last = (int)cdivl(Ci - (p.nb - 1) * pl.cw, 16);
   p.rb = 2 * (uint32_t)pl.cw;
@@ -504,7 +511,7 @@ xconv_status tc_run_conv(const xconv_desc* d, const TcConvPlan& pl, bool dgrad, 
   if (!image_map(&mi, in, Ci, pl.cw, p.P, p.ph + K - 1, KD) || !image_map(&mo, out, Co, pl.ocw, p.pw, p.ph, 1) ||
       !make_map(&mw, W, 3, dw, sw, bw, f16, swizzle_of(dgrad ? pl.nbw : pl.cw)))
     return XCONV_ERR_CUDA;
-  const size_t smem = 1024 + (size_t)p.o_off + 2 * (size_t)p.o_bytes;
+  const size_t smem = 1024 + (size_t)p.o_off + (size_t)(p.groups * p.o_per) * p.o_bytes;
   if (smem > (size_t)(SMEM_LIMIT - 1024)) return XCONV_ERR_UNSUPPORTED;
   const unsigned grid = std::min<uint32_t>(p.items, NUM_SMS);
   void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, ConvParams) =

@@ -42,6 +42,7 @@ struct TcConvPlan {
   int m_sub, acc_bufs;       // patches that share each weight tile; accumulator sets in tensor memory
   int cw, nbw, ocw;          // channels per input tile row, per MN-major weight block (dX), per staging tile
   int resident, w_slots, a_slots;   // all weights in shared memory, or a ring of w_slots tiles; input boxes
+  int o_per;                 // staging tiles per group of epilogue warps
   uint32_t a_sub_bytes;      // shared memory of one patch's box
   int groups;                // of epilogue warps: two where a patch is over quickly, one beside long mainloops, whose issue
                              // slots the second would only take
