@@ -111,9 +111,8 @@ struct TcParams {
   unsigned int tag;        // tag of this call
 };
 
-// All MMAs of one stage, fully unrolled.  The issuing thread runs alone in its warp, so every instruction
-// it executes costs a full dependent-issue slot (~6 cycles): a 128x64x16 MMA occupies the tensor pipe for
-// 32 cycles, i.e. about five instructions.  KS k-steps, TWO = two 128-row tiles share the B tile.
+// All MMAs of one stage, fully unrolled.  One warp's instructions are a dependent-issue slot (~6 cycles) each: a 128x64x16 MMA
+// occupies the tensor pipe for some 40 cycles, i.e. about seven instructions.  KS k-steps, TWO = two 128-row tiles share the B tile.
 // GROUPED: the stage holds KS/4 K-major tiles of 64 k each; after every fourth k-step the start
 // addresses jump to the next tile.
 template <int KS, bool TWO, bool GROUPED = false>
@@ -122,8 +121,8 @@ __device__ __forceinline__ void umma_stage(uint32_t d, uint32_t tile_n, uint32_t
                                            uint32_t a_sub, uint32_t a_jump = 0, uint32_t b_jump = 0) {
 #pragma unroll
   for (int k = 0; k < KS; ++k) {
-    umma_bf16(d, a_lo, hi, b_lo, hi, idesc, k == 0 ? acc : 1u);
-    if (TWO) umma_bf16(d + tile_n, a_lo + a_sub, hi, b_lo, hi, idesc, k == 0 ? acc : 1u);
+    umma_warp(d, a_lo, hi, b_lo, hi, idesc, k == 0 ? acc : 1u);
+    if (TWO) umma_warp(d + tile_n, a_lo + a_sub, hi, b_lo, hi, idesc, k == 0 ? acc : 1u);
     if (GROUPED && (k & 3) == 3) { a_lo += a_jump; b_lo += b_jump; }
     else { a_lo += a_step; b_lo += b_step; }
   }
@@ -138,11 +137,11 @@ __device__ __forceinline__ void umma_stage_taps(uint32_t d, uint32_t unit_cols, 
 #pragma unroll
   for (int k = 0; k < KS; ++k) {
     const uint32_t ac = k == 0 ? acc : 1u;
-    umma_bf16(d, a_lo, hi, b_lo, hi, id0, ac);
-    if (PIECES2) umma_bf16(d + piece0_cols, a_lo, hi, b_lo + b_piece, hi, id1, ac);
+    umma_warp(d, a_lo, hi, b_lo, hi, id0, ac);
+    if (PIECES2) umma_warp(d + piece0_cols, a_lo, hi, b_lo + b_piece, hi, id1, ac);
     if (TWO) {
-      umma_bf16(d + unit_cols, a_lo + a_sub, hi, b_lo, hi, id0, ac);
-      if (PIECES2) umma_bf16(d + unit_cols + piece0_cols, a_lo + a_sub, hi, b_lo + b_piece, hi, id1, ac);
+      umma_warp(d + unit_cols, a_lo + a_sub, hi, b_lo, hi, id0, ac);
+      if (PIECES2) umma_warp(d + unit_cols + piece0_cols, a_lo + a_sub, hi, b_lo + b_piece, hi, id1, ac);
     }
     a_lo += a_step;
     b_lo += b_step;
@@ -630,9 +629,13 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    // One thread.  With small tiles the time between two tcgen05.mma is set by this thread's own
-    // instruction stream, so the loop carries descriptors as 32-bit halves and does no division.
-    if (lane == 0) {
+    // The whole warp, converged: one lane is elected inside an MMA's or a commit's own instructions, and descriptors stay in uniform
+    // registers (one lane under a branch moved them there for every MMA, and waited 150 clocks longer per stage).  Measured, one lane ->
+    // warp, us: sketch of 64 samples, 32 probes, 401408 terms 18.7 -> 17.6; 96 -> 160 channels, 35 x 27, 50 probes, contraction 47.2 -> 43.3;
+    // 128 -> 192, 118 x 118 271 -> 245; 210 sketches, back-probes and contractions together 0.99, where memory bounds them 0.98 to 1.01,
+    // the slowest 303 -> 317 (160 -> 96, 33 x 22, 512 probes).  With small tiles the time between two tcgen05.mma is still set by the
+    // warp's instruction stream, so the loop carries descriptors as 32-bit halves and does no division.
+    {
       // instruction descriptor: float accumulator (bit 4), A and B formats (bits 7-9, 10-12: 0 = float16, 1 = bfloat16,
       // always the same for both), operand majorness (bits 15, 16), N >> 3 (bits 17-22), M >> 4 (bits 24-28)
       const uint32_t idesc = (1u << 4) | (F16 ? 0u : (1u << 7) | (1u << 10)) | ((uint32_t)p.a_mn_major << 15) |
@@ -654,8 +657,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       const uint32_t tile_n = (uint32_t)p.tile_n;
       int s = 0;
       uint32_t full_parity = 0, s16 = base16;
-      const uint32_t full_a0 = smem_u32(&full_bar[0]), empty_a0 = smem_u32(&empty_bar[0]);
-      uint32_t full_a = full_a0, empty_a = empty_a0;
       long lu = 0;
       bool ok = true;
       for (long u = blockIdx.x; u < p.units && ok; u += gridDim.x, ++lu) {
@@ -663,20 +664,20 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         const int buf = p.acc_bufs == 2 ? (int)(lu & 1) : 0;          // (no division: this thread's stream is the critical path)
         const long use = p.acc_bufs == 2 ? lu >> 1 : lu;
         if (use > 0) {                      // the epilogue must have emptied this accumulator set
-          ok = mbar_wait(&tmem_empty_bar[buf], (uint32_t)((use - 1) & 1), p.status, p.tag);
+          ok = mbar_wait_warp(&tmem_empty_bar[buf], (uint32_t)((use - 1) & 1), p.status, p.tag);
           if (!ok) break;
           tc_fence_after();
         }
         // Nothing to multiply: the barriers still take their turn, so that their phases keep counting units, and the
         // epilogue stores zeros without reading the accumulator.
-        if (w.nkb == 0) { mbar_arrive(&tmem_full_bar[buf]); continue; }
+        if (w.nkb == 0) { if (lane == 0) mbar_arrive(&tmem_full_bar[buf]); continue; }
         const uint32_t d_tmem = tmem_base + (uint32_t)(buf * acc_cols);
         uint32_t acc = 0;
         // BACKPROBE: the MMA spans the blocks this column tile has
         const uint32_t idesc_u = p.mode == MODE_BACKPROBE
                                      ? (idesc & ~(0x3Fu << 17)) | ((uint32_t)(w.nblk * 8) << 17) : idesc;
         for (int i = 0; i < w.nkb; ++i) {
-          if (!mbar_try_wait_a(full_a, full_parity)) ok = mbar_wait_slow(&full_bar[s], full_parity, p.status, p.tag);
+          ok = mbar_wait_warp(&full_bar[s], full_parity, p.status, p.tag);
           if (!ok) break;
           tc_fence_after();
           uint32_t a_lo = a_lo0 | s16;
@@ -740,11 +741,11 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 #undef XC_STAGE
 #undef XC_GROUP
           acc = 1u;
-          umma_commit_a(empty_a);            // stage s may be refilled once these MMAs have read it
-          s16 += stage16; full_a += 8; empty_a += 8;
-          if (++s == stages) { s = 0; s16 = base16; full_a = full_a0; empty_a = empty_a0; full_parity ^= 1u; }
+          umma_commit_warp(&empty_bar[s]);           // stage s may be refilled once these MMAs have read it
+          s16 += stage16;
+          if (++s == stages) { s = 0; s16 = base16; full_parity ^= 1u; }
         }
-        if (ok) umma_commit(&tmem_full_bar[buf]);
+        if (ok) umma_commit_warp(&tmem_full_bar[buf]);
       }
     }
   } else {
