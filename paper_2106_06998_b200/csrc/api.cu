@@ -128,6 +128,17 @@ static bool plan_backprobe_f32(const xconv_desc* d, GemmSplitPlan* p) {
   return 1.5 * p->clocks + 5000.0 < std::max(waves * d->B * 310.0, ((double)d->B + d->r) * 4.0 * Q / (148.0 * 16.0));
 }
 
+// The back-probe of 16-bit layers that neither tc_plan_wgrad's nor the streaming one serves: where the clocks of gemm_split.cu, with 5000 more for
+// the launch that splits S, are below those of the multiply-adds, 1270 a term of a wave of blocks or the stores of L at 7 bytes a clock and SM.  us,
+// multiply-adds -> this: 118 rows, 5 terms, 3.5 M positions 675 -> 371, 512 rows, 11 terms, 3136 positions 10.4 -> 7.2, 128 rows, 187
+// terms, 750000 positions 2325 -> 214, but 256 rows, 4 terms, 2400 positions 6.4 -> 7.5, 157 rows, 6 terms, 89856 positions 18.7 -> 19.7.
+static bool plan_backprobe_whole(const xconv_desc* d, GemmSplitPlan* p) {
+  if (d->dtype == XCONV_F32 || !plan_backprobe_split(d, p)) return false;
+  const double Q = (double)depth(d) * d->H * d->W * d->Cout;
+  const double waves = (double)cdiv(cdiv((long)Q, 1024) * cdiv(d->r, 16), 296);
+  return p->clocks + 5000.0 < std::max(waves * d->B * 1270.0, d->r * 2.0 * Q / (148.0 * 7.0));
+}
+
 static SketchPlan plan_sketch(const xconv_desc* d_, bool seeded = false) {
   const xconv_desc fl = flat(d_);
   const xconv_desc* d = &fl;
@@ -199,7 +210,7 @@ static xconv_status pad_channels(const void*& t, long rows, int C, char*& ws, cu
 
 struct WgradPlan {
   bool tc_bp, tc_ct;
-  bool split_bp; GemmSplitPlan g;      // back-probe of float layers on the tensor cores (gemm_split.cu)
+  bool split_bp; GemmSplitPlan g;      // back-probe with S in parts (gemm_split.cu): float layers, 16-bit ones that the others do not serve
   bool stream_bp;                      // back-probe of few rows (stream_tc.cu)
   bool halo;                           // contraction of few channels (contract_tc.cu) instead of the one of tc_kernels.cu
   TcHaloPlan h;                        // ... on the layer with its channels padded to multiples of 8
@@ -227,10 +238,10 @@ static WgradPlan plan_wgrad_core(const xconv_desc* d) {
   p.l_off = WS_HEADER;
   p.sb_off = p.l_off + align_up((size_t)d->r * Q * lsz, 256);
   const xconv_desc f = flat(d);
-  p.split_bp = plan_backprobe_f32(&f, &p.g);
-  p.part_off = p.sb_off + align_up(p.split_bp ? p.g.bytes : (size_t)d->r * d->B * 2, 256);
   p.tc_bp = (tc_plan_wgrad(&f, &p.tb) & 1) != 0;
   p.stream_bp = tc_backprobe_streams(&f, p.tc_bp);
+  p.split_bp = d->dtype == XCONV_F32 ? plan_backprobe_f32(&f, &p.g) : !p.tc_bp && !p.stream_bp && plan_backprobe_whole(&f, &p.g);
+  p.part_off = p.sb_off + align_up(p.split_bp ? p.g.bytes : (size_t)d->r * d->B * 2, 256);
   const xconv_desc c = planes_ct(d);    // the tensor-core contraction works plane by plane
   p.tc_ct = (tc_plan_wgrad(&c, &p.t) & 2) != 0;
   // The contraction for few channels: where the other one does not go (drained; if its channel blocks are not mostly padding, see
@@ -649,12 +660,12 @@ static xconv_status run_conv(const xconv_desc* d, bool dgrad, const void* in, co
                                  : run_conv_simt<bf16>(d, dgrad, in, Wt, out, st);
 }
 
-// L = S dY^T into `L`; `Sb` receives the bfloat16 copy of S that the tensor-core kernel reads.
+// L = S dY^T into `L`; `Sb` receives the 16-bit copy or the parts of S that the tensor-core kernels read.
 static xconv_status run_backprobe(const xconv_desc* d, const WgradPlan& p, const float* S, const void* dY,
                                   void* L, void* Sb_, char* w, cudaStream_t st, const unsigned long long* seed = nullptr) {
   if (p.split_bp) {
     const xconv_desc f = flat(d);
-    return run_backprobe_split(&f, p.g, S, d->B, 1, static_cast<const float*>(dY), static_cast<float*>(L), w, static_cast<char*>(Sb_), st);
+    return run_backprobe_split(&f, p.g, S, d->B, 1, dY, L, w, static_cast<char*>(Sb_), st);
   }
   if (p.stream_bp) {
     const xconv_desc f = flat(d);
@@ -730,7 +741,7 @@ static xconv_status run_wgrad(const xconv_desc* d, const float* S, const void* d
       s = tc_run_backprobe_stream(&f, S, 1, d->B, Z, w + sw.x_off, !sw.p1.tc_bp, w, st, seed);
     } else if (sw.p1.split_bp) {           // (so does this one)
       const xconv_desc f = flat(&sw.d1);
-      s = run_backprobe_split(&f, sw.p1.g, S, 1, d->B, static_cast<const float*>(Z), reinterpret_cast<float*>(w + sw.x_off), w, w + sw.sb_off, st);
+      s = run_backprobe_split(&f, sw.p1.g, S, 1, d->B, Z, w + sw.x_off, w, w + sw.sb_off, st);
     } else {
       float* St = reinterpret_cast<float*>(w + sw.st_off);
       const long n = (long)d->r * d->B;
@@ -870,7 +881,7 @@ int xconv_engine_for(const xconv_desc* desc, int op) {
     }
     case XCONV_OP_BACKPROBE: {
       const WgradPlan p = plan_wgrad(desc);
-      return p.split_bp ? f32 : p.stream_bp || p.tc_bp ? tc : XCONV_ENGINE_SIMT_F32;
+      return p.split_bp && desc->dtype == XCONV_F32 ? f32 : p.split_bp || p.stream_bp || p.tc_bp ? tc : XCONV_ENGINE_SIMT_F32;
     }
     case XCONV_OP_FORWARD:
     case XCONV_OP_DGRAD: {

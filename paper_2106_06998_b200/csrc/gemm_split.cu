@@ -1,4 +1,4 @@
-// Sketch S = Z^T X and back-probe L = S dY^T of float layers on the tensor cores (sm_100a): every float as three bfloat16 parts, a
+// Sketch S = Z^T X and back-probe L = S dY^T with float operands on the tensor cores (sm_100a): every float as three bfloat16 parts, a
 // product as six (split_f32.cuh).
 //
 // Both read one or two large float matrices once: the copy engine brings boxes of 32 terms of the reduction, twelve warps split them
@@ -12,6 +12,12 @@
 //               to the splits in turn, so that the CTAs read neighbouring bytes of every row at a time
 //   back-probe  rows = 128 positions of the flat (pixel, channel) axis, MN-major, columns = up to 64 rows of S, whose parts a small
 //               kernel writes as tile images; a CTA walks its tiles, a warp stores 128 bytes of a row of L at a time
+//   back-probe of 16-bit layers (those the kernels of tc_kernels.cu and stream_tc.cu do not serve; they were on multiply-adds, and S is
+//               not to be rounded): Y's tiles are copied as they are, two boxes of 64 positions, S goes in three parts (float16: its rows
+//               scaled first), one MMA a k-step.  us, multiply-adds -> this: 256 rows, 461 terms, 68208 positions 916 -> 91, 167 rows, 31 terms,
+//               591872 positions 353 -> 101 (memory 36), 512 rows, 4 terms, 295840 positions 180 -> 126 (memory 47).  Bound by S's
+//               images from L2 (20 KB a stage, 750 clocks) where the reduction is long, by the epilogue's chain of waits, loads and
+//               conversions (1850 clocks a tile) where it is short.
 #include "gemm_split.h"
 
 #include <algorithm>
@@ -20,12 +26,17 @@
 
 namespace xconv {
 
-constexpr int GS_STAGES = 4, GS_TERMS = 32;
+constexpr int GS_STAGES = 8, GS_TERMS = 32;
+constexpr uint32_t GS_OUT = 2048;                  // a staging tile of 16-bit results: 32 columns of 32 positions
+enum : int { GS_SKETCH = 0, GS_BACK = 1, GS_BACK_BF16 = 2, GS_BACK_F16 = 3 };
+template <int KIND> struct GsElement { using type = float; };
+template <> struct GsElement<GS_BACK_BF16> { using type = bf16; };
+template <> struct GsElement<GS_BACK_F16> { using type = f16; };
 
 struct GemmSplitParams {
-  const float *A, *B;                              // sketch: rows, columns [.][K]; back-probe: Y [K][M], and S
-  const uint8_t* img;
-  float* out;
+  const void* A; const float* B;                   // sketch: rows, columns [.][K]; back-probe: Y [K][M], and S
+  const uint8_t* img; const float* scale;
+  void* out;
   long M, K, N;
   long s_row, s_k;                                 // back-probe: S(j, k) = B[j * s_row + k * s_k]
   long o_m, o_n;                                   // out[m * o_m + n * o_n]
@@ -40,39 +51,72 @@ struct GemmSplitParams {
 };
 
 // A sum by multiply-adds: row m, column n, every `step`-th k-block from `kb` on.
-template <bool BACK>
+template <int KIND>
 __device__ __noinline__ float gs_plain_sum(const GemmSplitParams& p, long m, long n, long kb, long step) {
+  using T = typename GsElement<KIND>::type;
+  const T* A = static_cast<const T*>(p.A);
   float acc = 0.f;
   for (; kb < p.kblocks; kb += step)
     for (long k = kb * GS_TERMS; k < min(p.K, (kb + 1) * GS_TERMS); ++k)
-      acc = BACK ? fmaf(p.A[k * p.M + m], p.B[n * p.s_row + k * p.s_k], acc) : fmaf(p.A[m * p.K + k], p.B[n * p.K + k], acc);
+      acc = KIND != GS_SKETCH ? fmaf(to_f(A[k * p.M + m]), p.B[n * p.s_row + k * p.s_k], acc) : fmaf(to_f(A[m * p.K + k]), p.B[n * p.K + k], acc);
   return acc;
 }
 
-// The tile images of S for the back-probe: [column tile][k-block][3n rows of 32 terms], four terms a thread.
+// The tile images of S for the back-probe: [column tile][k-block][3n rows of 32 terms], four terms at a time.
+template <int KIND>
+__device__ __forceinline__ void write_image(const GemmSplitParams& p, uint8_t* img, long j, long kb, int q, float scale) {
+  const long tn = j / p.n, k = kb * GS_TERMS + 4 * q;
+  const int row = (int)(j - tn * p.n);
+  float v[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) v[e] = j < p.N && k + e < p.K ? p.B[j * p.s_row + (k + e) * p.s_k] * scale : 0.f;
+  const Split4 s = KIND == GS_BACK_F16 ? split4_f16(make_float4(v[0], v[1], v[2], v[3])) : split4(make_float4(v[0], v[1], v[2], v[3]));
+  uint8_t* base = img + (tn * p.kblocks + kb) * (long)p.b_bytes;
+  *reinterpret_cast<uint2*>(base + swizzled(6, (uint32_t)row, 8 * q)) = s.h;
+  *reinterpret_cast<uint2*>(base + swizzled(6, (uint32_t)(p.n + row), 8 * q)) = s.m;
+  *reinterpret_cast<uint2*>(base + swizzled(6, (uint32_t)(2 * p.n + row), 8 * q)) = s.l;
+}
+
 __global__ void __launch_bounds__(256) split_sketch_images(const GemmSplitParams p, uint8_t* __restrict__ img) {
   pdl_trigger();
   pdl_wait();
-  const long total = (long)p.tiles_n * p.kblocks * p.n * 8;
+  const long total = (long)p.tiles_n * p.n * p.kblocks * 8;
   for (long i = (long)blockIdx.x * 256 + threadIdx.x; i < total; i += (long)gridDim.x * 256) {
-    const int q = (int)(i & 7);
-    const long r = i >> 3, tile = r / p.n;
-    const int row = (int)(r - tile * p.n);
-    const long tn = tile / p.kblocks, j = tn * p.n + row, k = (tile - tn * p.kblocks) * GS_TERMS + 4 * q;
-    float v[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) v[e] = j < p.N && k + e < p.K ? p.B[j * p.s_row + (k + e) * p.s_k] : 0.f;
-    const Split4 s = split4(make_float4(v[0], v[1], v[2], v[3]));
-    uint8_t* base = img + tile * (long)p.b_bytes;
-    *reinterpret_cast<uint2*>(base + swizzled(6, (uint32_t)row, 8 * q)) = s.h;
-    *reinterpret_cast<uint2*>(base + swizzled(6, (uint32_t)(p.n + row), 8 * q)) = s.m;
-    *reinterpret_cast<uint2*>(base + swizzled(6, (uint32_t)(2 * p.n + row), 8 * q)) = s.l;
+    const long j = i / (p.kblocks * 8), k = i - j * (p.kblocks * 8);
+    write_image<GS_BACK>(p, img, j, k >> 3, (int)(k & 7), 1.0f);
   }
 }
 
-template <bool BACK>
-__global__ void __launch_bounds__(SP_THREADS, 1)
+// float16 parts.  A row of S is scaled by the power of two that brings its largest value to 2^14: the parts then hold what is above 2^-39 of
+// it, whatever the row's range.  (A row with a value that is not finite keeps its scale: its parts hold infinities or NaN.)  A warp per row.
+__global__ void __launch_bounds__(256) split_sketch_images_f16(const GemmSplitParams p, uint8_t* __restrict__ img, float* __restrict__ scale) {
+  pdl_trigger();
+  pdl_wait();
+  const int lane = threadIdx.x & 31;
+  for (long j = (long)blockIdx.x * 8 + (threadIdx.x >> 5); j < (long)p.tiles_n * p.n; j += (long)gridDim.x * 8) {
+    float top = 0.f;
+    bool finite = true;
+    if (j < p.N)
+      for (long k = lane; k < p.K; k += 32) {
+        const float v = fabsf(p.B[j * p.s_row + k * p.s_k]);
+        finite = finite && v - v == 0.f;
+        top = fmaxf(top, v);
+      }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+    finite = __all_sync(0xffffffffu, finite);
+    const int e = finite && top > 0.f ? max(-100, ilogbf(top) - 14) : 0;
+    if (lane == 0) scale[j] = ldexpf(1.f, e);
+    const float down = ldexpf(1.f, -e);
+    for (long i = lane; i < p.kblocks * 8; i += 32) write_image<GS_BACK_F16>(p, img, j, i >> 3, (int)(i & 7), down);
+  }
+}
+
+template <int KIND>
+__global__ void __launch_bounds__(KIND >= GS_BACK_BF16 ? SP_CONVERT * 32 : SP_THREADS, 1)
 gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, const __grid_constant__ GemmSplitParams p) {
+  using T = typename GsElement<KIND>::type;
+  constexpr bool BACK = KIND != GS_SKETCH, WHOLE = KIND >= GS_BACK_BF16;      // WHOLE: Y's tiles are copied as they are
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full[GS_STAGES], empty[GS_STAGES], acc_full[2], acc_empty[2];
   __shared__ __align__(8) uint64_t f_full[SP_FLOATS], f_empty[SP_FLOATS];
@@ -81,7 +125,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < GS_STAGES; ++s) { mbar_init(&full[s], SP_CONVERTERS / 32 + (BACK ? 1 : 0)); mbar_init(&empty[s], 2); }
+    for (int s = 0; s < GS_STAGES; ++s) { mbar_init(&full[s], WHOLE ? 2 : SP_CONVERTERS / 32 + (BACK ? 1 : 0)); mbar_init(&empty[s], 2); }
     for (int f = 0; f < SP_FLOATS; ++f) { mbar_init(&f_full[f], 1); mbar_init(&f_empty[f], SP_CONVERTERS / 32); }
     for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 8); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -113,12 +157,19 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     // ------------------------------------------------------------------ S's tile images (back-probe)
     if (BACK && lane == 0) {
       uint32_t s = 0, par = 1, i = 0, kb = 0;        // (a wait for the phase before the first returns at once)
-      long t = t0;
+      long tn = t0 / p.tiles_m, m = t0 - tn * p.tiles_m;      // (counted along: a division of longs for every stage held the copies up)
+      const uint8_t* tile = p.img + tn * p.kblocks * (long)p.b_bytes;
+      const uint8_t* src = tile;
       for (; i < total; ++i) {
         if (!mbar_wait(&empty[s], par, p.status, p.tag)) break;
         mbar_arrive_expect_tx(&full[s], p.b_bytes);
-        bulk_load(base + s * p.stage_bytes + p.a_bytes, p.img + ((t / p.tiles_m) * p.kblocks + kb) * (long)p.b_bytes, p.b_bytes, &full[s]);
-        if (++kb == per_unit) { kb = 0; ++t; }
+        bulk_load(base + s * p.stage_bytes + p.a_bytes, src, p.b_bytes, &full[s]);
+        src += p.b_bytes;
+        if (++kb == per_unit) {
+          kb = 0;
+          if (++m == p.tiles_m) { m = 0; tile = src; }
+          src = tile;
+        }
         if (++s == (uint32_t)p.stages) { s = 0; par ^= 1u; }
       }
       // every copy issued must have landed before the CTA exits
@@ -148,8 +199,8 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
           if (k == 1 && !two) break;
           const uint32_t ak = a + (k ? p.a_step : 0u);
           umma_warp(d, ak, a_hi, b + 2 * k, b_hi, p.idesc, acc);
-          umma_warp(d + n, ak + ap, a_hi, b + 2 * k, b_hi, p.idesc - narrower, 1u);
-          umma_warp(d + 2 * n, ak + 2 * ap, a_hi, b + 2 * k, b_hi, p.idesc - 2 * narrower, 1u);
+          if (!WHOLE) umma_warp(d + n, ak + ap, a_hi, b + 2 * k, b_hi, p.idesc - narrower, 1u);
+          if (!WHOLE) umma_warp(d + 2 * n, ak + 2 * ap, a_hi, b + 2 * k, b_hi, p.idesc - 2 * narrower, 1u);
           acc = 1u;
         }
         umma_commit_warp(&empty[s]);
@@ -162,6 +213,27 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
       }
       if (++kb == per_unit) kb = 0;
       if (++s == (uint32_t)p.stages) { s = 0; par ^= 1u; }
+    }
+  } else if (WHOLE && warp == SP_LOAD) {
+    // ------------------------------------------------------------------ copies of Y's tiles, as they are
+    if (lane == 0) {
+      long m = (t0 % p.tiles_m) * TILE_M;
+      uint32_t s = 0, par = 1, kb = 0, i = 0;
+      for (; i < total; ++i) {
+        if (!mbar_wait(&empty[s], par, p.status, p.tag)) break;
+        const uint32_t dst = base + s * p.stage_bytes;
+        mbar_arrive_expect_tx(&full[s], p.a_bytes);
+        tma_load_2d(dst, &map_a, (int)m, (int)(kb * GS_TERMS), &full[s]);
+        tma_load_2d(dst + (p.a_bytes >> 1), &map_a, (int)m + 64, (int)(kb * GS_TERMS), &full[s]);
+        if (++kb == per_unit) {
+          kb = 0;
+          if ((m += TILE_M) >= p.M) m = 0;
+        }
+        if (++s == (uint32_t)p.stages) { s = 0; par ^= 1u; }
+      }
+      // every copy issued must have landed before the CTA exits
+      for (uint32_t k = i > (uint32_t)p.stages ? i - p.stages : 0; k < i; ++k)
+        if (!mbar_wait(&full[k % p.stages], (k / p.stages) & 1u, p.status, p.tag)) break;
     }
   } else if (warp == SP_LOAD) {
     // ------------------------------------------------------------------ copies of the floats
@@ -195,9 +267,14 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     const int quad = warp & 3, half = (warp - SP_EPILOGUE) >> 2, groups = p.n >> 4;      // column groups half, half + 2 of 16
     const uint32_t tmem_q = tmem_base + ((uint32_t)(quad * 32) << 16);
     uint32_t buf = 0, par = 0;
+    const uint32_t stage = base + p.f_off + (uint32_t)(warp - SP_EPILOGUE) * GS_OUT;      // (WHOLE)
     bool ok = true;
+    long tn_at = t0 / p.tiles_m, m_at = (t0 - tn_at * p.tiles_m) * TILE_M;       // (WHOLE: counted along; the others have no registers for it)
     for (long t = t0; t < t1 && ok; ++t) {
-      const long tn = t / p.tiles_m, m = (t - tn * p.tiles_m) * TILE_M + quad * 32 + lane;
+      const long tn = WHOLE ? tn_at : t / p.tiles_m, m = (WHOLE ? m_at : (t - tn * p.tiles_m) * TILE_M) + quad * 32 + lane;
+      if ((m_at += TILE_M) >= p.M) { m_at = 0; ++tn_at; }
+      float scale = 0.f;                             // (float16) of column half * 16 + lane + (lane & 16), given to the others when it is needed
+      if (KIND == GS_BACK_F16 && half * 16 + lane + (lane & 16) < p.n) scale = __ldg(p.scale + tn * p.n + half * 16 + lane + (lane & 16));
       float sum[2][16];
 #pragma unroll
       for (int k = 0; k < 2; ++k)
@@ -214,8 +291,44 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         par ^= buf;
         buf ^= 1u;
       }
-      if (!ok || m >= p.M) continue;
-      float* out = p.out + (BACK ? 0 : kb0 * p.M * p.N) + m * p.o_m;
+      if (!ok) break;
+      if (WHOLE) {
+        // Results of 16 bits go through shared memory, so that a lane stores 16 bytes of a row (2 bytes a lane and store: 4900 clocks a tile;
+        // boxes of 16 rows of 64 bytes by the copy engine: 2080).
+        __syncwarp();                                // the last tile is read
+        float check = 0.f;                           // 0, or NaN
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          if (half + 2 * k >= groups) break;
+#pragma unroll
+          for (int e = 0; e < 16; ++e) {
+            if (KIND == GS_BACK_F16) sum[k][e] *= __shfl_sync(0xffffffffu, scale, k * 16 + e);
+            check = fmaf(sum[k][e], 0.f, check);
+            st_shared_16(stage + (uint32_t)((k * 16 + e) * 64 + lane * 2), from_f<T>(sum[k][e]));
+          }
+        }
+        // a value that cannot be split makes NaN of every sum it enters: those are taken again
+        if (!(check == 0.f) && m < p.M)
+          for (int c = 0; c < 32 && half * 16 + c + (c & 16) < p.n; ++c) {
+            const long n = tn * p.n + half * 16 + c + (c & 16);
+            if (n >= p.N) continue;
+            const float v = to_f(ld_shared_16<T>(stage + (uint32_t)(c * 64 + lane * 2)));
+            if (v - v != 0.f)
+              st_shared_16(stage + (uint32_t)(c * 64 + lane * 2), from_f<T>(gs_plain_sum<KIND>(p, m, n, kb0, kstep)));
+          }
+        __syncwarp();
+        const long at = m - lane + (lane & 3) * 8;   // (rows have a multiple of 8 positions)
+        T* to = static_cast<T*>(p.out) + at;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int row = i * 8 + (lane >> 2), c = half * 16 + row + (row & 16);
+          const long n = tn * p.n + c;
+          if (c < p.n && n < p.N && at < p.M) *reinterpret_cast<uint4*>(to + n * p.M) = ld_shared_v4(stage + (uint32_t)(row * 64 + (lane & 3) * 16));
+        }
+        continue;
+      }
+      if (m >= p.M) continue;
+      T* out = static_cast<T*>(p.out) + (BACK ? 0 : kb0 * p.M * p.N) + m * p.o_m;
       float check = 0.f;                             // 0, or NaN
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
@@ -224,17 +337,18 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
           check = fmaf(sum[k][e], 0.f, check);
-          if (n0 + e < p.N) out[(n0 + e) * p.o_n] = sum[k][e];
+          if (n0 + e < p.N) out[(n0 + e) * p.o_n] = from_f<T>(sum[k][e]);
         }
       }
       // a value that cannot be split makes NaN of every sum it enters: those are taken again
       if (!(check == 0.f))
         for (int c = half * 16; c < p.n && tn * p.n + c < p.N; c += (c & 15) == 15 ? 17 : 1) {
-          float* at = out + (tn * p.n + c) * p.o_n;
-          if (*at - *at != 0.f) *at = gs_plain_sum<BACK>(p, m, tn * p.n + c, kb0, kstep);
+          T* at = out + (tn * p.n + c) * p.o_n;
+          const float v = to_f(*at);
+          if (v - v != 0.f) *at = from_f<T>(gs_plain_sum<KIND>(p, m, tn * p.n + c, kb0, kstep));
         }
     }
-  } else if (warp >= SP_CONVERT) {
+  } else if (!WHOLE && warp >= SP_CONVERT) {
     // ------------------------------------------------------------------ conversion
     uint32_t s = 0, par = 1, f = 0, f_par = 0;
     for (uint32_t i = 0; i < total; ++i) {
@@ -261,15 +375,16 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
 
 // ------------------------------------------------------------------------------------ host side
 
-static void plan_columns(long M, long N, bool back, GemmSplitPlan* p) {
+static void plan_columns(long M, long N, int kind, GemmSplitPlan* p) {
+  const bool back = kind != GS_SKETCH, whole = kind >= GS_BACK_BF16;
   p->tiles_n = (int)cdivl(N, SP_MAX_N);
   p->n = round_up((int)cdivl(N, p->tiles_n), 16);
   p->f_rows_a = back ? GS_TERMS : (int)std::min<long>(TILE_M, (M + 7) / 8 * 8);
   p->f_rows_b = back ? 0 : (int)std::min<long>(p->n, (N + 7) / 8 * 8);
-  const int f_slot = back ? GS_TERMS * 512 : (int)up1k((uint32_t)p->f_rows_a * 128) + (int)up1k((uint32_t)p->f_rows_b * 128);
-  const int stage = 3 * 8192 + (int)up1k(3u * 64 * (uint32_t)p->n), room = SMEM_LIMIT - 4096 - 2 * stage - 2 * f_slot;
-  p->f_slots = 2 + std::min(SP_FLOATS - 2, room / f_slot);
-  p->stages = 2 + std::min(GS_STAGES - 2, (room - (p->f_slots - 2) * f_slot) / stage);
+  const int f_slot = whole ? (int)GS_OUT * 4 : back ? GS_TERMS * 512 : (int)up1k((uint32_t)p->f_rows_a * 128) + (int)up1k((uint32_t)p->f_rows_b * 128);
+  const int stage = (whole ? 1 : 3) * 8192 + (int)up1k(3u * 64 * (uint32_t)p->n), room = SMEM_LIMIT - 4096 - 2 * stage - 2 * f_slot;
+  p->f_slots = whole ? 2 : 2 + std::min(SP_FLOATS - 2, room / f_slot);      // (whole: the results' staging tiles)
+  p->stages = 2 + std::min((whole ? GS_STAGES : 4) - 2, (room - (p->f_slots - 2) * f_slot) / stage);
 }
 static const double HBM_SM = 22.0;                  // bytes per clock and SM from memory
 
@@ -278,7 +393,7 @@ bool plan_sketch_split(const xconv_desc* d, GemmSplitPlan* p) {
   if (d->dtype != XCONV_F32 || K % 4 != 0 || K >= (1L << 31) - 64) return false;      // (rows on 16-byte boundaries)
   p->swap = d->B > d->r ? 1 : 0;
   const long M = std::max(d->B, d->r), N = std::min(d->B, d->r);
-  plan_columns(M, N, false, p);
+  plan_columns(M, N, GS_SKETCH, p);
   p->tiles_m = cdivl(M, TILE_M);
   p->kblocks = cdivl(K, GS_TERMS);
   const long tiles = p->tiles_m * p->tiles_n;
@@ -291,33 +406,40 @@ bool plan_sketch_split(const xconv_desc* d, GemmSplitPlan* p) {
   return true;
 }
 
+static int back_kind(const xconv_desc* d) {
+  return d->dtype == XCONV_F32 ? GS_BACK : d->dtype == XCONV_F16 ? GS_BACK_F16 : GS_BACK_BF16;
+}
+
 bool plan_backprobe_split(const xconv_desc* d, GemmSplitPlan* p) {
   const long Q = (long)(d->D > 1 ? d->D : 1) * d->H * d->W * d->Cout;
+  const int kind = back_kind(d);
   p->swap = 0;
-  plan_columns(0, d->r, true, p);
+  plan_columns(0, d->r, kind, p);
   p->tiles_m = cdivl(Q, TILE_M);
   p->kblocks = cdivl(d->B, GS_TERMS);
   p->splits = 1;
-  if (d->dtype != XCONV_F32 || Q % 4 != 0 || Q >= (1L << 31) - 128) return false;
+  if (Q % (kind == GS_BACK ? 4 : 8) != 0 || Q >= (1L << 31) - 128) return false;      // (rows on 16-byte boundaries)
   const long tiles = p->tiles_m * p->tiles_n, ksteps = cdivl(d->B, 16);
-  const double clk = std::max({(double)ksteps * split_kstep_clocks(p->n), ksteps * 16 * 32 * 45.0 / 85,
-                               (d->B + std::min(d->r, p->n)) * 512 / HBM_SM}) + 200.0;
+  // (whole rows: measured, 1850 clocks a tile of one k-block, 3000 of three, 10800 of fifteen)
+  const double clk = kind == GS_BACK ? std::max({(double)ksteps * split_kstep_clocks(p->n), ksteps * 16 * 32 * 45.0 / 85,
+                                                 (d->B + std::min(d->r, p->n)) * 512 / HBM_SM}) + 200.0
+                                     : std::max(p->kblocks * 750.0 + 500.0, 1900.0);
   p->clocks = (long)((double)cdivl(tiles, NUM_SMS) * clk);
-  p->bytes = (size_t)p->tiles_n * p->kblocks * 3 * p->n * 64;
+  p->bytes = (size_t)p->tiles_n * p->kblocks * 3 * p->n * 64 + (kind == GS_BACK_F16 ? (size_t)p->tiles_n * p->n * sizeof(float) : 0);
   return true;
 }
 
-static void fill_common(const GemmSplitPlan& pl, char* ws_head, GemmSplitParams* p) {
+static void fill_common(const GemmSplitPlan& pl, int kind, char* ws_head, GemmSplitParams* p) {
   p->kblocks = pl.kblocks; p->tiles_m = pl.tiles_m; p->splits = pl.splits;
   p->n = pl.n; p->tiles_n = pl.tiles_n; p->stages = pl.stages;
   p->ks_last = (int)cdivl(p->K - (pl.kblocks - 1) * GS_TERMS, 16);
   p->a_plane = 8192; p->b_plane = 64 * (uint32_t)pl.n;
-  p->a_bytes = 3 * p->a_plane; p->b_bytes = 3 * p->b_plane;
+  p->a_bytes = (kind >= GS_BACK_BF16 ? 1 : 3) * p->a_plane; p->b_bytes = 3 * p->b_plane;
   p->stage_bytes = p->a_bytes + up1k(p->b_bytes);
   p->f_off = (uint32_t)pl.stages * p->stage_bytes;
   p->f_rows_a = pl.f_rows_a; p->f_rows_b = pl.f_rows_b; p->f_slots = pl.f_slots;
   p->a_hi = (512u >> 4) | (1u << 14) | (4u << 29);
-  p->idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(3 * pl.n >> 3) << 17) | ((uint32_t)(TILE_M >> 4) << 24);
+  p->idesc = (1u << 4) | (kind == GS_BACK_F16 ? 0u : (1u << 7) | (1u << 10)) | ((uint32_t)(3 * pl.n >> 3) << 17) | ((uint32_t)(TILE_M >> 4) << 24);
   p->tmem_cols = pow2_cols(6 * pl.n);
   p->status = reinterpret_cast<unsigned int*>(ws_head);
   p->tag = call_tag();
@@ -329,12 +451,13 @@ static bool matrix_map(CUtensorMap* m, const float* ptr, long cols, long rows, i
   return make_map_f32(m, ptr, 2, dims, str, box, CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
-template <bool BACK>
+template <int KIND>
 static xconv_status launch_gemm_split(const CUtensorMap& ma, const CUtensorMap& mb, const GemmSplitParams& p, unsigned grid, cudaStream_t st) {
   const size_t smem = 1024 + (size_t)p.f_off + (size_t)p.f_slots * p.f_slot;
+  const int threads = KIND >= GS_BACK_BF16 ? SP_CONVERT * 32 : SP_THREADS;
   if (smem > (size_t)(SMEM_LIMIT - 1024)) return XCONV_ERR_UNSUPPORTED;
-  cudaError_t e = cudaFuncSetAttribute(gemm_split_kernel<BACK>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT - 1024);
-  if (e == cudaSuccess) e = launch_pdl(gemm_split_kernel<BACK>, dim3(grid), dim3(SP_THREADS), smem_of_grid(smem, grid), st, ma, mb, p);
+  cudaError_t e = cudaFuncSetAttribute(gemm_split_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT - 1024);
+  if (e == cudaSuccess) e = launch_pdl(gemm_split_kernel<KIND>, dim3(grid), dim3(threads), smem_of_grid(smem, grid), st, ma, mb, p);
   count_launch();
   if (e != cudaSuccess) { set_cuda_error((int)e); return XCONV_ERR_CUDA; }
   return XCONV_OK;
@@ -343,26 +466,27 @@ static xconv_status launch_gemm_split(const CUtensorMap& ma, const CUtensorMap& 
 xconv_status run_sketch_split(const xconv_desc* d, const GemmSplitPlan& pl, const float* X, const float* Z, float* part, char* ws_head,
                               cudaStream_t st) {
   GemmSplitParams p{};
-  p.A = pl.swap ? X : Z;
-  p.B = pl.swap ? Z : X;
+  const float *rows = pl.swap ? X : Z, *cols = pl.swap ? Z : X;
+  p.A = rows; p.B = cols;
   p.out = part;
   p.M = pl.swap ? d->B : d->r;
   p.N = pl.swap ? d->r : d->B;
   p.K = (long)(d->D > 1 ? d->D : 1) * d->H * d->W * d->Cin;
   p.o_m = pl.swap ? 1 : d->B;
   p.o_n = pl.swap ? d->B : 1;
-  fill_common(pl, ws_head, &p);
+  fill_common(pl, GS_SKETCH, ws_head, &p);
   p.a_lo0 = 1u << 16; p.a_step = 2;
   p.f_b = up1k((uint32_t)p.f_rows_a * 128);
   p.f_slot = p.f_b + up1k((uint32_t)p.f_rows_b * 128);
   p.f_bytes = (uint32_t)(p.f_rows_a + p.f_rows_b) * 128;
   CUtensorMap ma, mb;
-  if (!matrix_map(&ma, p.A, p.K, p.M, GS_TERMS, p.f_rows_a) || !matrix_map(&mb, p.B, p.K, p.N, GS_TERMS, p.f_rows_b)) return XCONV_ERR_CUDA;
-  return launch_gemm_split<false>(ma, mb, p, (unsigned)(pl.tiles_m * pl.tiles_n * pl.splits), st);
+  if (!matrix_map(&ma, rows, p.K, p.M, GS_TERMS, p.f_rows_a) || !matrix_map(&mb, cols, p.K, p.N, GS_TERMS, p.f_rows_b)) return XCONV_ERR_CUDA;
+  return launch_gemm_split<GS_SKETCH>(ma, mb, p, (unsigned)(pl.tiles_m * pl.tiles_n * pl.splits), st);
 }
 
-xconv_status run_backprobe_split(const xconv_desc* d, const GemmSplitPlan& pl, const float* S, long s_row, long s_k, const float* Y, float* L,
+xconv_status run_backprobe_split(const xconv_desc* d, const GemmSplitPlan& pl, const float* S, long s_row, long s_k, const void* Y, void* L,
                                  char* ws_head, char* scratch, cudaStream_t st) {
+  const int kind = back_kind(d);
   GemmSplitParams p{};
   p.A = Y; p.B = S; p.s_row = s_row; p.s_k = s_k;
   p.img = reinterpret_cast<const uint8_t*>(scratch);
@@ -370,18 +494,32 @@ xconv_status run_backprobe_split(const xconv_desc* d, const GemmSplitPlan& pl, c
   p.M = (long)(d->D > 1 ? d->D : 1) * d->H * d->W * d->Cout;
   p.N = d->r; p.K = d->B;
   p.o_m = 1; p.o_n = p.M;
-  fill_common(pl, ws_head, &p);
+  fill_common(pl, kind, ws_head, &p);
   p.a_hi = (1024u >> 4) | (1u << 14) | (2u << 29);
   p.a_lo0 = (4096u >> 4) << 16; p.a_step = (16 * 128) >> 4; p.idesc |= 1u << 15;
-  p.f_slot = p.f_bytes = GS_TERMS * 512;
+  float* scale = reinterpret_cast<float*>(scratch + (size_t)pl.tiles_n * pl.kblocks * p.b_bytes);
+  p.scale = scale;
   CUtensorMap ma;
-  if (!matrix_map(&ma, Y, p.M, p.K, TILE_M, GS_TERMS)) return XCONV_ERR_CUDA;
+  if (kind == GS_BACK) {
+    p.f_slot = p.f_bytes = GS_TERMS * 512;
+    if (!matrix_map(&ma, static_cast<const float*>(Y), p.M, p.K, TILE_M, GS_TERMS)) return XCONV_ERR_CUDA;
+  } else {
+    const uint64_t dims[2] = {(uint64_t)p.M, (uint64_t)p.K}, str[1] = {(uint64_t)p.M * 2};
+    const uint32_t box[2] = {64, GS_TERMS};
+    if (!make_map(&ma, Y, 2, dims, str, box, kind == GS_BACK_F16)) return XCONV_ERR_CUDA;
+    p.f_slot = 4 * GS_OUT;
+  }
   const long pieces = (long)p.tiles_n * p.kblocks * p.n * 8;
-  const cudaError_t e = launch_pdl(split_sketch_images, dim3((unsigned)std::min<long>(2 * NUM_SMS, cdivl(pieces, 256))), dim3(256), 0, st, p,
-                                   reinterpret_cast<uint8_t*>(scratch));
+  const dim3 block(256);
+  const cudaError_t e = kind == GS_BACK_F16
+      ? launch_pdl(split_sketch_images_f16, dim3((unsigned)cdivl((long)p.tiles_n * p.n, 8)), block, 0, st, p, reinterpret_cast<uint8_t*>(scratch), scale)
+      : launch_pdl(split_sketch_images, dim3((unsigned)std::min<long>(2 * NUM_SMS, cdivl(pieces, 256))), block, 0, st, p,
+                   reinterpret_cast<uint8_t*>(scratch));
   count_launch();
   if (e != cudaSuccess) { set_cuda_error((int)e); return XCONV_ERR_CUDA; }
-  return launch_gemm_split<true>(ma, ma, p, (unsigned)std::min<long>(pl.tiles_m * pl.tiles_n, NUM_SMS), st);
+  const unsigned grid = (unsigned)std::min<long>(pl.tiles_m * pl.tiles_n, NUM_SMS);
+  return kind == GS_BACK ? launch_gemm_split<GS_BACK>(ma, ma, p, grid, st)
+         : kind == GS_BACK_F16 ? launch_gemm_split<GS_BACK_F16>(ma, ma, p, grid, st) : launch_gemm_split<GS_BACK_BF16>(ma, ma, p, grid, st);
 }
 
 }  // namespace xconv

@@ -1,4 +1,4 @@
-// Sketch and back-probe of float layers on the tensor cores (gemm_split.cu).
+// Sketch and back-probe of float layers, and back-probe of 16-bit layers with S in parts, on the tensor cores (gemm_split.cu).
 #pragma once
 
 #include "tc_api.h"
@@ -20,7 +20,7 @@ xconv_status run_sketch_split(const xconv_desc* d, const GemmSplitPlan& p, const
                               cudaStream_t st);
 // L[row][q] = sum over k of S[row * s_row + k * s_k] Y[k][q]: d->r rows, d->B terms.
 bool plan_backprobe_split(const xconv_desc* d, GemmSplitPlan* p);
-xconv_status run_backprobe_split(const xconv_desc* d, const GemmSplitPlan& p, const float* S, long s_row, long s_k, const float* Y, float* L,
+xconv_status run_backprobe_split(const xconv_desc* d, const GemmSplitPlan& p, const float* S, long s_row, long s_k, const void* Y, void* L,
                                  char* ws_head, char* scratch, cudaStream_t st);
 
 }  // namespace xconv

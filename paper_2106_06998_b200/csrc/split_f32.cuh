@@ -35,8 +35,37 @@ __device__ __forceinline__ Split4 split4(float4 v) {
   s.l.x = pack_bf16(v.x, v.y); s.l.y = pack_bf16(v.z, v.w);
   return s;
 }
+// Three float16 parts (11 + 11 + 11 bits; the caller scales, so that no part is out of the type's range).
+__device__ __forceinline__ uint32_t take_f16(float& a, float& b) {
+  const __half2 v = __floats2half2_rn(a, b);
+  const float2 f = __half22float2(v);
+  a -= f.x; b -= f.y;
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+__device__ __forceinline__ Split4 split4_f16(float4 v) {
+  Split4 s;
+  s.h.x = take_f16(v.x, v.y); s.h.y = take_f16(v.z, v.w);
+  s.m.x = take_f16(v.x, v.y); s.m.y = take_f16(v.z, v.w);
+  s.l.x = take_f16(v.x, v.y); s.l.y = take_f16(v.z, v.w);
+  return s;
+}
 __device__ __forceinline__ void st_shared_v2(uint32_t addr, uint2 v) {
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(v.x), "r"(v.y) : "memory");
+}
+template <typename T>
+__device__ __forceinline__ void st_shared_16(uint32_t addr, T v) {
+  asm volatile("st.shared.b16 [%0], %1;" ::"r"(addr), "h"(*reinterpret_cast<const uint16_t*>(&v)) : "memory");
+}
+template <typename T>
+__device__ __forceinline__ T ld_shared_16(uint32_t addr) {
+  uint16_t v;
+  asm volatile("ld.shared.b16 %0, [%1];" : "=h"(v) : "r"(addr) : "memory");
+  return *reinterpret_cast<const T*>(&v);
+}
+__device__ __forceinline__ uint4 ld_shared_v4(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+  return v;
 }
 // Byte offset of byte `b` of tile row `row` (2^rbs bytes a row, swizzled as the copy engine and the MMA descriptors have it).
 __device__ __forceinline__ uint32_t swizzled(int rbs, uint32_t row, uint32_t b) {

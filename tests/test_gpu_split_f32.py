@@ -89,6 +89,39 @@ def test_sketch_and_backprobe(r, B, C, H, W):
     check("L", L, np.tensordot(S.astype(np.float64), X.astype(np.float64), 1), TOL)
 
 
+@pytest.mark.parametrize("dt,u", [("bf16", 2.0 ** -8), ("f16", 2.0 ** -11)])
+@pytest.mark.parametrize("r,B,C,H,W", [
+    (70, 131, 24, 31, 28),       # two column tiles of 48, a last block of 3 terms, 96 positions in the last tile
+    (300, 45, 40, 33, 17),       # 8 positions in the last tile, 60 columns in the last column tile
+    (129, 97, 64, 8, 8),         # one term in the last block, fewer tiles than SMs
+])
+def test_backprobe_of_16_bit_rows(dt, u, r, B, C, H, W):
+    """S in three parts, the rows whole.  Bound: the rounding of the result, u of it, and TOL of its norm for the sums; float16 rows of S
+    scaled by 2^-30 and 2^20 keep their precision, and values that are not finite reach what the definition says, and nothing else."""
+    t = xb.to_device(inputs.draw("normal", (B, C, H, W), 21, dt, 1.0), dt)
+    if dt == "f16":
+        t = t * 2.0 ** -10
+    Y, S = host(t), _n((r, B), 22)
+    S[3] *= 2.0 ** -30
+    S[5] *= 2.0 ** 20
+    desc = xb.make_desc(B, C, C, H, W, r, t.dtype)
+    assert xb.engine_for(desc, xb.OP_BACKPROBE) == "tcgen05_" + dt
+    want = np.tensordot(S.astype(np.float64), Y, 1)
+    L = host(xb.xconv_backprobe(torch.from_numpy(S).cuda(), t)).astype(np.float64)
+    tiny = 2.0 ** -25 if dt == "f16" else 0.0                 # half the spacing of float16's subnormal numbers
+    norm = np.sqrt(np.square(want).mean(axis=(1, 2, 3), keepdims=True))
+    assert (np.abs(L - want) <= u * np.abs(want) * (1 + TOL) + 4 * TOL * norm + tiny).all()
+    S[r - 1, B - 1] = np.inf
+    t[2, 5, 1, 2] = float("nan")
+    L2 = host(xb.xconv_backprobe(torch.from_numpy(S).cuda(), t)).astype(np.float64)
+    assert np.isnan(L2[:, 5, 1, 2]).all()
+    got, exact = L2[r - 1], np.where(Y[B - 1] > 0, np.inf, np.where(Y[B - 1] < 0, -np.inf, np.nan))
+    got[5, 1, 2] = exact[5, 1, 2] = 0.0
+    assert np.array_equal(got, exact, equal_nan=True)
+    L[:, 5, 1, 2] = L2[:, 5, 1, 2] = 0.0
+    assert np.array_equal(L2[:r - 1], L[:r - 1])
+
+
 def test_values_that_cannot_be_split():
     """Infinities, NaN and the largest floats: every result they enter is what the definition gives, the others keep their bits."""
     r, B, Cin, Cout, H, W = 70, 64, 20, 36, 24, 30
