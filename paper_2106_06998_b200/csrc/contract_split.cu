@@ -138,7 +138,7 @@ contract_split_kernel(const __grid_constant__ CUtensorMap map_l, const __grid_co
     prefetch_tmap(&map_l);
     prefetch_tmap(&map_z);
   }
-  if (warp == 1) tmem_alloc_then_trigger(&tmem_slot, 256u);
+  if (warp == 1) split_take_columns(&tmem_slot, 256u);
   // (L between the rows of a patch and both tensors behind the last one stay zero)
   split_zero(base, (uint32_t)p.stages * p.stage_bytes);
   pdl_wait();

@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1) conv_split_kernel(const __grid_
     prefetch_tmap(&map_in);
     prefetch_tmap(&map_out);
   }
-  if (warp == 1) tmem_alloc_then_trigger(&tmem_slot, (uint32_t)p.tmem_cols);
+  if (warp == 1) split_take_columns(&tmem_slot, (uint32_t)p.tmem_cols);
   pdl_wait();
   if (threadIdx.x == 0) {
     go = (*reinterpret_cast<volatile unsigned int*>(p.status) != p.tag) ? 1 : 0;

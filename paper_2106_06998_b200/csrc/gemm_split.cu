@@ -133,7 +133,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     prefetch_tmap(&map_a);
     if (!BACK) prefetch_tmap(&map_b);
   }
-  if (warp == 1) tmem_alloc_then_trigger(&tmem_slot, (uint32_t)p.tmem_cols);
+  if (warp == 1) split_take_columns(&tmem_slot, (uint32_t)p.tmem_cols);
   if (!BACK) split_zero(base, (uint32_t)p.stages * p.stage_bytes);      // (rows that no conversion writes are multiplied all the same)
   pdl_wait();
   if (threadIdx.x == 0) {

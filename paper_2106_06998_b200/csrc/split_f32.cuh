@@ -90,6 +90,9 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
                ::"r"(dst), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
 
+// The accumulators' columns of tensor memory, for the kernels on split operands; the go-ahead for the next kernel is given behind them.
+__device__ __forceinline__ void split_take_columns(uint32_t* slot, uint32_t columns) { tmem_alloc_then_trigger(slot, columns); }
+
 // The roles of a block's 24 warps (80 registers a thread): 0 copies operands that were split before, 1 and 2 issue MMAs -- the chains of
 // accumulator set 0 and those of set 1, since one warp's instructions (some 40 clocks an MMA, and the waits between) do not keep the
 // tensor pipe busy beside the other warps -- 3 copies the floats, 4..11 add chains up, two per quarter of the MMA rows, 12..23 convert.

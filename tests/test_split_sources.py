@@ -1,0 +1,27 @@
+"""Source checks of the kernels on split operands that need no GPU."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2106_06998_b200", "csrc")
+
+
+def _code(name):
+    return re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+
+
+def test_they_take_tensor_memory_before_they_let_the_next_kernel_start():
+    """As for the other holders of tensor memory: it is taken through the function that gives the go-ahead behind the allocation (here by
+    way of split_take_columns), once, by one warp, and nothing else in those kernels gives it."""
+    helper = re.findall(r"void split_take_columns\([^)]*\) \{([^}]*)\}", _code("split_f32.cuh"))
+    assert helper == [" tmem_alloc_then_trigger(slot, columns); "]
+    holders = []
+    for name in sorted(os.listdir(CSRC)):
+        if not name.endswith((".cu", ".cuh")):
+            continue
+        for kernel in _code(name).split("__global__")[1:]:
+            body = kernel.split("\n}\n")[0]
+            if "split_take_columns" in body:
+                holders.append(name)
+                assert body.count("if (warp == 1) split_take_columns(") == 1 and body.count("split_take_columns") == 1, name
+                assert "tmem_alloc" not in body and "pdl_trigger(" not in body, name
+    assert holders == ["contract_split.cu", "conv_split.cu", "gemm_split.cu"]
