@@ -137,10 +137,14 @@ __device__ __forceinline__ void split_stage_done(uint64_t* full, uint64_t* float
   __syncwarp();
   if ((threadIdx.x & 31) == 0) { mbar_arrive(full); mbar_arrive(floats_empty); }
 }
+// A wait by a whole warp, one lane at the barrier.  What the barrier guards is ordered before the other lanes' reads by the warp barrier (a
+// shuffle orders no memory).
 __device__ __forceinline__ bool split_wait(uint64_t* bar, uint32_t parity, unsigned int* status, unsigned int tag) {
   bool ok = true;
   if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, status, tag);
-  return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+  ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+  __syncwarp();
+  return ok;
 }
 __device__ __forceinline__ void split_zero(uint32_t base, uint32_t bytes) {
   for (uint32_t i = threadIdx.x * 16; i < bytes; i += SP_THREADS * 16)

@@ -25,3 +25,14 @@ def test_they_take_tensor_memory_before_they_let_the_next_kernel_start():
                 assert body.count("if (warp == 1) split_take_columns(") == 1 and body.count("split_take_columns") == 1, name
                 assert "tmem_alloc" not in body and "pdl_trigger(" not in body, name
     assert holders == ["contract_split.cu", "conv_split.cu", "gemm_split.cu"]
+
+
+def _body(name, function):
+    """The text of a function of one source, from its name to the brace that closes it at the start of a line."""
+    return _code(name).split(function + "(", 1)[1].split("\n}\n")[0]
+
+
+def test_a_wait_by_one_lane_orders_the_reads_of_the_others():
+    """One lane asks the barrier for all: the lanes that read behind it need a warp barrier, since a shuffle orders no memory."""
+    body = _body("split_f32.cuh", "bool split_wait")
+    assert body.index("mbar_wait(") < body.index("__syncwarp()") and body.rindex("__shfl_sync") < body.index("__syncwarp()")
