@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1) conv_split_kernel(const __grid_
 }
 
 // [rows][C] floats to [rows][C4], C4 the next multiple of 4, with zeros: the copy engine steps through rows of 16 bytes.
-__global__ void __launch_bounds__(256) pad_floats_kernel(const float* __restrict__ in, float4* __restrict__ out, long pieces, int C, int per_row) {
+__global__ void __launch_bounds__(256) pad_floats_kernel(const float* in, float4* __restrict__ out, long pieces, int C, int per_row) {
   pdl_trigger();
   pdl_wait();
   const long i = (long)blockIdx.x * 256 + threadIdx.x;

@@ -274,7 +274,9 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
       const long tn = WHOLE ? tn_at : t / p.tiles_m, m = (WHOLE ? m_at : (t - tn * p.tiles_m) * TILE_M) + quad * 32 + lane;
       if ((m_at += TILE_M) >= p.M) { m_at = 0; ++tn_at; }
       float scale = 0.f;                             // (float16) of column half * 16 + lane + (lane & 16), given to the others when it is needed
-      if (KIND == GS_BACK_F16 && half * 16 + lane + (lane & 16) < p.n) scale = __ldg(p.scale + tn * p.n + half * 16 + lane + (lane & 16));
+      // (an ordinary load: the kernel before this one, which this one may start beside, writes the scales)
+      if (KIND == GS_BACK_F16 && half * 16 + lane + (lane & 16) < p.n)
+        scale = *const_cast<const volatile float*>(p.scale + tn * p.n + half * 16 + lane + (lane & 16));
       float sum[2][16];
 #pragma unroll
       for (int k = 0; k < 2; ++k)

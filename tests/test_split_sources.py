@@ -36,3 +36,12 @@ def test_a_wait_by_one_lane_orders_the_reads_of_the_others():
     """One lane asks the barrier for all: the lanes that read behind it need a warp barrier, since a shuffle orders no memory."""
     body = _body("split_f32.cuh", "bool split_wait")
     assert body.index("mbar_wait(") < body.index("__syncwarp()") and body.rindex("__shfl_sync") < body.index("__syncwarp()")
+
+
+def test_nothing_that_an_earlier_kernel_writes_is_read_as_constant():
+    """These kernels may start while the kernel before them still writes what they read: no load through the read-only cache, whose
+    lines nothing invalidates within a kernel."""
+    for name in ("contract_split.cu", "conv_split.cu", "gemm_split.cu", "split_f32.cuh"):
+        assert "__ldg" not in _code(name) and "ld.global.nc" not in _code(name), name
+    # (a const pointer that nothing else writes through may be read that way too; chan_scale is the caller's)
+    assert re.findall(r"const \w+\* __restrict__ (\w+)", "".join(map(_code, ("contract_split.cu", "conv_split.cu", "gemm_split.cu")))) == ["chan_scale"]
