@@ -369,6 +369,7 @@ bool plan_contract_split(const xconv_desc* d, ContractSplitPlan* p) {
   p->ng_n = (int)cdivl(d->Cin, 32 * p->ng_per);
   p->cols = KS > 1 ? p->j_per * 32 : p->ng_per * 32;
   const long units = (long)p->mg_n * p->dy_n * KD * p->ng_n * p->j_n;
+  if (units * (p->cols / 4) * TILE_M >= 1L << 31) return false;      // (the sum of the splits counts groups of four entries in 32 bits)
   const int qa = p->a_blocks * p->cwa / 4, qb = p->ng_per * 8;
   // clocks of an MMA: the tensor pipe, or the A tile and B at shared memory's rate
   const long mma = std::max(p->cols / 2, 32 + p->cols / 4);

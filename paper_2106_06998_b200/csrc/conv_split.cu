@@ -393,6 +393,7 @@ bool plan_conv_split(const xconv_desc* d, bool dgrad, ConvSplitPlan* p) {
   p->tiles_n = (int)cdivl(Co, SP_MAX_N);
   p->n = round_up((int)cdivl(Co, p->tiles_n), 16);
   p->ocw = p->n % 32 == 0 ? 32 : 16;
+  if ((long)p->tiles_n * p->nb * KD * T2 * p->n * (p->cw / 4) >= 1L << 31) return false;      // (conv_split_weights counts pieces in 32 bits)
   const uint32_t rb = 2 * (uint32_t)p->cw;
   p->w_tile = 3 * (uint32_t)p->n * rb;
   const uint32_t w_slot = up1k(p->w_tile), budget = SMEM_LIMIT - 4096;
