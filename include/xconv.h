@@ -48,7 +48,9 @@
  * Results are bit-reproducible run to run (fixed reduction order, no atomics).
  * A value that is not finite makes every result that it enters not finite.  In the offset contraction products with positions
  * outside the image are multiplications by zero, so that an infinity of an input or output channel can also make NaN of
- * entries of dW of that channel whose own terms are finite; other channels keep their bits.
+ * entries of dW of that channel whose own terms are finite; in the convolutions an infinite or NaN weight meets the
+ * zeros outside the image in the same way, and can make NaN of results of its channel at the border.  Other channels keep
+ * their bits.
  *
  * ERRORS.  Every entry point returns an xconv_status.  Every check of the arguments is made before the
  * first launch: a call that returns XCONV_ERR_INVALID_ARG, XCONV_ERR_UNSUPPORTED, XCONV_ERR_ALIGNMENT

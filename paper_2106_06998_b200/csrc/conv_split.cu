@@ -11,7 +11,7 @@
 // Three MMAs per k-step of 16 channels form the six products, in three groups of n accumulator columns:
 //   h x [h | m | l] -> columns 0..3n,   m x [h | m] -> columns n..3n,   l x h -> columns 2n..3n.
 // The A tile is then read three times instead of six (what bounds narrow MMAs), and the products hh have a column group of their
-// own.  Two accumulator sets take rows of offsets in turn (1 x 1: four blocks of channels), an issuing warp each; eight epilogue warps
+// own (which also decides results that are not finite: split_f32.cuh).  Two accumulator sets take rows of offsets in turn (1 x 1: four blocks of channels), an issuing warp each; eight epilogue warps
 // add the three groups of a set to float registers.
 //
 // Error against 64 bits on 120 random layers, times that of the FP32 multiply-adds (conv_fma.cu): 0.35 in the median, nowhere more
@@ -31,10 +31,9 @@ namespace xconv {
 constexpr int CS_A_SLOTS = 4, CS_W_SLOTS = 5;      // (weights: of each issuer's ring)
 
 struct ConvSplitParams {
-  const float *in, *wt;
+  const float* wt;
   const uint8_t* wimg;
-  int Ci, Co, W, H, dgrad;
-  int Cw;                                          // channels in of the weights (Ci counts padded ones)
+  int Co, Cw, dgrad;                               // channels out and in of the weights
   int KD, T, pad, pad_d;
   int P, pw, ph, patches_x, patches_y, depth;
   uint32_t patches, items;
@@ -62,19 +61,6 @@ __device__ __forceinline__ float cs_weight(const ConvSplitParams& p, int co, int
   return p.dgrad ? p.wt[((size_t)ci * p.T + (p.T - 1 - t)) * p.Co + co] : p.wt[((size_t)co * p.T + t) * p.Cw + ci];
 }
 
-// The sum of channel co at pixel (x, y, z) of image b by multiply-adds.
-template <int KS>
-__device__ __noinline__ float cs_plain_sum(const ConvSplitParams& p, int x, int y, int z, int b, int co) {
-  float acc = 0.f;
-  for (int t = 0; t < p.T; ++t) {
-    const int zz = z + t / (KS * KS) - p.pad_d, yy = y + t % (KS * KS) / KS - p.pad, xx = x + t % KS - p.pad;
-    if (zz < 0 || zz >= p.depth || yy < 0 || yy >= p.H || xx < 0 || xx >= p.W) continue;
-    const float* src = p.in + ((((size_t)b * p.depth + zz) * p.H + yy) * p.W + xx) * p.Ci;
-    for (int c = 0; c < p.Cw; ++c) acc = fmaf(src[c], cs_weight(p, co, c, t), acc);
-  }
-  return acc;
-}
-
 // The weights' tile images, a thread per four channels in of one row.  T here counts the offsets of all depths.
 __global__ void __launch_bounds__(256) conv_split_weights(const ConvSplitParams p, uint8_t* __restrict__ img, int tiles_n) {
   pdl_trigger();
@@ -94,7 +80,7 @@ __global__ void __launch_bounds__(256) conv_split_weights(const ConvSplitParams 
     float v[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) v[k] = co < p.Co && c + k < p.Cw ? cs_weight(p, co, c + k, t) : 0.f;
-    const Split4 s = split4(make_float4(v[0], v[1], v[2], v[3]));
+    const Split4 s = split4_apart<Bf16Parts>(make_float4(v[0], v[1], v[2], v[3]));
     uint8_t* base = img + (size_t)tile * p.w_tile;
     const auto at = [&](int plane) {
       const uint32_t rr = (uint32_t)(plane * p.n + row);
@@ -297,7 +283,6 @@ __global__ void __launch_bounds__(SP_THREADS, 1) conv_split_kernel(const __grid_
       if (!cs_epi_all(ok)) break;                    // the warps leave together
       const int n0 = (int)w.tn * p.n;
       if (live) {
-        float check = 0.f;                           // 0, or NaN
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
           const int g = half + 2 * k;
@@ -305,22 +290,10 @@ __global__ void __launch_bounds__(SP_THREADS, 1) conv_split_kernel(const __grid_
           const uint32_t row = base + p.o_off + (uint32_t)(p.ocw == 32 ? g >> 1 : g) * p.o_bytes + v * orb;
           const uint32_t piece = p.ocw == 32 ? (uint32_t)(g & 1) * 4 : 0u;
 #pragma unroll
-          for (int e = 0; e < 16; ++e) check = fmaf(sum[k][e], 0.f, check);
-#pragma unroll
           for (int e = 0; e < 16; e += 4)
             asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(row + (((piece + (e >> 2)) ^ swz) << 4)),
                          "f"(sum[k][e]), "f"(sum[k][e + 1]), "f"(sum[k][e + 2]), "f"(sum[k][e + 3]) : "memory");
         }
-        // a value that cannot be split makes NaN of every sum it enters: those are taken again
-        if (!(check == 0.f) && w.x + mx < p.W && w.y + my < p.H)
-          for (int c = half * 16; c < p.n && n0 + c < p.Co; c += (c & 15) == 15 ? 17 : 1) {
-            const uint32_t row = base + p.o_off + (uint32_t)(c / p.ocw) * p.o_bytes + v * orb, at = (uint32_t)(c % p.ocw);
-            const uint32_t addr = row + ((((at >> 2) ^ swz) << 4) | ((at & 3u) << 2));
-            float old;
-            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(old) : "r"(addr) : "memory");
-            if (old - old != 0.f)
-              asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(cs_plain_sum<KS>(p, w.x + mx, w.y + my, w.z, w.b, n0 + c)) : "memory");
-          }
       }
       fence_async_smem();
       cs_epi_sync();
@@ -440,9 +413,9 @@ xconv_status run_conv_split(const xconv_desc* d, const ConvSplitPlan& pl, bool d
   const ConvGeo g = conv_geo(d);
   if (xconv_status s = pad_floats(in, reinterpret_cast<float*>(scratch + pl.img_bytes), g.W * g.H * g.D * g.B, Ci, st)) return s;
   ConvSplitParams p{};
-  p.in = in; p.wt = Wt;
+  p.wt = Wt;
   p.wimg = reinterpret_cast<const uint8_t*>(scratch);
-  p.Ci = round_up(Ci, 4); p.Cw = Ci; p.Co = Co; p.W = (int)g.W; p.H = (int)g.H; p.dgrad = dgrad ? 1 : 0;
+  p.Cw = Ci; p.Co = Co; p.dgrad = dgrad ? 1 : 0;
   p.KD = KD; p.T = KD * K * K; p.pad = (K - 1) / 2; p.pad_d = (KD - 1) / 2;
   p.pw = pl.pw; p.ph = pl.ph; p.P = pl.pw + K - 1;
   p.patches_x = (int)cdivl(g.W, p.pw); p.patches_y = (int)cdivl(g.H, p.ph); p.depth = (int)g.D;
@@ -475,7 +448,7 @@ xconv_status run_conv_split(const xconv_desc* d, const ConvSplitPlan& pl, bool d
     const uint32_t box[5] = {(uint32_t)cb, (uint32_t)bw, (uint32_t)bh, 1, 1};
     return make_map_f32(m, ptr, 5, dims, str, box, swizzle);
   };
-  if (!image_map(&mi, in, p.Ci, p.cw, p.P, p.ph + K - 1, CU_TENSOR_MAP_SWIZZLE_NONE) ||
+  if (!image_map(&mi, in, round_up(Ci, 4), p.cw, p.P, p.ph + K - 1, CU_TENSOR_MAP_SWIZZLE_NONE) ||
       !image_map(&mo, out, Co, p.ocw, p.pw, p.ph, p.ocw == 32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B))
     return XCONV_ERR_CUDA;
   const size_t smem = 1024 + (size_t)p.f_off + (size_t)p.f_slots * p.f_slot;

@@ -34,7 +34,7 @@ template <> struct GsElement<GS_BACK_BF16> { using type = bf16; };
 template <> struct GsElement<GS_BACK_F16> { using type = f16; };
 
 struct GemmSplitParams {
-  const void* A; const float* B;                   // sketch: rows, columns [.][K]; back-probe: Y [K][M], and S
+  const float* B;                                  // back-probe: S
   const uint8_t* img; const float* scale;
   void* out;
   long M, K, N;
@@ -50,18 +50,6 @@ struct GemmSplitParams {
   unsigned int *status, tag;
 };
 
-// A sum by multiply-adds: row m, column n, every `step`-th k-block from `kb` on.
-template <int KIND>
-__device__ __noinline__ float gs_plain_sum(const GemmSplitParams& p, long m, long n, long kb, long step) {
-  using T = typename GsElement<KIND>::type;
-  const T* A = static_cast<const T*>(p.A);
-  float acc = 0.f;
-  for (; kb < p.kblocks; kb += step)
-    for (long k = kb * GS_TERMS; k < min(p.K, (kb + 1) * GS_TERMS); ++k)
-      acc = KIND != GS_SKETCH ? fmaf(to_f(A[k * p.M + m]), p.B[n * p.s_row + k * p.s_k], acc) : fmaf(to_f(A[m * p.K + k]), p.B[n * p.K + k], acc);
-  return acc;
-}
-
 // The tile images of S for the back-probe: [column tile][k-block][3n rows of 32 terms], four terms at a time.
 template <int KIND>
 __device__ __forceinline__ void write_image(const GemmSplitParams& p, uint8_t* img, long j, long kb, int q, float scale) {
@@ -70,7 +58,8 @@ __device__ __forceinline__ void write_image(const GemmSplitParams& p, uint8_t* i
   float v[4];
 #pragma unroll
   for (int e = 0; e < 4; ++e) v[e] = j < p.N && k + e < p.K ? p.B[j * p.s_row + (k + e) * p.s_k] * scale : 0.f;
-  const Split4 s = KIND == GS_BACK_F16 ? split4_f16(make_float4(v[0], v[1], v[2], v[3])) : split4(make_float4(v[0], v[1], v[2], v[3]));
+  const float4 v4 = make_float4(v[0], v[1], v[2], v[3]);
+  const Split4 s = KIND == GS_BACK_F16 ? split4_apart<F16Parts>(v4) : split4_apart<Bf16Parts>(v4);
   uint8_t* base = img + (tn * p.kblocks + kb) * (long)p.b_bytes;
   *reinterpret_cast<uint2*>(base + swizzled(6, (uint32_t)row, 8 * q)) = s.h;
   *reinterpret_cast<uint2*>(base + swizzled(6, (uint32_t)(p.n + row), 8 * q)) = s.m;
@@ -88,24 +77,21 @@ __global__ void __launch_bounds__(256) split_sketch_images(const GemmSplitParams
 }
 
 // float16 parts.  A row of S is scaled by the power of two that brings its largest value to 2^14: the parts then hold what is above 2^-39 of
-// it, whatever the row's range.  (A row with a value that is not finite keeps its scale: its parts hold infinities or NaN.)  A warp per row.
+// it, whatever the row's range.  (The largest finite one: infinities and NaN stay what they are.)  A warp per row.
 __global__ void __launch_bounds__(256) split_sketch_images_f16(const GemmSplitParams p, uint8_t* __restrict__ img, float* __restrict__ scale) {
   pdl_trigger();
   pdl_wait();
   const int lane = threadIdx.x & 31;
   for (long j = (long)blockIdx.x * 8 + (threadIdx.x >> 5); j < (long)p.tiles_n * p.n; j += (long)gridDim.x * 8) {
     float top = 0.f;
-    bool finite = true;
     if (j < p.N)
       for (long k = lane; k < p.K; k += 32) {
         const float v = fabsf(p.B[j * p.s_row + k * p.s_k]);
-        finite = finite && v - v == 0.f;
-        top = fmaxf(top, v);
+        if (v - v == 0.f) top = fmaxf(top, v);
       }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
-    finite = __all_sync(0xffffffffu, finite);
-    const int e = finite && top > 0.f ? max(-100, ilogbf(top) - 14) : 0;
+    const int e = top > 0.f ? max(-100, ilogbf(top) - 14) : 0;
     if (lane == 0) scale[j] = ldexpf(1.f, e);
     const float down = ldexpf(1.f, -e);
     for (long i = lane; i < p.kblocks * 8; i += 32) write_image<GS_BACK_F16>(p, img, j, i >> 3, (int)(i & 7), down);
@@ -298,26 +284,15 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         // Results of 16 bits go through shared memory, so that a lane stores 16 bytes of a row (2 bytes a lane and store: 4900 clocks a tile;
         // boxes of 16 rows of 64 bytes by the copy engine: 2080).
         __syncwarp();                                // the last tile is read
-        float check = 0.f;                           // 0, or NaN
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
           if (half + 2 * k >= groups) break;
 #pragma unroll
           for (int e = 0; e < 16; ++e) {
             if (KIND == GS_BACK_F16) sum[k][e] *= __shfl_sync(0xffffffffu, scale, k * 16 + e);
-            check = fmaf(sum[k][e], 0.f, check);
             st_shared_16(stage + (uint32_t)((k * 16 + e) * 64 + lane * 2), from_f<T>(sum[k][e]));
           }
         }
-        // a value that cannot be split makes NaN of every sum it enters: those are taken again
-        if (!(check == 0.f) && m < p.M)
-          for (int c = 0; c < 32 && half * 16 + c + (c & 16) < p.n; ++c) {
-            const long n = tn * p.n + half * 16 + c + (c & 16);
-            if (n >= p.N) continue;
-            const float v = to_f(ld_shared_16<T>(stage + (uint32_t)(c * 64 + lane * 2)));
-            if (v - v != 0.f)
-              st_shared_16(stage + (uint32_t)(c * 64 + lane * 2), from_f<T>(gs_plain_sum<KIND>(p, m, n, kb0, kstep)));
-          }
         __syncwarp();
         const long at = m - lane + (lane & 3) * 8;   // (rows have a multiple of 8 positions)
         T* to = static_cast<T*>(p.out) + at;
@@ -331,24 +306,14 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
       }
       if (m >= p.M) continue;
       T* out = static_cast<T*>(p.out) + (BACK ? 0 : kb0 * p.M * p.N) + m * p.o_m;
-      float check = 0.f;                             // 0, or NaN
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
         if (half + 2 * k >= groups) break;
         const long n0 = tn * p.n + (half + 2 * k) * 16;
 #pragma unroll
-        for (int e = 0; e < 16; ++e) {
-          check = fmaf(sum[k][e], 0.f, check);
+        for (int e = 0; e < 16; ++e)
           if (n0 + e < p.N) out[(n0 + e) * p.o_n] = from_f<T>(sum[k][e]);
-        }
       }
-      // a value that cannot be split makes NaN of every sum it enters: those are taken again
-      if (!(check == 0.f))
-        for (int c = half * 16; c < p.n && tn * p.n + c < p.N; c += (c & 15) == 15 ? 17 : 1) {
-          T* at = out + (tn * p.n + c) * p.o_n;
-          const float v = to_f(*at);
-          if (v - v != 0.f) *at = from_f<T>(gs_plain_sum<KIND>(p, m, tn * p.n + c, kb0, kstep));
-        }
     }
   } else if (!WHOLE && warp >= SP_CONVERT) {
     // ------------------------------------------------------------------ conversion
@@ -469,7 +434,6 @@ xconv_status run_sketch_split(const xconv_desc* d, const GemmSplitPlan& pl, cons
                               cudaStream_t st) {
   GemmSplitParams p{};
   const float *rows = pl.swap ? X : Z, *cols = pl.swap ? Z : X;
-  p.A = rows; p.B = cols;
   p.out = part;
   p.M = pl.swap ? d->B : d->r;
   p.N = pl.swap ? d->r : d->B;
@@ -490,7 +454,7 @@ xconv_status run_backprobe_split(const xconv_desc* d, const GemmSplitPlan& pl, c
                                  char* ws_head, char* scratch, cudaStream_t st) {
   const int kind = back_kind(d);
   GemmSplitParams p{};
-  p.A = Y; p.B = S; p.s_row = s_row; p.s_k = s_k;
+  p.B = S; p.s_row = s_row; p.s_k = s_k;
   p.img = reinterpret_cast<const uint8_t*>(scratch);
   p.out = L;
   p.M = (long)(d->D > 1 ? d->D : 1) * d->H * d->W * d->Cout;

@@ -8,10 +8,15 @@
 // so the products hh are summed apart from the small ones, or behind them, in chains of a few MMAs, and the chains are added in
 // float registers (see the kernels for the errors measured).
 //
-// A value that no part can hold as such -- an infinity, NaN, a finite one that rounds up to an infinity -- leaves NaN in one of
-// its parts, so every sum it enters becomes NaN, and no other one: the kernels take sums that are not finite again by plain
-// multiply-adds.  (Below 2^-110 the last part runs out of exponents: what is lost there is 2^-134 in itself.)
+// Values that are not finite.  The first part of an infinity or NaN is the value itself, so the products hh are what the definition makes of
+// it; the other parts are NaN then.  Where the products hh have a column group of their own, a chain whose group is not finite counts
+// with that group alone (split_add_set): results that are not finite cost no more than others, and no other result changes.  The contraction, whose
+// products share an accumulator, and whose zeros between image rows would meet them, takes sums that are not finite again.
+// The first part of a finite value is finite (a value that would round up to an infinity is cut to the largest bfloat16 instead).
+// (Below 2^-110 the last part runs out of exponents: what is lost there is 2^-134 in itself.)
 #pragma once
+
+#include <type_traits>
 
 #include "common.cuh"
 #include "tc_ptx.cuh"
@@ -20,34 +25,58 @@ namespace xconv {
 
 // The parts of four neighbouring floats, packed in pairs.
 struct Split4 { uint2 h, m, l; };
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
-  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<const uint32_t*>(&v);
-}
-__device__ __forceinline__ float low_f(uint32_t v) { return __uint_as_float(v << 16); }
-__device__ __forceinline__ float high_f(uint32_t v) { return __uint_as_float(v & 0xFFFF0000u); }
-__device__ __forceinline__ Split4 split4(float4 v) {
-  Split4 s;
-  s.h.x = pack_bf16(v.x, v.y); s.h.y = pack_bf16(v.z, v.w);
-  v.x -= low_f(s.h.x); v.y -= high_f(s.h.x); v.z -= low_f(s.h.y); v.w -= high_f(s.h.y);
-  s.m.x = pack_bf16(v.x, v.y); s.m.y = pack_bf16(v.z, v.w);
-  v.x -= low_f(s.m.x); v.y -= high_f(s.m.x); v.z -= low_f(s.m.y); v.w -= high_f(s.m.y);
-  s.l.x = pack_bf16(v.x, v.y); s.l.y = pack_bf16(v.z, v.w);
-  return s;
-}
-// Three float16 parts (11 + 11 + 11 bits; the caller scales, so that no part is out of the type's range).
-__device__ __forceinline__ uint32_t take_f16(float& a, float& b) {
-  const __half2 v = __floats2half2_rn(a, b);
-  const float2 f = __half22float2(v);
+struct Bf16Parts {
+  static __device__ __forceinline__ uint32_t pack(float a, float b) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&v);
+  }
+  static __device__ __forceinline__ float2 floats(uint32_t v) { return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xFFFF0000u)); }
+};
+// (11 + 11 + 11 bits; the caller scales, so that no part is out of the type's range.)
+struct F16Parts {
+  static __device__ __forceinline__ uint32_t pack(float a, float b) {
+    const __half2 v = __floats2half2_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&v);
+  }
+  static __device__ __forceinline__ float2 floats(uint32_t v) { return __half22float2(*reinterpret_cast<const __half2*>(&v)); }
+};
+template <class Parts>
+__device__ __forceinline__ void take_part(float& a, float& b, uint32_t v) {
+  const float2 f = Parts::floats(v);
   a -= f.x; b -= f.y;
-  return *reinterpret_cast<const uint32_t*>(&v);
 }
-__device__ __forceinline__ Split4 split4_f16(float4 v) {
+// The parts of v, the first one given; `v` is what is left of it behind the second one then.
+template <class Parts>
+__device__ __forceinline__ Split4 split_behind(float4& v, uint2 h) {
   Split4 s;
-  s.h.x = take_f16(v.x, v.y); s.h.y = take_f16(v.z, v.w);
-  s.m.x = take_f16(v.x, v.y); s.m.y = take_f16(v.z, v.w);
-  s.l.x = take_f16(v.x, v.y); s.l.y = take_f16(v.z, v.w);
+  s.h = h;
+  take_part<Parts>(v.x, v.y, h.x); take_part<Parts>(v.z, v.w, h.y);
+  s.m = make_uint2(Parts::pack(v.x, v.y), Parts::pack(v.z, v.w));
+  take_part<Parts>(v.x, v.y, s.m.x); take_part<Parts>(v.z, v.w, s.m.y);
+  s.l = make_uint2(Parts::pack(v.x, v.y), Parts::pack(v.z, v.w));
   return s;
+}
+constexpr float BF16_MAX = 3.3895313892515355e38f;
+__device__ __forceinline__ float cut_to_bf16(float v) { return v - v == 0.f ? fminf(fmaxf(v, -BF16_MAX), BF16_MAX) : v; }
+__device__ __forceinline__ Split4 split4(float4 v) {
+  float4 left = v;
+  Split4 s = split_behind<Bf16Parts>(left, make_uint2(Bf16Parts::pack(v.x, v.y), Bf16Parts::pack(v.z, v.w)));
+  const float check = (left.x + left.y) + (left.z + left.w);        // NaN: one of the first parts is not finite
+  if (check != check)
+    s = split_behind<Bf16Parts>(v, make_uint2(Bf16Parts::pack(cut_to_bf16(v.x), cut_to_bf16(v.y)), Bf16Parts::pack(cut_to_bf16(v.z), cut_to_bf16(v.w))));
+  return s;
+}
+// A first part that rounded to zero of values that are not zero becomes the type's smallest number, so that an infinity times it is
+// one.  (For operands that a kernel of their own splits.  Where the boxes are split, an infinity times a float below 2^-134 is NaN.)
+__device__ __forceinline__ uint32_t never_zero(uint32_t h, float a, float b) {
+  if (a != 0.f && !(h & 0x7FFFu)) h |= 1u;
+  if (b != 0.f && !(h & 0x7FFF0000u)) h |= 0x10000u;
+  return h;
+}
+template <class Parts>
+__device__ __forceinline__ Split4 split4_apart(float4 v) {
+  const float4 c = std::is_same<Parts, Bf16Parts>::value ? make_float4(cut_to_bf16(v.x), cut_to_bf16(v.y), cut_to_bf16(v.z), cut_to_bf16(v.w)) : v;
+  return split_behind<Parts>(v, make_uint2(never_zero(Parts::pack(c.x, c.y), v.x, v.y), never_zero(Parts::pack(c.z, c.w), v.z, v.w)));
 }
 __device__ __forceinline__ void st_shared_v2(uint32_t addr, uint2 v) {
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(v.x), "r"(v.y) : "memory");
@@ -55,12 +84,6 @@ __device__ __forceinline__ void st_shared_v2(uint32_t addr, uint2 v) {
 template <typename T>
 __device__ __forceinline__ void st_shared_16(uint32_t addr, T v) {
   asm volatile("st.shared.b16 [%0], %1;" ::"r"(addr), "h"(*reinterpret_cast<const uint16_t*>(&v)) : "memory");
-}
-template <typename T>
-__device__ __forceinline__ T ld_shared_16(uint32_t addr) {
-  uint16_t v;
-  asm volatile("ld.shared.b16 %0, [%1];" : "=h"(v) : "r"(addr) : "memory");
-  return *reinterpret_cast<const T*>(&v);
 }
 __device__ __forceinline__ uint4 ld_shared_v4(uint32_t addr) {
   uint4 v;
@@ -151,7 +174,8 @@ __device__ __forceinline__ void split_zero(uint32_t base, uint32_t bytes) {
     asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(base + i), "r"(0) : "memory");
   fence_async_smem();
 }
-// An accumulator set's three groups of n columns added to the sums of an epilogue warp's column groups (`half`, `half` + 2 of 16).
+// An accumulator set's three groups of n columns added to the sums of an epilogue warp's column groups (`half`, `half` + 2 of 16).  A sum
+// of products hh that is not finite counts alone.
 __device__ __forceinline__ void split_add_set(uint32_t set, uint32_t n, int half, float (&sum)[2][16]) {
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
@@ -161,13 +185,26 @@ __device__ __forceinline__ void split_add_set(uint32_t set, uint32_t n, int half
     tmem_ld16_issue(set + n + c, x);
     tmem_ld16_issue(set + 2 * n + c, y);
     tmem_ld_wait(x); tmem_ld_wait(y);
-    float small[16];
+    float t[16];
 #pragma unroll
-    for (int e = 0; e < 16; ++e) small[e] = __uint_as_float(x[e]) + __uint_as_float(y[e]);
+    for (int e = 0; e < 16; ++e) t[e] = __uint_as_float(x[e]) + __uint_as_float(y[e]);
     tmem_ld16_issue(set + c, x);
     tmem_ld_wait(x);
+    float check = 0.f;                               // 0, or NaN
 #pragma unroll
-    for (int e = 0; e < 16; ++e) sum[k][e] += __uint_as_float(x[e]) + small[e];
+    for (int e = 0; e < 16; ++e) {
+      t[e] += __uint_as_float(x[e]);
+      check = fmaf(t[e], 0.f, check);
+    }
+    if (!(check == 0.f)) {
+#pragma unroll
+      for (int e = 0; e < 16; ++e) {
+        const float hh = __uint_as_float(x[e]);
+        if (hh - hh != 0.f) t[e] = hh;
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 16; ++e) sum[k][e] += t[e];
   }
 }
 
