@@ -98,25 +98,121 @@ struct SplitWalk {
   }
 };
 
-// One entry's sum over this split's patches by multiply-adds.
-__device__ __noinline__ float split_plain_sum(const ContractSplitParams& p, uint32_t i0, uint32_t n, int dz, SplitEntry e) {
+// The sums of 32 entries with one offset over this split's patches by multiply-adds, a lane each: over the patches in the set `only`, or all; rows
+// of patches that are `piece` modulo `pieces`.  Ends early when no lane's sum can change any more: NaN, or not finite among finite terms.
+constexpr int CT_SET = 2048;                       // patches of a CTA that a set tells apart (patch i: bit i modulo this)
+__device__ __forceinline__ float split_line(const ContractSplitParams& p, uint32_t i0, uint32_t n, int dz, int dy, int dx, int ch_l, int ch_z, bool wanted,
+                                            const uint32_t* only, uint32_t piece, uint32_t pieces) {
+  constexpr int U = 16;                              // terms whose loads are under way together
   float acc = 0.f;
+  uint32_t turn = 0;
   SplitWalk w(p, i0);
   for (uint32_t i = 0; i < n; ++i, w.step(p)) {
+    if (only && !((only[i % CT_SET / 32] >> (i % 32)) & 1u)) continue;
     const int zz = w.z + dz - p.pad_d;
     if (zz < 0 || zz >= p.depth) continue;
-    const float* Lp = p.L + ((size_t)w.b * p.depth + w.z) * p.H * p.W * p.Lc + e.m;
-    const float* Zp = p.Z + ((size_t)w.b * p.depth + zz) * p.H * p.W * p.Zc + e.n;
+    const float* Lp = p.L + (((size_t)w.b * p.depth + w.z) * p.H * p.W + w.x) * p.Lc + ch_l;
+    const float* Zp = p.Z + (((size_t)w.b * p.depth + zz) * p.H * p.W + w.x) * p.Zc + ch_z;
+    const int x0 = max(0, p.pad - dx - w.x), x1 = min(min(p.pw, p.W - w.x), p.W - w.x + p.pad - dx);
     for (int y = 0; y < p.ph; ++y) {
-      const int yz = p.rows_on_a ? w.y + y : w.y + y + e.dy - p.pad, yl = yz - (e.dy - p.pad);
+      const int yz = p.rows_on_a ? w.y + y : w.y + y + dy - p.pad, yl = yz - (dy - p.pad);
       if (yz < 0 || yz >= p.H || yl < 0 || yl >= p.H) continue;
-      for (int x = 0; x < p.pw; ++x) {
-        const int xl = w.x + x, xz = xl + e.dx - p.pad;
-        if (xl < p.W && xz >= 0 && xz < p.W) acc = fmaf(Lp[((size_t)yl * p.W + xl) * p.Lc], Zp[((size_t)yz * p.W + xz) * p.Zc], acc);
+      if (turn++ % pieces != piece) continue;
+      const float *l = Lp + (size_t)yl * p.W * p.Lc, *z = Zp + (ptrdiff_t)(yz * (ptrdiff_t)p.W + dx - p.pad) * p.Zc;
+      for (int x = x0; x < x1; x += U) {
+        float a[U], b[U];
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+          const bool in = x + k < x1;
+          a[k] = in ? l[(size_t)(x + k) * p.Lc] : 0.f;
+          b[k] = in ? z[(size_t)(x + k) * p.Zc] : 0.f;
+        }
+#pragma unroll
+        for (int k = 0; k < U; ++k) acc = fmaf(a[k], b[k], acc);
+        if (__all_sync(0xffffffffu, !wanted || (only ? acc != acc : acc - acc != 0.f))) return acc;
       }
     }
   }
   return acc;
+}
+
+// A value that cannot be split makes NaN of every sum it enters, and of those that it meets with a zero between image rows or outside the
+// image: the sums of the unit's tile that are not finite are taken again, by all warps of the block.  A warp takes 32 columns of a row, or 32
+// rows of a column, whichever leaves fewer of them to do: one infinity among the values of L is rows, one in Z columns.  First over the patches that
+// hold values that are not finite (`odd`): what comes out not finite is the result.  The others met such a value with a zero, or ran over;
+// they are summed over all patches, which finite terms alone enter.
+// us a call (contraction and sum of the splits), 64 -> 64 channels, 64 probes of 32 x 32: finite values 53; one infinity in L 93, in Z 72; all of L
+// NaN 118, or so large that every sum runs over 165.  One thread a sum, serially, took 16900 and 1060 for one infinity.
+__device__ __noinline__ void split_again(const ContractSplitParams& p, const SplitUnit& u, float* tile, uint32_t i0, uint32_t n, const uint32_t* odd,
+                                         uint32_t* scratch) {
+  constexpr int WARPS = SP_THREADS / 32, MAP = TILE_M * 3, LIST = MAP + 8, SUMS = LIST + CT_COLS * 4;
+  uint32_t *map = scratch, *lines = scratch + MAP, *list = scratch + LIST, &count = lines[7];      // map: sums to do, [row][column / 32]; lines: rows, columns with one
+  float* sums = reinterpret_cast<float*>(scratch + SUMS);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const auto at = [&](int row, int c) { return tile + (size_t)(c >> 2) * 4 * TILE_M + row * 4 + (c & 3); };
+  for (int i = tid; i < LIST; i += SP_THREADS) scratch[i] = 0;
+  bool any = tid < CT_SET / 32 && odd[tid] != 0;
+  const bool some_odd = __syncthreads_or(any);
+#pragma unroll 4
+  for (int i = tid; i < p.cols / 4 * TILE_M; i += SP_THREADS) {
+    const float4 v = reinterpret_cast<const float4*>(tile)[i];
+    const float f[4] = {v.x, v.y, v.z, v.w};
+    const int row = i % TILE_M, c0 = i / TILE_M * 4;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (f[k] - f[k] != 0.f && split_live(p, split_entry(p, u, row, c0 + k))) {
+        atomicOr(&map[row * 3 + (c0 >> 5)], 1u << ((c0 + k) & 31));
+        atomicOr(&lines[row >> 5], 1u << (row & 31));
+        atomicOr(&lines[4 + (c0 >> 5)], 1u << ((c0 + k) & 31));
+      }
+  }
+  __syncthreads();
+  const bool by_row = __popc(lines[0]) + __popc(lines[1]) + __popc(lines[2]) + __popc(lines[3]) <= __popc(lines[4]) + __popc(lines[5]) + __popc(lines[6]);
+  const int wide = (by_row ? p.cols : TILE_M) / 32, words = (by_row ? TILE_M : p.cols) * wide;
+  struct Word { int row, c; bool wanted; unsigned lanes; SplitEntry e; int dy, dx; };
+  const auto word_at = [&](int word) {
+    Word t;
+    const int line = word / wide, other = word % wide * 32 + lane;
+    t.row = by_row ? line : other; t.c = by_row ? other : line;
+    t.wanted = (map[t.row * 3 + (t.c >> 5)] >> (t.c & 31)) & 1u;
+    t.lanes = __ballot_sync(0xffffffffu, t.wanted);
+    t.e = split_entry(p, u, t.row, t.c);
+    const int first = max(0, __ffs(t.lanes) - 1);               // (the offset is that of all wanted lanes)
+    t.dy = __shfl_sync(0xffffffffu, t.e.dy, first); t.dx = __shfl_sync(0xffffffffu, t.e.dx, first);
+    return t;
+  };
+  const auto line_sum = [&](const Word& t, const uint32_t* only, uint32_t piece, uint32_t pieces) {
+    return split_line(p, i0, n, u.dz, t.dy, t.dx, t.wanted ? t.e.m : 0, t.wanted ? t.e.n : 0, t.wanted, only, piece, pieces);
+  };
+  for (int word = warp; word < words; word += WARPS) {
+    const Word t = word_at(word);
+    if (!t.lanes) continue;
+    bool left = t.wanted;
+    if (some_odd) {
+      const float s = line_sum(t, odd, 0, 1);
+      if (left && s - s != 0.f) {
+        *at(t.row, t.c) = s;
+        atomicAnd(&map[t.row * 3 + (t.c >> 5)], ~(1u << (t.c & 31)));
+        left = false;
+      }
+    }
+    if (__any_sync(0xffffffffu, left) && lane == 0) list[atomicAdd(&count, 1u)] = (uint32_t)word;
+  }
+  __syncthreads();
+  const int todo = (int)count, pieces = max(1, WARPS / max(1, todo));
+  for (int item = warp; item < todo * pieces; item += WARPS) {
+    const Word t = word_at((int)list[item / pieces]);
+    const float s = line_sum(t, nullptr, (uint32_t)(item % pieces), (uint32_t)pieces);
+    if (pieces > 1) sums[item * 32 + lane] = s;
+    else if (t.wanted) *at(t.row, t.c) = s;
+  }
+  if (pieces == 1) return;
+  __syncthreads();
+  if (warp >= todo) return;
+  const Word t = word_at((int)list[warp]);
+  float s = 0.f;
+  for (int k = 0; k < pieces; ++k) s += sums[(warp * pieces + k) * 32 + lane];
+  if (t.wanted) *at(t.row, t.c) = s;
 }
 
 template <int RBA, int QA, int QB>
@@ -125,7 +221,7 @@ contract_split_kernel(const __grid_constant__ CUtensorMap map_l, const __grid_co
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full[CT_STAGES], empty[CT_STAGES], acc_full[2], acc_empty[2];
   __shared__ __align__(8) uint64_t f_full[SP_FLOATS], f_empty[SP_FLOATS];
-  __shared__ uint32_t tmem_slot;
+  __shared__ uint32_t tmem_slot, odd[CT_SET / 32];      // odd: patches with a value that is not finite
   __shared__ int go;
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -139,6 +235,7 @@ contract_split_kernel(const __grid_constant__ CUtensorMap map_l, const __grid_co
     prefetch_tmap(&map_z);
   }
   if (warp == 1) split_take_columns(&tmem_slot, 256u);
+  if (threadIdx.x < CT_SET / 32) odd[threadIdx.x] = 0;
   // (L between the rows of a patch and both tensors behind the last one stay zero)
   split_zero(base, (uint32_t)p.stages * p.stage_bytes);
   pdl_wait();
@@ -155,6 +252,7 @@ contract_split_kernel(const __grid_constant__ CUtensorMap map_l, const __grid_co
   const uint32_t n = (uint32_t)((unsigned long long)p.items * (split + 1) / p.splits) - i0;     // patches of this CTA (>= 1)
   const SplitUnit u = split_unit(p, ug);
   const int chains = (p.ksteps + p.chunk - 1) / p.chunk;
+  int again = 0;                                     // a sum is not finite
 
   if (!go) {
     // fall through to the teardown
@@ -213,8 +311,9 @@ contract_split_kernel(const __grid_constant__ CUtensorMap map_l, const __grid_co
     for (uint32_t i = 0; i < n; ++i) {
       if (!split_wait(&empty[s], par, p.status, p.tag) || !split_wait(&f_full[f], f_par, p.status, p.tag)) break;
       const uint32_t from = base + p.f_off + f * p.f_slot, to = base + s * p.stage_bytes;
-      split_box<RBA == 128 ? 7 : 6, QA, true>(from, p.pw * p.a_rows, to, p.a_plane, p.a_blk, (uint32_t)(p.KS - 1), p.inv_pw);
-      split_box<6, QB, false>(from + p.f_b, p.P * p.ph, to + p.a_bytes, p.b_plane, p.b_blk, 0u, 0u);
+      const bool odd_l = split_box<RBA == 128 ? 7 : 6, QA, true>(from, p.pw * p.a_rows, to, p.a_plane, p.a_blk, (uint32_t)(p.KS - 1), p.inv_pw);
+      const bool odd_z = split_box<6, QB, false>(from + p.f_b, p.P * p.ph, to + p.a_bytes, p.b_plane, p.b_blk, 0u, 0u);
+      if (odd_l || odd_z) atomicOr(&odd[i % CT_SET / 32], 1u << (i % 32));
       split_stage_done(&full[s], &f_empty[f]);
       if (++s == (uint32_t)p.stages) { s = 0; par ^= 1u; }
       if (++f == (uint32_t)p.f_slots) { f = 0; f_par ^= 1u; }
@@ -281,21 +380,17 @@ contract_split_kernel(const __grid_constant__ CUtensorMap map_l, const __grid_co
         for (int e = 0; e < 16; e += 4)
           *reinterpret_cast<float4*>(dst + (size_t)e * TILE_M) = make_float4(sum[k][e], sum[k][e + 1], sum[k][e + 2], sum[k][e + 3]);
       }
-      // a value that cannot be split makes NaN of every sum it enters: those are taken again
-      if (!(check == 0.f))
-        for (int c = half * 16; c < p.cols; c += (c & 15) == 15 ? 17 : 1) {
-          float* at = part + (size_t)(c >> 2) * 4 * TILE_M + (c & 3);
-          const SplitEntry e = split_entry(p, u, row, c);
-          if (split_live(p, e) && *at - *at != 0.f) *at = split_plain_sum(p, i0, n, u.dz, e);
-        }
+      again = !(check == 0.f);
     }
   }
   tc_fence_before();
-  __syncthreads();
+  again = __syncthreads_or(again);
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, 256u);
   }
+  if (again) split_again(p, u, p.part + ((size_t)ug * p.splits + split) * (size_t)p.cols * TILE_M, i0, n, odd,
+                         reinterpret_cast<uint32_t*>(smem_raw));
 }
 
 // dW[m][offset][n] = scale(n) * sum over splits, four neighbouring columns of one accumulator row per group.  LANES threads share a

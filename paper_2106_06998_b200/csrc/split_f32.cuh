@@ -58,12 +58,16 @@ __device__ __forceinline__ Split4 split_behind(float4& v, uint2 h) {
 }
 constexpr float BF16_MAX = 3.3895313892515355e38f;
 __device__ __forceinline__ float cut_to_bf16(float v) { return v - v == 0.f ? fminf(fmaxf(v, -BF16_MAX), BF16_MAX) : v; }
-__device__ __forceinline__ Split4 split4(float4 v) {
+// (`odd`: a value is not finite.)
+__device__ __forceinline__ Split4 split4(float4 v, bool& odd) {
   float4 left = v;
   Split4 s = split_behind<Bf16Parts>(left, make_uint2(Bf16Parts::pack(v.x, v.y), Bf16Parts::pack(v.z, v.w)));
   const float check = (left.x + left.y) + (left.z + left.w);        // NaN: one of the first parts is not finite
-  if (check != check)
+  if (check != check) {
+    const float finite = (v.x - v.x) + (v.y - v.y) + (v.z - v.z) + (v.w - v.w);      // 0, or NaN
+    odd = odd || finite != 0.f;
     s = split_behind<Bf16Parts>(v, make_uint2(Bf16Parts::pack(cut_to_bf16(v.x), cut_to_bf16(v.y)), Bf16Parts::pack(cut_to_bf16(v.z), cut_to_bf16(v.w))));
+  }
   return s;
 }
 // A first part that rounded to zero of values that are not zero becomes the type's smallest number, so that an infinity times it is
@@ -127,12 +131,14 @@ constexpr int SP_FLOATS = 4;                         // float boxes under way at
 // three tiles of 2^RBS bytes a row in blocks `block` bytes apart, the parts `plane` bytes apart.  Position i goes to row i, or with PITCH to
 // row i + (KS - 1) floor(i / width): `gap` = KS - 1, `inv` = ceil(2^20 / width).  By the twelve conversion warps; some 40 instructions for four
 // values (with copies of single pieces by the threads, their addresses and bounds, it was 100, and the conversion bounded every kernel).
+// Returns whether this thread met a value that is not finite.
 template <int RBS, int QSHIFT, bool PITCH>
-__device__ __forceinline__ void split_box(uint32_t src, int positions, uint32_t dst, uint32_t plane, uint32_t block, uint32_t gap, uint32_t inv) {
+__device__ __forceinline__ bool split_box(uint32_t src, int positions, uint32_t dst, uint32_t plane, uint32_t block, uint32_t gap, uint32_t inv) {
   constexpr int U = 4;
   const int tid = threadIdx.x - SP_CONVERT * 32, items = positions << QSHIFT;
   const uint32_t q = (uint32_t)tid & ((1u << QSHIFT) - 1u), byte = (q & ((1u << (RBS - 3)) - 1u)) * 8;
   const uint32_t to = dst + (QSHIFT > RBS - 3 ? (q >> (RBS - 3)) * block : 0u);
+  bool odd = false;
   src += (uint32_t)tid * 16;
   for (int i = tid; i < items; i += U * SP_CONVERTERS, src += U * SP_CONVERTERS * 16) {
     float4 v[U];
@@ -146,13 +152,14 @@ __device__ __forceinline__ void split_box(uint32_t src, int positions, uint32_t 
       if (u > 0 && i + u * SP_CONVERTERS >= items) break;
       uint32_t row = (uint32_t)(i + u * SP_CONVERTERS) >> QSHIFT;
       if (PITCH) row += ((row * inv) >> 20) * gap;
-      const Split4 s = split4(v[u]);
+      const Split4 s = split4(v[u], odd);
       const uint32_t at = to + swizzled(RBS, row, byte);
       st_shared_v2(at, s.h);
       st_shared_v2(at + plane, s.m);
       st_shared_v2(at + 2 * plane, s.l);
     }
   }
+  return odd;
 }
 // What the converters do when a stage's tiles are written and its floats read.
 __device__ __forceinline__ void split_stage_done(uint64_t* full, uint64_t* floats_empty) {
