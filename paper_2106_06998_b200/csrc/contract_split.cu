@@ -11,7 +11,8 @@
 // per k-step whatever the width of the patch (7 pixels: 7 of 9 are work, where whole k-steps per row left 7 of 16).
 //
 // The copy engine brings the floats of both boxes, twelve warps write their parts; six passes over a chain of k-steps, the products of the small parts
-// first and hh last, leave an accumulator that was rounded towards zero a few times at its full size only.  Two accumulator
+// first (scaled up, split_f32.cuh; the MMA scales the accumulator down between them) and hh last, leave an accumulator that was rounded towards
+// zero a few times at its full size only.  Two accumulator
 // sets take the chains in turn, eight epilogue warps add them in float registers (48 sums a thread), and the
 // sums of the splits are added in fixed order by a second kernel.
 //
@@ -141,30 +142,32 @@ __device__ __forceinline__ float split_line(const ContractSplitParams& p, uint32
 // rows of a column, whichever leaves fewer of them to do: one infinity among the values of L is rows, one in Z columns.  First over the patches that
 // hold values that are not finite (`odd`): what comes out not finite is the result.  The others met such a value with a zero, or ran over;
 // they are summed over all patches, which finite terms alone enter.
-// us a call (contraction and sum of the splits), 64 -> 64 channels, 64 probes of 32 x 32: finite values 53; one infinity in L 93, in Z 72; all of L
-// NaN 118, or so large that every sum runs over 165.  One thread a sum, serially, took 16900 and 1060 for one infinity.
+// us a call (contraction and sum of the splits), 64 -> 64 channels, 64 probes of 32 x 32: finite values 53; one infinity in L 97, in Z 72; all of L
+// NaN 123, or so large that every sum runs over 173.  One thread a sum, serially, took 16900 and 1060 for one infinity.
 __device__ __noinline__ void split_again(const ContractSplitParams& p, const SplitUnit& u, float* tile, uint32_t i0, uint32_t n, const uint32_t* odd,
                                          uint32_t* scratch) {
-  constexpr int WARPS = SP_THREADS / 32, MAP = TILE_M * 3, LIST = MAP + 8, SUMS = LIST + CT_COLS * 4;
-  uint32_t *map = scratch, *lines = scratch + MAP, *list = scratch + LIST, &count = lines[7];      // map: sums to do, [row][column / 32]; lines: rows, columns with one
+  constexpr int WARPS = SP_THREADS / 32, MAP = CT_COLS * 4, LIST = MAP + 8, SUMS = LIST + CT_COLS * 4;
+  uint32_t *map = scratch, *lines = scratch + MAP, *list = scratch + LIST, &count = lines[7];      // map: sums to do, [column][row / 32]; lines: rows, columns with one
   float* sums = reinterpret_cast<float*>(scratch + SUMS);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const auto at = [&](int row, int c) { return tile + (size_t)(c >> 2) * 4 * TILE_M + row * 4 + (c & 3); };
   for (int i = tid; i < LIST; i += SP_THREADS) scratch[i] = 0;
   bool any = tid < CT_SET / 32 && odd[tid] != 0;
   const bool some_odd = __syncthreads_or(any);
-#pragma unroll 4
-  for (int i = tid; i < p.cols / 4 * TILE_M; i += SP_THREADS) {
+#pragma unroll 2
+  for (int i = tid; i < p.cols / 4 * TILE_M; i += SP_THREADS) {      // (a warp: four columns of 32 rows)
     const float4 v = reinterpret_cast<const float4*>(tile)[i];
     const float f[4] = {v.x, v.y, v.z, v.w};
     const int row = i % TILE_M, c0 = i / TILE_M * 4;
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (f[k] - f[k] != 0.f && split_live(p, split_entry(p, u, row, c0 + k))) {
-        atomicOr(&map[row * 3 + (c0 >> 5)], 1u << ((c0 + k) & 31));
-        atomicOr(&lines[row >> 5], 1u << (row & 31));
-        atomicOr(&lines[4 + (c0 >> 5)], 1u << ((c0 + k) & 31));
-      }
+    for (int k = 0; k < 4; ++k) {
+      if (!__any_sync(0xffffffffu, f[k] - f[k] != 0.f)) continue;
+      const unsigned rows = __ballot_sync(0xffffffffu, f[k] - f[k] != 0.f && split_live(p, split_entry(p, u, row, c0 + k)));
+      if (lane != 0 || !rows) continue;
+      map[(c0 + k) * 4 + (row >> 5)] = rows;
+      atomicOr(&lines[row >> 5], rows);
+      atomicOr(&lines[4 + (c0 >> 5)], 1u << ((c0 + k) & 31));
+    }
   }
   __syncthreads();
   const bool by_row = __popc(lines[0]) + __popc(lines[1]) + __popc(lines[2]) + __popc(lines[3]) <= __popc(lines[4]) + __popc(lines[5]) + __popc(lines[6]);
@@ -174,7 +177,7 @@ __device__ __noinline__ void split_again(const ContractSplitParams& p, const Spl
     Word t;
     const int line = word / wide, other = word % wide * 32 + lane;
     t.row = by_row ? line : other; t.c = by_row ? other : line;
-    t.wanted = (map[t.row * 3 + (t.c >> 5)] >> (t.c & 31)) & 1u;
+    t.wanted = (map[t.c * 4 + (t.row >> 5)] >> (t.row & 31)) & 1u;
     t.lanes = __ballot_sync(0xffffffffu, t.wanted);
     t.e = split_entry(p, u, t.row, t.c);
     const int first = max(0, __ffs(t.lanes) - 1);               // (the offset is that of all wanted lanes)
@@ -192,7 +195,7 @@ __device__ __noinline__ void split_again(const ContractSplitParams& p, const Spl
       const float s = line_sum(t, odd, 0, 1);
       if (left && s - s != 0.f) {
         *at(t.row, t.c) = s;
-        atomicAnd(&map[t.row * 3 + (t.c >> 5)], ~(1u << (t.c & 31)));
+        atomicAnd(&map[t.c * 4 + (t.row >> 5)], ~(1u << (t.row & 31)));
         left = false;
       }
     }
@@ -281,23 +284,24 @@ contract_split_kernel(const __grid_constant__ CUtensorMap map_l, const __grid_co
         tc_fence_after();
         const int kn = min(p.chunk, p.ksteps - k0);
         uint32_t acc = 0;
-        // lh, hl, mm, mh, hm, hh
-        auto pass = [&](uint32_t a, uint32_t b) {
+        // lh, hl, mm (times 2^14), mh, hm (2^7), hh: the accumulator is scaled down between them
+        auto pass = [&](uint32_t a, uint32_t b, bool down) {
 #pragma unroll
           for (int k = 0; k < CT_CHAIN; ++k) {
             if (k >= kn) break;
-            umma_warp(d, a, a_hi, b, b_hi, idesc, acc);
+            if (k == 0 && down) umma_warp_down<7>(d, a, a_hi, b, b_hi, idesc);
+            else umma_warp(d, a, a_hi, b, b_hi, idesc, acc);
             acc = 1u;
             a += a_step;
             b += b_step;
           }
         };
-        pass(a0 + 2 * ap, b0);
-        pass(a0, b0 + 2 * bp);
-        pass(a0 + ap, b0 + bp);
-        pass(a0 + ap, b0);
-        pass(a0, b0 + bp);
-        pass(a0, b0);
+        pass(a0 + 2 * ap, b0, false);
+        pass(a0, b0 + 2 * bp, false);
+        pass(a0 + ap, b0 + bp, false);
+        pass(a0 + ap, b0, true);
+        pass(a0, b0 + bp, false);
+        pass(a0, b0, true);
         umma_commit_warp(&acc_full[own]);
       }
       if (!ok) break;
@@ -311,10 +315,15 @@ contract_split_kernel(const __grid_constant__ CUtensorMap map_l, const __grid_co
     for (uint32_t i = 0; i < n; ++i) {
       if (!split_wait(&empty[s], par, p.status, p.tag) || !split_wait(&f_full[f], f_par, p.status, p.tag)) break;
       const uint32_t from = base + p.f_off + f * p.f_slot, to = base + s * p.stage_bytes;
-      const bool odd_l = split_box<RBA == 128 ? 7 : 6, QA, true>(from, p.pw * p.a_rows, to, p.a_plane, p.a_blk, (uint32_t)(p.KS - 1), p.inv_pw);
-      const bool odd_z = split_box<6, QB, false>(from + p.f_b, p.P * p.ph, to + p.a_bytes, p.b_plane, p.b_blk, 0u, 0u);
-      if (odd_l || odd_z) atomicOr(&odd[i % CT_SET / 32], 1u << (i % 32));
-      split_stage_done(&full[s], &f_empty[f]);
+      const SplitBox of_l{from, p.pw * p.a_rows, to, p.a_plane, p.a_blk, (uint32_t)(p.KS - 1), p.inv_pw};
+      const SplitBox of_z{from + p.f_b, p.P * p.ph, to + p.a_bytes, p.b_plane, p.b_blk, 0u, 0u};
+      float2 check = make_float2(0.f, 0.f);
+      split_box<RBA == 128 ? 7 : 6, QA, true>(of_l, check);
+      split_box<6, QB, false>(of_z, check);
+      split_stage_done(&full[s], &f_empty[f], check, [&] {
+        const bool odd_l = split_box_again<RBA == 128 ? 7 : 6, QA, true>(of_l), odd_z = split_box_again<6, QB, false>(of_z);
+        if (odd_l || odd_z) atomicOr(&odd[i % CT_SET / 32], 1u << (i % 32));
+      });
       if (++s == (uint32_t)p.stages) { s = 0; par ^= 1u; }
       if (++f == (uint32_t)p.f_slots) { f = 0; f_par ^= 1u; }
     }

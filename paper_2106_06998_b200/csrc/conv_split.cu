@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1) conv_split_kernel(const __grid_
         ok = split_wait(&t_full[buf], par, p.status, p.tag);
         if (!ok) break;
         tc_fence_after();
-        split_add_set(tmem_q + buf * (uint32_t)(3 * p.n), (uint32_t)p.n, half, sum);
+        split_add_set<Bf16Parts>(tmem_q + buf * (uint32_t)(3 * p.n), (uint32_t)p.n, half, sum);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&t_empty[buf]);
@@ -310,8 +310,10 @@ __global__ void __launch_bounds__(SP_THREADS, 1) conv_split_kernel(const __grid_
     uint32_t s = 0, par = 1, f = 0, f_par = 0;
     for (uint32_t j = 0; j < total; ++j) {
       if (!split_wait(&a_empty[s], par, p.status, p.tag) || !split_wait(&f_full[f], f_par, p.status, p.tag)) break;
-      split_box<RB == 64 ? 6 : 5, RB == 64 ? 3 : 2, false>(base + p.f_off + f * p.f_slot, p.npos, base + s * p.a_slot, p.a_plane, 0u, 0u, 0u);
-      split_stage_done(&a_full[s], &f_empty[f]);
+      const SplitBox box{base + p.f_off + f * p.f_slot, p.npos, base + s * p.a_slot, p.a_plane, 0u, 0u, 0u};
+      float2 check = make_float2(0.f, 0.f);
+      split_box<RB == 64 ? 6 : 5, RB == 64 ? 3 : 2, false>(box, check);
+      split_stage_done(&a_full[s], &f_empty[f], check, [&] { split_box_again<RB == 64 ? 6 : 5, RB == 64 ? 3 : 2, false>(box); });
       if (++s == (uint32_t)p.a_slots) { s = 0; par ^= 1u; }
       if (++f == (uint32_t)p.f_slots) { f = 0; f_par ^= 1u; }
     }

@@ -29,9 +29,9 @@ namespace xconv {
 constexpr int GS_STAGES = 8, GS_TERMS = 32;
 constexpr uint32_t GS_OUT = 2048;                  // a staging tile of 16-bit results: 32 columns of 32 positions
 enum : int { GS_SKETCH = 0, GS_BACK = 1, GS_BACK_BF16 = 2, GS_BACK_F16 = 3 };
-template <int KIND> struct GsElement { using type = float; };
-template <> struct GsElement<GS_BACK_BF16> { using type = bf16; };
-template <> struct GsElement<GS_BACK_F16> { using type = f16; };
+template <int KIND> struct GsElement { using type = float; using parts = Bf16Parts; };
+template <> struct GsElement<GS_BACK_BF16> { using type = bf16; using parts = Bf16Parts; };
+template <> struct GsElement<GS_BACK_F16> { using type = f16; using parts = F16Parts; };
 
 struct GemmSplitParams {
   const float* B;                                  // back-probe: S
@@ -58,8 +58,7 @@ __device__ __forceinline__ void write_image(const GemmSplitParams& p, uint8_t* i
   float v[4];
 #pragma unroll
   for (int e = 0; e < 4; ++e) v[e] = j < p.N && k + e < p.K ? p.B[j * p.s_row + (k + e) * p.s_k] * scale : 0.f;
-  const float4 v4 = make_float4(v[0], v[1], v[2], v[3]);
-  const Split4 s = KIND == GS_BACK_F16 ? split4_apart<F16Parts>(v4) : split4_apart<Bf16Parts>(v4);
+  const Split4 s = split4_apart<typename GsElement<KIND>::parts>(make_float4(v[0], v[1], v[2], v[3]));
   uint8_t* base = img + (tn * p.kblocks + kb) * (long)p.b_bytes;
   *reinterpret_cast<uint2*>(base + swizzled(6, (uint32_t)row, 8 * q)) = s.h;
   *reinterpret_cast<uint2*>(base + swizzled(6, (uint32_t)(p.n + row), 8 * q)) = s.m;
@@ -272,7 +271,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         ok = split_wait(&acc_full[buf], par, p.status, p.tag);
         if (!ok) break;
         tc_fence_after();
-        split_add_set(tmem_q + buf * (uint32_t)(3 * p.n), (uint32_t)p.n, half, sum);
+        split_add_set<typename GsElement<KIND>::parts>(tmem_q + buf * (uint32_t)(3 * p.n), (uint32_t)p.n, half, sum);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&acc_empty[buf]);
@@ -321,13 +320,17 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     for (uint32_t i = 0; i < total; ++i) {
       if (!split_wait(&empty[s], par, p.status, p.tag) || !split_wait(&f_full[f], f_par, p.status, p.tag)) break;
       const uint32_t from = base + p.f_off + f * p.f_slot, to = base + s * p.stage_bytes;
+      float2 check = make_float2(0.f, 0.f);
       if (BACK) {
-        split_box<7, 5, false>(from, GS_TERMS, to, p.a_plane, p.a_plane >> 1, 0u, 0u);
+        const SplitBox box{from, GS_TERMS, to, p.a_plane, p.a_plane >> 1, 0u, 0u};
+        split_box<7, 5, false>(box, check);
+        split_stage_done(&full[s], &f_empty[f], check, [&] { split_box_again<7, 5, false>(box); });
       } else {
-        split_box<6, 3, false>(from, p.f_rows_a, to, p.a_plane, 0u, 0u, 0u);
-        split_box<6, 3, false>(from + p.f_b, p.f_rows_b, to + p.a_bytes, p.b_plane, 0u, 0u, 0u);
+        const SplitBox rows{from, p.f_rows_a, to, p.a_plane, 0u, 0u, 0u}, cols{from + p.f_b, p.f_rows_b, to + p.a_bytes, p.b_plane, 0u, 0u, 0u};
+        split_box<6, 3, false>(rows, check);
+        split_box<6, 3, false>(cols, check);
+        split_stage_done(&full[s], &f_empty[f], check, [&] { split_box_again<6, 3, false>(rows); split_box_again<6, 3, false>(cols); });
       }
-      split_stage_done(&full[s], &f_empty[f]);
       if (++s == (uint32_t)p.stages) { s = 0; par ^= 1u; }
       if (++f == (uint32_t)p.f_slots) { f = 0; f_par ^= 1u; }
     }

@@ -3,17 +3,19 @@
 //   x = h + m + l,   h = rn(x), m = rn(x - h), l = rn(x - h - m)      (8 + 8 + 8 significand bits: exact)
 //
 // and a product of two floats as the six products hh, hm, mh, hl, mm, lh of their parts (each exact in a float; the three
-// left out are below 2^-25 of the product together).  What keeps the sums as precise as FP32 multiply-adds is where they are
-// taken: the accumulators of the tensor cores are not rounded to nearest and lose about 2e-8 of their value with every MMA,
-// so the products hh are summed apart from the small ones, or behind them, in chains of a few MMAs, and the chains are added in
-// float registers (see the kernels for the errors measured).
+// left out are below 2^-24 of the product together: |m| <= 2^-8 |x|, |l| <= 2^-17 |x|).  The second and third parts are kept times 2^7 and
+// 2^14, so that they have the range of the first one: floats below 2^-110 would lose bits of their last part otherwise.  hm and mh then carry
+// 2^7, hl, mm and lh 2^14, none larger than the product itself, and their sums are scaled back (exactly) where they are added.
+//
+// What keeps the sums as precise as FP32 multiply-adds is where they are taken: the accumulators of the tensor cores are not rounded to
+// nearest and lose about 2e-8 of their value with every MMA, so the products hh are summed apart from the small ones, or behind them, in
+// chains of a few MMAs, and the chains are added in float registers (see the kernels for the errors measured).
 //
 // Values that are not finite.  The first part of an infinity or NaN is the value itself, so the products hh are what the definition makes of
 // it; the other parts are NaN then.  Where the products hh have a column group of their own, a chain whose group is not finite counts
 // with that group alone (split_add_set): results that are not finite cost no more than others, and no other result changes.  The contraction, whose
 // products share an accumulator, and whose zeros between image rows would meet them, takes sums that are not finite again.
 // The first part of a finite value is finite (a value that would round up to an infinity is cut to the largest bfloat16 instead).
-// (Below 2^-110 the last part runs out of exponents: what is lost there is 2^-134 in itself.)
 #pragma once
 
 #include <type_traits>
@@ -26,6 +28,7 @@ namespace xconv {
 // The parts of four neighbouring floats, packed in pairs.
 struct Split4 { uint2 h, m, l; };
 struct Bf16Parts {
+  static constexpr float STEP = 128.f;               // between the scales of two parts
   static __device__ __forceinline__ uint32_t pack(float a, float b) {
     const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<const uint32_t*>(&v);
@@ -34,16 +37,18 @@ struct Bf16Parts {
 };
 // (11 + 11 + 11 bits; the caller scales, so that no part is out of the type's range.)
 struct F16Parts {
+  static constexpr float STEP = 1.f;
   static __device__ __forceinline__ uint32_t pack(float a, float b) {
     const __half2 v = __floats2half2_rn(a, b);
     return *reinterpret_cast<const uint32_t*>(&v);
   }
   static __device__ __forceinline__ float2 floats(uint32_t v) { return __half22float2(*reinterpret_cast<const __half2*>(&v)); }
 };
+// (a, b) - (the two values of v), times the scale of the next part; two floats an instruction.
 template <class Parts>
 __device__ __forceinline__ void take_part(float& a, float& b, uint32_t v) {
-  const float2 f = Parts::floats(v);
-  a -= f.x; b -= f.y;
+  const float2 left = __fmul2_rn(__ffma2_rn(Parts::floats(v), make_float2(-1.f, -1.f), make_float2(a, b)), make_float2(Parts::STEP, Parts::STEP));
+  a = left.x; b = left.y;
 }
 // The parts of v, the first one given; `v` is what is left of it behind the second one then.
 template <class Parts>
@@ -58,16 +63,23 @@ __device__ __forceinline__ Split4 split_behind(float4& v, uint2 h) {
 }
 constexpr float BF16_MAX = 3.3895313892515355e38f;
 __device__ __forceinline__ float cut_to_bf16(float v) { return v - v == 0.f ? fminf(fmaxf(v, -BF16_MAX), BF16_MAX) : v; }
-// (`odd`: a value is not finite.)
-__device__ __forceinline__ Split4 split4(float4 v, bool& odd) {
-  float4 left = v;
-  Split4 s = split_behind<Bf16Parts>(left, make_uint2(Bf16Parts::pack(v.x, v.y), Bf16Parts::pack(v.z, v.w)));
-  const float check = (left.x + left.y) + (left.z + left.w);        // NaN: one of the first parts is not finite
-  if (check != check) {
-    const float finite = (v.x - v.x) + (v.y - v.y) + (v.z - v.z) + (v.w - v.w);      // 0, or NaN
-    odd = odd || finite != 0.f;
-    s = split_behind<Bf16Parts>(v, make_uint2(Bf16Parts::pack(cut_to_bf16(v.x), cut_to_bf16(v.y)), Bf16Parts::pack(cut_to_bf16(v.z), cut_to_bf16(v.w))));
-  }
+// 2^7 (c - the two values of v): the multiply-add takes the bfloat16 halves as they are (unpacking them cost four instructions of ten).
+__device__ __forceinline__ float2 left_behind(float2 c, uint32_t v) {
+  const float2 up = __fmul2_rn(c, make_float2(Bf16Parts::STEP, Bf16Parts::STEP));
+  float2 d;
+  asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %2;\n\tfma.rn.f32.bf16 %0, l, %5, %3;\n\tfma.rn.f32.bf16 %1, h, %5, %4;\n\t}"
+      : "=f"(d.x), "=f"(d.y) : "r"(v), "f"(up.x), "f"(up.y), "h"((uint16_t)0xC300));      // -128
+  return d;
+}
+// The parts where the first part of every value is finite and 2^7 times the value is; `check` becomes NaN where not.
+__device__ __forceinline__ Split4 split4(float4 v, float2& check) {
+  Split4 s;
+  s.h = make_uint2(Bf16Parts::pack(v.x, v.y), Bf16Parts::pack(v.z, v.w));
+  float2 a = left_behind(make_float2(v.x, v.y), s.h.x), b = left_behind(make_float2(v.z, v.w), s.h.y);
+  s.m = make_uint2(Bf16Parts::pack(a.x, a.y), Bf16Parts::pack(b.x, b.y));
+  a = left_behind(a, s.m.x); b = left_behind(b, s.m.y);
+  s.l = make_uint2(Bf16Parts::pack(a.x, a.y), Bf16Parts::pack(b.x, b.y));
+  check = __ffma2_rn(a, b, check);
   return s;
 }
 // A first part that rounded to zero of values that are not zero becomes the type's smallest number, so that an infinity times it is
@@ -77,10 +89,12 @@ __device__ __forceinline__ uint32_t never_zero(uint32_t h, float a, float b) {
   if (b != 0.f && !(h & 0x7FFF0000u)) h |= 0x10000u;
   return h;
 }
-template <class Parts>
+template <class Parts, bool NEVER_ZERO = true>
 __device__ __forceinline__ Split4 split4_apart(float4 v) {
   const float4 c = std::is_same<Parts, Bf16Parts>::value ? make_float4(cut_to_bf16(v.x), cut_to_bf16(v.y), cut_to_bf16(v.z), cut_to_bf16(v.w)) : v;
-  return split_behind<Parts>(v, make_uint2(never_zero(Parts::pack(c.x, c.y), v.x, v.y), never_zero(Parts::pack(c.z, c.w), v.z, v.w)));
+  uint2 h = make_uint2(Parts::pack(c.x, c.y), Parts::pack(c.z, c.w));
+  if (NEVER_ZERO) h = make_uint2(never_zero(h.x, v.x, v.y), never_zero(h.y, v.z, v.w));
+  return split_behind<Parts>(v, h);
 }
 __device__ __forceinline__ void st_shared_v2(uint32_t addr, uint2 v) {
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(v.x), "r"(v.y) : "memory");
@@ -92,6 +106,11 @@ __device__ __forceinline__ void st_shared_16(uint32_t addr, T v) {
 __device__ __forceinline__ uint4 ld_shared_v4(uint32_t addr) {
   uint4 v;
   asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ float4 ld_shared_f4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
   return v;
 }
 // Byte offset of byte `b` of tile row `row` (2^rbs bytes a row, swizzled as the copy engine and the MMA descriptors have it).
@@ -129,41 +148,75 @@ constexpr int SP_FLOATS = 4;                         // float boxes under way at
 
 // A box of floats as the copy engine left it at `src` (2^QSHIFT pieces of four per position, one position behind the other), converted to
 // three tiles of 2^RBS bytes a row in blocks `block` bytes apart, the parts `plane` bytes apart.  Position i goes to row i, or with PITCH to
-// row i + (KS - 1) floor(i / width): `gap` = KS - 1, `inv` = ceil(2^20 / width).  By the twelve conversion warps; some 40 instructions for four
+// row i + (KS - 1) floor(i / width): `gap` = KS - 1, `inv` = ceil(2^20 / width).  By the twelve conversion warps; some 35 instructions for four
 // values (with copies of single pieces by the threads, their addresses and bounds, it was 100, and the conversion bounded every kernel).
-// Returns whether this thread met a value that is not finite.
+// `check` becomes NaN where this form cannot split a value: the box then goes through split_box_again.
+struct SplitBox { uint32_t src; int positions; uint32_t dst, plane, block, gap, inv; };
 template <int RBS, int QSHIFT, bool PITCH>
-__device__ __forceinline__ bool split_box(uint32_t src, int positions, uint32_t dst, uint32_t plane, uint32_t block, uint32_t gap, uint32_t inv) {
+struct SplitPlaces {
+  uint32_t to, byte, plane, gap, inv;
+  __device__ __forceinline__ SplitPlaces(const SplitBox& b, int tid) : plane(b.plane), gap(b.gap), inv(b.inv) {
+    const uint32_t q = (uint32_t)tid & ((1u << QSHIFT) - 1u);
+    byte = (q & ((1u << (RBS - 3)) - 1u)) * 8;
+    to = b.dst + (QSHIFT > RBS - 3 ? (q >> (RBS - 3)) * b.block : 0u);
+  }
+  __device__ __forceinline__ uint32_t of(int i) const {
+    uint32_t row = (uint32_t)i >> QSHIFT;
+    if (PITCH) row += ((row * inv) >> 20) * gap;
+    return to + swizzled(RBS, row, byte);
+  }
+  __device__ __forceinline__ void store(uint32_t at, const Split4& s) const {
+    st_shared_v2(at, s.h);
+    st_shared_v2(at + plane, s.m);
+    st_shared_v2(at + 2 * plane, s.l);
+  }
+};
+template <int RBS, int QSHIFT, bool PITCH>
+__device__ __forceinline__ void split_box(const SplitBox& b, float2& check) {
   constexpr int U = 4;
-  const int tid = threadIdx.x - SP_CONVERT * 32, items = positions << QSHIFT;
-  const uint32_t q = (uint32_t)tid & ((1u << QSHIFT) - 1u), byte = (q & ((1u << (RBS - 3)) - 1u)) * 8;
-  const uint32_t to = dst + (QSHIFT > RBS - 3 ? (q >> (RBS - 3)) * block : 0u);
-  bool odd = false;
-  src += (uint32_t)tid * 16;
-  for (int i = tid; i < items; i += U * SP_CONVERTERS, src += U * SP_CONVERTERS * 16) {
+  // Without PITCH the items of a thread lie ROWS rows apart, and the swizzle of every other one differs in one bit at most: the addresses are
+  // constants apart, where working each out took five instructions of forty.
+  constexpr uint32_t ROWS = SP_CONVERTERS >> QSHIFT, FLIP = ((ROWS >> (7 - RBS)) & ((1u << (RBS - 4)) - 1u)) << 4;
+  static_assert(PITCH || ((FLIP == 0 || FLIP == 64) && (2 * ROWS >> (7 - RBS)) % (1u << (RBS - 4)) == 0), "two items ahead the swizzle is the same");
+  const int tid = threadIdx.x - SP_CONVERT * 32, items = b.positions << QSHIFT;
+  const SplitPlaces<RBS, QSHIFT, PITCH> places(b, tid);
+  uint32_t from = b.src + (uint32_t)tid * 16, at = PITCH ? 0u : places.of(tid);
+  for (int i = tid; i < items; i += U * SP_CONVERTERS, from += U * SP_CONVERTERS * 16, at += U * ROWS << RBS) {
     float4 v[U];
 #pragma unroll
     for (int u = 0; u < U; ++u)
-      if (u == 0 || i + u * SP_CONVERTERS < items)
-        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[u].x), "=f"(v[u].y), "=f"(v[u].z), "=f"(v[u].w)
-                     : "r"(src + u * SP_CONVERTERS * 16) : "memory");
+      if (u == 0 || i + u * SP_CONVERTERS < items) v[u] = ld_shared_f4(from + u * SP_CONVERTERS * 16);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       if (u > 0 && i + u * SP_CONVERTERS >= items) break;
-      uint32_t row = (uint32_t)(i + u * SP_CONVERTERS) >> QSHIFT;
-      if (PITCH) row += ((row * inv) >> 20) * gap;
-      const Split4 s = split4(v[u], odd);
-      const uint32_t at = to + swizzled(RBS, row, byte);
-      st_shared_v2(at, s.h);
-      st_shared_v2(at + plane, s.m);
-      st_shared_v2(at + 2 * plane, s.l);
+      places.store(PITCH ? places.of(i + u * SP_CONVERTERS) : (u & 1 ? at ^ FLIP : at) + (u * ROWS << RBS), split4(v[u], check));
     }
+  }
+}
+// The thread's part of a box again, any values; returns whether one is not finite.
+template <int RBS, int QSHIFT, bool PITCH>
+__device__ __noinline__ bool split_box_again(const SplitBox b) {
+  const int tid = threadIdx.x - SP_CONVERT * 32, items = b.positions << QSHIFT;
+  const SplitPlaces<RBS, QSHIFT, PITCH> places(b, tid);
+  bool odd = false;
+#pragma unroll 2
+  for (int i = tid; i < items; i += SP_CONVERTERS) {
+    const float4 v = ld_shared_f4(b.src + (uint32_t)i * 16);
+    odd = odd || (v.x - v.x) + (v.y - v.y) + (v.z - v.z) + (v.w - v.w) != 0.f;
+    places.store(places.of(i), split4_apart<Bf16Parts, false>(v));
   }
   return odd;
 }
-// What the converters do when a stage's tiles are written and its floats read.
-__device__ __forceinline__ void split_stage_done(uint64_t* full, uint64_t* floats_empty) {
+// What the converters do when a stage's tiles are written and its floats read: `again` converts them once more, where a value asks for that
+// (behind the fence, whose time hides the check's).
+template <class Again>
+__device__ __forceinline__ void split_stage_done(uint64_t* full, uint64_t* floats_empty, float2 check, const Again& again) {
   fence_async_smem();
+  const float c = check.x + check.y;
+  if (c != c) {
+    again();
+    fence_async_smem();
+  }
   __syncwarp();
   if ((threadIdx.x & 31) == 0) { mbar_arrive(full); mbar_arrive(floats_empty); }
 }
@@ -183,6 +236,7 @@ __device__ __forceinline__ void split_zero(uint32_t base, uint32_t bytes) {
 }
 // An accumulator set's three groups of n columns added to the sums of an epilogue warp's column groups (`half`, `half` + 2 of 16).  A sum
 // of products hh that is not finite counts alone.
+template <class Parts>
 __device__ __forceinline__ void split_add_set(uint32_t set, uint32_t n, int half, float (&sum)[2][16]) {
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
@@ -192,26 +246,32 @@ __device__ __forceinline__ void split_add_set(uint32_t set, uint32_t n, int half
     tmem_ld16_issue(set + n + c, x);
     tmem_ld16_issue(set + 2 * n + c, y);
     tmem_ld_wait(x); tmem_ld_wait(y);
-    float t[16];
+    const float2 down = make_float2(1.f / Parts::STEP, 1.f / Parts::STEP);
+    const auto pair = [](const uint32_t (&v)[16], int e) { return make_float2(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1])); };
+    float2 t[8];
 #pragma unroll
-    for (int e = 0; e < 16; ++e) t[e] = __uint_as_float(x[e]) + __uint_as_float(y[e]);
+    for (int e = 0; e < 8; ++e) t[e] = __ffma2_rn(pair(y, e), down, pair(x, e));
     tmem_ld16_issue(set + c, x);
     tmem_ld_wait(x);
-    float check = 0.f;                               // 0, or NaN
+    float2 check = make_float2(0.f, 0.f);            // 0, or NaN
 #pragma unroll
-    for (int e = 0; e < 16; ++e) {
-      t[e] += __uint_as_float(x[e]);
-      check = fmaf(t[e], 0.f, check);
+    for (int e = 0; e < 8; ++e) {
+      t[e] = __ffma2_rn(t[e], down, pair(x, e));
+      check = __ffma2_rn(t[e], make_float2(0.f, 0.f), check);
     }
-    if (!(check == 0.f)) {
+    if (!(check.x + check.y == 0.f)) {
 #pragma unroll
-      for (int e = 0; e < 16; ++e) {
-        const float hh = __uint_as_float(x[e]);
-        if (hh - hh != 0.f) t[e] = hh;
+      for (int e = 0; e < 8; ++e) {
+        const float2 hh = pair(x, e);
+        if (hh.x - hh.x != 0.f) t[e].x = hh.x;
+        if (hh.y - hh.y != 0.f) t[e].y = hh.y;
       }
     }
 #pragma unroll
-    for (int e = 0; e < 16; ++e) sum[k][e] += t[e];
+    for (int e = 0; e < 8; ++e) {
+      const float2 a = __fadd2_rn(make_float2(sum[k][2 * e], sum[k][2 * e + 1]), t[e]);
+      sum[k][2 * e] = a.x; sum[k][2 * e + 1] = a.y;
+    }
   }
 }
 
