@@ -263,11 +263,11 @@ __global__ void __launch_bounds__(SP_THREADS, 1) conv_split_kernel(const __grid_
     uint32_t buf = 0, par = 0;
     bool ok = true;
     for (CvWalk w(p, i0, i1); w.it < i1; w.step(p)) {
-      float sum[2][16];                              // channel groups half, half + 2 of 16
+      float2 sum[2][8];                              // channel groups half, half + 2 of 16
 #pragma unroll
       for (int k = 0; k < 2; ++k)
 #pragma unroll
-        for (int e = 0; e < 16; ++e) sum[k][e] = 0.f;
+        for (int e = 0; e < 8; ++e) sum[k][e] = make_float2(0.f, 0.f);
       for (int c = 0; c < chains && ok; ++c) {
         ok = split_wait(&t_full[buf], par, p.status, p.tag);
         if (!ok) break;
@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1) conv_split_kernel(const __grid_
 #pragma unroll
           for (int e = 0; e < 16; e += 4)
             asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(row + (((piece + (e >> 2)) ^ swz) << 4)),
-                         "f"(sum[k][e]), "f"(sum[k][e + 1]), "f"(sum[k][e + 2]), "f"(sum[k][e + 3]) : "memory");
+                         "f"(sum[k][e / 2].x), "f"(sum[k][e / 2].y), "f"(sum[k][e / 2 + 1].x), "f"(sum[k][e / 2 + 1].y) : "memory");
         }
       }
       fence_async_smem();

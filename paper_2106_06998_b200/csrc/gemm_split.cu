@@ -34,7 +34,7 @@ template <> struct GsElement<GS_BACK_BF16> { using type = bf16; using parts = Bf
 template <> struct GsElement<GS_BACK_F16> { using type = f16; using parts = F16Parts; };
 
 struct GemmSplitParams {
-  const float* B;                                  // back-probe: S
+  const float* B; const void* Y;                   // back-probe: S, and Y [K][M]
   const uint8_t* img; const float* scale;
   void* out;
   long M, K, N;
@@ -75,26 +75,69 @@ __global__ void __launch_bounds__(256) split_sketch_images(const GemmSplitParams
   }
 }
 
-// float16 parts.  A row of S is scaled by the power of two that brings its largest value to 2^14: the parts then hold what is above 2^-39 of
-// it, whatever the row's range.  (The largest finite one: infinities and NaN stay what they are.)  A warp per row.
+// float16 parts.  A row of S is scaled by the power of two that brings its largest finite value to 2^14 (infinities and NaN stay what they are).
+// Its parts then hold it down to 2^-61 of that value, all 24 bits of entries above 2^-36 of it.  A row with smaller entries than that (they
+// count where the large ones meet zeros of Y) is marked by the sign of its scale: its sums are taken by multiply-adds.  A warp per row.
 __global__ void __launch_bounds__(256) split_sketch_images_f16(const GemmSplitParams p, uint8_t* __restrict__ img, float* __restrict__ scale) {
   pdl_trigger();
   pdl_wait();
   const int lane = threadIdx.x & 31;
   for (long j = (long)blockIdx.x * 8 + (threadIdx.x >> 5); j < (long)p.tiles_n * p.n; j += (long)gridDim.x * 8) {
-    float top = 0.f;
+    float top = 0.f, low = INFINITY;
     if (j < p.N)
       for (long k = lane; k < p.K; k += 32) {
         const float v = fabsf(p.B[j * p.s_row + k * p.s_k]);
         if (v - v == 0.f) top = fmaxf(top, v);
+        if (v > 0.f) low = fminf(low, v);
       }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
-    const int e = top > 0.f ? max(-100, ilogbf(top) - 14) : 0;
-    if (lane == 0) scale[j] = ldexpf(1.f, e);
-    const float down = ldexpf(1.f, -e);
+    for (int o = 16; o > 0; o >>= 1) {
+      top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+      low = fminf(low, __shfl_xor_sync(0xffffffffu, low, o));
+    }
+    const int e = top > 0.f ? max(-100, (int)(__float_as_uint(top) >> 23) - 127 - 14) : 0;
+    if (lane == 0) scale[j] = copysignf(__uint_as_float((uint32_t)(127 + e) << 23), low - top * 1.4551915228366852e-11f);      // 2^-36
+    const float down = __uint_as_float((uint32_t)(127 - e) << 23);
     for (long i = lane; i < p.kblocks * 8; i += 32) write_image<GS_BACK_F16>(p, img, j, i >> 3, (int)(i & 7), down);
   }
+}
+
+// The results of marked columns (a bit per column of an epilogue warp's staging tile) at 32 positions, by multiply-adds: Q columns, U terms under
+// way at a time.  us, 256 rows, 461 terms, 68208 positions: no row marked 97, one 440, all 8000.  (No more registers than the kernel has: with
+// 150 a thread the next one no longer fits beside it, 12.6 -> 14.4 us for 70 rows, 131 terms.)
+template <int Q, int U>
+__device__ __noinline__ unsigned gs_wide_columns(const GemmSplitParams& p, uint32_t stage, unsigned wide, long n0, long m, int lane) {
+  const f16* Y = static_cast<const f16*>(p.Y) + min(m, p.M - 1);
+  int c[Q];
+  const float* S[Q];
+  float acc[Q];
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    c[q] = __ffs(wide) - 1;
+    wide &= wide - 1;
+    S[q] = p.B + (n0 + c[q] + (c[q] & 16)) * p.s_row;
+    acc[q] = 0.f;
+  }
+#pragma unroll 1
+  for (long k = 0; k < p.K; k += U) {
+    f16 y[U];
+    float s[U][Q];
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+      const long at = min(k + i, p.K - 1);
+      y[i] = Y[at * p.M];
+#pragma unroll
+      for (int q = 0; q < Q; ++q) s[i][q] = S[q][at * p.s_k];
+    }
+#pragma unroll
+    for (int i = 0; i < U; ++i)
+#pragma unroll
+      for (int q = 0; q < Q; ++q)
+        if (k + i < p.K) acc[q] = fmaf(s[i][q], to_f(y[i]), acc[q]);
+  }
+#pragma unroll
+  for (int q = 0; q < Q; ++q) st_shared_16(stage + (uint32_t)(c[q] * 64 + lane * 2), from_f<f16>(acc[q]));
+  return wide;
 }
 
 template <int KIND>
@@ -262,16 +305,16 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
       // (an ordinary load: the kernel before this one, which this one may start beside, writes the scales)
       if (KIND == GS_BACK_F16 && half * 16 + lane + (lane & 16) < p.n)
         scale = *const_cast<const volatile float*>(p.scale + tn * p.n + half * 16 + lane + (lane & 16));
-      float sum[2][16];
+      float2 sum[2][8];
 #pragma unroll
       for (int k = 0; k < 2; ++k)
 #pragma unroll
-        for (int e = 0; e < 16; ++e) sum[k][e] = 0.f;
+        for (int e = 0; e < 8; ++e) sum[k][e] = make_float2(0.f, 0.f);
       for (uint32_t i = 0; i < per_unit; i += 2) {
         ok = split_wait(&acc_full[buf], par, p.status, p.tag);
         if (!ok) break;
         tc_fence_after();
-        split_add_set<typename GsElement<KIND>::parts>(tmem_q + buf * (uint32_t)(3 * p.n), (uint32_t)p.n, half, sum);
+        split_add_set<typename GsElement<KIND>::parts, WHOLE>(tmem_q + buf * (uint32_t)(3 * p.n), (uint32_t)p.n, half, sum);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&acc_empty[buf]);
@@ -288,9 +331,15 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
           if (half + 2 * k >= groups) break;
 #pragma unroll
           for (int e = 0; e < 16; ++e) {
-            if (KIND == GS_BACK_F16) sum[k][e] *= __shfl_sync(0xffffffffu, scale, k * 16 + e);
-            st_shared_16(stage + (uint32_t)((k * 16 + e) * 64 + lane * 2), from_f<T>(sum[k][e]));
+            float v = split_sum(sum, k, e);
+            if (KIND == GS_BACK_F16) v *= __shfl_sync(0xffffffffu, fabsf(scale), k * 16 + e);
+            st_shared_16(stage + (uint32_t)((k * 16 + e) * 64 + lane * 2), from_f<T>(v));
           }
+        }
+        if (KIND == GS_BACK_F16) {
+          unsigned wide = __ballot_sync(0xffffffffu, scale < 0.f);
+          while (wide) wide = __popc(wide) >= 4 ? gs_wide_columns<4, 4>(p, stage, wide, tn * p.n + half * 16, m, lane)
+                                                : gs_wide_columns<1, 8>(p, stage, wide, tn * p.n + half * 16, m, lane);
         }
         __syncwarp();
         const long at = m - lane + (lane & 3) * 8;   // (rows have a multiple of 8 positions)
@@ -311,7 +360,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         const long n0 = tn * p.n + (half + 2 * k) * 16;
 #pragma unroll
         for (int e = 0; e < 16; ++e)
-          if (n0 + e < p.N) out[(n0 + e) * p.o_n] = from_f<T>(sum[k][e]);
+          if (n0 + e < p.N) out[(n0 + e) * p.o_n] = from_f<T>(split_sum(sum, k, e));
       }
     }
   } else if (!WHOLE && warp >= SP_CONVERT) {
@@ -389,6 +438,9 @@ bool plan_backprobe_split(const xconv_desc* d, GemmSplitPlan* p) {
   p->kblocks = cdivl(d->B, GS_TERMS);
   p->splits = 1;
   if (Q % (kind == GS_BACK ? 4 : 8) != 0 || Q >= (1L << 31) - 128) return false;      // (rows on 16-byte boundaries)
+  // (float16: a tile whose rows of S are all marked takes its sums by multiply-adds in the epilogue, some 1500 clocks a term, and the other warps
+  // wait for a second at most)
+  if (kind == GS_BACK_F16 && d->B > 1 << 18) return false;
   const long tiles = p->tiles_m * p->tiles_n, ksteps = cdivl(d->B, 16);
   // (whole rows: measured, 1850 clocks a tile of one k-block, 3000 of three, 10800 of fifteen)
   const double clk = kind == GS_BACK ? std::max({(double)ksteps * split_kstep_clocks(p->n), ksteps * 16 * 32 * 45.0 / 85,
@@ -457,7 +509,7 @@ xconv_status run_backprobe_split(const xconv_desc* d, const GemmSplitPlan& pl, c
                                  char* ws_head, char* scratch, cudaStream_t st) {
   const int kind = back_kind(d);
   GemmSplitParams p{};
-  p.B = S; p.s_row = s_row; p.s_k = s_k;
+  p.B = S; p.Y = Y; p.s_row = s_row; p.s_k = s_k;
   p.img = reinterpret_cast<const uint8_t*>(scratch);
   p.out = L;
   p.M = (long)(d->D > 1 ? d->D : 1) * d->H * d->W * d->Cout;

@@ -35,9 +35,10 @@ struct Bf16Parts {
   }
   static __device__ __forceinline__ float2 floats(uint32_t v) { return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xFFFF0000u)); }
 };
-// (11 + 11 + 11 bits; the caller scales, so that no part is out of the type's range.)
+// Three float16 parts (11 + 11 + 11 bits, of values that the caller scales to below 2^15; the second part times 2^12, the third times 2^24, so
+// that what is left of a value below 2^15 is below 2^-47 whatever its size).
 struct F16Parts {
-  static constexpr float STEP = 1.f;
+  static constexpr float STEP = 4096.f;
   static __device__ __forceinline__ uint32_t pack(float a, float b) {
     const __half2 v = __floats2half2_rn(a, b);
     return *reinterpret_cast<const uint32_t*>(&v);
@@ -235,31 +236,39 @@ __device__ __forceinline__ void split_zero(uint32_t base, uint32_t bytes) {
   fence_async_smem();
 }
 // An accumulator set's three groups of n columns added to the sums of an epilogue warp's column groups (`half`, `half` + 2 of 16).  A sum
-// of products hh that is not finite counts alone.
-template <class Parts>
-__device__ __forceinline__ void split_add_set(uint32_t set, uint32_t n, int half, float (&sum)[2][16]) {
+// of products hh that is not finite counts alone.  AT_ONCE: all three groups are loaded together, where there are registers for it.
+template <class Parts, bool AT_ONCE = false>
+__device__ __forceinline__ void split_add_set(uint32_t set, uint32_t n, int half, float2 (&sum)[2][8]) {
+  const float2 down = make_float2(1.f / Parts::STEP, 1.f / Parts::STEP), zero = make_float2(0.f, 0.f);
+  const auto pair = [](const uint32_t (&v)[16], int e) { return make_float2(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1])); };
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
     const uint32_t c = (uint32_t)(half + 2 * k) * 16;
     if (c >= n) break;
-    uint32_t x[16], y[16];
-    tmem_ld16_issue(set + n + c, x);
-    tmem_ld16_issue(set + 2 * n + c, y);
-    tmem_ld_wait(x); tmem_ld_wait(y);
-    const float2 down = make_float2(1.f / Parts::STEP, 1.f / Parts::STEP);
-    const auto pair = [](const uint32_t (&v)[16], int e) { return make_float2(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1])); };
+    uint32_t x[16], y[16], z[16];
+    tmem_ld16_issue(set + n + c, y);
+    tmem_ld16_issue(set + 2 * n + c, z);
+    if (AT_ONCE) tmem_ld16_issue(set + c, x);
+    tmem_ld_wait(y); tmem_ld_wait(z);
     float2 t[8];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) t[e] = __ffma2_rn(pair(y, e), down, pair(x, e));
-    tmem_ld16_issue(set + c, x);
+    for (int e = 0; e < 8; ++e) t[e] = __ffma2_rn(pair(z, e), down, pair(y, e));
+    if (!AT_ONCE) tmem_ld16_issue(set + c, x);
     tmem_ld_wait(x);
-    float2 check = make_float2(0.f, 0.f);            // 0, or NaN
+    constexpr int CHECKS = AT_ONCE ? 4 : 2;          // (chains of multiply-adds: their latency counts)
+    float2 check[CHECKS];                            // 0, or NaN
+#pragma unroll
+    for (int i = 0; i < CHECKS; ++i) check[i] = zero;
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       t[e] = __ffma2_rn(t[e], down, pair(x, e));
-      check = __ffma2_rn(t[e], make_float2(0.f, 0.f), check);
+      check[e & (CHECKS - 1)] = __ffma2_rn(t[e], zero, check[e & (CHECKS - 1)]);
     }
-    if (!(check.x + check.y == 0.f)) {
+#pragma unroll
+    for (int i = CHECKS / 2; i > 0; i >>= 1)
+#pragma unroll
+      for (int j = 0; j < i; ++j) check[j] = __fadd2_rn(check[j], check[j + i]);
+    if (!(check[0].x + check[0].y == 0.f)) {
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         const float2 hh = pair(x, e);
@@ -268,12 +277,10 @@ __device__ __forceinline__ void split_add_set(uint32_t set, uint32_t n, int half
       }
     }
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const float2 a = __fadd2_rn(make_float2(sum[k][2 * e], sum[k][2 * e + 1]), t[e]);
-      sum[k][2 * e] = a.x; sum[k][2 * e + 1] = a.y;
-    }
+    for (int e = 0; e < 8; ++e) sum[k][e] = __fadd2_rn(sum[k][e], t[e]);
   }
 }
+__device__ __forceinline__ float split_sum(const float2 (&sum)[2][8], int k, int e) { return e & 1 ? sum[k][e >> 1].y : sum[k][e >> 1].x; }
 
 static inline uint32_t up1k(uint32_t v) { return (v + 1023u) & ~1023u; }
 // Clocks of the three MMAs of a k-step with n columns per group: the tensor pipe's half clock per column, or shared memory's 128 bytes a clock.

@@ -43,3 +43,26 @@ def test_small_floats(which):
     check("dX", host(xb.xconv_dgrad(dev(dY), dev(Wt))) * up, O.dx_exact(dY, Wt) * up, TOL)
     check("L", host(xb.xconv_backprobe(torch.from_numpy(S).cuda(), dev(dY))) * up, np.tensordot(S.astype(np.float64), dY.astype(np.float64), 1) * up, TOL)
     check("dW", host(xb.xconv_contract(dev(L), dev(Z))) * up, O.wgrad_contract(L, Z, 3, 3) * up, TOL)
+
+
+@pytest.mark.parametrize("dt,u,tiny", [("bf16", 2.0 ** -8, 0.0), ("f16", 2.0 ** -11, 2.0 ** -25)])
+@pytest.mark.parametrize("r,B,C,H,W", [(70, 131, 24, 31, 28), (300, 45, 40, 33, 17)])
+def test_rows_of_the_sketch_with_a_wide_range(dt, u, tiny, r, B, C, H, W):
+    """Large entries of S meet a sample of zeros, so that the small ones decide.  Bound: the rounding of the result (u of it, half the spacing
+    of float16's subnormal numbers), and TOL of the sum of the terms' magnitudes."""
+    Y, S = inputs.draw("normal", (B, C, H, W), 7, dt, 2.0 ** -6), _n((r, B), 8)
+    Y[7] = 0.0
+    S[4] *= np.float32(2.0 ** -10); S[4, 7] = 2.0 ** 20                     # 2^30 within the row: parts
+    S[6, 7] = 2.0 ** 34
+    S[9] *= (2.0 ** -np.linspace(0, 60, B)).astype(np.float32)              # every size down to 2^-60 of the largest: multiply-adds
+    S[r - 1, 7] = 2.0 ** 50
+    S[33, 7] = -2.0 ** 90
+    desc = xb.make_desc(B, C, C, H, W, r, torch.bfloat16 if dt == "bf16" else torch.float16)
+    assert xb.engine_for(desc, xb.OP_BACKPROBE) == "tcgen05_" + dt
+    Yd = xb.to_device(Y, dt)
+    exact = host(Yd)
+    L = host(xb.xconv_backprobe(torch.from_numpy(S).cuda(), Yd))
+    S64 = S.astype(np.float64)
+    want, size = np.tensordot(S64, exact, 1), np.tensordot(np.abs(S64), np.abs(exact), 1)
+    over = np.abs(L - want) > u * np.abs(want) * (1 + TOL) + TOL * size + tiny
+    assert not over.any(), np.unique(np.argwhere(over)[:, 0])
