@@ -677,7 +677,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         const uint32_t idesc_u = p.mode == MODE_BACKPROBE
                                      ? (idesc & ~(0x3Fu << 17)) | ((uint32_t)(w.nblk * 8) << 17) : idesc;
         for (int i = 0; i < w.nkb; ++i) {
-          ok = mbar_wait_warp(&full_bar[s], full_parity, p.status, p.tag);
+          ok = mbar_wait_warp_long(&full_bar[s], full_parity, p.status, p.tag);
           if (!ok) break;
           tc_fence_after();
           uint32_t a_lo = a_lo0 | s16;

@@ -161,9 +161,44 @@ __device__ __forceinline__ void umma_commit_warp(uint64_t* bar) {
   asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
                "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar)) : "memory");
 }
+// One lane asks the barrier, the whole, converged warp gets the answer.
+__device__ __forceinline__ bool mbar_try_warp(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred e, p;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "setp.ne.b32 p, 0, 0;\n\t"
+      "@e mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "vote.sync.any.pred p, p, 0xffffffff;\n\t"
+      "selp.b32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+  return ok != 0;
+}
+static __device__ __noinline__ bool mbar_wait_warp_slow(uint64_t* bar, uint32_t parity, unsigned int* status, unsigned int tag) {
+  for (int i = 0; i < 4096; ++i)
+    if (mbar_try_warp(bar, parity)) return true;
+  const unsigned long long t0 = global_ns();
+  for (;;) {
+    for (int i = 0; i < 256; ++i)
+      if (mbar_try_warp(bar, parity)) return true;
+    if (__any_sync(0xffffffffu, global_ns() - t0 > 1000000000ull)) {
+      atomicExch(status, tag);
+      return false;
+    }
+  }
+}
 // A wait by a whole warp whose outcome is the same in every lane.
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, unsigned int* status, unsigned int tag) {
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, status, tag));
+}
+// The same where the wait is long as a rule (the copies bound the kernel): after the first try one lane asks, the warp stays converged.  32
+// lanes asking for microseconds took shared memory's time from the copies (tc_gemm_kernel: 160 -> 96 channels, 33 x 22, 512 probes 317 -> 287 us); where
+// the wait is short the answer's way is what counts (contract_halo_kernel that way: volumes of 48^3, 32 channels 65 -> 69).
+__device__ __forceinline__ bool mbar_wait_warp_long(uint64_t* bar, uint32_t parity, unsigned int* status, unsigned int tag) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  const bool ok = mbar_wait_warp_slow(bar, parity, status, tag);
+  __syncwarp();                                      // (orders what the one lane has seen before the others' MMAs)
+  return ok;
 }
 
 // mbarrier arrive once every MMA issued so far by this thread has finished.
