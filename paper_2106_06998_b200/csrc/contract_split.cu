@@ -237,19 +237,9 @@ contract_split_kernel(const __grid_constant__ CUtensorMap map_l, const __grid_co
     prefetch_tmap(&map_l);
     prefetch_tmap(&map_z);
   }
-  if (warp == 1) split_take_columns(&tmem_slot, 256u);
   if (threadIdx.x < CT_SET / 32) odd[threadIdx.x] = 0;
   // (L between the rows of a patch and both tensors behind the last one stay zero)
-  split_zero(base, (uint32_t)p.stages * p.stage_bytes);
-  pdl_wait();
-  if (threadIdx.x == 0) {
-    go = (*reinterpret_cast<volatile unsigned int*>(p.status) != p.tag) ? 1 : 0;
-    if (blockIdx.x == 0) reinterpret_cast<volatile unsigned int*>(p.status)[1] = p.tag;
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(&tmem_slot);
+  const uint32_t tmem_base = split_begin(warp, &tmem_slot, 256u, base, (uint32_t)p.stages * p.stage_bytes, p.status, p.tag, &go);
   const uint32_t ug = blockIdx.x / p.splits, split = blockIdx.x - ug * p.splits;
   const uint32_t i0 = (uint32_t)((unsigned long long)p.items * split / p.splits);
   const uint32_t n = (uint32_t)((unsigned long long)p.items * (split + 1) / p.splits) - i0;     // patches of this CTA (>= 1)

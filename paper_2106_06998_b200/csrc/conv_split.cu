@@ -127,16 +127,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1) conv_split_kernel(const __grid_
     prefetch_tmap(&map_in);
     prefetch_tmap(&map_out);
   }
-  if (warp == 1) split_take_columns(&tmem_slot, (uint32_t)p.tmem_cols);
-  pdl_wait();
-  if (threadIdx.x == 0) {
-    go = (*reinterpret_cast<volatile unsigned int*>(p.status) != p.tag) ? 1 : 0;
-    if (blockIdx.x == 0) reinterpret_cast<volatile unsigned int*>(p.status)[1] = p.tag;
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(&tmem_slot);
+  const uint32_t tmem_base = split_begin(warp, &tmem_slot, (uint32_t)p.tmem_cols, 0u, 0u, p.status, p.tag, &go);
   const uint32_t i0 = (uint32_t)((unsigned long long)p.items * blockIdx.x / gridDim.x);
   const uint32_t i1 = (uint32_t)((unsigned long long)p.items * (blockIdx.x + 1) / gridDim.x);
   const int stages = p.nb * p.KD;                   // of a unit: blocks of channels, one depth offset after the other

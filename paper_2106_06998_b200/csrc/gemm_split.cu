@@ -161,17 +161,8 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     prefetch_tmap(&map_a);
     if (!BACK) prefetch_tmap(&map_b);
   }
-  if (warp == 1) split_take_columns(&tmem_slot, (uint32_t)p.tmem_cols);
-  if (!BACK) split_zero(base, (uint32_t)p.stages * p.stage_bytes);      // (rows that no conversion writes are multiplied all the same)
-  pdl_wait();
-  if (threadIdx.x == 0) {
-    go = (*reinterpret_cast<volatile unsigned int*>(p.status) != p.tag) ? 1 : 0;
-    if (blockIdx.x == 0) reinterpret_cast<volatile unsigned int*>(p.status)[1] = p.tag;
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(&tmem_slot);
+  // (the sketch: rows that no conversion writes are multiplied all the same)
+  const uint32_t tmem_base = split_begin(warp, &tmem_slot, (uint32_t)p.tmem_cols, base, BACK ? 0u : (uint32_t)p.stages * p.stage_bytes, p.status, p.tag, &go);
   // this CTA's units -- back-probe: a run of tiles; sketch: one -- and the k-blocks of a unit
   const long tiles = p.tiles_m * p.tiles_n;
   const long t0 = BACK ? tiles * blockIdx.x / gridDim.x : (long)blockIdx.x / p.splits;

@@ -137,9 +137,6 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
                ::"r"(dst), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
 
-// The accumulators' columns of tensor memory, for the kernels on split operands; the go-ahead for the next kernel is given behind them.
-__device__ __forceinline__ void split_take_columns(uint32_t* slot, uint32_t columns) { tmem_alloc_then_trigger(slot, columns); }
-
 // The roles of a block's 24 warps (80 registers a thread): 0 copies operands that were split before, 1 and 2 issue MMAs -- the chains of
 // accumulator set 0 and those of set 1, since one warp's instructions (some 40 clocks an MMA, and the waits between) do not keep the
 // tensor pipe busy beside the other warps -- 3 copies the floats, 4..11 add chains up, two per quarter of the MMA rows, 12..23 convert.
@@ -234,6 +231,22 @@ __device__ __forceinline__ void split_zero(uint32_t base, uint32_t bytes) {
   for (uint32_t i = threadIdx.x * 16; i < bytes; i += SP_THREADS * 16)
     asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(base + i), "r"(0) : "memory");
   fence_async_smem();
+}
+// What a block does between its barriers' set-up and its roles: the accumulators' columns of tensor memory (the go-ahead for the next kernel is
+// given behind them), `bytes` of zeros at `at`, the wait for the kernel before, the tag of this call in the header.  Returns where the
+// columns are; *go: no earlier kernel of the call ran into its time limit.
+__device__ __forceinline__ uint32_t split_begin(int warp, uint32_t* slot, uint32_t columns, uint32_t at, uint32_t bytes, unsigned int* status, unsigned int tag, int* go) {
+  if (warp == 1) tmem_alloc_then_trigger(slot, columns);
+  if (bytes) split_zero(at, bytes);
+  pdl_wait();
+  if (threadIdx.x == 0) {
+    *go = (*reinterpret_cast<volatile unsigned int*>(status) != tag) ? 1 : 0;
+    if (blockIdx.x == 0) reinterpret_cast<volatile unsigned int*>(status)[1] = tag;
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  return *reinterpret_cast<volatile uint32_t*>(slot);
 }
 // An accumulator set's three groups of n columns added to the sums of an epilogue warp's column groups (`half`, `half` + 2 of 16).  A sum
 // of products hh that is not finite counts alone.  AT_ONCE: all three groups are loaded together, where there are registers for it.

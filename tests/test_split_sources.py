@@ -9,22 +9,42 @@ def _code(name):
     return re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
 
 
-def test_they_take_tensor_memory_before_they_let_the_next_kernel_start():
-    """As for the other holders of tensor memory: it is taken through the function that gives the go-ahead behind the allocation (here by
-    way of split_take_columns), once, by one warp, and nothing else in those kernels gives it."""
-    helper = re.findall(r"void split_take_columns\([^)]*\) \{([^}]*)\}", _code("split_f32.cuh"))
-    assert helper == [" tmem_alloc_then_trigger(slot, columns); "]
-    holders = []
+def _functions():
+    """Name, whether it is a kernel, and body of every device function of the sources."""
     for name in sorted(os.listdir(CSRC)):
-        if not name.endswith((".cu", ".cuh")):
-            continue
-        for kernel in _code(name).split("__global__")[1:]:
-            body = kernel.split("\n}\n")[0]
-            if "split_take_columns" in body:
-                holders.append(name)
-                assert body.count("if (warp == 1) split_take_columns(") == 1 and body.count("split_take_columns") == 1, name
-                assert "tmem_alloc" not in body and "pdl_trigger(" not in body, name
-    assert holders == ["contract_split.cu", "conv_split.cu", "gemm_split.cu"]
+        if name.endswith((".cu", ".cuh")):
+            code = re.sub(r"__launch_bounds__\((?:[^()]|\([^()]*\))*\)", "", _code(name))
+            for chunk in code.split("\n}\n"):
+                found = re.findall(r"__(device|global)__[^;{}]*?\b(\w+)\s*\([^;]*?\)\s*\{", chunk)
+                for kind, function in found:
+                    yield function, kind == "global", chunk
+
+
+def test_every_kernel_that_takes_tensor_memory_does_so_before_it_lets_the_next_one_start():
+    """Whatever functions it goes through: a kernel that reaches the allocation does so once, by one warp, and the go-ahead for the next kernel is
+    given behind the allocation and nowhere else."""
+    functions = list(_functions())
+    reach = {f for f, _, body in functions if "tcgen05.alloc." in body}
+    assert reach == {"tmem_alloc"}
+    calls = lambda body, names: re.findall(r"\b(%s)\(" % "|".join(sorted(names)), body)
+    while True:
+        more = {f for f, _, body in functions if set(calls(body, reach)) - {f}} | reach
+        if more == reach:
+            break
+        reach = more
+    kernels = {f for f, kernel, _ in functions if kernel} & reach
+    assert kernels == {"tc_gemm_kernel", "conv_tc_kernel", "contract_halo_kernel", "conv_split_kernel", "contract_split_kernel", "gemm_split_kernel"}
+    helpers = reach - kernels
+    assert helpers == {"tmem_alloc", "tmem_alloc_then_trigger", "split_begin"}
+    bodies = {f: body.split(f + "(", 1)[1] for f, _, body in functions if f in reach}
+    order = bodies["tmem_alloc_then_trigger"]
+    assert 0 <= order.index("tmem_alloc(") < order.index("pdl_trigger(") and order.count("pdl_trigger(") == 1
+    assert "pdl_trigger(" not in bodies["tmem_alloc"]
+    for f in kernels | {"split_begin"}:
+        taken = calls(bodies[f], helpers - {"tmem_alloc"})
+        assert len(taken) == 1 and "tmem_alloc(" not in bodies[f] and "pdl_trigger(" not in bodies[f], f
+        if taken == ["tmem_alloc_then_trigger"]:
+            assert re.search(r"if \(warp == 1\) \{?\s*tmem_alloc_then_trigger\(", bodies[f]), f
 
 
 def _body(name, function):
