@@ -67,13 +67,13 @@ def layer_work(c, r):
 
 # DRAM bytes (read + write) of one launch of the dominant kernel, from the ncu capture summarised in
 # profiles/ (None where the kernel has changed since, or was never captured).
-NCU_TRAFFIC = {   # (config, r, phase): bytes; profiles/tc_gemm_kernel_config*.md, profiles/simt_kernels_config2_r64.md
+NCU_TRAFFIC = {   # (config, r, phase): bytes; profiles/tc_gemm_kernel_config*.md
     # (config 4's contraction has another kernel since its capture)
     (5, 64, "sketch"): 235.9e6, (5, 64, "backprobe"): 221.4e6, (5, 64, "contract"): 55.0e6,
     (5, 16, "contract"): 12.9e6, (5, 256, "contract"): 205.8e6,
     (4, 64, "sketch"): 339.6e6, (4, 64, "backprobe"): 277.1e6,
     (3, 32, "sketch"): 79.1e6, (3, 32, "backprobe"): 53.2e6, (3, 32, "contract"): 53.8e6,
-    (2, 64, "sketch"): 50.4e6, (2, 64, "backprobe"): 33.6e6, (2, 64, "contract"): 33.6e6,
+    # (config 2's three have other kernels too)
 }
 
 
@@ -490,9 +490,10 @@ def run_xconv(args):
         for n, ms in ph_ms.items():
             gbs = work[n]["bytes"] / (ms * 1e-3) / 1e9
             tfs = work[n]["flops"] / (ms * 1e-3) / 1e12
-            comp_peak = tensor_peak if eng[n] == "tcgen05_bf16" else fma_tflops
+            # float storage on the tensor cores: six bfloat16 products for one of floats
+            comp_peak = fma_tflops if eng[n] == "simt_f32" else tensor_peak / (6 if eng[n] == "tcgen05_f32" else 1)
             t_mem, t_comp = work[n]["bytes"] / (peaks["hbm_gbs"] * 1e9), work[n]["flops"] / (comp_peak * 1e12)
-            bound = "hbm" if t_mem >= t_comp else ("tensor" if eng[n] == "tcgen05_bf16" else "alu")
+            bound = "hbm" if t_mem >= t_comp else ("alu" if eng[n] == "simt_f32" else "tensor")
             out[n] = {"ms": ms, "engine": eng[n], "GBps": gbs, "TFLOPps": tfs, "bound": bound,
                       "peak": peaks["hbm_gbs"] if bound == "hbm" else comp_peak,
                       "roofline_ms": 1e3 * max(t_mem, t_comp),
