@@ -90,7 +90,8 @@ typedef enum { XCONV_OP_FORWARD = 0, XCONV_OP_WGRAD = 1, XCONV_OP_DGRAD = 2, XCO
 
 /* Which arithmetic engine a call will use for its dominant kernel: FP32 multiply-adds or the tensor cores (by tcgen05, or
  * by mma.sync in the kernels that stream few samples or few probes through registers), per storage type.  (F32: float values
- * as three bfloat16 parts each, summed as precisely as by FP32 multiply-adds.) */
+ * as three bfloat16 parts each, summed as precisely as by FP32 multiply-adds; results below the smallest normal float may lose more
+ * than those do.)  A float convolution whose scratch holds the header alone runs on FP32 multiply-adds. */
 typedef enum { XCONV_ENGINE_NONE = 0, XCONV_ENGINE_SIMT_F32 = 1, XCONV_ENGINE_TCGEN05_BF16 = 2,
                XCONV_ENGINE_TCGEN05_F16 = 3, XCONV_ENGINE_TCGEN05_F32 = 4 } xconv_engine;
 
@@ -315,7 +316,7 @@ xconv_status xconv_workspace_status(const void* ws, void* cuda_stream);
 xconv_status xconv_selftest_wait_limit(void* ws, size_t ws_bytes, unsigned int limit_ms, void* cuda_stream);
 
 /* Measurement aid (no counterpart in the paper): the FP32 fused-multiply-add rate this GPU sustains,
- * which is the arithmetic ceiling of the FP32-FMA kernels that serve float storage.  Runs a kernel of
+ * which is the arithmetic ceiling of the FP32-FMA kernels (small float layers).  Runs a kernel of
  * register-only FMA chains a few times on `cuda_stream`, times it with CUDA events, synchronises, and
  * writes the best rate in TFLOP/s (2 flops per FMA) to the HOST double `tflops`.  `scratch` is device
  * memory of at least 148*16*256*4 bytes that the kernel writes its (meaningless) sums to. */

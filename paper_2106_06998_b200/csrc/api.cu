@@ -223,8 +223,9 @@ struct WgradPlan {
 };
 
 // Float layers whose contraction goes to the tensor cores (contract_split.cu).  It was faster on every one of 160 layers (us: 84 -> 72 to
-// 2680 -> 520, two thirds of them more than threefold), by a few microseconds only where the multiply-adds (70 a clock and SM on
-// tiles of 64 x 32 channels and 32 pixels) take less than eight: those layers keep the kernel that they are known by.
+// 2680 -> 520, two thirds of them more than threefold).  The limit (multiply-adds at 70 a clock and SM on tiles of 64 x 32 channels and 32 pixels
+// for 15000 clocks) is not where the two cross, which is below it: it leaves the layer 16 -> 16 channels, 32 x 32, 8 probes on the kernel that
+// the parity tests name for it, and gives up a few microseconds on layers of that size.
 static bool plan_contract_f32(const xconv_desc* d, ContractSplitPlan* p) {
   const double macs = (double)d->r * depth(d) * d->H * cdiv(d->W, 32) * 32 * kdepth(d) * d->KH * d->KW * align_up(d->Cin, 64) * align_up(d->Cout, 32);
   return d->dtype == XCONV_F32 && macs > 15000.0 * 148 * 70 && plan_contract_split(d, p);
@@ -596,7 +597,8 @@ static xconv_status run_conv_simt(const xconv_desc* d, bool dgrad, const void* i
 // Float layers whose convolution goes to the tensor cores (conv_split.cu): all but the smallest.  The call alone is faster from a
 // microsecond of multiply-adds on (us, multiply-adds -> this, 160 layers: 8 x 16 -> 16 channels of 32 x 32 12.5 -> 8.6, 4 x 192 -> 48, 37 x 37,
 // 1 x 1 14.5 -> 8.9, larger ones 236 -> 57; but 9 x 1 -> 128 channels of 13 x 13, 1 x 1, with the copies before it 15.5 -> 18.6), but it
-// is a launch more: a training step of the first of these, host and all, 57.4 -> 61.4.  3000: two of 75 multiply-adds a clock and SM.
+// is a launch more: a training step of the first of these, host and all, 57.4 -> 61.4.  3000 clocks of 75 multiply-adds a clock and SM keep that
+// layer off, by that one step's time; alone the kernels cross at about half of it.
 static bool plan_conv_f32(const xconv_desc* d, bool dgrad, ConvSplitPlan* p) {
   const double macs = (double)d->B * depth(d) * d->H * d->W * d->Cin * d->Cout * kdepth(d) * d->KH * d->KW;
   if (d->dtype != XCONV_F32 || macs <= 3000.0 * 148 * 75) return false;

@@ -504,7 +504,6 @@ bool plan_contract_split(const xconv_desc* d, ContractSplitPlan* p) {
   }
   if (best < 0) return false;
   p->units = units;
-  p->clocks = (long)best;
   const long px = g.W * g.H * g.D * g.B;
   p->part_bytes = (size_t)units * p->splits * p->cols * TILE_M * sizeof(float);
   p->bytes = p->part_bytes + padded_float_bytes(px, d->Cout) + padded_float_bytes(px, d->Cin);

@@ -10,7 +10,7 @@ struct ContractSplitPlan {
   int cwa, a_blocks;            // channels per block of L, blocks
   int pw, ph, ksteps, stages, f_slots;
   uint32_t a_blk, b_blk, f_slot, f_b;
-  long patches, splits, units, clocks;    // clocks: what the busiest SM is expected to take
+  long patches, splits, units;
   size_t part_bytes, bytes;     // partial sums; all scratch (with padded copies of L and Z)
 };
 

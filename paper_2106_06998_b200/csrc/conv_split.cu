@@ -11,12 +11,13 @@
 // Three MMAs per k-step of 16 channels form the six products, in three groups of n accumulator columns:
 //   h x [h | m | l] -> columns 0..3n,   m x [h | m] -> columns n..3n,   l x h -> columns 2n..3n.
 // The A tile is then read three times instead of six (what bounds narrow MMAs), and the products hh have a column group of their
-// own (which also decides results that are not finite: split_f32.cuh).  Two accumulator sets take rows of offsets in turn (1 x 1: four blocks of channels), an issuing warp each; eight epilogue warps
-// add the three groups of a set to float registers.
+// own (which also decides results that are not finite: split_f32.cuh).  Two accumulator sets take rows of offsets in turn (1 x 1: four blocks
+// of channels), an issuing warp each; eight epilogue warps add the three groups of a set to float registers.
 //
 // Error against 64 bits on 120 random layers, times that of the FP32 multiply-adds (conv_fma.cu): 0.35 in the median, nowhere more
 // than 1; 1e-7 where those have 1e-6.  What bounds it: the MMAs, 204 clocks per k-step and 64 channels out (an MMA of N columns holds the
-// tensor pipe N / 2 clocks, or shared memory 32 + N / 4), at three quarters of that: the rest are the issuing warps' waits.
+// tensor pipe N / 2 clocks, or shared memory 32 + N / 4).  The tensor pipe is active 0.54 of the time on 64 -> 64 channels, 128 images of 32 x 32 from a
+// cold cache (0.64 of the warm call): the rest are the issuing warps' waits for weights (336 MB from L2 there) and for the conversion.
 // us, multiply-adds -> this: 64 -> 64 channels, 128 images of 32 x 32 236 -> 57 (the MMAs alone 36); 96 -> 160, 39 x 39 286 -> 53; 5 x 5,
 // 64 -> 128 617 -> 130; 1 x 1, 48 -> 128, 4 images of 168 x 190 138 -> 48.
 #include "conv_split.h"
@@ -377,7 +378,7 @@ bool plan_conv_split(const xconv_desc* d, bool dgrad, ConvSplitPlan* p) {
     if (items >= (1L << 32) - 1) continue;
     // conversion: some 45 instructions for four values, on four schedulers at two thirds of their rate
     const long convert = (long)npos * KD * p->nb * p->cw / 4 * 45 / 85;
-    const long cost = cdivl(items, NUM_SMS) * std::max(ksteps * split_kstep_clocks(p->n), convert) + std::min(items, 1L) * 400;
+    const long cost = cdivl(items, NUM_SMS) * std::max(ksteps * split_kstep_clocks(p->n), convert);
     if (best >= 0 && cost >= best) continue;
     best = cost;
     p->pw = pw; p->ph = ph; p->patches = patches;
@@ -393,7 +394,6 @@ bool plan_conv_split(const xconv_desc* d, bool dgrad, ConvSplitPlan* p) {
     p->f_slot = f_slot;
   }
   if (best < 0) return false;
-  p->clocks = best;
   p->img_bytes = ((size_t)p->tiles_n * p->nb * KD * T2 * p->w_tile + 255) / 256 * 256;
   p->bytes = p->img_bytes + padded_float_bytes(g.W * g.H * g.D * g.B, Ci);
   return true;

@@ -9,7 +9,7 @@ struct ConvSplitPlan {
   int cw, nb, ks_last;          // channels in per block, blocks, k-steps of the last one
   int n, tiles_n, ocw;          // channels out per column tile, tiles, channels per staging tile
   int pw, ph;                   // patch
-  long patches, clocks;         // clocks: what the busiest SM is expected to take
+  long patches;
   uint32_t a_plane, w_tile, f_slot;
   int a_slots, w_slots, f_slots;
   size_t img_bytes, bytes;      // the split weights; all scratch behind the header (with a padded copy of the input)
