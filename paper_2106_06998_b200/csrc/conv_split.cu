@@ -264,10 +264,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1) conv_split_kernel(const __grid_
         ok = split_wait(&t_full[buf], par, p.status, p.tag);
         if (!ok) break;
         tc_fence_after();
-        split_add_set<Bf16Parts>(tmem_q + buf * (uint32_t)(3 * p.n), (uint32_t)p.n, half, sum);
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&t_empty[buf]);
+        split_add_set<Bf16Parts>(tmem_q + buf * (uint32_t)(3 * p.n), (uint32_t)p.n, half, sum, &t_empty[buf]);
         par ^= buf;
         buf ^= 1u;
       }

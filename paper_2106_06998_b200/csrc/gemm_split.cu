@@ -305,10 +305,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         ok = split_wait(&acc_full[buf], par, p.status, p.tag);
         if (!ok) break;
         tc_fence_after();
-        split_add_set<typename GsElement<KIND>::parts, WHOLE>(tmem_q + buf * (uint32_t)(3 * p.n), (uint32_t)p.n, half, sum);
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&acc_empty[buf]);
+        split_add_set<typename GsElement<KIND>::parts, WHOLE>(tmem_q + buf * (uint32_t)(3 * p.n), (uint32_t)p.n, half, sum, &acc_empty[buf]);
         par ^= buf;
         buf ^= 1u;
       }

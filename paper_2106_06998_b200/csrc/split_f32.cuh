@@ -249,11 +249,21 @@ __device__ __forceinline__ uint32_t split_begin(int warp, uint32_t* slot, uint32
   return *reinterpret_cast<volatile uint32_t*>(slot);
 }
 // An accumulator set's three groups of n columns added to the sums of an epilogue warp's column groups (`half`, `half` + 2 of 16).  A sum
-// of products hh that is not finite counts alone.  AT_ONCE: all three groups are loaded together, where there are registers for it.
+// of products hh that is not finite counts alone.  AT_ONCE: all three groups are loaded together, where there are registers for it.  The set is
+// given back to the MMAs (`empty`) as soon as it is read: they do not wait for the look at its sums.
 template <class Parts, bool AT_ONCE = false>
-__device__ __forceinline__ void split_add_set(uint32_t set, uint32_t n, int half, float2 (&sum)[2][8]) {
+__device__ __forceinline__ void split_add_set(uint32_t set, uint32_t n, int half, float2 (&sum)[2][8], uint64_t* empty) {
   const float2 down = make_float2(1.f / Parts::STEP, 1.f / Parts::STEP), zero = make_float2(0.f, 0.f);
   const auto pair = [](const uint32_t (&v)[16], int e) { return make_float2(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1])); };
+  const auto give_back = [&] {
+    tc_fence_before();
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive(empty);
+  };
+  if ((uint32_t)half * 16 >= n) {                    // (a warp without columns)
+    give_back();
+    return;
+  }
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
     const uint32_t c = (uint32_t)(half + 2 * k) * 16;
@@ -268,6 +278,7 @@ __device__ __forceinline__ void split_add_set(uint32_t set, uint32_t n, int half
     for (int e = 0; e < 8; ++e) t[e] = __ffma2_rn(pair(z, e), down, pair(y, e));
     if (!AT_ONCE) tmem_ld16_issue(set + c, x);
     tmem_ld_wait(x);
+    if (k == 1 || c + 32 >= n) give_back();
     constexpr int CHECKS = AT_ONCE ? 4 : 2;          // (chains of multiply-adds: their latency counts)
     float2 check[CHECKS];                            // 0, or NaN
 #pragma unroll
