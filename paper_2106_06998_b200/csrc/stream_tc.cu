@@ -12,7 +12,7 @@
 //    fragments of 8 column tiles with one byte permutation each, and its accumulators are 16 neighbouring columns of the
 //    result (back-probe).
 // Probing vectors redrawn from a seed are drawn into the fragments: a fragment register is two sign bits of a Philox word
-// moved to bits 15 and 31, two instructions.
+// moved to bits 15 and 31, a multiplication and a logic instruction.
 #include "common.cuh"
 #include "tc_api.h"
 
@@ -20,14 +20,17 @@
 
 namespace xconv {
 
-template <bool F16>
+// (FREE: the compiler may move it among other instructions; the loads of the kernels with stored operands run ahead in program order.)
+template <bool F16, bool FREE = false>
 __device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  if (F16)
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-  else
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+#define XC_MMA(T) "mma.sync.aligned.m16n8k16.row.col.f32." T "." T ".f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};" \
+                : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1)
+  if (F16) {
+    if (FREE) asm(XC_MMA("f16")); else asm volatile(XC_MMA("f16"));
+  } else {
+    if (FREE) asm(XC_MMA("bf16")); else asm volatile(XC_MMA("bf16"));
+  }
+#undef XC_MMA
 }
 __device__ __forceinline__ uint4 ldg_stream(const void* p) {
   uint4 v;
@@ -49,6 +52,22 @@ __device__ __forceinline__ float from16(unsigned short v) {
 template <bool F16>
 __device__ __forceinline__ uint32_t pack16(float a, float b) { return (uint32_t)to16<F16>(a) | ((uint32_t)to16<F16>(b) << 16); }
 
+// Two signs at bits 15 and 31 of `bits`, as two values +-1: one instruction, with both constants in registers (as constants they are put
+// into two instructions).
+struct SignPair { uint32_t mask, ones; };
+template <bool F16>
+__device__ __forceinline__ SignPair sign_pair() {
+  SignPair s;
+  asm volatile("mov.b32 %0, %1;" : "=r"(s.mask) : "n"(0x80008000u));
+  asm volatile("mov.b32 %0, %1;" : "=r"(s.ones) : "n"(F16 ? 0x3C003C00u : 0x3F803F80u));
+  return s;
+}
+__device__ __forceinline__ uint32_t signed_ones(uint32_t bits, const SignPair& s) {
+  uint32_t v;
+  asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(v) : "r"(bits), "r"(s.mask), "r"(s.ones));       // (bits & mask) | ones
+  return v;
+}
+
 // Two packed values with infinities and NaN replaced by zeros.
 template <bool F16>
 __device__ __forceinline__ uint32_t finite16(uint32_t v) {
@@ -60,12 +79,34 @@ __device__ __forceinline__ uint32_t finite16(uint32_t v) {
   return v & __hlt2_mask(__habs2(h), __nv_bfloat162(__ushort_as_bfloat16(0x7F80), __ushort_as_bfloat16(0x7F80)));
 }
 
+// What the kernels that draw signs take from constant memory: the keys of the ten rounds (added up per block they are a fifth of Philox's
+// instructions), and powers of two.  Signs are moved into place by multiplications with these: what bounds the drawing is the pipe of
+// shifts and logic (60 % busy, two instructions a register), and a multiplication goes to another.  (A constant factor the compiler would
+// make a shift again.)
+struct SignKeys {
+  uint32_t key[10][2], pow2[16];
+  void set(unsigned long long seed) {
+    uint32_t k0 = (uint32_t)(seed & 0xFFFFFFFFull), k1 = (uint32_t)(seed >> 32);
+    for (auto& k : key) { k[0] = k0; k[1] = k1; k0 += 0x9E3779B9u; k1 += 0xBB67AE85u; }
+    for (int i = 0; i < 16; ++i) pow2[i] = 1u << i;
+  }
+};
+// Philox block b (philox4x32_10 in common.cuh).
+__device__ __forceinline__ uint4 sign_block(unsigned long long b, const SignKeys& s) {
+  uint32_t c0 = (uint32_t)b, c1 = (uint32_t)(b >> 32), c2 = 0u, c3 = 0u;
+#pragma unroll
+  for (int i = 0; i < 10; ++i) {
+    const unsigned long long m0 = (unsigned long long)0xD2511F53u * c0, m1 = (unsigned long long)0xCD9E8D57u * c2;
+    c0 = (uint32_t)(m1 >> 32) ^ c1 ^ s.key[i][0]; c1 = (uint32_t)m1;
+    c2 = (uint32_t)(m0 >> 32) ^ c3 ^ s.key[i][1]; c3 = (uint32_t)m0;
+  }
+  return make_uint4(c0, c1, c2, c3);
+}
 // The 128 sign bits of entries e0 .. e0+127 of Z (e0 a multiple of 64, `whole`: of 128).
-__device__ __forceinline__ uint4 sign_bits128(unsigned long long e0, bool whole, uint32_t k0, uint32_t k1) {
-  const unsigned long long b = e0 >> 7;
-  uint4 w = philox4x32_10((uint32_t)b, (uint32_t)(b >> 32), k0, k1);
+__device__ __forceinline__ uint4 sign_bits128(unsigned long long e0, bool whole, const SignKeys& s) {
+  uint4 w = sign_block(e0 >> 7, s);
   if (!whole && (e0 & 64)) {                          // the second half of this block, the first of the next
-    const uint4 v = philox4x32_10((uint32_t)(b + 1), (uint32_t)((b + 1) >> 32), k0, k1);
+    const uint4 v = sign_block((e0 >> 7) + 1, s);
     w = make_uint4(w.z, w.w, v.x, v.y);
   }
   return w;
@@ -81,7 +122,7 @@ struct SketchStream {
   float* part;
   int M, N, swap;
   long K;
-  uint32_t seed_lo, seed_hi;
+  SignKeys signs;
   unsigned int *status, tag;                          // workspace header: this call is the last to use it
 };
 
@@ -138,10 +179,23 @@ __global__ void __launch_bounds__(256, 2) sketch_stream_kernel(const SketchStrea
   } else {
     // A = the signs of the seed.  128 k at a time: each lane draws one row's 128 signs (MT / 2 of them), the rows' words go
     // through shared memory.  In a step of 32 k (one word) the pairs are (s, s + 16), s = 4t .. 4t+3.
-    const uint32_t ones = F16 ? 0x3C003C00u : 0x3F803F80u;
+    // What bounds it: a product holds a scheduler for some 8 clocks, and the instructions beside it, 8 a product, take theirs one after
+    // the other (17 of 19 clocks a product; no pipe above 43 %).  256 probes x 16 samples, 2.1 M terms 91 -> 80 us against two logic
+    // instructions and an addition of keys more.
+    const SignPair pm = sign_pair<F16>();
+    const uint32_t place = p.signs.pow2[12 - 4 * t];
     const bool whole = (p.K & 127) == 0;
     const uint16_t* brow = p.Bm + (long)g * p.K + 4 * t;
-    for (long k0 = (long)blockIdx.x * 1024 + warp * 128; k0 < p.K; k0 += (long)gridDim.x * 1024) {
+    constexpr int DR = (16 * MT + 31) / 32;            // rows a lane draws
+    uint4 drawn[DR];
+    auto draw = [&](long k) {
+#pragma unroll
+      for (int i = 0; i < DR; ++i)
+        drawn[i] = sign_bits128((unsigned long long)(m0 + 32 * i + lane) * (unsigned long long)p.K + (unsigned long long)k, whole, p.signs);
+    };
+    long k0 = (long)blockIdx.x * 1024 + warp * 128;
+    if (k0 < p.K) draw(k0);
+    for (; k0 < p.K; k0 += (long)gridDim.x * 1024) {
       uint2 x[4][NT][2];
 #pragma unroll
       for (int w = 0; w < 4; ++w)
@@ -153,16 +207,13 @@ __global__ void __launch_bounds__(256, 2) sketch_stream_kernel(const SketchStrea
                              ? *reinterpret_cast<const uint2*>(brow + (long)(8 * j) * p.K + k0 + 32 * w + 16 * h) : make_uint2(0u, 0u);
       __syncwarp();
 #pragma unroll
-      for (int i = 0; i < (16 * MT + 31) / 32; ++i) {
-        const int row = 32 * i + lane;
-        if (row < 16 * MT)
-          bits[warp][row] = sign_bits128((unsigned long long)(m0 + row) * (unsigned long long)p.K + (unsigned long long)k0, whole,
-                                         p.seed_lo, p.seed_hi);
-      }
+      for (int i = 0; i < DR; ++i)
+        if (32 * i + lane < 16 * MT) bits[warp][32 * i + lane] = drawn[i];
       __syncwarp();
+      if (k0 + (long)gridDim.x * 1024 < p.K) draw(k0 + (long)gridDim.x * 1024);      // the next piece's signs, between this one's products
 #pragma unroll
       for (int w = 0; w < 4; ++w) {
-        uint32_t b[NT][4];
+        uint32_t b[NT][4], w0[MT], w1[MT];
 #pragma unroll
         for (int j = 0; j < NT; ++j) {
           const uint2 lo = x[w][j][0], hi = x[w][j][1];
@@ -171,18 +222,19 @@ __global__ void __launch_bounds__(256, 2) sketch_stream_kernel(const SketchStrea
         }
 #pragma unroll
         for (int i = 0; i < MT; ++i) {
-          const uint32_t w0 = reinterpret_cast<const uint32_t*>(&bits[warp][16 * i + g])[w] << (12 - 4 * t);
-          const uint32_t w1 = reinterpret_cast<const uint32_t*>(&bits[warp][16 * i + 8 + g])[w] << (12 - 4 * t);
-          const uint32_t f0[4] = {((w0 << 3) & 0x80008000u) ^ ones, ((w1 << 3) & 0x80008000u) ^ ones,
-                                  ((w0 << 2) & 0x80008000u) ^ ones, ((w1 << 2) & 0x80008000u) ^ ones};
-          const uint32_t f1[4] = {((w0 << 1) & 0x80008000u) ^ ones, ((w1 << 1) & 0x80008000u) ^ ones,
-                                  (w0 & 0x80008000u) ^ ones, (w1 & 0x80008000u) ^ ones};
-#pragma unroll
-          for (int j = 0; j < NT; ++j) {
-            mma16816<F16>(acc[i][j], f0, b[j][0], b[j][1]);
-            mma16816<F16>(acc[i][j], f1, b[j][2], b[j][3]);
-          }
+          w0[i] = reinterpret_cast<const uint32_t*>(&bits[warp][16 * i + g])[w] * place;
+          w1[i] = reinterpret_cast<const uint32_t*>(&bits[warp][16 * i + 8 + g])[w] * place;
         }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)                    // all row tiles of one half, so that no product waits for the one before it
+#pragma unroll
+          for (int i = 0; i < MT; ++i) {
+            const uint32_t c0 = p.signs.pow2[3 - 2 * h], c1 = h ? 1u : p.signs.pow2[2];
+            const uint32_t f[4] = {signed_ones(w0[i] * c0, pm), signed_ones(w1[i] * c0, pm), signed_ones(w0[i] * c1, pm),
+                                   signed_ones(w1[i] * c1, pm)};
+#pragma unroll
+            for (int j = 0; j < NT; ++j) mma16816<F16, true>(acc[i][j], f, b[j][2 * h], b[j][2 * h + 1]);
+          }
       }
     }
   }
@@ -210,7 +262,7 @@ __global__ void __launch_bounds__(256, 2) sketch_stream_kernel(const SketchStrea
 
 // L[row][q] = sum over k of S(row, k) * Y[k][q], rounded to storage: up to 16 MT rows, a warp owns 64 columns.  S(row, k) =
 // S[row * s_row + k * s_k] (float, rounded to storage in shared memory, so that neither a transposed nor a 16-bit copy of it
-// is written).  SEEDED: Y = the signs of the seed.
+// is written).
 struct BackprobeStream {
   const float* S;
   long s_row, s_k;
@@ -218,27 +270,12 @@ struct BackprobeStream {
   uint16_t* L;
   int rows, K, K16, ld;                               // K16: K rounded up to 64; ld: row pitch of S in shared memory
   long Q, groups;                                     // groups of 64 columns
-  uint32_t seed_lo, seed_hi;
   unsigned int *status, tag;
 };
 
-// SPLIT: S as the sum of two 16-bit values, multiplied one after the other: for the layers whose sums used the float S (24 bits)
-// before.  The two keep 16 bits of it in bfloat16 and 22 in float16 (where every row is scaled by a power of two into the range
-// first), far below the rounding of the result: relative error against 64 bits on 76 random layers 1.6e-3 to 1.7e-3 (bfloat16)
-// and 2.1e-4 (float16), 1.00001 times that of the float S at most; 2.4e-3 with S rounded once.
-// Y's infinities and NaN count once, with the first value: the second is zero or of either sign, and its product with an
-// infinity would make a NaN of the sum.  So an entry of S that is not zero has a first value that is not zero either.
-// KC: k-steps of 16 that are loaded together.  ALL: they are the whole reduction; a warp then takes 4 / KC groups of
-// columns at a time, so that as many bytes are in flight as with a long reduction.  Otherwise the loads of the next
-// KC k-steps (of the next group behind the last) are under way while these are multiplied.
-template <bool F16, int MT, bool SEEDED, int KC, bool ALL, bool SPLIT>
-__global__ void __launch_bounds__(256, MT >= 4 ? 1 : 2) backprobe_stream_kernel(const BackprobeStream p) {
-  extern __shared__ __align__(16) uint16_t s16[];     // [16 MT][ld], then (SEEDED) 8 warps x 32 rows x 8 bytes of signs
-  pdl_trigger();
-  pdl_wait();
-  if (threadIdx.x == 0 && blockIdx.x == 0) p.status[1] = p.tag;
-  __shared__ float unscale[SPLIT ? 16 * MT : 1];      // SPLIT: what the row's sums are multiplied by
-  uint16_t* s16lo = s16 + 16 * MT * p.ld;             // SPLIT: the second values
+// S in shared memory, rounded to storage (SPLIT: as two values, the second ones at s16lo, and what the sums of a row are multiplied by in `unscale`).
+template <bool F16, int MT, bool SPLIT>
+__device__ __forceinline__ void stage_sketch(const BackprobeStream& p, uint16_t* s16, uint16_t* s16lo, float* unscale) {
   if (SPLIT) {
     // a warp's rows side by side, so that their loads are in flight together (one row after the other, a wait for memory
     // each: 64 rows of 5 terms 11.8 us a launch in float16)
@@ -289,9 +326,27 @@ __global__ void __launch_bounds__(256, MT >= 4 ? 1 : 2) backprobe_stream_kernel(
     }
   }
   __syncthreads();
+}
+
+// SPLIT: S as the sum of two 16-bit values, multiplied one after the other: for the layers whose sums used the float S (24 bits)
+// before.  The two keep 16 bits of it in bfloat16 and 22 in float16 (where every row is scaled by a power of two into the range
+// first), far below the rounding of the result: relative error against 64 bits on 76 random layers 1.6e-3 to 1.7e-3 (bfloat16)
+// and 2.1e-4 (float16), 1.00001 times that of the float S at most; 2.4e-3 with S rounded once.
+// Y's infinities and NaN count once, with the first value: the second is zero or of either sign, and its product with an
+// infinity would make a NaN of the sum.  So an entry of S that is not zero has a first value that is not zero either.
+// KC: k-steps of 16 that are loaded together.  ALL: they are the whole reduction; a warp then takes 4 / KC groups of
+// columns at a time, so that as many bytes are in flight as with a long reduction.  Otherwise the loads of the next
+// KC k-steps (of the next group behind the last) are under way while these are multiplied.
+template <bool F16, int MT, int KC, bool ALL, bool SPLIT>
+__global__ void __launch_bounds__(256, MT >= 4 ? 1 : 2) backprobe_stream_kernel(const BackprobeStream p) {
+  extern __shared__ __align__(16) uint16_t s16[];     // [16 MT][ld]
+  pdl_trigger();
+  pdl_wait();
+  if (threadIdx.x == 0 && blockIdx.x == 0) p.status[1] = p.tag;
+  __shared__ float unscale[SPLIT ? 16 * MT : 1];      // SPLIT: what the row's sums are multiplied by
+  uint16_t* s16lo = s16 + 16 * MT * p.ld;             // SPLIT: the second values
+  stage_sketch<F16, MT, SPLIT>(p, s16, s16lo, unscale);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const uint32_t ones = F16 ? 0x3C003C00u : 0x3F803F80u;
-  uint2* bits = reinterpret_cast<uint2*>(s16 + (SPLIT ? 2 : 1) * 16 * MT * p.ld) + warp * 32;
   constexpr int GB = ALL ? 4 / KC : 1, VB = ALL ? GB : 2;
   const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
   float acc[MT][8][4];
@@ -306,14 +361,6 @@ __global__ void __launch_bounds__(256, MT >= 4 ? 1 : 2) backprobe_stream_kernel(
         v[gb][u][r] = k < p.K && q < p.Q ? ldg_stream(p.Y + (long)k * p.Q + q) : zero;
       }
   };
-  auto draw = [&](long grp, int k0) {                 // the signs of 32 rows, one row's 64 bits per lane (half a Philox block)
-    __syncwarp();
-    const unsigned long long e0 = (unsigned long long)(k0 + lane) * (unsigned long long)p.Q + (unsigned long long)(grp * 64);
-    const unsigned long long blk = e0 >> 7;
-    const uint4 w = philox4x32_10((uint32_t)blk, (uint32_t)(blk >> 32), p.seed_lo, p.seed_hi);
-    bits[lane] = (e0 & 64) ? make_uint2(w.z, w.w) : make_uint2(w.x, w.y);
-    __syncwarp();
-  };
   auto multiply = [&](int gb, int k0) {
 #pragma unroll
     for (int u = 0; u < KC; ++u) {
@@ -326,35 +373,23 @@ __global__ void __launch_bounds__(256, MT >= 4 ? 1 : 2) backprobe_stream_kernel(
         a[i][2] = *reinterpret_cast<const uint32_t*>(s + 8);
         a[i][3] = *reinterpret_cast<const uint32_t*>(s + 8 * p.ld + 8);
       }
-      uint32_t x0 = 0, x1 = 0;                        // SEEDED: eight signs of the two rows of a pair, at bits 0 and 16
-      if (SEEDED) {
-        const uint8_t* sb = reinterpret_cast<const uint8_t*>(bits) + (16 * u + 2 * t) * 8 + g;
-        x0 = (uint32_t)sb[0] | ((uint32_t)sb[8] << 16);
-        x1 = (uint32_t)sb[64] | ((uint32_t)sb[72] << 16);
-      }
 #pragma unroll
       for (int c = 0; c < 8; ++c) {                   // column 8 g + c is column g of tile c
-        uint32_t b0, b1;
-        if (SEEDED) {
-          b0 = ((x0 << (15 - c)) & 0x80008000u) ^ ones;
-          b1 = ((x1 << (15 - c)) & 0x80008000u) ^ ones;
-        } else {
-          b0 = __byte_perm(word(v[gb][u][0], c >> 1), word(v[gb][u][1], c >> 1), (c & 1) ? 0x7632 : 0x5410);
-          b1 = __byte_perm(word(v[gb][u][2], c >> 1), word(v[gb][u][3], c >> 1), (c & 1) ? 0x7632 : 0x5410);
-        }
+        uint32_t b0 = __byte_perm(word(v[gb][u][0], c >> 1), word(v[gb][u][1], c >> 1), (c & 1) ? 0x7632 : 0x5410);
+        uint32_t b1 = __byte_perm(word(v[gb][u][2], c >> 1), word(v[gb][u][3], c >> 1), (c & 1) ? 0x7632 : 0x5410);
 #pragma unroll
         for (int i = 0; i < MT; ++i) mma16816<F16>(acc[i][c], a[i], b0, b1);
         if (SPLIT) {
-          if (!SEEDED) { b0 = finite16<F16>(b0); b1 = finite16<F16>(b1); }
+          b0 = finite16<F16>(b0); b1 = finite16<F16>(b1);
 #pragma unroll
           for (int i = 0; i < MT; ++i) mma16816<F16>(acc[i][c], a[MT + i], b0, b1);
         }
       }
     }
   };
-  if (!ALL && !SEEDED) fetch(0, (long)blockIdx.x * 8 + warp, 0);
+  if (!ALL) fetch(0, (long)blockIdx.x * 8 + warp, 0);
   for (long grp0 = ((long)blockIdx.x * 8 + warp) * GB; grp0 < p.groups; grp0 += (long)gridDim.x * 8 * GB) {
-    if (ALL && !SEEDED)
+    if (ALL)
 #pragma unroll
       for (int gb = 0; gb < GB; ++gb) fetch(gb, grp0 + gb, 0);
 #pragma unroll
@@ -371,12 +406,10 @@ __global__ void __launch_bounds__(256, MT >= 4 ? 1 : 2) backprobe_stream_kernel(
         multiply(gb, 0);
       } else {
         for (int k0 = 0; k0 < p.K16; k0 += 32 * KC) {       // (K16 is a multiple of 64)
-          if (SEEDED) draw(grp, k0);
-          else fetch(1, grp, k0 + 16 * KC);
+          fetch(1, grp, k0 + 16 * KC);
           multiply(0, k0);
           const bool last = k0 + 32 * KC >= p.K16;
-          if (SEEDED) draw(grp, k0 + 16 * KC);
-          else fetch(0, last ? grp + (long)gridDim.x * 8 : grp, last ? 0 : k0 + 32 * KC);
+          fetch(0, last ? grp + (long)gridDim.x * 8 : grp, last ? 0 : k0 + 32 * KC);
           // (padding of the reduction: zeros; left out by halves, a test per k-step keeps the loads from running ahead)
           if (!SPLIT || k0 + 16 * KC < p.K) multiply(1, k0 + 16 * KC);
         }
@@ -404,6 +437,107 @@ __global__ void __launch_bounds__(256, MT >= 4 ? 1 : 2) backprobe_stream_kernel(
           }
         }
     }
+  }
+}
+
+// The same with Y = the signs of the seed.  Bounded as the sketch that draws them (above); 16 rows, 256 terms, 2.1 M columns 96 -> 76 us, 16 rows,
+// 8 terms, 3.5 M columns 45 -> 24.
+template <bool F16, int MT, int GP, bool SPLIT>
+__global__ void __launch_bounds__(256, MT >= 4 ? 1 : 2) backprobe_seeded_kernel(const BackprobeStream p, const __grid_constant__ SignKeys signs) {
+  extern __shared__ __align__(16) uint16_t s16[];     // [16 MT][ld], then 8 warps x 32 rows x 16 bytes of signs
+  pdl_trigger();
+  pdl_wait();
+  if (threadIdx.x == 0 && blockIdx.x == 0) p.status[1] = p.tag;
+  __shared__ float unscale[SPLIT ? 16 * MT : 1];
+  stage_sketch<F16, MT, SPLIT>(p, s16, s16 + 16 * MT * p.ld, unscale);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  // S of k-step k: the first values in a[0 .. MT-1], the second ones behind
+  auto load_s = [&](uint32_t (&a)[SPLIT ? 2 * MT : MT][4], int k) {
+#pragma unroll
+    for (int i = 0; i < (SPLIT ? 2 * MT : MT); ++i) {
+      const uint16_t* s = s16 + (16 * i + g) * p.ld + k + 2 * t;
+      a[i][0] = *reinterpret_cast<const uint32_t*>(s);
+      a[i][1] = *reinterpret_cast<const uint32_t*>(s + 8 * p.ld);
+      a[i][2] = *reinterpret_cast<const uint32_t*>(s + 8);
+      a[i][3] = *reinterpret_cast<const uint32_t*>(s + 8 * p.ld + 8);
+    }
+  };
+  // accumulator columns 2t and 2t+1 of tile c are the columns 16 t + c and 16 t + 8 + c
+  auto store = [&](float (&acc)[MT][8][4], long grp) {
+    const long qo = grp * 64 + 16 * t;
+#pragma unroll
+    for (int i = 0; i < MT; ++i)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int row = 16 * i + 8 * h + g;
+        if (row >= p.rows) continue;
+        if (SPLIT && F16) {
+          const float d = unscale[row];
+#pragma unroll
+          for (int c = 0; c < 8; ++c) { acc[i][c][2 * h] *= d; acc[i][c][2 * h + 1] *= d; }
+        }
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+          if (qo + 8 * s >= p.Q) continue;
+          uint4 o;
+          o.x = pack16<F16>(acc[i][0][2 * h + s], acc[i][1][2 * h + s]); o.y = pack16<F16>(acc[i][2][2 * h + s], acc[i][3][2 * h + s]);
+          o.z = pack16<F16>(acc[i][4][2 * h + s], acc[i][5][2 * h + s]); o.w = pack16<F16>(acc[i][6][2 * h + s], acc[i][7][2 * h + s]);
+          *reinterpret_cast<uint4*>(p.L + (long)row * p.Q + qo + 8 * s) = o;
+        }
+      }
+  };
+  // A warp takes GP groups side by side, a whole Philox block of every row where GP is 2.  The signs of 32 rows, a row per lane, go
+  // through shared memory, and the next 32 are drawn between the products of these.
+  const SignPair pm = sign_pair<F16>();
+  uint4* bits = reinterpret_cast<uint4*>(s16 + (SPLIT ? 2 : 1) * 16 * MT * p.ld) + warp * 32;
+  const bool whole = GP == 2 && (p.Q & 127) == 0;
+  for (long grp0 = ((long)blockIdx.x * 8 + warp) * GP; grp0 < p.groups; grp0 += (long)gridDim.x * 8 * GP) {
+    float acc[GP][MT][8][4];
+#pragma unroll
+    for (int gp = 0; gp < GP; ++gp)
+#pragma unroll
+      for (int i = 0; i < MT; ++i)
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) acc[gp][i][c][e] = 0.f;
+    uint4 drawn;
+    auto draw = [&](int k0) {
+      const unsigned long long e0 = (unsigned long long)(k0 + lane) * (unsigned long long)p.Q + (unsigned long long)(grp0 * 64);
+      if (GP == 2) {
+        drawn = sign_bits128(e0, whole, signs);
+      } else {
+        const uint4 w = sign_block(e0 >> 7, signs);
+        drawn = (e0 & 64) ? make_uint4(w.z, w.w, 0u, 0u) : make_uint4(w.x, w.y, 0u, 0u);
+      }
+    };
+    draw(0);
+    for (int k0 = 0; k0 < p.K; k0 += 32) {                // (S is padded with zeros to a multiple of 64 terms)
+      __syncwarp();
+      bits[lane] = drawn;
+      __syncwarp();
+      if (k0 + 32 < p.K) draw(k0 + 32);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        uint32_t a[SPLIT ? 2 * MT : MT][4];
+        load_s(a, k0 + 16 * u);
+#pragma unroll
+        for (int gp = 0; gp < GP; ++gp) {
+          // eight signs of the two rows of a pair, at bits 0 and 16
+          const uint8_t* sb = reinterpret_cast<const uint8_t*>(bits) + (16 * u + 2 * t) * 16 + 8 * gp + g;
+          const uint32_t x0 = (uint32_t)sb[0] | ((uint32_t)sb[16] << 16), x1 = (uint32_t)sb[128] | ((uint32_t)sb[144] << 16);
+#pragma unroll
+          for (int c = 0; c < 8; ++c) {                   // column 8 g + c is column g of tile c
+            const uint32_t place = signs.pow2[15 - c], b0 = signed_ones(x0 * place, pm), b1 = signed_ones(x1 * place, pm);
+#pragma unroll
+            for (int i = 0; i < (SPLIT ? 2 * MT : MT); ++i) mma16816<F16, true>(acc[gp][i % MT][c], a[i], b0, b1);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int gp = 0; gp < GP; ++gp)
+      if (grp0 + gp < p.groups) store(acc[gp], grp0 + gp);
   }
 }
 
@@ -471,7 +605,7 @@ xconv_status tc_run_sketch_stream(const xconv_desc* d, const StreamSketchPlan& p
   q.N = pl.swap ? d->r : d->B;
   q.swap = pl.swap;
   q.K = (long)d->H * d->W * d->Cin;
-  if (seed) { q.seed_lo = (uint32_t)(*seed & 0xFFFFFFFFull); q.seed_hi = (uint32_t)(*seed >> 32); }
+  if (seed) q.signs.set(*seed);
   const cudaError_t e = d->dtype == XCONV_F16 ? launch_sketch_stream<true>(pl, seed != nullptr, q, st)
                                               : launch_sketch_stream<false>(pl, seed != nullptr, q, st);
   count_launch();
@@ -481,7 +615,7 @@ xconv_status tc_run_sketch_stream(const xconv_desc* d, const StreamSketchPlan& p
 
 static int stream_k(int K) { return (int)(cdiv_(K, 64) * 64); }
 static size_t stream_smem(int mt, int K, bool seeded, bool split) {
-  return (size_t)(16 * mt) * (stream_k(K) + 8) * (split ? 4 : 2) + (seeded ? 8 * 32 * 8 : 0);
+  return (size_t)(16 * mt) * (stream_k(K) + 8) * (split ? 4 : 2) + (seeded ? 8 * 32 * 16 : 0);
 }
 
 // `other`: the tcgen05 back-probe serves the layer.  Up to 16 rows this one is faster where every warp has two groups of columns
@@ -492,21 +626,36 @@ static size_t stream_smem(int mt, int K, bool seeded, bool split) {
 bool tc_backprobe_streams(const xconv_desc* d, bool other) {
   if (d->dtype != XCONV_BF16 && d->dtype != XCONV_F16) return false;
   const long Q = (long)d->H * d->W * d->Cout;
-  if (Q % 8 != 0 || Q < 2048 || d->r > 64 || stream_smem(d->r > 32 ? 4 : d->r > 16 ? 2 : 1, d->B, true, !other) > 96 * 1024) return false;
+  if (Q % 8 != 0 || Q < 2048 || d->r > 64 || stream_smem(d->r > 32 ? 4 : d->r > 16 ? 2 : 1, d->B, true, !other) > 98 * 1024) return false;
   return !other || (d->r <= 16 && (d->B <= 64 || Q >= 2L * 64 * 16 * 148));
 }
 
 template <bool F16, int MT>
-static cudaError_t launch_backprobe_stream(const BackprobeStream& q, bool seeded, bool split, unsigned grid, size_t smem, cudaStream_t st) {
+static cudaError_t launch_backprobe_seeded(const BackprobeStream& q, const SignKeys& signs, bool split, unsigned grid, size_t smem, cudaStream_t st) {
+  // Pairs of groups draw half the blocks, but only where every warp of the grid has a group of its own all the same (16 rows: 256 terms, 2.1 M
+  // columns 91 -> 77 us, 498 terms, 4608 columns 28 -> 34).
+  constexpr int PAIR = MT == 1 ? 2 : 1;
+  const bool pairs = q.groups > 8L * 148 * 2;
+  void (*kernel)(BackprobeStream, SignKeys);
+  if (split) kernel = pairs ? backprobe_seeded_kernel<F16, MT, PAIR, true> : backprobe_seeded_kernel<F16, MT, 1, true>;
+  else if (MT > 1) return cudaErrorInvalidValue;
+  else kernel = pairs ? backprobe_seeded_kernel<F16, 1, 2, false> : backprobe_seeded_kernel<F16, 1, 1, false>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+  if (e == cudaSuccess) e = want_l1(reinterpret_cast<const void*>(kernel), smem);
+  return e != cudaSuccess ? e : launch_pdl(kernel, dim3(grid), dim3(256), smem, st, q, signs);
+}
+
+template <bool F16, int MT>
+static cudaError_t launch_backprobe_stream(const BackprobeStream& q, const SignKeys* signs, bool split, unsigned grid, size_t smem, cudaStream_t st) {
+  if (signs) return launch_backprobe_seeded<F16, MT>(q, *signs, split, grid, smem, st);
   constexpr int KC = MT == 1 ? 2 : 1;
   void (*kernel)(BackprobeStream);
-  if (split) kernel = seeded ? backprobe_stream_kernel<F16, MT, true, 2, false, true> : backprobe_stream_kernel<F16, MT, false, KC, false, true>;
+  if (split) kernel = backprobe_stream_kernel<F16, MT, KC, false, true>;
   else if (MT > 1) return cudaErrorInvalidValue;      // (one value per entry of S: up to 16 rows only)
   else
-    kernel = seeded ? backprobe_stream_kernel<F16, 1, true, 2, false, false>
-             : q.K <= 16 ? backprobe_stream_kernel<F16, 1, false, 1, true, false>
-             : q.K <= 32 ? backprobe_stream_kernel<F16, 1, false, 2, true, false>
-             : q.K <= 64 ? backprobe_stream_kernel<F16, 1, false, 4, true, false> : backprobe_stream_kernel<F16, 1, false, 2, false, false>;
+    kernel = q.K <= 16 ? backprobe_stream_kernel<F16, 1, 1, true, false>
+             : q.K <= 32 ? backprobe_stream_kernel<F16, 1, 2, true, false>
+             : q.K <= 64 ? backprobe_stream_kernel<F16, 1, 4, true, false> : backprobe_stream_kernel<F16, 1, 2, false, false>;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
   if (e == cudaSuccess) e = want_l1(reinterpret_cast<const void*>(kernel), smem);
   return e != cudaSuccess ? e : launch_pdl(kernel, dim3(grid), dim3(256), smem, st, q);
@@ -523,19 +672,21 @@ xconv_status tc_run_backprobe_stream(const xconv_desc* d, const float* S, long s
   q.rows = d->r; q.K = d->B; q.K16 = stream_k(d->B); q.ld = q.K16 + 8;
   q.Q = (long)d->H * d->W * d->Cout;
   q.groups = cdiv_(q.Q, 64);
-  if (seed) { q.seed_lo = (uint32_t)(*seed & 0xFFFFFFFFull); q.seed_hi = (uint32_t)(*seed >> 32); }
+  SignKeys keys;
+  if (seed) keys.set(*seed);
+  const SignKeys* signs = seed ? &keys : nullptr;
   const int mt = d->r > 32 ? 4 : d->r > 16 ? 2 : 1;
   const unsigned grid = (unsigned)std::min<long>(cdiv_(q.groups, 8), 148L * (mt == 4 ? 1 : 2));
   const size_t smem = stream_smem(mt, d->B, seed != nullptr, split);
   cudaError_t e;
   if (d->dtype == XCONV_F16)
-    e = mt == 4 ? launch_backprobe_stream<true, 4>(q, seed != nullptr, split, grid, smem, st)
-        : mt == 2 ? launch_backprobe_stream<true, 2>(q, seed != nullptr, split, grid, smem, st)
-                  : launch_backprobe_stream<true, 1>(q, seed != nullptr, split, grid, smem, st);
+    e = mt == 4 ? launch_backprobe_stream<true, 4>(q, signs, split, grid, smem, st)
+        : mt == 2 ? launch_backprobe_stream<true, 2>(q, signs, split, grid, smem, st)
+                  : launch_backprobe_stream<true, 1>(q, signs, split, grid, smem, st);
   else
-    e = mt == 4 ? launch_backprobe_stream<false, 4>(q, seed != nullptr, split, grid, smem, st)
-        : mt == 2 ? launch_backprobe_stream<false, 2>(q, seed != nullptr, split, grid, smem, st)
-                  : launch_backprobe_stream<false, 1>(q, seed != nullptr, split, grid, smem, st);
+    e = mt == 4 ? launch_backprobe_stream<false, 4>(q, signs, split, grid, smem, st)
+        : mt == 2 ? launch_backprobe_stream<false, 2>(q, signs, split, grid, smem, st)
+                  : launch_backprobe_stream<false, 1>(q, signs, split, grid, smem, st);
   count_launch();
   if (e != cudaSuccess) { set_cuda_error((int)e); return XCONV_ERR_CUDA; }
   return XCONV_OK;
