@@ -30,11 +30,12 @@
 #include "tc_api.h"
 #include "tc_ptx.cuh"
 #include "conv_walk.cuh"
+#include "conv_slide.cuh"
 
 namespace xconv {
 
 constexpr int CV_THREADS = 384;            // launch bound; a launch has 128 + 128 * groups threads
-constexpr int CV_A_SLOTS = 4, CV_W_SLOTS = 8;
+constexpr int CV_A_SLOTS = 8, CV_W_SLOTS = 8, CV_RING = 32;
 
 struct ConvParams {
   int KD, T, pad, pad_d, dgrad;
@@ -51,18 +52,12 @@ struct ConvParams {
   uint32_t w_off, o_off, o_bytes;                 // shared memory behind the input ring: weights, staging tiles
   uint32_t a_hi, b_hi, b_lo0, b_step, idesc;      // descriptor words
   int ocw, co;                                    // channels per staging tile, channels of the output
+  // walking along an axis (conv_slide.cuh): its extent, padding and kernel offsets; rows of offsets in the plane; images per tile; accumulators
+  int extent, pad_s, ks, ki, planar, img_step, ring;
+  uint32_t w_blk_bytes;                           // weights of one of the ks offsets that an MMA takes together
   unsigned int* status;
   unsigned int tag;
 };
-
-// The 128 threads of one group of epilogue warps: true if `ok` holds in every one of them.
-__device__ __forceinline__ bool epi_all(int group, bool ok) {
-  uint32_t r;
-  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbarrier.cta.red.and.pred q, %2, 128, p;\n\t"
-               "selp.b32 %0, 1, 0, q;\n\t}" : "=r"(r) : "r"(ok ? 1u : 0u), "r"(1 + group) : "memory");
-  return r != 0;
-}
-__device__ __forceinline__ void epi_sync(int group) { asm volatile("barrier.cta.sync %0, 128;" ::"r"(1 + group) : "memory"); }
 
 // The MMAs of one channel block: every offset, KSTEPS k-steps for each of the unit's patches (TWO: two, which share the
 // weight tile).  Run by the whole warp.  Returns false if a wait ran out.  The warp issues one instruction per some six
@@ -135,14 +130,16 @@ __device__ __forceinline__ void cv_issue_one_block(const ConvParams& p, const Cv
   }
 }
 
-template <bool F16, int KS>
+// SLIDE: the layer is walked along an axis (conv_slide.cuh).
+template <bool F16, int KS, bool SLIDE>
 __global__ void __launch_bounds__(CV_THREADS, 1)
 conv_tc_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant__ CUtensorMap map_w,
                const __grid_constant__ CUtensorMap map_out, const __grid_constant__ ConvParams p) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t a_full[CV_A_SLOTS], a_empty[CV_A_SLOTS];
   __shared__ __align__(8) uint64_t w_full[CV_W_SLOTS], w_empty[CV_W_SLOTS];
-  __shared__ __align__(8) uint64_t t_full[2], t_empty[2];
+  constexpr int SETS = SLIDE ? CV_RING : 2;          // accumulators that change hands
+  __shared__ __align__(8) uint64_t t_full[SETS], t_empty[SETS];
   __shared__ uint32_t tmem_slot;
   __shared__ int go;
 
@@ -151,7 +148,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
   if (threadIdx.x == 0) {
     for (int s = 0; s < CV_A_SLOTS; ++s) { mbar_init(&a_full[s], 1); mbar_init(&a_empty[s], 1); }
     for (int s = 0; s < CV_W_SLOTS; ++s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(&t_full[b], 1); mbar_init(&t_empty[b], p.acc_bufs == 2 ? 4 : 4 * p.groups); }
+    for (int b = 0; b < SETS; ++b) { mbar_init(&t_full[b], 1); mbar_init(&t_empty[b], SLIDE || p.acc_bufs == 2 ? 4 : 4 * p.groups); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
     prefetch_tmap(&map_in);
@@ -175,6 +172,33 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
 
   if (!go) {
     // fall through to the teardown
+  } else if (SLIDE) {
+    if (warp == 0) {
+      if (lane == 0) sl_copy(p, &map_in, base, i0, i1, a_full, a_empty);
+    } else if (warp == 2) {
+      if (lane == 0 && i0 < i1) {                // all weights once: per block of channels and offset in the plane the ks offsets, the last first
+        mbar_arrive_expect_tx(&w_full[0], (uint32_t)(p.nb * p.ki * KS) * p.w_tile_bytes);
+        uint32_t dst = base + p.w_off;
+        for (int blk = 0; blk < p.nb; ++blk)
+          for (int o = 0; o < p.ki * KS; ++o)
+            for (int k = p.ks - 1; k >= 0; --k) {
+              const int t = k * p.ki * KS + o;
+              if (!p.dgrad) tma_load_3d(dst, &map_w, blk * p.cw, t, 0, &w_full[0]);
+              else
+                for (int j = 0; j < p.w_boxes; ++j) tma_load_3d(dst + (uint32_t)j * p.w_box_bytes, &map_w, j * p.w_nbw, p.T - 1 - t, blk * p.cw, &w_full[0]);
+              dst += p.w_blk_bytes;
+            }
+        mbar_wait(&w_full[0], 0, p.status, p.tag);
+      }
+    } else if (warp == 1) {
+      if (i0 < i1 && mbar_wait_warp(&w_full[0], 0, p.status, p.tag)) {
+        tc_fence_after();
+        sl_issue<KS>(p, tmem_base, (base & 0x3FFFFu) >> 4, ((base + p.w_off) & 0x3FFFFu) >> 4, i0, i1,
+                     SlBars{a_full, a_empty, t_full, t_empty});
+      }
+    } else if (warp >= 4) {
+      sl_epilogue<F16>(p, &map_out, base, tmem_base, i0, i1, t_full, t_empty);
+    }
   } else if (warp == 0) {
     // ------------------------------------------------------------------ input boxes
     if (lane == 0) {
@@ -303,11 +327,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
     // ------------------------------------------------------------------ epilogue
     const int quad = warp & 3, group = (warp - 4) >> 2;
     const uint32_t set_cols = (uint32_t)(p.tile_n * p.m_sub);
-    const int m = quad * 32 + lane, my = m / p.P, mx = m - my * p.P;      // this thread's position in the box
-    const bool live = mx < p.pw && my < p.ph;
-    const int v = my * p.pw + mx;                                         // ... and its pixel of the patch
-    const uint32_t orb = (uint32_t)p.ocw * 2;
-    const uint32_t swz = p.ocw == 64 ? (uint32_t)v & 7u : p.ocw == 32 ? ((uint32_t)v >> 1) & 3u : ((uint32_t)v >> 2) & 1u;
+    const EpiPixel px(p, quad * 32 + lane);                               // this thread's pixel
     const bool leader = quad == 0 && lane == 0;
     uint32_t lu = 0, ob = 0;                                              // ob: which of the group's staging tiles
     for (CvWalk w(p, i0, i1); w.it < i1; ++lu) {
@@ -327,25 +347,10 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_constant
       for (int sub = 0; sub < n; ++sub, w.step(p)) {
         if (share && sub != group) continue;
         for (int c = 0; c < cols; c += p.ocw) {
-          const uint32_t tile = base + p.o_off + ((uint32_t)(group * p.o_per) + ob) * p.o_bytes, row = tile + (uint32_t)v * orb;
+          const uint32_t tile = base + p.o_off + ((uint32_t)(group * p.o_per) + ob) * p.o_bytes;
           if (leader) { if (p.o_per == 1) bulk_wait_read<0>(); else bulk_wait_read<1>(); }     // the tile's last store has read it
           epi_sync(group);
-          for (int h = 0; h < p.ocw && c + h < p.tile_n; h += 32) {
-            uint32_t r[32];
-            const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + buf * set_cols + (uint32_t)(sub * p.tile_n + c + h);
-            if (p.tile_n - c - h >= 32) tmem_ld32(taddr, r);
-            else tmem_ld16(taddr, r);
-            const int n16 = min(32, min(p.ocw, p.tile_n - c) - h) >> 3;   // 16-byte pieces
-            if (live) {
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                if (i >= n16) break;
-                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(row + ((((uint32_t)(h >> 3) + i) ^ swz) << 4)),
-                             "r"(pack2(r[8 * i + 0], r[8 * i + 1], F16)), "r"(pack2(r[8 * i + 2], r[8 * i + 3], F16)),
-                             "r"(pack2(r[8 * i + 4], r[8 * i + 5], F16)), "r"(pack2(r[8 * i + 6], r[8 * i + 7], F16)) : "memory");
-              }
-            }
-          }
+          epi_row<F16>(p, px, tile, tmem_base + ((uint32_t)(quad * 32) << 16) + buf * set_cols + (uint32_t)(sub * p.tile_n + c), p.tile_n - c);
           if (sub == last && c + p.ocw >= cols) {                         // this group has read what it reads of the set
             tc_fence_before();
             __syncwarp();
@@ -385,6 +390,54 @@ static CUtensorMapSwizzle swizzle_of(int row_elems) {
 static uint32_t layout_of(int row_elems) { return row_elems == 64 ? 2u : row_elems == 32 ? 4u : 6u; }
 static int block_width(int c) { return c > 32 ? 64 : c > 16 ? 32 : 16; }
 
+// The plan of conv_slide.cuh and the clocks of its busiest CTA, as measured: the MMAs of a plane hold the pipe N/2 clocks each or as long as their operands take
+// from shared memory, or the warp that issues them some 45 and 230 a plane; the planes at the ends of a CTA's segments and where the ring of accumulators
+// ends take 750 and 105 an MMA; an epilogue warp waits some 250 clocks for its turn beside what its columns take, and there are two groups.
+static long plan_slide(const xconv_desc* d, bool dgrad, TcConvPlan* p) {
+  const int Ci = dgrad ? d->Cout : d->Cin, Co = dgrad ? d->Cin : d->Cout;
+  const ConvGeo g = conv_geo(d);
+  const int K = d->KH, ks = K, planar = d->KD > 1 ? 0 : 1, ki = planar ? 1 : K;
+  if (K < 3) return -1;
+  const long extent = planar ? g.H : g.D;
+  const int nbw = dgrad ? (Co % 64 == 0 ? 64 : 32) : 16, tile_n = round_up(Co, nbw), ocw = block_width(Co);
+  if (ks * tile_n > 256) return -1;
+  const int ring = std::min(CV_RING, 512 / tile_n);
+  const uint32_t budget = SMEM_LIMIT - 4096;
+  long best = -1;
+  for (int cw = block_width(Ci); cw >= 16 && best < 0; cw /= 2) {      // (narrower blocks only where no plan fits)
+    const int nb = (int)cdivl(Ci, cw), ksteps = (nb - 1) * (cw / 16) + (int)cdivl(Ci - (nb - 1) * cw, 16);
+    const uint32_t rb = 2 * (uint32_t)cw;
+    const long w_bytes = (long)nb * ki * K * ks * tile_n * rb;
+    for (long nx = cdivl(g.W, 128); nx <= std::max(cdivl(g.W, 128), std::min(32L, g.W)); ++nx) {
+      const int pw = (int)cdivl(g.W, nx), P = pw + K - 1;
+      if (P > 256) continue;
+      const long across = planar ? g.B : g.H;                       // what a tile takes several rows of: images or rows
+      const int ph_max = (int)std::min<long>(across, (128 - pw) / P + 1), ph = (int)cdivl(across, cdivl(across, ph_max));
+      const int box_rows = P * (planar ? ph : ph + K - 1), need_rows = (ki - 1) * P + K - 1 + TILE_M;
+      const uint32_t a_sub = align1k((uint32_t)std::max(box_rows, need_rows) * rb), o_bytes = align1k((uint32_t)(pw * ph) * 2 * ocw);
+      const long room = (long)budget - w_bytes - 1024 - 2L * o_bytes;
+      if (room < 2L * a_sub) continue;
+      const int o_per = room >= 4L * a_sub + 2L * o_bytes ? 2 : 1;
+      const int a_slots = (int)std::min<long>(CV_A_SLOTS, (room - (o_per - 1) * 2L * o_bytes) / a_sub);
+      const long columns = cdivl(g.W, pw) * cdivl(across, ph) * (planar ? 1 : g.B), items = columns * extent;
+      if (items >= (1L << 31)) continue;
+      const long per_cta = cdivl(items, std::min<long>(items, NUM_SMS));
+      const long segments = per_cta >= extent ? cdivl(per_cta, extent) : (extent % per_cta ? 2 : 1), planes = per_cta + (ks - 1) * std::min(2L, segments);
+      const long products = (long)ki * K * ksteps + 1, pipe = std::max({62, ks * tile_n / 2, 40 + ks * tile_n / 4});
+      const long bytes = (long)nb * box_rows * rb, copy = std::max(bytes / 45, bytes * 2200 / ((long)a_slots * a_sub));
+      const long odd = std::min(planes, nb > 1 ? planes : 2 * (ks - 1) * segments + per_cta * (ks - 1) / ring);      // planes that are not like the one before
+      const long inner = std::max({230 + 45 * products, products * pipe, copy, (250 + 7L * tile_n) / 2}), other = 750 + 500 * (nb - 1) + products * std::max(105L, pipe);
+      const long cost = (planes - odd) * inner + odd * std::max(other, copy) + w_bytes / 45;
+      if (best >= 0 && cost >= best) continue;
+      best = cost;
+      p->slide = 1; p->ring = ring;
+      p->cw = cw; p->m_sub = 1; p->tile_n = tile_n; p->tiles_n = 1; p->acc_bufs = 2; p->patch_w = pw; p->patch_h = ph;
+      p->resident = 1; p->w_slots = 0; p->groups = 2; p->nbw = nbw; p->ocw = ocw; p->patches = items; p->o_per = o_per; p->a_slots = a_slots; p->a_sub_bytes = a_sub;
+    }
+  }
+  return best;
+}
+
 // Picks patch, column tile, patches per weight tile and the place of the weights by the time a CTA would take, in
 // clocks: the MMAs (a k-step of N columns holds the pipe N/2 clocks, and at least the 34 it takes to read its A tile),
 // or the copies where they take longer (an SM pulls about 45 bytes per clock from L2), times the items of the busiest CTA.
@@ -396,7 +449,7 @@ bool tc_plan_conv(const xconv_desc* d, bool dgrad, TcConvPlan* p) {
   if (g.W >= (1L << 31) || g.B >= (1L << 31)) return false;
   const int K = d->KH, KD = d->KD > 1 ? d->KD : 1, T = KD * K * K;
   const uint32_t budget = SMEM_LIMIT - 4096;
-  long best = -1;
+  long best = -1, real = 0;
   for (int cw = block_width(Ci); cw >= 16 && best < 0; cw /= 2) {   // (narrower blocks only where no plan fits)
     const int nb = (int)cdivl(Ci, cw), ks_last = (int)cdivl(Ci - (nb - 1) * cw, 16), ksteps = (nb - 1) * (cw / 16) + ks_last;
     const uint32_t rb = 2 * (uint32_t)cw;
@@ -443,15 +496,26 @@ bool tc_plan_conv(const xconv_desc* d, bool dgrad, TcConvPlan* p) {
           // sketch; in the place of boxes 256 -> 192 channels, 1 x 1 53.4 -> 55.9).
           p->w_slots = 0;
           if (room - w_all >= 2 * o_bytes + 2 * a_slot) p->o_per = 2;
-          p->a_slots = (int)std::min<uint32_t>(CV_A_SLOTS, 2 + (room - w_all - (p->o_per == 2 ? 2 * o_bytes : 0)) / a_slot);
+          p->a_slots = (int)std::min<uint32_t>(4, 2 + (room - w_all - (p->o_per == 2 ? 2 * o_bytes : 0)) / a_slot);
         } else {
           p->a_slots = room >= a_slot + 4 * w_tile ? 3 : 2;
           p->w_slots = (int)std::min<uint32_t>(CV_W_SLOTS, (budget - (uint32_t)p->a_slots * a_slot - 2 * o_bytes) / w_tile);
         }
         p->a_sub_bytes = a_sub;
+        p->slide = 0;
+        // ... and what its patches take as measured: an MMA 56 clocks at least, 250 from one patch to the next, and a ring of weight tiles hands on as many as
+        // it holds in the time of one copy
+        const long turns = std::max({(long)T * ksteps * m_sub * std::max(56, tile_n / 2) + 250, resident ? 0 : (long)nb * T * 2200 / p->w_slots, m_sub * copy, m_sub * epi});
+        real = cdivl(per_cta, m_sub) * turns + (resident ? (long)w_all / 45 : 0);
       }
     }
   }
+  // Both counts leave out the same 5 us of launch, first copies and last stores, and the walk's last planes complete several outputs at once: it is taken
+  // for a tenth and 2000 clocks less, or where the weights would be streamed.  (Of 104 convolutions with at most 64 channels on one side 14 are walked,
+  // 0.39 to 0.95 of the time; without the 2000 clocks also 5 x 5, 8 -> 16 channels of 4 images of 224 x 224, 20.2 -> 22.6 us.)
+  TcConvPlan slide{};
+  const long sliding = best >= 0 && real < 8000 ? -1 : plan_slide(d, dgrad, &slide);      // (a walk takes that much for its first and last planes)
+  if (sliding >= 0 && (best < 0 || sliding + 2000 < (p->resident ? real - real / 10 : real))) { *p = slide; return true; }
   return best >= 0;
 }
 
@@ -465,11 +529,17 @@ xconv_status tc_run_conv(const xconv_desc* d, const TcConvPlan& pl, bool dgrad, 
   p.KD = KD; p.T = T; p.pad = (K - 1) / 2; p.pad_d = (KD - 1) / 2; p.dgrad = dgrad ? 1 : 0;
   p.pw = pl.patch_w; p.ph = pl.patch_h; p.P = pl.patch_w + K - 1;
   p.patches_x = (int)cdivl(g.W, p.pw); p.patches_y = (int)cdivl(g.H, p.ph); p.depth = (int)g.D;
+  if (pl.slide) {
+    p.planar = KD == 1 ? 1 : 0;
+    p.ks = K; p.ki = p.planar ? 1 : K; p.pad_s = (K - 1) / 2; p.ring = pl.ring;
+    p.extent = (int)(p.planar ? g.H : g.D); p.img_step = p.planar ? p.ph : 1;
+    if (p.planar) p.patches_y = 1;
+  }
   p.patches = (uint32_t)pl.patches; p.items = (uint32_t)(pl.patches * pl.tiles_n);
   p.plane_rows = (uint32_t)(p.P * (p.ph + K - 1));
   p.m_sub = pl.m_sub; p.acc_bufs = pl.acc_bufs; p.groups = pl.groups; p.tile_n = pl.tile_n;
   p.o_per = pl.o_per;
-  p.tmem_cols = pow2_cols(pl.acc_bufs * pl.m_sub * pl.tile_n);
+  p.tmem_cols = pow2_cols(pl.slide ? pl.ring * pl.tile_n : pl.acc_bufs * pl.m_sub * pl.tile_n);
   p.cw = pl.cw; p.nb = (int)cdivl(Ci, pl.cw); p.ks_full = pl.cw / 16; p.ks_last = (int)cdivl(Ci - (p.nb - 1) * pl.cw, 16);
   p.rb = 2 * (uint32_t)pl.cw;
   p.a_sub_bytes = pl.a_sub_bytes; p.a_tx = p.plane_rows * KD * p.rb; p.a_slots = pl.a_slots;
@@ -477,8 +547,13 @@ xconv_status tc_run_conv(const xconv_desc* d, const TcConvPlan& pl, bool dgrad, 
   p.w_tile_bytes = (uint32_t)pl.tile_n * p.rb;
   p.w_boxes = dgrad ? pl.tile_n / pl.nbw : 1;
   p.w_box_bytes = p.w_tile_bytes / (uint32_t)p.w_boxes;
+  p.w_blk_bytes = p.w_tile_bytes;
+  if (pl.slide) {                                // a tile: the weights of the axis' ks offsets
+    p.w_tile_bytes *= (uint32_t)p.ks;
+    p.a_tx = (uint32_t)(p.P * (p.planar ? p.ph : p.ph + K - 1)) * p.rb;
+  }
   p.w_off = (uint32_t)(pl.a_slots * pl.m_sub) * pl.a_sub_bytes;
-  p.o_off = align1k(p.w_off + (uint32_t)(pl.resident ? p.nb * T : pl.w_slots) * p.w_tile_bytes);
+  p.o_off = align1k(p.w_off + (uint32_t)(pl.resident ? p.nb * T : pl.w_slots) * p.w_blk_bytes);
   p.ocw = pl.ocw; p.co = Co;
   p.o_bytes = align1k((uint32_t)(p.pw * p.ph * 2 * pl.ocw));
   p.a_hi = ((8 * p.rb) >> 4) | (1u << 14) | (layout_of(pl.cw) << 29);
@@ -492,32 +567,36 @@ xconv_status tc_run_conv(const xconv_desc* d, const TcConvPlan& pl, bool dgrad, 
     p.b_lo0 = 1u << 16;
     p.b_step = 2;
   }
-  p.idesc = (1u << 4) | (f16 ? 0u : (1u << 7) | (1u << 10)) | (dgrad ? 1u << 16 : 0u) | ((uint32_t)(pl.tile_n >> 3) << 17) |
+  p.idesc = (1u << 4) | (f16 ? 0u : (1u << 7) | (1u << 10)) | (dgrad ? 1u << 16 : 0u) | (pl.slide ? 0u : (uint32_t)(pl.tile_n >> 3) << 17) |
             ((uint32_t)(TILE_M >> 4) << 24);
   p.status = reinterpret_cast<unsigned int*>(ws_head);
   p.tag = call_tag();
 
   CUtensorMap mi, mw, mo;
-  auto image_map = [&](CUtensorMap* m, const void* ptr, int C, int cb, int bw, int bh, int bd) {
+  auto image_map = [&](CUtensorMap* m, const void* ptr, int C, int cb, int bw, int bh, int bd, int bb) {
     const uint64_t dims[5] = {(uint64_t)C, (uint64_t)g.W, (uint64_t)g.H, (uint64_t)g.D, (uint64_t)g.B};
     const uint64_t row = (uint64_t)C * 2;
     const uint64_t str[4] = {row, row * g.W, row * g.W * g.H, row * g.W * g.H * g.D};
-    const uint32_t box[5] = {(uint32_t)cb, (uint32_t)bw, (uint32_t)bh, (uint32_t)bd, 1};
+    const uint32_t box[5] = {(uint32_t)cb, (uint32_t)bw, (uint32_t)bh, (uint32_t)bd, (uint32_t)bb};
     return make_map(m, ptr, 5, dims, str, box, f16, swizzle_of(cb));
   };
   const uint64_t dw[3] = {(uint64_t)d->Cin, (uint64_t)T, (uint64_t)d->Cout};
   const uint64_t sw[2] = {(uint64_t)d->Cin * 2, (uint64_t)T * d->Cin * 2};
   const uint32_t bw[3] = {(uint32_t)(dgrad ? pl.nbw : pl.cw), 1, (uint32_t)(dgrad ? pl.cw : pl.tile_n)};
-  if (!image_map(&mi, in, Ci, pl.cw, p.P, p.ph + K - 1, KD) || !image_map(&mo, out, Co, pl.ocw, p.pw, p.ph, 1) ||
+  const bool rows = pl.slide && p.planar;        // a tile's rows are of several images
+  if (!image_map(&mi, in, Ci, pl.cw, p.P, rows ? 1 : p.ph + K - 1, pl.slide ? 1 : KD, rows ? p.ph : 1) ||
+      !image_map(&mo, out, Co, pl.ocw, p.pw, rows ? 1 : p.ph, 1, rows ? p.ph : 1) ||
       !make_map(&mw, W, 3, dw, sw, bw, f16, swizzle_of(dgrad ? pl.nbw : pl.cw)))
     return XCONV_ERR_CUDA;
   const size_t smem = 1024 + (size_t)p.o_off + (size_t)(p.groups * p.o_per) * p.o_bytes;
   if (smem > (size_t)(SMEM_LIMIT - 1024)) return XCONV_ERR_UNSUPPORTED;
   const unsigned grid = std::min<uint32_t>(p.items, NUM_SMS);
   void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, ConvParams) =
-      K == 3 ? (f16 ? conv_tc_kernel<true, 3> : conv_tc_kernel<false, 3>)
-      : K == 5 ? (f16 ? conv_tc_kernel<true, 5> : conv_tc_kernel<false, 5>)
-               : (f16 ? conv_tc_kernel<true, 1> : conv_tc_kernel<false, 1>);
+      K == 1 ? (f16 ? conv_tc_kernel<true, 1, false> : conv_tc_kernel<false, 1, false>)
+      : pl.slide ? (K == 3 ? (f16 ? conv_tc_kernel<true, 3, true> : conv_tc_kernel<false, 3, true>)
+                           : (f16 ? conv_tc_kernel<true, 5, true> : conv_tc_kernel<false, 5, true>))
+      : K == 3 ? (f16 ? conv_tc_kernel<true, 3, false> : conv_tc_kernel<false, 3, false>)
+               : (f16 ? conv_tc_kernel<true, 5, false> : conv_tc_kernel<false, 5, false>);
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT - 1024);
   if (e == cudaSuccess)
     e = launch_pdl(kernel, dim3(grid), dim3(128 + 128 * p.groups), smem_of_grid(smem, grid), st, mi, mw, mo, p);

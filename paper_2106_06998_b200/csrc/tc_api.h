@@ -47,6 +47,7 @@ struct TcConvPlan {
   int groups;                // of epilogue warps: two where a patch is over quickly, one beside long mainloops, whose issue
                              // slots the second would only take
   long patches;
+  int slide, ring;           // walk along an axis (conv_slide.cuh), patches then counts outputs; accumulators in the ring
 };
 
 struct TcHaloPlan {            // contraction of layers with few channels (contract_tc.cu)
