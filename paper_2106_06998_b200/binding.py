@@ -7,6 +7,7 @@ library is missing or a layer has no kernel, a RuntimeError is raised.
 """
 from __future__ import annotations
 
+import atexit
 import ctypes
 import os
 import threading
@@ -53,9 +54,10 @@ _lib = None
 
 def lib() -> ctypes.CDLL:
     """The loaded shared library; raises if it has not been built (no fallback exists)."""
-    global _lib
+    global _lib, _native
     if _lib is not None:
         return _lib
+    _native = None                              # (it calls the library that was loaded before)
     if not os.path.exists(LIB_PATH):
         raise RuntimeError(f"{LIB_PATH} is missing: build it with `python -m paper_2106_06998_b200.build` "
                            "(libxconv has no CPU or library fallback)")
@@ -114,6 +116,26 @@ def lib() -> ctypes.CDLL:
     L.xconv_status_string.argtypes = [c_int]; L.xconv_status_string.restype = c_char_p
     _lib = L
     return L
+
+
+# csrc/marshal.cpp: the calls below on ordinary tensors, in native code.  It answers None where the call is not that simple; the Python path behind it
+# takes everything, and raises every error.
+_native = None
+_NATIVE_CALLS = ("xconv_workspace_bytes", "xconv_forward", "xconv_sketch", "xconv_wgrad", "xconv_dgrad", "xconv_sketch_seeded", "xconv_wgrad_seeded",
+                 "xconv_backprobe", "xconv_contract")
+
+
+def _load_native():
+    global _native
+    try:
+        from . import _marshal
+    except ImportError as e:
+        raise RuntimeError(f"{os.path.join(_HERE, '_marshal.so')} cannot be loaded ({e}): build it with `python -m paper_2106_06998_b200.build`") from e
+    L = lib()                                   # (before `_native` is set)
+    _marshal.use_library(*(ctypes.cast(getattr(L, name), c_void_p).value for name in _NATIVE_CALLS), _check)
+    atexit.register(_marshal.release)
+    _native = _marshal
+    return _marshal
 
 
 def _dtype_code(t: torch.dtype) -> int:
@@ -295,6 +317,9 @@ def last_launch_count() -> int:
 
 def xconv_sketch(X: torch.Tensor, Z: torch.Tensor) -> torch.Tensor:
     """S = Z^T X (Algorithm 1 forward step 3): float32 tensor [r, B].  X (B, Cin, [D,] H, W), Z (r, Cin, [D,] H, W)."""
+    out = (_native or _load_native()).sketch(X, Z)
+    if out is not None:
+        return out
     _cl(X, "X"); _cl(Z, "Z")
     B, Cin = X.shape[:2]
     D, H, W = _geo(X)
@@ -336,6 +361,10 @@ def xconv_block_sparse_probes_from_seed(seed: int, p: float, r: int, Cin: int, H
 def xconv_sketch_seeded(X: torch.Tensor, seed: int, r: int, gaussian: bool = False) -> torch.Tensor:
     """S = Z[seed]^T X without a stored Z (Algorithm 1 keeps the seed): float32 tensor [r, B].  ``gaussian``: standard
     normal probing vectors (drawn into the workspace) instead of Rademacher ones."""
+    if gaussian is False:
+        out = (_native or _load_native()).sketch_seeded(X, seed, r)
+        if out is not None:
+            return out
     _cl(X, "X")
     B, Cin = X.shape[:2]
     D, H, W = _geo(X)
@@ -356,6 +385,10 @@ def xconv_wgrad_seeded(sketch: torch.Tensor, dY: torch.Tensor, seed: int, Cin: i
     """dW estimate from the sketch and the seed (Algorithm 1 backward steps 2-4): Z[seed] is redrawn on chip or into
     the workspace, never passed in.  float32 (Cout, Cin, [KD,] K, K), channels-last.  ``gaussian``: standard normal
     probing vectors instead of Rademacher ones."""
+    if gaussian is False:
+        out = (_native or _load_native()).wgrad_seeded(sketch, dY, seed, Cin, kernel_size, kernel_depth, circular)
+        if out is not None:
+            return out
     _cl(dY, "dY")
     B, Cout = dY.shape[:2]
     D, H, Wd = _geo(dY)
@@ -394,6 +427,9 @@ def xconv_sketch_static(X: torch.Tensor, Z: torch.Tensor, out: torch.Tensor | No
 
 def xconv_forward(X: torch.Tensor, W: torch.Tensor, Z: torch.Tensor, circular: bool = False):
     """Y = conv(X, W) and the sketch S = Z^T X (Algorithm 1 forward steps 1 and 3).  5-d tensors are volumes."""
+    out = (_native or _load_native()).forward(X, W, Z, circular)
+    if out is not None:
+        return out
     _cl(X, "X"); _cl(W, "W"); _cl(Z, "Z")
     B, Cin = X.shape[:2]
     D, H, Wd = _geo(X)
@@ -415,6 +451,10 @@ def xconv_wgrad(sketch: torch.Tensor, dY: torch.Tensor, Z: torch.Tensor, kernel_
                 chan_scale: torch.Tensor | None = None, kernel_depth: int = 1,
                 zero_blocks: torch.Tensor | None = None, circular: bool = False) -> torch.Tensor:
     """dW estimate (Algorithm 1 backward steps 3-4): float32 (Cout, Cin, [KD,] K, K), channels-last."""
+    if chan_scale is None and zero_blocks is None:
+        out = (_native or _load_native()).wgrad(sketch, dY, Z, kernel_size, kernel_depth, circular)
+        if out is not None:
+            return out
     _cl(dY, "dY"); _cl(Z, "Z")
     B, Cout = dY.shape[:2]
     D, H, Wd = _geo(dY)
@@ -472,6 +512,9 @@ def xconv_wgrad_independent(sketch: torch.Tensor, dY: torch.Tensor, Z: torch.Ten
 
 def xconv_backprobe(sketch: torch.Tensor, dY: torch.Tensor) -> torch.Tensor:
     """L = S dY^T (Algorithm 1 backward step 3): (r, Cout, [D,] H, W) in dY's dtype, channels-last."""
+    out = (_native or _load_native()).backprobe(sketch, dY)
+    if out is not None:
+        return out
     _cl(dY, "dY")
     B, Cout = dY.shape[:2]
     D, H, Wd = _geo(dY)
@@ -489,6 +532,10 @@ def xconv_contract(L: torch.Tensor, Z: torch.Tensor, kernel_size: int = 3,
                    chan_scale: torch.Tensor | None = None, kernel_depth: int = 1,
                    zero_blocks: torch.Tensor | None = None, circular: bool = False) -> torch.Tensor:
     """dW[m,n,k] = scale[n] * sum L[j,m,.] Z[j,n,.+k] (Algorithm 1 backward step 4)."""
+    if chan_scale is None and zero_blocks is None:
+        out = (_native or _load_native()).contract(L, Z, kernel_size, kernel_depth, circular)
+        if out is not None:
+            return out
     _cl(L, "L"); _cl(Z, "Z")
     r, Cout = L.shape[:2]
     D, H, Wd = _geo(L)
@@ -506,6 +553,9 @@ def xconv_contract(L: torch.Tensor, Z: torch.Tensor, kernel_size: int = 3,
 
 def xconv_dgrad(dY: torch.Tensor, W: torch.Tensor, circular: bool = False) -> torch.Tensor:
     """Exact dX (transposed convolution)."""
+    out = (_native or _load_native()).dgrad(dY, W, circular)
+    if out is not None:
+        return out
     _cl(dY, "dY"); _cl(W, "W")
     B, Cout = dY.shape[:2]
     D, H, Wd = _geo(dY)

@@ -1,4 +1,4 @@
-"""Builds libxconv.so in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Builds libxconv.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and the binding's native part with the host compiler."""
 from __future__ import annotations
 
 import os
@@ -8,6 +8,7 @@ import subprocess
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libxconv.so")
+MARSHAL, MARSHAL_SOURCE = os.path.join(HERE, "_marshal.so"), os.path.join(HERE, "csrc", "marshal.cpp")
 SOURCES = ["api.cu", "tc_kernels.cu", "conv_tc.cu", "contract_tc.cu", "stream_tc.cu", "conv_fma.cu", "conv_split.cu", "contract_split.cu", "gemm_split.cu",
            "static_scratch.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -25,14 +26,31 @@ def _stale() -> bool:
     if not os.path.exists(LIB):
         return True
     t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(HERE, "..", "include", "xconv.h")]
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if not f.endswith(".cpp")] + [os.path.join(HERE, "..", "include", "xconv.h")]
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def build_marshal(force: bool = False) -> str:
+    """Compiles the binding's calls on ordinary tensors (csrc/marshal.cpp) against the installed torch; returns the module's path."""
+    header = os.path.join(HERE, "..", "include", "xconv.h")
+    if not force and os.path.exists(MARSHAL) and os.path.getmtime(MARSHAL) >= max(map(os.path.getmtime, (MARSHAL_SOURCE, header))):
+        return MARSHAL
+    import sysconfig
+    import torch
+    top = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
+    subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+                    "-isystem", os.path.join(top, "include"), "-isystem", os.path.join(top, "include", "torch", "csrc", "api", "include"),
+                    "-isystem", sysconfig.get_paths()["include"], "-isystem", os.path.join(cuda, "include"), MARSHAL_SOURCE, "-o", MARSHAL,
+                    "-L" + os.path.join(top, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-L" + os.path.join(cuda, "lib64"), "-lcudart"], check=True)
+    return MARSHAL
 
 
 def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     """Compile every CUDA source into one shared library; returns its path.
     ``extra_flags`` go to nvcc."""
     if not force and not _stale():
+        build_marshal()
         return LIB
     objs, jobs = [], []
     for src in SOURCES:
@@ -48,6 +66,7 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
         if code != 0:
             raise subprocess.CalledProcessError(code, cmd)
     subprocess.run([_nvcc(), "-shared", "-cudart", "static", "-o", LIB, *objs, "-ldl"], check=True)
+    build_marshal(force)
     return LIB
 
 
