@@ -9,7 +9,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libxconv.so")
 MARSHAL, MARSHAL_SOURCE = os.path.join(HERE, "_marshal.so"), os.path.join(HERE, "csrc", "marshal.cpp")
-SOURCES = ["api.cu", "tc_kernels.cu", "conv_tc.cu", "contract_tc.cu", "stream_tc.cu", "conv_fma.cu", "conv_split.cu", "contract_split.cu", "gemm_split.cu",
+SOURCES = ["api.cu", "tc_kernels.cu", "conv_tc.cu", "contract_tc.cu", "stream_tc.cu", "conv_fma.cu", "small_f32.cu", "conv_split.cu", "contract_split.cu", "gemm_split.cu",
            "static_scratch.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "--use_fast_math=false", "-Xcompiler", "-fPIC,-O2", "-cudart", "static"]

@@ -13,6 +13,7 @@
 #include "conv_split.h"
 #include "contract_split.h"
 #include "gemm_split.h"
+#include "small_f32.h"
 #include "tc_api.h"
 #include <type_traits>
 
@@ -470,11 +471,13 @@ static xconv_status run_sketch_simt(const xconv_desc* d, const SketchPlan& p, co
     const size_t smem = (size_t)GT_STAGES * 128 * GT_LD * sizeof(float);
     cudaError_t ea = cudaFuncSetAttribute(gemm_tn_simt_async, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (ea != cudaSuccess) { g_last_cuda_error = (int)ea; return XCONV_ERR_CUDA; }
-    gemm_tn_simt_async<<<grid, 256, smem, st>>>(reinterpret_cast<const float*>(Z), reinterpret_cast<const float*>(X), part,
-                                                d->r, d->B, K, p.k_per_split);
+    ea = launch_pdl(gemm_tn_simt_async, grid, dim3(256), smem, st, reinterpret_cast<const float*>(Z), reinterpret_cast<const float*>(X), part,
+                    d->r, d->B, K, p.k_per_split);
+    if (ea != cudaSuccess) { g_last_cuda_error = (int)ea; return XCONV_ERR_CUDA; }
   } else {
-    gemm_tn_simt<T><<<grid, 256, 0, st>>>(static_cast<const T*>(Z), static_cast<const T*>(X), part, d->r, d->B, K,
-                                          p.k_per_split, (K % 4 == 0) ? 1 : 0);
+    const cudaError_t ea = launch_pdl(gemm_tn_simt<T>, grid, dim3(256), 0, st, static_cast<const T*>(Z), static_cast<const T*>(X), part, d->r, d->B, K,
+                                      p.k_per_split, (K % 4 == 0) ? 1 : 0);
+    if (ea != cudaSuccess) { g_last_cuda_error = (int)ea; return XCONV_ERR_CUDA; }
   }
   xconv_status s = check_launch();
   if (s != XCONV_OK) return s;
@@ -535,8 +538,9 @@ static xconv_status run_backprobe_simt(const xconv_desc* d, const float* S, cons
     if (best < 0 || cost < best) { best = cost; threads = t; }
   }
   dim3 g1((unsigned)cdiv(cdiv(Q, 4), threads), (unsigned)cdiv(d->r, 16));
-  backprobe_simt<T, TL><<<g1, threads, 0, st>>>(S, static_cast<const T*>(dY), static_cast<TL*>(Lv), d->r, d->B, Q,
-                                                (Q % 4 == 0) ? 1 : 0);
+  const cudaError_t e = launch_pdl(backprobe_simt<T, TL>, g1, dim3(threads), 0, st, S, static_cast<const T*>(dY), static_cast<TL*>(Lv), d->r, d->B, Q,
+                                   (Q % 4 == 0) ? 1 : 0);
+  if (e != cudaSuccess) { g_last_cuda_error = (int)e; return XCONV_ERR_CUDA; }
   return check_launch();
 }
 
@@ -548,6 +552,11 @@ static xconv_status run_contract_simt(const xconv_desc* d, const WgradPlan& p, c
   const T* Zt = static_cast<const T*>(Z);
   const bool vec = d->Cin % 4 == 0 && d->Cout % 4 == 0;      // rows of L and Z then start on 4-element boundaries
   const unsigned gx = (unsigned)cdiv(d->Cin, 64), gy = (unsigned)cdiv(d->Cout, 32), gz = (unsigned)p.splits;
+  if constexpr (std::is_same<T, float>::value)
+    if (small_contract_serves(d)) {
+      const xconv_status ss = run_small_contract(d, p.splits, p.items_per_split, L, Zt, part, st);
+      return ss == XCONV_OK ? run_reduce(part, dW, (long)d->Cout * T9 * d->Cin, p.splits, alpha, d->chan_scale, d->Cin, st) : ss;
+    }
 #define XC_CONTRACT(KS, KD, DYS) do { \
     dim3 g2(gx * (KD * KS / DYS), gy, gz); \
     if (vec && std::is_same<TL, float>::value && std::is_same<T, float>::value) { \
@@ -575,9 +584,12 @@ static xconv_status run_conv_simt(const xconv_desc* d, bool dgrad, const void* i
   const int Ci = dgrad ? d->Cout : d->Cin, Co = dgrad ? d->Cin : d->Cout;
   const int D = depth(d), planes = d->B * D;
   ConvFma g;
-  if constexpr (std::is_same<T, float>::value)
+  if constexpr (std::is_same<T, float>::value) {
+    if (small_conv_serves(d))
+      return run_small_conv(d, dgrad, static_cast<const float*>(in), static_cast<const float*>(Wt), static_cast<float*>(out), st);
     if (plan_conv_fma(d, dgrad, &g))
       return run_conv_fma(d, g, dgrad, static_cast<const float*>(in), static_cast<const float*>(Wt), static_cast<float*>(out), st);
+  }
   dim3 grid((unsigned)((long)planes * d->H * cdiv(d->W, 32)), (unsigned)cdiv(Co, 64));
   const T* i_ = static_cast<const T*>(in);
   const T* w_ = static_cast<const T*>(Wt);

@@ -16,14 +16,15 @@ __device__ __forceinline__ int wrap_index(int v, int n) { v %= n; return v < 0 ?
 // Split over k: block z writes its partial tile to part[z][M][N]; reduce_partials sums them in order.
 // ---------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(256) gemm_tn_simt(const T* __restrict__ A, const T* __restrict__ Bm,
-                                                    float* __restrict__ part, int M, int N, long K,
+__global__ void __launch_bounds__(256) gemm_tn_simt(const T* A, const T* Bm, float* part, int M, int N, long K,
                                                     long k_per_split, int vec) {
   // 64 x 64 outputs per block, 32 k per step (128 consecutive bytes of a row; rows lie K elements apart);
   // the loads of the next step are issued before the arithmetic of this one.
   constexpr int KS = 32;
   __shared__ __align__(16) float As[KS][68];
   __shared__ __align__(16) float Bs[KS][68];
+  pdl_trigger();
+  pdl_wait();
   const int tid = threadIdx.x;
   const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
   const long kb = (long)blockIdx.z * k_per_split;
@@ -98,9 +99,10 @@ __device__ __forceinline__ void cp_async16_f(float* dst, const float* src, bool 
   asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
                "r"(valid ? 16 : 0) : "memory");
 }
-static __global__ void __launch_bounds__(256) gemm_tn_simt_async(const float* __restrict__ A, const float* __restrict__ Bm,
-                                                          float* __restrict__ part, int M, int N, long K, long k_per_split) {
+static __global__ void __launch_bounds__(256) gemm_tn_simt_async(const float* A, const float* Bm, float* part, int M, int N, long K, long k_per_split) {
   extern __shared__ __align__(16) float gt_tiles[];       // [stage][A rows 0..63 | B rows 0..63][GT_LD]
+  pdl_trigger();
+  pdl_wait();
   const int tid = threadIdx.x;
   const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
   const long kb = (long)blockIdx.z * k_per_split;
@@ -205,9 +207,10 @@ reduce_partials(const float* __restrict__ part, float* __restrict__ out, long co
 // size, a multiple of 32 up to 256, so that the grid fills whole waves of the SMs).
 // ---------------------------------------------------------------------------------------------
 template <typename T, typename TL>
-__global__ void __launch_bounds__(256) backprobe_simt(const float* __restrict__ S, const T* __restrict__ dY,
-                                                      TL* __restrict__ L, int r, int B, long Q, int vec) {
+__global__ void __launch_bounds__(256) backprobe_simt(const float* S, const T* dY, TL* L, int r, int B, long Q, int vec) {
   __shared__ __align__(16) float Ss[128][16];
+  pdl_trigger();
+  pdl_wait();
   const int tid = threadIdx.x;
   const long q = ((long)blockIdx.x * blockDim.x + tid) * 4;
   const int j0 = blockIdx.y * 16;
