@@ -180,15 +180,19 @@ static SketchPlan plan_sketch(const xconv_desc* d_, bool seeded = false) {
 static inline int pad8(int c) { return (c + 7) / 8 * 8; }
 static size_t padded_bytes(long rows, int c) { return c % 8 ? align_up((size_t)rows * pad8(c) * 2, 256) : 0; }
 
-template <typename T>
-__global__ void __launch_bounds__(256) pad_channels_kernel(const T* __restrict__ in, T* __restrict__ out, long pieces, int C,
-                                                           int per_row) {
-  pdl_trigger();
-  pdl_wait();
-  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;      // one 16-byte piece of the padded tensor
-  if (i >= pieces) return;
+// One or two tensors of C channels; a thread writes one 16-byte piece.
+struct PadJob { const unsigned short* in; unsigned short* out; long pieces; };
+static __global__ void __launch_bounds__(256) pad_channels_kernel(const PadJob one, const PadJob two, int C, int per_row) {
+  const long at = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool second = at >= one.pieces;
+  const long i = second ? at - one.pieces : at;
+  const unsigned short* in = second ? two.in : one.in;
+  unsigned short* out = second ? two.out : one.out;
   const long row = i / per_row;
   const int c0 = (int)(i - row * per_row) * 8;
+  pdl_wait();
+  pdl_trigger();
+  if (i >= (second ? two.pieces : one.pieces)) return;
   uint32_t w[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
   for (int k = 0; k < 8; ++k)
@@ -196,16 +200,21 @@ __global__ void __launch_bounds__(256) pad_channels_kernel(const T* __restrict__
   *reinterpret_cast<uint4*>(out + i * 8) = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// `t` itself, or its padded copy at *ws (which then moves on behind it).
-static xconv_status pad_channels(const void*& t, long rows, int C, char*& ws, cudaStream_t st) {
+// `t` (and `u`, where there is one) themselves, or their padded copies at *ws (which then moves on behind them).
+static xconv_status pad_channels(const void*& t, long rows, int C, char*& ws, cudaStream_t st, const void** u = nullptr, long rows_u = 0) {
   if (C % 8 == 0) return XCONV_OK;
-  const long pieces = rows * (pad8(C) / 8);
-  const cudaError_t e = launch_pdl(pad_channels_kernel<unsigned short>, dim3((unsigned)cdiv(pieces, 256)), dim3(256), 0, st,
-                                   static_cast<const unsigned short*>(t), reinterpret_cast<unsigned short*>(ws), pieces, C, pad8(C) / 8);
-  ++g_launches;
-  if (e != cudaSuccess) { g_last_cuda_error = (int)e; return XCONV_ERR_CUDA; }
+  const int per_row = pad8(C) / 8;
+  PadJob one{static_cast<const unsigned short*>(t), reinterpret_cast<unsigned short*>(ws), rows * per_row}, two{nullptr, nullptr, 0};
   t = ws;
   ws += padded_bytes(rows, C);
+  if (u) {
+    two = PadJob{static_cast<const unsigned short*>(*u), reinterpret_cast<unsigned short*>(ws), rows_u * per_row};
+    *u = ws;
+    ws += padded_bytes(rows_u, C);
+  }
+  const cudaError_t e = launch_pdl(pad_channels_kernel, dim3((unsigned)cdiv(one.pieces + two.pieces, 256)), dim3(256), 0, st, one, two, C, per_row);
+  ++g_launches;
+  if (e != cudaSuccess) { g_last_cuda_error = (int)e; return XCONV_ERR_CUDA; }
   return XCONV_OK;
 }
 
@@ -448,12 +457,17 @@ static size_t probes_bytes(const xconv_desc* d) {
 static const unsigned REDUCE_PDL_BLOCKS = 6000;
 static xconv_status run_reduce(const float* part, float* out, long count, int splits, float alpha, const float* chan_scale,
                                int period, cudaStream_t st) {
-  const dim3 grid((unsigned)cdiv(count, RP_OUT)), block(RP_OUT * RP_LANES);
+  // Many splits of few outputs: four times the threads to an output, and twice the loads in flight (us a launch, 441 to 4096 outputs of 128 to 296 splits:
+  // 5.9 -> 4.0; with the loads alone few splits of many outputs lose, 65536 of 7 3.8 -> 5.1).
+  const bool few = splits >= 64 && count <= 16384;
+  const dim3 grid((unsigned)cdiv(count, few ? 8 : 32)), block(256);
   cudaError_t e;
-  if (grid.x <= REDUCE_PDL_BLOCKS) {
-    e = launch_pdl(reduce_partials<true>, grid, block, 0, st, part, out, count, splits, alpha, chan_scale, period);
+  if (few) {
+    e = launch_pdl(reduce_partials<true, 32>, grid, block, 0, st, part, out, count, splits, alpha, chan_scale, period);
+  } else if (grid.x <= REDUCE_PDL_BLOCKS) {
+    e = launch_pdl(reduce_partials<true, 8>, grid, block, 0, st, part, out, count, splits, alpha, chan_scale, period);
   } else {
-    reduce_partials<false><<<grid, block, 0, st>>>(part, out, count, splits, alpha, chan_scale, period);
+    reduce_partials<false, 8><<<grid, block, 0, st>>>(part, out, count, splits, alpha, chan_scale, period);
     e = cudaGetLastError();
   }
   ++g_launches;
@@ -467,17 +481,20 @@ static xconv_status run_sketch_simt(const xconv_desc* d, const SketchPlan& p, co
   const long K = (long)d->H * d->W * d->Cin;
   float* part = reinterpret_cast<float*>(ws + p.part_off);
   dim3 grid((unsigned)cdiv(d->B, 64), (unsigned)cdiv(d->r, 64), (unsigned)p.splits);
+  // (Started under the kernel before only if it is over at once: grids of a whole wave are dealt unevenly to SMs that that one still uses, 512 x 32 rows, 1176
+  // terms 10 -> 12.8 us, and the copies go through what L1 it leaves, 16 x 53 rows, 10816 terms in a training step 83 -> 86; 8 x 8 rows, 16384 terms 10.3 -> 8.0.)
+  const bool small = (long)grid.x * grid.y * grid.z <= 148 && (d->r + d->B) * K <= 1L << 19;
   if (std::is_same<T, float>::value && K % 4 == 0 && p.k_per_split % GT_KS == 0) {
     const size_t smem = (size_t)GT_STAGES * 128 * GT_LD * sizeof(float);
     cudaError_t ea = cudaFuncSetAttribute(gemm_tn_simt_async, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (ea != cudaSuccess) { g_last_cuda_error = (int)ea; return XCONV_ERR_CUDA; }
-    ea = launch_pdl(gemm_tn_simt_async, grid, dim3(256), smem, st, reinterpret_cast<const float*>(Z), reinterpret_cast<const float*>(X), part,
+    ea = launch_if_pdl(small, gemm_tn_simt_async, grid, dim3(256), smem, st, reinterpret_cast<const float*>(Z), reinterpret_cast<const float*>(X), part,
                     d->r, d->B, K, p.k_per_split);
     if (ea != cudaSuccess) { g_last_cuda_error = (int)ea; return XCONV_ERR_CUDA; }
   } else {
-    const cudaError_t ea = launch_pdl(gemm_tn_simt<T>, grid, dim3(256), 0, st, static_cast<const T*>(Z), static_cast<const T*>(X), part, d->r, d->B, K,
-                                      p.k_per_split, (K % 4 == 0) ? 1 : 0);
-    if (ea != cudaSuccess) { g_last_cuda_error = (int)ea; return XCONV_ERR_CUDA; }
+    // (an ordinary launch: it loads through L1, of which SMs split for the kernel before have little; 16 x 8 rows, 1440 terms behind a convolution 8 us, 17 started under it)
+    gemm_tn_simt<T><<<grid, 256, 0, st>>>(static_cast<const T*>(Z), static_cast<const T*>(X), part, d->r, d->B, K,
+                                          p.k_per_split, (K % 4 == 0) ? 1 : 0);
   }
   xconv_status s = check_launch();
   if (s != XCONV_OK) return s;
@@ -538,8 +555,11 @@ static xconv_status run_backprobe_simt(const xconv_desc* d, const float* S, cons
     if (best < 0 || cost < best) { best = cost; threads = t; }
   }
   dim3 g1((unsigned)cdiv(cdiv(Q, 4), threads), (unsigned)cdiv(d->r, 16));
-  const cudaError_t e = launch_pdl(backprobe_simt<T, TL>, g1, dim3(threads), 0, st, S, static_cast<const T*>(dY), static_cast<TL*>(Lv), d->r, d->B, Q,
-                                   (Q % 4 == 0) ? 1 : 0);
+  // Small ones start under the kernel before.  Large ones would find their SMs split for that one, with little of the L1 that their loads are in flight
+  // through (us with the contraction behind, ordinary -> dependent: 8 rows of 8 terms, 57600 positions 20.4 -> 19.2, but 16 rows of 22, 251008 positions 84 -> 105).
+  const bool small = (long)g1.x * g1.y <= 296 && (d->r + d->B) * Q <= 1L << 20;
+  const cudaError_t e = launch_if_pdl(small, backprobe_simt<T, TL>, g1, dim3(threads), 0, st, S, static_cast<const T*>(dY), static_cast<TL*>(Lv), d->r, d->B, Q,
+                                      (Q % 4 == 0) ? 1 : 0);
   if (e != cudaSuccess) { g_last_cuda_error = (int)e; return XCONV_ERR_CUDA; }
   return check_launch();
 }
@@ -663,8 +683,7 @@ static xconv_status run_conv(const xconv_desc* d, bool dgrad, const void* in, co
   if (plan_conv(d, dgrad, &e, &t)) {
     char* copies = ws + WS_HEADER;
     if (!dgrad) {
-      xconv_status s = pad_channels(in, (long)d->B * depth(d) * d->H * d->W, d->Cin, copies, st);
-      if (s == XCONV_OK) s = pad_channels(Wt, (long)d->Cout * kdepth(d) * d->KH * d->KW, d->Cin, copies, st);
+      const xconv_status s = pad_channels(in, (long)d->B * depth(d) * d->H * d->W, d->Cin, copies, st, &Wt, (long)d->Cout * kdepth(d) * d->KH * d->KW);
       if (s != XCONV_OK) return s;
     }
     return tc_run_conv(&e, t, dgrad, in, Wt, out, ws, st);
@@ -757,12 +776,21 @@ static xconv_status run_wgrad(const xconv_desc* d, const float* S, const void* d
       const xconv_desc f = flat(&sw.d1);
       s = run_backprobe_split(&f, sw.p1.g, S, 1, d->B, Z, w + sw.x_off, w, w + sw.sb_off, st);
     } else {
+      // the transposed sketch, in the form that its reader takes
+      const dim3 grid((unsigned)cdiv(d->B, 32), (unsigned)cdiv(d->r, 32)), block(32, 8);
       float* St = reinterpret_cast<float*>(w + sw.st_off);
-      const long n = (long)d->r * d->B;
-      transpose_f32<<<(unsigned)cdiv(n, 256), 256, 0, st>>>(S, St, d->r, d->B);
-      s = check_launch();
-      if (s != XCONV_OK) return s;
-      s = run_backprobe(&sw.d1, sw.p1, St, Z, w + sw.x_off, w + sw.sb_off, w, st, seed);
+      cudaError_t e;
+      if (!sw.p1.tc_bp) e = launch_pdl(transpose_sketch<float>, grid, block, 0, st, S, St, (int)d->r, (int)d->B);
+      else if (d->dtype == XCONV_F16) e = launch_pdl(transpose_sketch<f16>, grid, block, 0, st, S, reinterpret_cast<f16*>(w + sw.sb_off), (int)d->r, (int)d->B);
+      else e = launch_pdl(transpose_sketch<bf16>, grid, block, 0, st, S, reinterpret_cast<bf16*>(w + sw.sb_off), (int)d->r, (int)d->B);
+      ++g_launches;
+      if (e != cudaSuccess) { g_last_cuda_error = (int)e; return XCONV_ERR_CUDA; }
+      if (sw.p1.tc_bp) {
+        const xconv_desc f = flat(&sw.d1);
+        s = tc_run_backprobe(&f, sw.p1.tb, w + sw.sb_off, Z, w + sw.x_off, w, st, seed);
+      } else {
+        s = run_backprobe(&sw.d1, sw.p1, St, Z, w + sw.x_off, w + sw.sb_off, w, st, seed);
+      }
     }
     if (s != XCONV_OK) return s;
     return run_contract(&sw.d2, sw.p2, dY, w + sw.x_off, dW, alpha, w + sw.part_off, w, st);

@@ -19,13 +19,16 @@ enum : unsigned int { WS_OK = 0u };
 
 // Programmatic dependent launch: a kernel launched with launch_pdl may start while the kernel before
 // it in the stream is still draining; it must call pdl_wait() before it reads or overwrites anything
-// that kernel touches.  pdl_trigger() lets the kernel after this one start its own preamble early.
+// that kernel touches.  pdl_trigger() lets the kernel after this one start its own preamble early.  Where a kernel is short and small the go-ahead is
+// given behind its loads: given at its start, the kernels behind it pile up on the SMs, and one of them that loads through L1 starts on an SM that is still
+// split for the shared memory of a kernel before (training step of 8 images of 32 x 32, float, 30 -> 28 us; sketch of 39 x 220 rows, 1152 terms in its step 45 -> 35).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// (`dependent` false: an ordinary launch, behind the end of the kernel before.)
 template <typename... KArgs, typename... Args>
-static inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                                     Args&&... args) {
+static inline cudaError_t launch_if_pdl(bool dependent, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                        Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -35,8 +38,42 @@ static inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 b
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = dependent ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+static inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+  return launch_if_pdl(true, kernel, grid, block, smem, st, static_cast<Args&&>(args)...);
+}
+
+// The sum of every LANES-th of `splits` partial sums from the g-th on, four columns (or one) of each, in order.  DEEP loads are in flight at once: these kernels
+// are chains of waits for L2.  By ld.global.cg: the kernel before wrote them.
+template <int LANES, int DEEP = 8>
+__device__ __forceinline__ float4 sum_splits4(const float* src, size_t stride, int g, int splits) {
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int k = g; k < splits; k += DEEP * LANES) {
+    float4 v[DEEP];
+#pragma unroll
+    for (int i = 0; i < DEEP; ++i)
+      v[i] = k + i * LANES < splits ? __ldcg(reinterpret_cast<const float4*>(src + (size_t)(k + i * LANES) * stride)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < DEEP; ++i)
+      if (k + i * LANES < splits) { s.x += v[i].x; s.y += v[i].y; s.z += v[i].z; s.w += v[i].w; }
+  }
+  return s;
+}
+template <int LANES, int DEEP>
+__device__ __forceinline__ float sum_splits(const float* src, size_t stride, int g, int splits) {
+  float s = 0.f;
+  for (int k = g; k < splits; k += DEEP * LANES) {
+    float v[DEEP];
+#pragma unroll
+    for (int i = 0; i < DEEP; ++i) v[i] = k + i * LANES < splits ? __ldcg(src + (size_t)(k + i * LANES) * stride) : 0.f;
+#pragma unroll
+    for (int i = 0; i < DEEP; ++i)
+      if (k + i * LANES < splits) s += v[i];
+  }
+  return s;
 }
 
 __device__ __forceinline__ float to_f(float v) { return v; }

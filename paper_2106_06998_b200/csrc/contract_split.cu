@@ -399,24 +399,17 @@ __global__ void __launch_bounds__(256) reduce_split_partials(const ContractSplit
                                                              float alpha, const float* __restrict__ chan_scale) {
   constexpr int GROUPS = 256 / LANES;
   __shared__ float4 acc[LANES][GROUPS];
-  pdl_trigger();
-  pdl_wait();
   const int o = threadIdx.x % GROUPS, g = threadIdx.x / GROUPS;
   const uint32_t idx = blockIdx.x * GROUPS + o, q4 = (uint32_t)p.cols >> 2;
   const uint32_t row = idx % TILE_M, q = idx / TILE_M % q4, ug = idx / TILE_M / q4;
   const SplitUnit u = split_unit(p, ug);
   const SplitEntry e = split_entry(p, u, (int)row, (int)q * 4);
   const bool live = idx < groups && split_live(p, e);
-  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (live) {
-    const size_t tile = (size_t)p.cols * TILE_M;
-    const float* src = p.part + (size_t)ug * p.splits * tile + ((size_t)q * TILE_M + row) * 4;
-#pragma unroll 4
-    for (uint32_t k = g; k < p.splits; k += LANES) {
-      const float4 v = *reinterpret_cast<const float4*>(src + (size_t)k * tile);
-      s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
-    }
-  }
+  const size_t tile = (size_t)p.cols * TILE_M;
+  const float* src = p.part + (size_t)ug * p.splits * tile + ((size_t)q * TILE_M + row) * 4;
+  pdl_wait();                                        // (what is above runs under the kernel before)
+  float4 s = live ? sum_splits4<LANES>(src, tile, g, (int)p.splits) : make_float4(0.f, 0.f, 0.f, 0.f);
+  pdl_trigger();
   if (LANES > 1) {
     acc[g][o] = s;
     __syncthreads();

@@ -329,12 +329,10 @@ contract_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
 // threads share a group and take the splits in turn; their sums are added in lane order.  `cout_out`, `cin_out`: channels
 // of dW (the padded channels behind them have no place in it).
 template <int LANES>
-__global__ void __launch_bounds__(256) reduce_halo_partials(const HaloParams p, float* __restrict__ out, uint32_t groups,
-                                                            int cout_out, int cin_out, float alpha, const float* __restrict__ chan_scale) {
+__global__ void __launch_bounds__(256) reduce_halo_partials(const HaloParams p, float* out, uint32_t groups, int cout_out, int cin_out, float alpha,
+                                                            const float* chan_scale) {
   constexpr int GROUPS = 256 / LANES;
   __shared__ float4 acc[LANES][GROUPS];
-  pdl_trigger();
-  pdl_wait();
   const int o = threadIdx.x % GROUPS, g = threadIdx.x / GROUPS;
   const uint32_t idx = blockIdx.x * GROUPS + o;
   const uint32_t row = idx % TILE_M, q4 = (uint32_t)p.cols >> 2;
@@ -355,16 +353,11 @@ __global__ void __launch_bounds__(256) reduce_halo_partials(const HaloParams p, 
   const int nb = u.ng * p.ng_per + grp % p.ng_per, dz = u.dzg * p.dz_per + grp / p.ng_per;
   const int n = nb * p.cwb + (c - grp * per) % p.cwb;
   const bool live = idx < groups && dy >= 0 && j < p.KS && m < cout_out && n < cin_out;
-  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (live) {
-    const size_t tile = (size_t)p.mt * p.cols * TILE_M;
-    const float* src = p.part + (size_t)ug * p.splits * tile + ((size_t)mt * q4 * TILE_M + (size_t)q * TILE_M + row) * 4;
-#pragma unroll 4
-    for (uint32_t k = g; k < p.splits; k += LANES) {
-      const float4 v = *reinterpret_cast<const float4*>(src + (size_t)k * tile);
-      s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
-    }
-  }
+  const size_t tile = (size_t)p.mt * p.cols * TILE_M;
+  const float* src = p.part + (size_t)ug * p.splits * tile + ((size_t)mt * q4 * TILE_M + (size_t)q * TILE_M + row) * 4;
+  pdl_wait();                                        // (what is above runs under the kernel before)
+  float4 s = live ? sum_splits4<LANES>(src, tile, g, (int)p.splits) : make_float4(0.f, 0.f, 0.f, 0.f);
+  pdl_trigger();
   if (LANES > 1) {
     acc[g][o] = s;
     __syncthreads();

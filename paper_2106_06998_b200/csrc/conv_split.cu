@@ -64,8 +64,8 @@ __device__ __forceinline__ float cs_weight(const ConvSplitParams& p, int co, int
 
 // The weights' tile images, a thread per four channels in of one row.  T here counts the offsets of all depths.
 __global__ void __launch_bounds__(256) conv_split_weights(const ConvSplitParams p, uint8_t* __restrict__ img, int tiles_n) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int quads = p.cw >> 2, T2 = p.T / p.KD;
   const uint32_t total = (uint32_t)(tiles_n * p.nb * p.T) * (uint32_t)(p.n * quads);
   for (uint32_t i = blockIdx.x * 256 + threadIdx.x; i < total; i += gridDim.x * 256) {

@@ -66,8 +66,8 @@ __device__ __forceinline__ void write_image(const GemmSplitParams& p, uint8_t* i
 }
 
 __global__ void __launch_bounds__(256) split_sketch_images(const GemmSplitParams p, uint8_t* __restrict__ img) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const long total = (long)p.tiles_n * p.n * p.kblocks * 8;
   for (long i = (long)blockIdx.x * 256 + threadIdx.x; i < total; i += (long)gridDim.x * 256) {
     const long j = i / (p.kblocks * 8), k = i - j * (p.kblocks * 8);
@@ -79,8 +79,8 @@ __global__ void __launch_bounds__(256) split_sketch_images(const GemmSplitParams
 // Its parts then hold it down to 2^-61 of that value, all 24 bits of entries above 2^-36 of it.  A row with smaller entries than that (they
 // count where the large ones meet zeros of Y) is marked by the sign of its scale: its sums are taken by multiply-adds.  A warp per row.
 __global__ void __launch_bounds__(256) split_sketch_images_f16(const GemmSplitParams p, uint8_t* __restrict__ img, float* __restrict__ scale) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   for (long j = (long)blockIdx.x * 8 + (threadIdx.x >> 5); j < (long)p.tiles_n * p.n; j += (long)gridDim.x * 8) {
     float top = 0.f, low = INFINITY;

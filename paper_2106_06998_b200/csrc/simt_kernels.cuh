@@ -23,7 +23,6 @@ __global__ void __launch_bounds__(256) gemm_tn_simt(const T* A, const T* Bm, flo
   constexpr int KS = 32;
   __shared__ __align__(16) float As[KS][68];
   __shared__ __align__(16) float Bs[KS][68];
-  pdl_trigger();
   pdl_wait();
   const int tid = threadIdx.x;
   const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
@@ -101,7 +100,6 @@ __device__ __forceinline__ void cp_async16_f(float* dst, const float* src, bool 
 }
 static __global__ void __launch_bounds__(256) gemm_tn_simt_async(const float* A, const float* Bm, float* part, int M, int N, long K, long k_per_split) {
   extern __shared__ __align__(16) float gt_tiles[];       // [stage][A rows 0..63 | B rows 0..63][GT_LD]
-  pdl_trigger();
   pdl_wait();
   const int tid = threadIdx.x;
   const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
@@ -158,6 +156,7 @@ static __global__ void __launch_bounds__(256) gemm_tn_simt_async(const float* A,
         }
     }
   }
+  pdl_trigger();
   float* out = part + (long)blockIdx.z * M * N;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -171,33 +170,33 @@ static __global__ void __launch_bounds__(256) gemm_tn_simt_async(const float* A,
   }
 }
 
-// out[i] = scale(i) * sum_s part[s][i].  Eight threads share an output and take the splits in turn (one
-// thread per output would walk a chain of `splits` dependent loads); their eight sums are added in a
+// out[i] = scale(i) * sum_s part[s][i].  LANES threads share an output and take the splits in turn; their sums are added in a
 // fixed order, so results are reproducible.  scale(i) = chan_scale[i % period] if chan_scale else alpha.
-// Launch with 256 threads: 32 outputs per block.
-constexpr int RP_OUT = 32, RP_LANES = 8;
-template <bool PDL>
-static __global__ void __launch_bounds__(RP_OUT * RP_LANES)
-reduce_partials(const float* __restrict__ part, float* __restrict__ out, long count, int splits, float alpha,
-                const float* __restrict__ chan_scale, int period) {
-  __shared__ float acc[RP_LANES][RP_OUT];
-  if (PDL) {
-    pdl_trigger();
-    pdl_wait();
-  }
-  const int o = threadIdx.x % RP_OUT, g = threadIdx.x / RP_OUT;
-  const long i = (long)blockIdx.x * RP_OUT + o;
+// Launch with 256 threads: 256 / LANES outputs per block.
+template <bool PDL, int LANES>
+static __global__ void __launch_bounds__(256)
+reduce_partials(const float* part, float* out, long count, int splits, float alpha, const float* chan_scale, int period) {
+  constexpr int OUT = 256 / LANES;
+  __shared__ float acc[LANES][OUT];
+  if (PDL) pdl_wait();
+  const int o = threadIdx.x % OUT, g = threadIdx.x / OUT;
+  const long i = (long)blockIdx.x * OUT + o;
   float s = 0.f;
   if (i < count) {
+    if (LANES == 32) {
+      s = sum_splits<LANES, 8>(part + i, (size_t)count, g, splits);
+    } else {
 #pragma unroll 4
-    for (int k = g; k < splits; k += RP_LANES) s += part[(long)k * count + i];
+      for (int k = g; k < splits; k += LANES) s += __ldcg(part + (size_t)k * count + i);
+    }
   }
+  if (PDL) pdl_trigger();
   acc[g][o] = s;
   __syncthreads();
   if (g != 0 || i >= count) return;
   float t = acc[0][o];
 #pragma unroll
-  for (int l = 1; l < RP_LANES; ++l) t += acc[l][o];
+  for (int l = 1; l < LANES; ++l) t += acc[l][o];
   out[i] = t * (chan_scale ? chan_scale[i % period] : alpha);
 }
 
@@ -209,7 +208,6 @@ reduce_partials(const float* __restrict__ part, float* __restrict__ out, long co
 template <typename T, typename TL>
 __global__ void __launch_bounds__(256) backprobe_simt(const float* S, const T* dY, TL* L, int r, int B, long Q, int vec) {
   __shared__ __align__(16) float Ss[128][16];
-  pdl_trigger();
   pdl_wait();
   const int tid = threadIdx.x;
   const long q = ((long)blockIdx.x * blockDim.x + tid) * 4;
@@ -253,6 +251,7 @@ __global__ void __launch_bounds__(256) backprobe_simt(const float* S, const T* d
     }
     __syncthreads();
   }
+  pdl_trigger();                 // (not earlier: the next kernel's shared memory is taken from the L1 that the loads above are in flight through)
   if (q < Q) {
 #pragma unroll
     for (int j = 0; j < 16; ++j)
@@ -660,21 +659,28 @@ __global__ void __launch_bounds__(256) rebuild_indep_simt(const float* __restric
   }
 }
 
-// out[b][j] = in[j][b] for a small [rows][cols] float matrix (the sketch, transposed).
-static __global__ void transpose_f32(const float* __restrict__ in, float* __restrict__ out, int rows, int cols) {
-  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long)rows * cols) return;
-  const int j = (int)(i / cols), b = (int)(i % cols);
-  out[(long)b * rows + j] = in[i];
+// out[b][j] = in[j][b] for a small [rows][cols] float matrix (the sketch), as float or in the storage type of the tensor-core operand.  A block turns 32 x 32
+// entries around in shared memory.  Launch with (32, 8) threads.
+template <typename T>
+static __global__ void __launch_bounds__(256) transpose_sketch(const float* in, T* out, int rows, int cols) {
+  __shared__ float tile[32][33];
+  pdl_wait();
+  pdl_trigger();
+  const int j0 = blockIdx.y * 32, b0 = blockIdx.x * 32;
+  for (int i = threadIdx.y; i < 32; i += 8)
+    if (j0 + i < rows && b0 + (int)threadIdx.x < cols) tile[i][threadIdx.x] = __ldcg(in + (long)(j0 + i) * cols + b0 + threadIdx.x);
+  __syncthreads();
+  for (int i = threadIdx.y; i < 32; i += 8)
+    if (b0 + i < cols && j0 + (int)threadIdx.x < rows) out[(long)(b0 + i) * rows + j0 + threadIdx.x] = from_f<T>(tile[threadIdx.x][i]);
 }
 
 // float -> 16-bit storage type copy (the sketch as tensor-core operand).
 template <typename T>
-static __global__ void cast_f32_to_16(const float* __restrict__ in, T* __restrict__ out, long n) {
-  pdl_trigger();
+static __global__ void cast_f32_to_16(const float* in, T* out, long n) {
   pdl_wait();
+  pdl_trigger();
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) out[i] = from_f<T>(in[i]);
+  if (i < n) out[i] = from_f<T>(__ldcg(in + i));
 }
 
 }  // namespace xconv

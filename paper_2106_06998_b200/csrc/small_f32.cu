@@ -39,7 +39,6 @@ __global__ void __launch_bounds__(128) small_conv_kernel(const float* in, const 
   __shared__ int sx[G::NS], sy[G::NS], sz[G::NS];
   __shared__ long sb[G::NS];                                    // the strip's plane, or -1
   const int tid = threadIdx.x, per_row = (W + 3) / 4;
-  pdl_trigger();
   if (tid < G::NS) {
     const long s = (long)blockIdx.x * G::NS + tid, row = s / per_row, plane = row / H;
     sx[tid] = (int)(s - row * per_row) * 4;
@@ -129,6 +128,7 @@ __global__ void __launch_bounds__(128) small_conv_kernel(const float* in, const 
     }
     __syncthreads();             // all reads of this buffer are done before the copies of the step after next land in it
   }
+  pdl_trigger();
   int p0 = 0, p1 = 4;                                           // the pixels that this thread writes
   if (KG == 4) {
     float* red = small_smem;                                    // [channels in][pixel, channel][thread]
@@ -217,7 +217,6 @@ __global__ void __launch_bounds__(256) small_contract_kernel(const float* L, con
   const int nblocks = (Cin + 15) / 16, kz = blockIdx.x / nblocks, n0 = (int)(blockIdx.x % nblocks) * 16, m0 = blockIdx.y * 16;
   const int chunks = (W + SC_X - 1) / SC_X;
   const long ib = (long)blockIdx.z * items_per_split, ie = min(items, ib + items_per_split);
-  pdl_trigger();
   // coordinates of the item whose tiles are fetched next
   int xc = (int)(ib % chunks), y = (int)((ib / chunks) % H);
   long jz = ib / ((long)chunks * H);                            // plane: probe * D + z
@@ -275,6 +274,7 @@ __global__ void __launch_bounds__(256) small_contract_kernel(const float* L, con
     }
     __syncthreads();             // all reads of this buffer are done before the copies of the item after next land in it
   }
+  pdl_trigger();
   if (m0 + m >= Cout || n0 + n >= Cin) return;
   float* o = part + ((long)blockIdx.z * Cout * TALL + (long)(m0 + m) * TALL + kz * T) * Cin + n0 + n;
 #pragma unroll

@@ -1013,7 +1013,6 @@ __global__ void __launch_bounds__(RS_LANES * RS_GROUPS)
 reduce_sketch_partials(const float* __restrict__ part, float* __restrict__ S, long groups, long split_stride,
                        int splits, int tiles_n, int m_sub, int tile_n, int rows, int cols, int B, int swapped) {
   __shared__ float4 acc[RS_LANES][RS_GROUPS];
-  pdl_trigger();
   pdl_wait();
   const int o = threadIdx.x % RS_GROUPS, g = threadIdx.x / RS_GROUPS;
   const long idx = (long)blockIdx.x * RS_GROUPS + o;   // group of four columns, in stored order
@@ -1025,6 +1024,7 @@ reduce_sketch_partials(const float* __restrict__ part, float* __restrict__ S, lo
       s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
     }
   }
+  pdl_trigger();
   acc[g][o] = s;
   __syncthreads();
   if (g != 0 || idx >= groups) return;
@@ -1066,7 +1066,6 @@ __global__ void __launch_bounds__(256) reduce_contract_partials(const float* __r
                                                                 const float* __restrict__ chan_scale) {
   constexpr int GROUPS = 256 / LANES;
   __shared__ float4 acc[LANES][GROUPS];
-  pdl_trigger();
   pdl_wait();
   const int o = threadIdx.x % GROUPS, g = threadIdx.x / GROUPS;
   const long idx = (long)blockIdx.x * GROUPS + o;
@@ -1078,6 +1077,7 @@ __global__ void __launch_bounds__(256) reduce_contract_partials(const float* __r
       s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
     }
   }
+  pdl_trigger();
   if (LANES > 1) {
     acc[g][o] = s;
     __syncthreads();
