@@ -80,37 +80,66 @@ __host__ __device__ __forceinline__ HaloUnit halo_unit(const HaloParams& p, uint
 }
 
 // The MMAs of `rows` image rows of a patch.  FORM 1 and 2: as many row tiles and one piece; 12 and 13: one row tile, two or three
-// pieces; 0: any number of both.  (With the pieces known to the compiler a k-step is straight-line code; in a loop that looks them up it
-// took 135 clocks an MMA of 56: volumes of 48^3, 32 channels 49 -> 34 us.)
-template <int FORM>
+// pieces; 0: any number of both.  KX: k-steps of a row, 0 for any number.  The warp issues an instruction per some six clocks, so a loop that looks the
+// pieces up took 135 clocks an MMA of 56 (volumes of 48^3, 32 channels 49 -> 34 us), and a loop over a row's k-steps 143 an MMA of 62 where there is one (images of 16 columns), 96
+// for two, 69 for three.  us a call with its reduction, that loop -> rows unrolled: 64 -> 16 channels, 12 planes of 13 x 13, 290 probes 112 -> 73; 48 -> 64, 256 images of 86 x 86 36.6 -> 27.8;
+// volumes of 48^3, 32 channels 44 -> 36; 32 -> 32, 64 probes of 256 x 256 106 -> 90.  (Asking for the next patch before this one's commit gains 1 % where the MMAs bound it
+// and loses 5 % where the copies do.)
+template <int FORM, int KX>
 __device__ __forceinline__ void halo_mmas(const HaloParams& p, int rows, uint32_t tmem, uint32_t a0, uint32_t b0, uint32_t& acc,
                                           uint32_t id0) {
-  const int kx = p.pw >> 4;
+  const int kx = KX > 0 ? KX : p.pw >> 4;
   const uint32_t a_step = p.a_step16, b_step = p.b_step16;
-  for (int y = 0; y < rows; ++y) {
-    uint32_t a = a0, b = b0;
-    for (int x = 0; x < kx; ++x) {
-      if (FORM > 10) {
+  auto kstep = [&](uint32_t a, uint32_t b) {
+    if (FORM > 10) {
 #pragma unroll
-        for (int i = 0; i < FORM - 10; ++i)
-          umma_warp(tmem + p.piece_col[i], a, p.a_hi, b + p.piece_off[i], p.b_hi, p.piece_idesc[i], acc);
-      } else if (FORM > 0) {
-        umma_warp(tmem, a, p.a_hi, b, p.b_hi, id0, acc);
-        if (FORM == 2) umma_warp(tmem + (uint32_t)p.cols, a + p.a_mt16, p.a_hi, b, p.b_hi, id0, acc);
-      } else {
-        for (int i = 0; i < p.pieces; ++i) {
-          const uint32_t bb = b + p.piece_off[i], d = tmem + p.piece_col[i], id = p.piece_idesc[i];
-          umma_warp(d, a, p.a_hi, bb, p.b_hi, id, acc);
-          if (p.mt > 1) umma_warp(d + (uint32_t)p.cols, a + p.a_mt16, p.a_hi, bb, p.b_hi, id, acc);
-          if (p.mt > 2) umma_warp(d + 2u * (uint32_t)p.cols, a + 2u * p.a_mt16, p.a_hi, bb, p.b_hi, id, acc);
-        }
+      for (int i = 0; i < FORM - 10; ++i)
+        umma_warp(tmem + p.piece_col[i], a, p.a_hi, b + p.piece_off[i], p.b_hi, p.piece_idesc[i], acc);
+    } else if (FORM > 0) {
+      umma_warp(tmem, a, p.a_hi, b, p.b_hi, id0, acc);
+      if (FORM == 2) umma_warp(tmem + (uint32_t)p.cols, a + p.a_mt16, p.a_hi, b, p.b_hi, id0, acc);
+    } else {
+      for (int i = 0; i < p.pieces; ++i) {
+        const uint32_t bb = b + p.piece_off[i], d = tmem + p.piece_col[i], id = p.piece_idesc[i];
+        umma_warp(d, a, p.a_hi, bb, p.b_hi, id, acc);
+        if (p.mt > 1) umma_warp(d + (uint32_t)p.cols, a + p.a_mt16, p.a_hi, bb, p.b_hi, id, acc);
+        if (p.mt > 2) umma_warp(d + 2u * (uint32_t)p.cols, a + 2u * p.a_mt16, p.a_hi, bb, p.b_hi, id, acc);
       }
-      acc = 1u;
-      a += a_step;
-      b += b_step;
     }
-    a0 += p.a_row16;
-    b0 += p.b_row16;
+    acc = 1u;
+  };
+  if (KX > 0) {
+    constexpr int ROWS = KX == 1 ? 4 : KX == 2 ? 2 : 1;            // unrolled together
+    int y = 0;
+#pragma unroll 1
+    for (; y + ROWS <= rows; y += ROWS) {
+#pragma unroll
+      for (int r = 0; r < ROWS; ++r) {
+#pragma unroll
+        for (int x = 0; x < KX; ++x) kstep(a0 + (uint32_t)x * a_step, b0 + (uint32_t)x * b_step);
+        a0 += p.a_row16;
+        b0 += p.b_row16;
+      }
+    }
+    if (ROWS > 1)
+#pragma unroll 1
+      for (; y < rows; ++y) {
+#pragma unroll
+        for (int x = 0; x < KX; ++x) kstep(a0 + (uint32_t)x * a_step, b0 + (uint32_t)x * b_step);
+        a0 += p.a_row16;
+        b0 += p.b_row16;
+      }
+  } else {
+    for (int y = 0; y < rows; ++y) {
+      uint32_t a = a0, b = b0;
+      for (int x = 0; x < kx; ++x) {
+        kstep(a, b);
+        a += a_step;
+        b += b_step;
+      }
+      a0 += p.a_row16;
+      b0 += p.b_row16;
+    }
   }
 }
 
@@ -119,7 +148,7 @@ struct HaloBars { uint64_t *full, *empty, *acc_full, *acc_empty; };
 // The issuing warp of a drained contraction: two accumulator sets in turn, each for chunk_patches patches or for chunk_rows rows
 // of one (a loop per chunk and nothing to decide per row: the warp issues an instruction per some six clocks).  `a_add`, `b_add`,
 // `id0`: what the unit moves the two tiles by, and the instruction descriptor for its pixel shifts (FORM > 0).
-template <int FORM>
+template <int FORM, int KX>
 __device__ __forceinline__ void halo_issue_drained(const HaloParams& p, const HaloBars& bar, uint32_t n, uint32_t tmem_base,
                                                    uint32_t s0, uint32_t a_add, uint32_t b_add, uint32_t id0) {
   const uint32_t stage16 = p.stage_bytes >> 4, set_cols = (uint32_t)(p.mt * p.cols);
@@ -136,7 +165,7 @@ __device__ __forceinline__ void halo_issue_drained(const HaloParams& p, const Ha
         acc = 0;
         left = p.chunk_patches;
       }
-      halo_mmas<FORM>(p, min(p.chunk_rows, p.ph - y), tmem, a, b, acc, id0);
+      halo_mmas<FORM, KX>(p, min(p.chunk_rows, p.ph - y), tmem, a, b, acc, id0);
       if (--left == 0 || (i + 1 == n && y + p.chunk_rows >= p.ph)) {
         umma_commit_warp(&bar.acc_full[buf]);
         left = 0;
@@ -151,6 +180,22 @@ __device__ __forceinline__ void halo_issue_drained(const HaloParams& p, const Ha
     st += stage16;
     if (++s == (uint32_t)p.stages) { s = 0; par ^= 1u; st = s0; }
   }
+}
+
+// ... of an undrained one: a single chain.
+template <int FORM, int KX>
+__device__ __forceinline__ void halo_issue_chain(const HaloParams& p, const HaloBars& bar, uint32_t n, uint32_t tmem_base, uint32_t b0, uint32_t a_bytes16) {
+  const uint32_t stage16 = p.stage_bytes >> 4;
+  uint32_t s = 0, par = 0, acc = 0, st = b0;
+  for (uint32_t i = 0; i < n; ++i) {
+    if (!mbar_wait_warp(&bar.full[s], par, p.status, p.tag)) return;
+    tc_fence_after();
+    halo_mmas<FORM, KX>(p, p.ph, tmem_base, p.a_lo0 | st, p.b_lo0 | (st + a_bytes16), acc, p.piece_idesc[0]);
+    umma_commit_warp(&bar.empty[s]);
+    st += stage16;
+    if (++s == (uint32_t)p.stages) { s = 0; par ^= 1u; st = b0; }
+  }
+  umma_commit_warp(&bar.acc_full[0]);
 }
 
 template <bool F16, bool DRAIN>
@@ -219,7 +264,7 @@ contract_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (the whole warp)
-    const uint32_t b0 = ((base & 0x3FFFFu) >> 4), stage16 = p.stage_bytes >> 4, a_bytes16 = p.a_bytes >> 4;
+    const uint32_t b0 = ((base & 0x3FFFFu) >> 4), a_bytes16 = p.a_bytes >> 4;
     const bool one = p.mt == 1 && p.pieces == 1;
     if (DRAIN) {
       const HaloUnit u = halo_unit(p, ug);
@@ -228,29 +273,25 @@ contract_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
       const uint32_t b_add = a_bytes16 + (uint32_t)(u.jg * p.j_per) * (p.b_step16 >> 4);
       const int fewer = max(0, (u.jg + 1) * p.j_per - p.KS) * p.cwb;           // columns of shifts behind the last one
       const uint32_t id0 = p.piece_idesc[0] - ((uint32_t)(fewer >> 3) << 17);
-      if (one) halo_issue_drained<1>(p, bar, n, tmem_base, b0, a_add, b_add, id0);
-      else if (p.mt == 2 && p.pieces == 1) halo_issue_drained<2>(p, bar, n, tmem_base, b0, a_add, b_add, id0);
-      else if (p.mt == 1 && p.pieces == 2) halo_issue_drained<12>(p, bar, n, tmem_base, b0, a_add, b_add, id0);
-      else if (p.mt == 1 && p.pieces == 3) halo_issue_drained<13>(p, bar, n, tmem_base, b0, a_add, b_add, id0);
-      else halo_issue_drained<0>(p, bar, n, tmem_base, b0, a_add, b_add, id0);
+#define XC_ISSUE(FORM, KX) halo_issue_drained<FORM, KX>(p, bar, n, tmem_base, b0, a_add, b_add, id0)
+#define XC_ROWS(FORM) switch (p.pw >> 4) { case 1: XC_ISSUE(FORM, 1); break; case 2: XC_ISSUE(FORM, 2); break; case 3: XC_ISSUE(FORM, 3); break; \
+                                           case 4: XC_ISSUE(FORM, 4); break; default: XC_ISSUE(FORM, 0); }
+      if (one) XC_ROWS(1)
+      else if (p.mt == 2 && p.pieces == 1) XC_ROWS(2)
+      else if (p.mt == 1 && p.pieces == 2) XC_ROWS(12)
+      else if (p.mt == 1 && p.pieces == 3) XC_ROWS(13)
+      else XC_ISSUE(0, 0);
+#undef XC_ISSUE
     } else {
-      uint32_t s = 0, par = 0, acc = 0, st = b0;
-      bool ok = true;
-      for (uint32_t i = 0; i < n; ++i) {
-        ok = mbar_wait_warp(&full[s], par, p.status, p.tag);
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t a = p.a_lo0 | st, b = p.b_lo0 | (st + a_bytes16);
-        if (one) halo_mmas<1>(p, p.ph, tmem_base, a, b, acc, p.piece_idesc[0]);
-        else if (p.mt == 2 && p.pieces == 1) halo_mmas<2>(p, p.ph, tmem_base, a, b, acc, p.piece_idesc[0]);
-        else if (p.mt == 1 && p.pieces == 2) halo_mmas<12>(p, p.ph, tmem_base, a, b, acc, 0u);
-        else if (p.mt == 1 && p.pieces == 3) halo_mmas<13>(p, p.ph, tmem_base, a, b, acc, 0u);
-        else halo_mmas<0>(p, p.ph, tmem_base, a, b, acc, 0u);
-        umma_commit_warp(&empty[s]);
-        st += stage16;
-        if (++s == (uint32_t)p.stages) { s = 0; par ^= 1u; st = b0; }
-      }
-      if (ok) umma_commit_warp(&acc_full[0]);
+      const HaloBars bar{full, empty, acc_full, acc_empty};
+#define XC_ISSUE(FORM, KX) halo_issue_chain<FORM, KX>(p, bar, n, tmem_base, b0, a_bytes16)
+      if (one) XC_ROWS(1)
+      else if (p.mt == 2 && p.pieces == 1) XC_ROWS(2)
+      else if (p.mt == 1 && p.pieces == 2) XC_ROWS(12)
+      else if (p.mt == 1 && p.pieces == 3) XC_ROWS(13)
+      else XC_ISSUE(0, 0);
+#undef XC_ROWS
+#undef XC_ISSUE
     }
   } else {
     // ------------------------------------------------------------------ epilogue: partial sums in accumulator order
