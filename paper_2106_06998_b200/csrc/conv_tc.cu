@@ -503,9 +503,10 @@ bool tc_plan_conv(const xconv_desc* d, bool dgrad, TcConvPlan* p) {
         }
         p->a_sub_bytes = a_sub;
         p->slide = 0;
-        // ... and what its patches take as measured: an MMA 56 clocks at least, 250 from one patch to the next, and a ring of weight tiles hands on as many as
-        // it holds in the time of one copy
-        const long turns = std::max({(long)T * ksteps * m_sub * std::max(56, tile_n / 2) + 250, resident ? 0 : (long)nb * T * 2200 / p->w_slots, m_sub * copy, m_sub * epi});
+        // ... and what its patches take as measured: an MMA 56 clocks at least, 250 from one patch to the next, a ring of weight tiles hands on as many as
+        // it holds in the time of one copy, and a box of one plane comes in at 5 clocks a pixel however narrow its rows are (16 -> 16 channels, 3 x 3, 25 images of
+        // 154 x 154: walked 20.7 us where it was taken for slower than patches at 23.8, 64 of 95 x 157 36.8 -> 32.2)
+        const long turns = std::max({(long)T * ksteps * m_sub * std::max(56, tile_n / 2) + 250, KD == 1 ? 5L * nb * m_sub * box_rows : 0, resident ? 0 : (long)nb * T * 2200 / p->w_slots, m_sub * copy, m_sub * epi});
         real = cdivl(per_cta, m_sub) * turns + (resident ? (long)w_all / 45 : 0);
       }
     }
