@@ -1,6 +1,6 @@
 """The convolutions that walk along an axis (conv_slide.cuh), at the edges of their walk: runs of outputs that start and end inside a column, columns shorter
 than the kernel, rows of several images in a tile with a last group that is not full, several blocks of channels, accumulators whose ring ends
-inside an MMA, rows longer than a tile, volumes.  Bars as in test_gpu_parity.py: one rounding to the storage type."""
+inside an MMA, rows longer than a tile, volumes; and the ones done in patches with more than four input boxes in flight.  Bars as in test_gpu_parity.py: one rounding to the storage type."""
 import numpy as np
 import pytest
 import torch
@@ -34,6 +34,20 @@ def _built():
     ("bf16", 2, 64, 24, 27, 33, 40, 3),       # ... whose weights were streamed
 ])
 def test_walked_convolution_and_input_gradient(dtype, B, Cin, Cout, D, H, W, K):
+    convolutions_against_64_bits(dtype, B, Cin, Cout, D, H, W, K)
+
+
+@pytest.mark.parametrize("dtype,B,Cin,Cout,H,W,K", [
+    ("f16", 19, 72, 8, 131, 128, 1),          # pointwise: sixteen patches a CTA and some CTAs with fewer, two blocks of channels
+    ("bf16", 46, 192, 24, 129, 129, 1),       # ... forty, three blocks, a last patch of few pixels
+    ("f16", 37, 24, 64, 83, 83, 3),           # patches, whose input gradient walks
+    ("bf16", 9, 96, 16, 133, 131, 3),         # ... whose input gradient is done in patches
+])
+def test_long_runs_of_patches(dtype, B, Cin, Cout, H, W, K):
+    convolutions_against_64_bits(dtype, B, Cin, Cout, 1, H, W, K)
+
+
+def convolutions_against_64_bits(dtype, B, Cin, Cout, D, H, W, K):
     g = np.random.Generator(np.random.PCG64([B, Cin, Cout, H, W, K]))
     geo, kgeo, KD = ((D, H, W), (K, K, K), K) if D > 1 else ((H, W), (K, K), 1)
     X, dY = (inputs.round_to_storage(g.standard_normal((B, c) + geo, dtype=np.float32), dtype) for c in (Cin, Cout))
