@@ -13,6 +13,7 @@ struct TcSketchPlan {
   int swap;            // 0: MMA rows = probes, columns = samples; 1: rows = samples, columns = probes
   int tile_m, tile_n, m_sub;  // output tile of one work unit; m_sub 128-row MMA tiles share the other operand
   int tiles_m, tiles_n, splits;
+  bool row_boxes;            // operands are copied in boxes of eight rows x kgroup blocks
   int kgroup, rows_box;      // 64-wide k-blocks per stage; rows of the A box
   long kblocks, kblocks_per_split, kb_rem;   // the first kb_rem splits take one k-block more
   int stages;

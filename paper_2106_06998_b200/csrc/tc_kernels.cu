@@ -37,6 +37,7 @@ struct TcParams {
   int stages;
   int ksteps;              // UMMA k-steps (of 16) per stage
   int kgroup;              // SKETCH: 64-wide k-blocks per stage (each its own K-major tile), 1 elsewhere
+  int row_boxes_a, row_boxes_b;   // SKETCH, kgroup > 1: boxes of eight rows x kgroup blocks per operand and stage (0: one box of all rows)
   uint32_t a_jump, b_jump; // kgroup > 1: descriptor start-address step (>>4) from the last k-step of a block to the next block
   uint32_t a_stage_bytes, b_stage_bytes, tx_bytes;
   int a_boxes, b_boxes;    // TMA boxes per stage: A per 128-row tile, B in all
@@ -294,8 +295,9 @@ __device__ __forceinline__ Unit decode_unit(const TcParams& p, long u_) {
 // ------------------------------------------------------------------------------------ the kernel
 
 // F16: the 16-bit storage type is float16 instead of bfloat16 (a compile-time constant, so that the epilogues'
-// conversions carry no selection between the two).
-template <bool F16>
+// conversions carry no selection between the two).  ROWS: SKETCH with operands in boxes of eight rows (a constant too: with its copies beside the
+// others' the short kernels took 1 % longer, 65.0 -> 65.9 and 84.6 -> 85.9 us a training step).
+template <bool F16, bool ROWS>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                const __grid_constant__ CUtensorMap map_c, const TcParams p) {
@@ -553,6 +555,39 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     }
   } else if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
+    if (ROWS) {
+      // SKETCH in boxes of eight rows, issued by the whole, converged warp: some 80 clocks a box under `if (lane == 0)` were more than its bytes
+      // take (256 probes 263 -> 168 us, 128 135 -> 95)
+      const int stages = p.stages;
+      const uint32_t box = 1024u * (uint32_t)p.kgroup;
+      int s = 0;
+      long fill = 0, it = 0;
+      bool ok = true;
+      for (long u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
+        const Unit w = decode_unit(p, u);
+        const int row0 = w.tm * p.m_sub * TILE_M, col0 = w.tn * p.tile_n;
+        int kb = (int)w.split * p.kgroup;
+        for (int i = 0; i < w.nkb; ++i) {
+          if (fill > 0) {
+            ok = mbar_wait_warp_long(&empty_bar[s], (uint32_t)((fill - 1) & 1), p.status, p.tag);
+            if (!ok) break;
+          }
+          if (lane == 0) mbar_arrive_expect_tx(&full_bar[s], p.tx_bytes);
+          __syncwarp();
+          const uint32_t bar = smem_u32(&full_bar[s]);
+          uint32_t dst = tiles_base + (uint32_t)s * stage_bytes;
+#pragma unroll 4
+          for (int g = 0; g < p.row_boxes_a; ++g, dst += box) tma_load_3d_warp(dst, &map_a, 0, row0 + 8 * g, kb, bar);
+#pragma unroll 4
+          for (int g = 0; g < p.row_boxes_b; ++g, dst += box) tma_load_3d_warp(dst, &map_b, 0, col0 + 8 * g, kb, bar);
+          kb += p.kgroup * p.k_weave;
+          ++it;
+          if (++s == stages) { s = 0; ++fill; }
+        }
+      }
+      for (long i = max(0L, it - stages); i < it; ++i)      // (as below)
+        if (!mbar_wait_warp(&full_bar[i % stages], (uint32_t)((i / stages) & 1), p.status, p.tag)) break;
+    } else
     // One thread; its loop is kept free of divisions (coordinates advance incrementally).
     if (lane == 0) {
       const int stages = p.stages;
@@ -1124,7 +1159,8 @@ static xconv_status launch(const CUtensorMap& ma, const CUtensorMap& mb, const T
   while (table && q.stages > 2 && bytes() > (size_t)(SMEM_LIMIT - 1024)) --q.stages;
   const size_t smem = bytes();
   if (smem > (size_t)(SMEM_LIMIT - 1024) || p.tmem_cols > 512 || p.stages > MAX_STAGES) return XCONV_ERR_UNSUPPORTED;
-  void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, TcParams) = p.f16 ? tc_gemm_kernel<true> : tc_gemm_kernel<false>;
+  void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, TcParams) = p.row_boxes_a ? (p.f16 ? tc_gemm_kernel<true, true> : tc_gemm_kernel<false, true>)
+                                                                            : p.f16 ? tc_gemm_kernel<true, false> : tc_gemm_kernel<false, false>;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT - 1024);
   if (e != cudaSuccess) { set_cuda_error((int)e); return XCONV_ERR_CUDA; }
   q.tag = call_tag();
@@ -1159,6 +1195,11 @@ bool tc_plan_sketch(const xconv_desc* d, TcSketchPlan* p, bool redraw) {
   const uint32_t block = (uint32_t)p->rows_box * 128 + p->tile_n * 128;
   p->kgroup = 1;
   if (K % 64 == 0) p->kgroup = block <= 12 * 1024 ? 4 : block <= 36 * 1024 ? 2 : 1;
+  // Rows 1.5 MB apart or more: a box of all rows has each 128 bytes of it in another page of memory, and goes round all pages once per k-block.
+  // Boxes of eight rows take the blocks of a row close together (16 samples, 64 probes of 2^21 entries 77 -> 62 us, 256 probes 271 -> 165, 32 and
+  // 32 135 -> 94: 4.0 -> 5.7 TB/s; with rows of 1.6 MB, 64 and 256 93 -> 82; of 1.4 and 1 MB 1.00, and below the copies' number costs up to 1.4).
+  p->row_boxes = !redraw && K % 64 == 0 && K >= (3L << 18) && block <= 50 * 1024;
+  if (p->row_boxes) p->kgroup = block <= 25 * 1024 ? 4 : 2;      // (four against two: 168 -> 165, 95 -> 93, 56.0 -> 55.2)
   // Z redrawn in the kernel: a Philox block covers 128 consecutive entries of a row, i.e. two k-blocks
   if (redraw && K % 128 == 0 && p->kgroup == 1 && 2 * 2 * block + TILE_M * 128 <= (uint32_t)(SMEM_LIMIT - STATIC_SMEM_SLACK))
     p->kgroup = 2;
@@ -1195,11 +1236,11 @@ xconv_status tc_run_sketch(const xconv_desc* d, const TcSketchPlan& pl, const vo
   // box never writes only feed accumulator rows that are never stored.
   const uint32_t rows_box = (uint32_t)pl.rows_box;
   if (pl.kgroup > 1) {
-    // (64 k, rows, k-blocks): one box brings kgroup K-major tiles, one behind the other in shared memory
+    // (64 k, rows, k-blocks): one box brings kgroup K-major tiles, one behind the other in shared memory (or eight rows of each)
     const uint64_t da[3] = {64, (uint64_t)rows, (uint64_t)(K / 64)}, db[3] = {64, (uint64_t)cols, (uint64_t)(K / 64)};
     const uint64_t sa[2] = {(uint64_t)K * 2, 128};
-    const uint32_t box_a[3] = {64, rows_box, (uint32_t)pl.kgroup};
-    const uint32_t box_b[3] = {64, (uint32_t)pl.tile_n, (uint32_t)pl.kgroup};
+    const uint32_t box_a[3] = {64, pl.row_boxes ? 8u : rows_box, (uint32_t)pl.kgroup};
+    const uint32_t box_b[3] = {64, pl.row_boxes ? 8u : (uint32_t)pl.tile_n, (uint32_t)pl.kgroup};
     if (!make_map(&ma, A, 3, da, sa, box_a, f16) || !make_map(&mb, Bm, 3, db, sa, box_b, f16)) return XCONV_ERR_CUDA;
   } else {
     const uint64_t da[2] = {(uint64_t)K, (uint64_t)rows}, db[2] = {(uint64_t)K, (uint64_t)cols};
@@ -1237,6 +1278,16 @@ xconv_status tc_run_sketch(const xconv_desc* d, const TcSketchPlan& pl, const vo
   // The MMA always reads 128 rows of A.  Behind a shorter tile it reads whatever follows (the rows it
   // produces are never stored), which must still be this CTA's shared memory.
   p.smem_pad = TILE_M * 128 - std::min<uint32_t>(a_tile, TILE_M * 128);
+  if (pl.row_boxes) {
+    // 8-row groups kgroup KB apart, the k-blocks of a group behind one another; the 128 rows of the MMA then reach further, and stages make room for that
+    p.row_boxes_a = (int)rows_box / 8; p.row_boxes_b = pl.tile_n / 8;
+    p.layout = 2; p.sbo = 1024u * pl.kgroup; p.mn_step = 2048; p.cw_shift = 6;
+    p.a_jump = p.b_jump = 64 - 6;
+    p.a_sub_bytes = TILE_M * 128 * pl.kgroup;
+    const uint32_t reach = TILE_M * 128u * pl.kgroup, stage = p.a_stage_bytes + p.b_stage_bytes;
+    p.smem_pad = reach > stage ? reach - stage : 0;
+    while (p.stages > 2 && p.stages * stage + p.smem_pad + 1024 > (uint32_t)(SMEM_LIMIT - STATIC_SMEM_SLACK)) --p.stages;
+  }
   p.a_boxes = p.b_boxes = 1;
   p.a_mn_major = p.b_mn_major = 0;
   p.tiles_m = pl.tiles_m;
