@@ -37,7 +37,8 @@ struct TcParams {
   int stages;
   int ksteps;              // UMMA k-steps (of 16) per stage
   int kgroup;              // SKETCH: 64-wide k-blocks per stage (each its own K-major tile), 1 elsewhere
-  int row_boxes_a, row_boxes_b;   // SKETCH, kgroup > 1: boxes of eight rows x kgroup blocks per operand and stage (0: one box of all rows)
+  int row_boxes_a, row_boxes_b;   // boxes of eight rows per operand and stage (0: boxes of all rows).  SKETCH: x kgroup blocks; BACKPROBE: dY, x b_boxes
+  uint32_t sbo_b;          // ... the B descriptor's stride between 8-row groups there
   uint32_t a_jump, b_jump; // kgroup > 1: descriptor start-address step (>>4) from the last k-step of a block to the next block
   uint32_t a_stage_bytes, b_stage_bytes, tx_bytes;
   int a_boxes, b_boxes;    // TMA boxes per stage: A per 128-row tile, B in all
@@ -118,12 +119,12 @@ struct TcParams {
 // addresses jump to the next tile.
 template <int KS, bool TWO, bool GROUPED = false>
 __device__ __forceinline__ void umma_stage(uint32_t d, uint32_t tile_n, uint32_t a_lo, uint32_t b_lo, uint32_t hi,
-                                           uint32_t idesc, uint32_t acc, uint32_t a_step, uint32_t b_step,
+                                           uint32_t hi_b, uint32_t idesc, uint32_t acc, uint32_t a_step, uint32_t b_step,
                                            uint32_t a_sub, uint32_t a_jump = 0, uint32_t b_jump = 0) {
 #pragma unroll
   for (int k = 0; k < KS; ++k) {
-    umma_warp(d, a_lo, hi, b_lo, hi, idesc, k == 0 ? acc : 1u);
-    if (TWO) umma_warp(d + tile_n, a_lo + a_sub, hi, b_lo, hi, idesc, k == 0 ? acc : 1u);
+    umma_warp(d, a_lo, hi, b_lo, hi_b, idesc, k == 0 ? acc : 1u);
+    if (TWO) umma_warp(d + tile_n, a_lo + a_sub, hi, b_lo, hi_b, idesc, k == 0 ? acc : 1u);
     if (GROUPED && (k & 3) == 3) { a_lo += a_jump; b_lo += b_jump; }
     else { a_lo += a_step; b_lo += b_step; }
   }
@@ -295,7 +296,7 @@ __device__ __forceinline__ Unit decode_unit(const TcParams& p, long u_) {
 // ------------------------------------------------------------------------------------ the kernel
 
 // F16: the 16-bit storage type is float16 instead of bfloat16 (a compile-time constant, so that the epilogues'
-// conversions carry no selection between the two).  ROWS: SKETCH with operands in boxes of eight rows (a constant too: with its copies beside the
+// conversions carry no selection between the two).  ROWS: SKETCH and BACKPROBE with operands in boxes of eight rows (a constant too: with its copies beside the
 // others' the short kernels took 1 % longer, 65.0 -> 65.9 and 84.6 -> 85.9 us a training step).
 template <bool F16, bool ROWS>
 __global__ void __launch_bounds__(TC_THREADS, 1)
@@ -556,17 +557,18 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   } else if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     if (ROWS) {
-      // SKETCH in boxes of eight rows, issued by the whole, converged warp: some 80 clocks a box under `if (lane == 0)` were more than its bytes
+      // SKETCH and BACKPROBE in boxes of eight rows, issued by the whole, converged warp: some 80 clocks a box under `if (lane == 0)` were more than its bytes
       // take (256 probes 263 -> 168 us, 128 135 -> 95)
       const int stages = p.stages;
-      const uint32_t box = 1024u * (uint32_t)p.kgroup;
+      const uint32_t box = 1024u * (uint32_t)(p.mode == MODE_SKETCH ? p.kgroup : p.b_boxes);
       int s = 0;
       long fill = 0, it = 0;
       bool ok = true;
       for (long u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
         const Unit w = decode_unit(p, u);
         const int row0 = w.tm * p.m_sub * TILE_M, col0 = w.tn * p.tile_n;
-        int kb = (int)w.split * p.kgroup;
+        const bool sketch = p.mode == MODE_SKETCH;
+        int kb = sketch ? (int)w.split * p.kgroup : 0;         // block of the row; back-probe: row of dY
         for (int i = 0; i < w.nkb; ++i) {
           if (fill > 0) {
             ok = mbar_wait_warp_long(&empty_bar[s], (uint32_t)((fill - 1) & 1), p.status, p.tag);
@@ -576,11 +578,20 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           __syncwarp();
           const uint32_t bar = smem_u32(&full_bar[s]);
           uint32_t dst = tiles_base + (uint32_t)s * stage_bytes;
+          if (sketch) {
 #pragma unroll 4
-          for (int g = 0; g < p.row_boxes_a; ++g, dst += box) tma_load_3d_warp(dst, &map_a, 0, row0 + 8 * g, kb, bar);
+            for (int g = 0; g < p.row_boxes_a; ++g, dst += box) tma_load_3d_warp(dst, &map_a, 0, row0 + 8 * g, kb, bar);
 #pragma unroll 4
-          for (int g = 0; g < p.row_boxes_b; ++g, dst += box) tma_load_3d_warp(dst, &map_b, 0, col0 + 8 * g, kb, bar);
-          kb += p.kgroup * p.k_weave;
+            for (int g = 0; g < p.row_boxes_b; ++g, dst += box) tma_load_3d_warp(dst, &map_b, 0, col0 + 8 * g, kb, bar);
+            kb += p.kgroup * p.k_weave;
+          } else {
+            // (the blocks past the tile's own are the next tile's: nothing reads them here)
+            tma_load_2d_warp(dst, &map_a, kb, row0, bar);
+            dst += p.a_stage_bytes;
+#pragma unroll 2
+            for (int g = 0; g < p.row_boxes_b; ++g, dst += box) tma_load_3d_warp(dst, &map_b, 0, kb + 8 * g, w.blk0, bar);
+            kb += p.ksteps * 16;
+          }
           ++it;
           if (++s == stages) { s = 0; ++fill; }
         }
@@ -684,6 +695,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       const uint32_t a_lo0 = ((p.a_mn_major ? p.a_lbo : 16u) >> 4) << 16;
       const uint32_t b_lo0 = ((p.b_mn_major ? p.b_lbo : 16u) >> 4) << 16;
       const uint32_t desc_hi = (p.sbo >> 4) | (1u << 14) | (p.layout << 29);
+      const uint32_t desc_hi_b = ROWS ? (p.sbo_b >> 4) | (1u << 14) | (p.layout << 29) : desc_hi;
       const uint32_t a_sub = p.a_sub_bytes >> 4;
       const uint32_t a_stage16 = p.a_stage_bytes >> 4, stage16 = stage_bytes >> 4;
       const uint32_t base16 = (tiles_base & 0x3FFFFu) >> 4;
@@ -717,8 +729,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           tc_fence_after();
           uint32_t a_lo = a_lo0 | s16;
           uint32_t b_lo = b_lo0 | (s16 + a_stage16);
-#define XC_STAGE(KS, TWO) umma_stage<KS, TWO>(d_tmem, tile_n, a_lo, b_lo, desc_hi, idesc_u, acc, a_step, b_step, a_sub)
-#define XC_GROUP(KS, TWO) umma_stage<KS, TWO, true>(d_tmem, tile_n, a_lo, b_lo, desc_hi, idesc, acc, a_step, b_step, \
+#define XC_STAGE(KS, TWO) umma_stage<KS, TWO>(d_tmem, tile_n, a_lo, b_lo, desc_hi, desc_hi_b, idesc_u, acc, a_step, b_step, a_sub)
+#define XC_GROUP(KS, TWO) umma_stage<KS, TWO, true>(d_tmem, tile_n, a_lo, b_lo, desc_hi, desc_hi, idesc, acc, a_step, b_step, \
                                                     a_sub, p.a_jump, p.b_jump)
           if (p.mode == MODE_CONTRACT && p.tpu > 1) {
             // several offsets per unit: per k-step one MMA per piece (and row tile), each spanning whole
@@ -1281,7 +1293,7 @@ xconv_status tc_run_sketch(const xconv_desc* d, const TcSketchPlan& pl, const vo
   if (pl.row_boxes) {
     // 8-row groups kgroup KB apart, the k-blocks of a group behind one another; the 128 rows of the MMA then reach further, and stages make room for that
     p.row_boxes_a = (int)rows_box / 8; p.row_boxes_b = pl.tile_n / 8;
-    p.layout = 2; p.sbo = 1024u * pl.kgroup; p.mn_step = 2048; p.cw_shift = 6;
+    p.layout = 2; p.sbo = p.sbo_b = 1024u * pl.kgroup; p.mn_step = 2048; p.cw_shift = 6;
     p.a_jump = p.b_jump = 64 - 6;
     p.a_sub_bytes = TILE_M * 128 * pl.kgroup;
     const uint32_t reach = TILE_M * 128u * pl.kgroup, stage = p.a_stage_bytes + p.b_stage_bytes;
@@ -1484,7 +1496,10 @@ xconv_status tc_run_backprobe(const xconv_desc* d, const TcWgradPlan& pl, const 
   const uint64_t db[3] = {64, (uint64_t)d->B, (uint64_t)(Q / 64)};
   const uint64_t sa[1] = {(uint64_t)d->B * 2}, sb[2] = {(uint64_t)Q * 2, 128};
   const uint32_t box_a[2] = {64, (uint32_t)pl.bp_rows_box};           // 128-byte rows whatever bk is (zero fill past B)
-  const uint32_t box_b[3] = {64, (uint32_t)bk, 1};
+  // Rows of dY 2 MB apart or more: boxes of eight rows, as in the sketch (plan there).  64 channels of 160 x 160, 128 samples and probes 200 -> 155 us,
+  // 200 samples, 80 probes 217 -> 159 (4.2 -> 5.8 TB/s), 64 and 128 152 -> 137; rows of 1.6 MB 78 -> 79 and 85 -> 88.
+  const bool row_boxes = !seed && Q >= (1L << 20);
+  const uint32_t box_b[3] = {64, row_boxes ? 8u : (uint32_t)bk, row_boxes ? (uint32_t)pl.bp_tile_n / 64 : 1};
   // (seeded: the streamed operand is never read, and its map stands in with the output's address)
   if (!make_map(&ma, S_bf16, 2, da, sa, box_a, f16) || !make_map(&mb, seed ? L : dY, 3, db, sb, box_b, f16)) return XCONV_ERR_CUDA;
   // L [r][Q] for the epilogue's stores, as (64 positions, r rows, Q/64 groups): one box = the 32 rows of one
@@ -1525,6 +1540,11 @@ xconv_status tc_run_backprobe(const xconv_desc* d, const TcWgradPlan& pl, const 
   p.a_mn_major = 0;
   p.b_mn_major = 1;
   p.b_lbo = p.b_box_bytes;
+  if (row_boxes) {
+    p.row_boxes_a = 1; p.row_boxes_b = bk / 8;
+    p.layout = 2; p.sbo = 1024; p.cw_shift = 6;
+    p.b_lbo = 1024; p.sbo_b = 1024u * p.b_boxes; p.mn_step = 2 * p.sbo_b;
+  }
   p.epi_groups = pl.bp_groups;
   p.epi_bytes = (uint32_t)slots * (BP_SLOT_BYTES / 4) * staging_quads * pl.bp_groups;
   p.epi_slots = slots;

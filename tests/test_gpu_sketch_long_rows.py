@@ -1,5 +1,5 @@
-"""Sketches of long rows (tc_kernels.cu: operands copied in boxes of eight rows), on whole numbers: signs times samples of -3 .. 3 sum to
-less than 2^24, so the sketch is exact in any order of summation."""
+"""Sketches and back-probes of long rows (tc_kernels.cu: operands copied in boxes of eight rows), on whole numbers: signs times samples of
+-3 .. 3 sum to less than 2^24, so the sketch is exact in any order of summation; a back-probe of whole numbers is its exact sum rounded once."""
 import pytest
 import torch
 
@@ -35,3 +35,19 @@ def test_sketch_of_long_rows_is_exact(dtype, r, B, C, H, W):
     for j in range(0, r, 16):
         want[j:j + 16] = Z[j:j + 16].reshape(-1, H * W * C).double() @ X.reshape(B, -1).double().T
     assert torch.equal(S.double().reshape(r, B), want)
+
+
+@pytest.mark.parametrize("dtype,r,B,C,H,W", [
+    ("bf16", 72, 66, 64, 128, 128),       # the shortest row served; two stages of samples, the second of two rows
+    ("f16", 131, 128, 64, 127, 131),      # blocks that are no multiple of four; three rows in the second tile of probes
+    ("bf16", 300, 21, 32, 257, 130),      # one stage of two k-steps, its last box of eight rows past the samples
+    ("bf16", 65, 130, 64, 128, 127),      # below the line: boxes of all rows
+])
+def test_backprobe_of_long_rows_is_rounded_once(dtype, r, B, C, H, W):
+    g = torch.Generator(device="cuda").manual_seed(r * 1000 + B)
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float16
+    S = torch.randint(-8, 9, (r, B), generator=g, device="cuda").float()
+    dY = torch.randint(-3, 4, (B, H, W, C), generator=g, device="cuda", dtype=torch.int8).to(dt)
+    L = xb.xconv_backprobe(S, dY.permute(0, 3, 1, 2))
+    want = (S.double() @ dY.reshape(B, -1).double()).to(dt)
+    assert torch.equal(L.permute(0, 2, 3, 1).reshape(r, -1), want)
