@@ -1,13 +1,13 @@
 // Sketch S = Z^T X and back-probe L = S dY^T with float operands on the tensor cores (sm_100a): every float as three bfloat16 parts, a
 // product as six (split_f32.cuh).
 //
-// Both read one or two large float matrices once: the copy engine brings boxes of 32 terms of the reduction, twelve warps split them
-// and write the parts as MMA tiles.  The columns' parts lie one under another, so that three MMAs per k-step of 16 form the six products
+// Both read one or two large float matrices once: the copy engine brings boxes of 32 terms of the reduction, twelve warps in three
+// teams split them and write the parts as MMA tiles.  The columns' parts lie one under another, so that three MMAs per k-step of 16 form the six products
 // in three groups of n accumulator columns, as in conv_split.cu; two accumulator sets take chains of four k-steps (two stages) in
 // turn and eight epilogue warps add them in float registers.
 // Error against 64 bits, times that of the FP32 multiply-adds: 0.47 in the median, nowhere more than 1.  us, multiply-adds -> this: sketch of
-// 128 x 64 rows, 65536 terms 39 -> 26 (memory 8: the stages' chain of copy, split and MMA is some 2000 clocks, and a CTA has 14), back-probe
-// of 64 rows, 128 terms, 65536 positions 37 -> 23 (memory 8).
+// 128 x 64 rows, 65536 terms 39 -> 20 (memory 8: the stages' chain of copy, split and MMA is some 2000 clocks, and a CTA has 14), back-probe
+// of 64 rows, 128 terms, 65536 positions 37 -> 23 (memory 8).  Long sketches run at 3 to 4 TB/s: the conversion.
 //   sketch      rows = the larger of probes and samples (tiles of 128), columns = the other (up to 64); both K-major; the k-blocks are dealt
 //               to the splits in turn, so that the CTAs read neighbouring bytes of every row at a time
 //   back-probe  rows = 128 positions of the flat (pixel, channel) axis, MN-major, columns = up to 64 rows of S, whose parts a small
@@ -26,7 +26,7 @@
 
 namespace xconv {
 
-constexpr int GS_STAGES = 8, GS_TERMS = 32;
+constexpr int GS_STAGES = 8, GS_TERMS = 32, GS_TEAMS = 3;
 constexpr uint32_t GS_OUT = 2048;                  // a staging tile of 16-bit results: 32 columns of 32 positions
 enum : int { GS_SKETCH = 0, GS_BACK = 1, GS_BACK_BF16 = 2, GS_BACK_F16 = 3 };
 template <int KIND> struct GsElement { using type = float; using parts = Bf16Parts; };
@@ -144,6 +144,7 @@ template <int KIND>
 __global__ void __launch_bounds__(KIND >= GS_BACK_BF16 ? SP_CONVERT * 32 : SP_THREADS, 1)
 gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, const __grid_constant__ GemmSplitParams p) {
   using T = typename GsElement<KIND>::type;
+  constexpr int TEAMS = GS_TEAMS;
   constexpr bool BACK = KIND != GS_SKETCH, WHOLE = KIND >= GS_BACK_BF16;      // WHOLE: Y's tiles are copied as they are
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full[GS_STAGES], empty[GS_STAGES], acc_full[2], acc_empty[2];
@@ -153,8 +154,8 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < GS_STAGES; ++s) { mbar_init(&full[s], WHOLE ? 2 : SP_CONVERTERS / 32 + (BACK ? 1 : 0)); mbar_init(&empty[s], 2); }
-    for (int f = 0; f < SP_FLOATS; ++f) { mbar_init(&f_full[f], 1); mbar_init(&f_empty[f], SP_CONVERTERS / 32); }
+    for (int s = 0; s < GS_STAGES; ++s) { mbar_init(&full[s], WHOLE ? 2 : SP_CONVERTERS / 32 / TEAMS + (BACK ? 1 : 0)); mbar_init(&empty[s], 2); }
+    for (int f = 0; f < SP_FLOATS; ++f) { mbar_init(&f_full[f], 1); mbar_init(&f_empty[f], SP_CONVERTERS / 32 / TEAMS); }
     for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 8); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
@@ -353,23 +354,31 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     }
   } else if (!WHOLE && warp >= SP_CONVERT) {
     // ------------------------------------------------------------------ conversion
-    uint32_t s = 0, par = 1, f = 0, f_par = 0;
-    for (uint32_t i = 0; i < total; ++i) {
-      if (!split_wait(&empty[s], par, p.status, p.tag) || !split_wait(&f_full[f], f_par, p.status, p.tag)) break;
+    // In three teams of four warps that take the stages in turn: with all twelve on each a stage took 1500 to 1800 clocks whatever its rows (two waits,
+    // the way through shared memory, the proxy's fence, the arrivals), and nothing hid them.  us, one team -> two -> three:
+    // sketch of 64 x 16 rows, 2^21 terms 355 -> 225 -> 226, 64 x 64, 131072 terms 36.1 -> 29.6 -> 27.8, 300 x 100, 51200 terms 76.5 -> 60.8 -> 58.3.
+    // A ring has as many stages as there are teams, so that a stage's barriers see one team: the parity of a lap tells it from the lap before only.
+    // (Float boxes, three or four, change teams: that the stage `f_slots` before is converted is known from `empty`, which says that the MMAs have
+    // gone through all stages up to three before.)
+    constexpr int THREADS = SP_CONVERTERS / TEAMS;
+    const uint32_t team = (uint32_t)(warp - SP_CONVERT) / (THREADS / 32);
+    SplitTurn turn(team, (uint32_t)p.stages), f_turn(team, (uint32_t)p.f_slots);
+    for (uint32_t i = team; i < total; i += TEAMS) {
+      const uint32_t s = turn.at, f = f_turn.at;
+      if (!split_wait(&empty[s], turn.lap ^ 1u, p.status, p.tag) || !split_wait(&f_full[f], f_turn.lap, p.status, p.tag)) break;
       const uint32_t from = base + p.f_off + f * p.f_slot, to = base + s * p.stage_bytes;
       float2 check = make_float2(0.f, 0.f);
       if (BACK) {
         const SplitBox box{from, GS_TERMS, to, p.a_plane, p.a_plane >> 1, 0u, 0u};
-        split_box<7, 5, false>(box, check);
-        split_stage_done(&full[s], &f_empty[f], check, [&] { split_box_again<7, 5, false>(box); });
+        split_box<7, 5, false, THREADS>(box, check);
+        split_stage_done(&full[s], &f_empty[f], check, [&] { split_box_again<7, 5, false, THREADS>(box); });
       } else {
         const SplitBox rows{from, p.f_rows_a, to, p.a_plane, 0u, 0u, 0u}, cols{from + p.f_b, p.f_rows_b, to + p.a_bytes, p.b_plane, 0u, 0u, 0u};
-        split_box<6, 3, false>(rows, check);
-        split_box<6, 3, false>(cols, check);
-        split_stage_done(&full[s], &f_empty[f], check, [&] { split_box_again<6, 3, false>(rows); split_box_again<6, 3, false>(cols); });
+        split_box<6, 3, false, THREADS>(rows, check);
+        split_box<6, 3, false, THREADS>(cols, check);
+        split_stage_done(&full[s], &f_empty[f], check, [&] { split_box_again<6, 3, false, THREADS>(rows); split_box_again<6, 3, false, THREADS>(cols); });
       }
-      if (++s == (uint32_t)p.stages) { s = 0; par ^= 1u; }
-      if (++f == (uint32_t)p.f_slots) { f = 0; f_par ^= 1u; }
+      turn.next(TEAMS); f_turn.next(TEAMS);
     }
   }
   tc_fence_before();
@@ -390,8 +399,13 @@ static void plan_columns(long M, long N, int kind, GemmSplitPlan* p) {
   p->f_rows_b = back ? 0 : (int)std::min<long>(p->n, (N + 7) / 8 * 8);
   const int f_slot = whole ? (int)GS_OUT * 4 : back ? GS_TERMS * 512 : (int)up1k((uint32_t)p->f_rows_a * 128) + (int)up1k((uint32_t)p->f_rows_b * 128);
   const int stage = (whole ? 1 : 3) * 8192 + (int)up1k(3u * 64 * (uint32_t)p->n), room = SMEM_LIMIT - 4096 - 2 * stage - 2 * f_slot;
-  p->f_slots = whole ? 2 : 2 + std::min(SP_FLOATS - 2, room / f_slot);      // (whole: the results' staging tiles)
-  p->stages = 2 + std::min((whole ? GS_STAGES : 4) - 2, (room - (p->f_slots - 2) * f_slot) / stage);
+  if (whole) {
+    p->f_slots = 2;                                  // (the results' staging tiles)
+    p->stages = 2 + std::min(GS_STAGES - 2, room / stage);
+  } else {                                           // (every n has room for that: 3 x 36 KB and 3 x 24 KB)
+    p->stages = GS_TEAMS;
+    p->f_slots = 2 + std::min(SP_FLOATS - 2, (room - (GS_TEAMS - 2) * stage) / f_slot);
+  }
 }
 static const double HBM_SM = 22.0;                  // bytes per clock and SM from memory
 
@@ -465,7 +479,7 @@ template <int KIND>
 static xconv_status launch_gemm_split(const CUtensorMap& ma, const CUtensorMap& mb, const GemmSplitParams& p, unsigned grid, cudaStream_t st) {
   const size_t smem = 1024 + (size_t)p.f_off + (size_t)p.f_slots * p.f_slot;
   const int threads = KIND >= GS_BACK_BF16 ? SP_CONVERT * 32 : SP_THREADS;
-  if (smem > (size_t)(SMEM_LIMIT - 1024)) return XCONV_ERR_UNSUPPORTED;
+  if (smem > (size_t)(SMEM_LIMIT - 1024) || (KIND < GS_BACK_BF16 && (p.stages != GS_TEAMS || p.f_slots < GS_TEAMS))) return XCONV_ERR_UNSUPPORTED;
   cudaError_t e = cudaFuncSetAttribute(gemm_split_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT - 1024);
   if (e == cudaSuccess) e = launch_pdl(gemm_split_kernel<KIND>, dim3(grid), dim3(threads), smem_of_grid(smem, grid), st, ma, mb, p);
   count_launch();

@@ -169,36 +169,45 @@ struct SplitPlaces {
     st_shared_v2(at + 2 * plane, s.l);
   }
 };
-template <int RBS, int QSHIFT, bool PITCH>
+// Where the converting warps take stages in turn, in teams: the slot of a ring that a team comes to next, and the parity of its lap.
+struct SplitTurn {
+  uint32_t at, lap, slots;
+  __device__ __forceinline__ SplitTurn(uint32_t first, uint32_t n) : at(first), lap(0), slots(n) { next(0); }
+  __device__ __forceinline__ void next(uint32_t teams) {
+    at += teams;
+    while (at >= slots) { at -= slots; lap ^= 1u; }
+  }
+};
+template <int RBS, int QSHIFT, bool PITCH, int THREADS = SP_CONVERTERS>
 __device__ __forceinline__ void split_box(const SplitBox& b, float2& check) {
   constexpr int U = 4;
   // Without PITCH the items of a thread lie ROWS rows apart, and the swizzle of every other one differs in one bit at most: the addresses are
   // constants apart, where working each out took five instructions of forty.
-  constexpr uint32_t ROWS = SP_CONVERTERS >> QSHIFT, FLIP = ((ROWS >> (7 - RBS)) & ((1u << (RBS - 4)) - 1u)) << 4;
+  constexpr uint32_t ROWS = THREADS >> QSHIFT, FLIP = ((ROWS >> (7 - RBS)) & ((1u << (RBS - 4)) - 1u)) << 4;
   static_assert(PITCH || ((FLIP == 0 || FLIP == 64) && (2 * ROWS >> (7 - RBS)) % (1u << (RBS - 4)) == 0), "two items ahead the swizzle is the same");
-  const int tid = threadIdx.x - SP_CONVERT * 32, items = b.positions << QSHIFT;
+  const int tid = (threadIdx.x - SP_CONVERT * 32) % THREADS, items = b.positions << QSHIFT;
   const SplitPlaces<RBS, QSHIFT, PITCH> places(b, tid);
   uint32_t from = b.src + (uint32_t)tid * 16, at = PITCH ? 0u : places.of(tid);
-  for (int i = tid; i < items; i += U * SP_CONVERTERS, from += U * SP_CONVERTERS * 16, at += U * ROWS << RBS) {
+  for (int i = tid; i < items; i += U * THREADS, from += U * THREADS * 16, at += U * ROWS << RBS) {
     float4 v[U];
 #pragma unroll
     for (int u = 0; u < U; ++u)
-      if (u == 0 || i + u * SP_CONVERTERS < items) v[u] = ld_shared_f4(from + u * SP_CONVERTERS * 16);
+      if (u == 0 || i + u * THREADS < items) v[u] = ld_shared_f4(from + u * THREADS * 16);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      if (u > 0 && i + u * SP_CONVERTERS >= items) break;
-      places.store(PITCH ? places.of(i + u * SP_CONVERTERS) : (u & 1 ? at ^ FLIP : at) + (u * ROWS << RBS), split4(v[u], check));
+      if (u > 0 && i + u * THREADS >= items) break;
+      places.store(PITCH ? places.of(i + u * THREADS) : (u & 1 ? at ^ FLIP : at) + (u * ROWS << RBS), split4(v[u], check));
     }
   }
 }
 // The thread's part of a box again, any values; returns whether one is not finite.
-template <int RBS, int QSHIFT, bool PITCH>
+template <int RBS, int QSHIFT, bool PITCH, int THREADS = SP_CONVERTERS>
 __device__ __noinline__ bool split_box_again(const SplitBox b) {
-  const int tid = threadIdx.x - SP_CONVERT * 32, items = b.positions << QSHIFT;
+  const int tid = (threadIdx.x - SP_CONVERT * 32) % THREADS, items = b.positions << QSHIFT;
   const SplitPlaces<RBS, QSHIFT, PITCH> places(b, tid);
   bool odd = false;
 #pragma unroll 2
-  for (int i = tid; i < items; i += SP_CONVERTERS) {
+  for (int i = tid; i < items; i += THREADS) {
     const float4 v = ld_shared_f4(b.src + (uint32_t)i * 16);
     odd = odd || (v.x - v.x) + (v.y - v.y) + (v.z - v.z) + (v.w - v.w) != 0.f;
     places.store(places.of(i), split4_apart<Bf16Parts, false>(v));
