@@ -1,4 +1,5 @@
-"""Python binding of libxconv: argument marshalling only -- every step runs in the CUDA library.
+"""Python binding of libxconv: argument marshalling only -- every step runs in the CUDA library.  Calls on ordinary tensors are
+marshalled in native code (csrc/marshal.cpp); everything else, and every error, takes the ctypes path of this file.
 
 Tensors are torch CUDA tensors of logical shape (batch, channel, H, W) / (Cout, Cin, KH, KW) /
 (r, Cin, H, W) held in ``torch.channels_last`` memory format (the library's layout), in float32 or

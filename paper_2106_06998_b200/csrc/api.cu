@@ -628,9 +628,9 @@ static xconv_status run_conv_simt(const xconv_desc* d, bool dgrad, const void* i
 
 // Float layers whose convolution goes to the tensor cores (conv_split.cu): all but the smallest.  The call alone is faster from a
 // microsecond of multiply-adds on (us, multiply-adds -> this, 160 layers: 8 x 16 -> 16 channels of 32 x 32 12.5 -> 8.6, 4 x 192 -> 48, 37 x 37,
-// 1 x 1 14.5 -> 8.9, larger ones 236 -> 57; but 9 x 1 -> 128 channels of 13 x 13, 1 x 1, with the copies before it 15.5 -> 18.6), but it
-// is a launch more: a training step of the first of these, host and all, 57.4 -> 61.4.  3000 clocks of 75 multiply-adds a clock and SM keep that
-// layer off, by that one step's time; alone the kernels cross at about half of it.
+// 1 x 1 14.5 -> 8.9, larger ones 236 -> 57; but 9 x 1 -> 128 channels of 13 x 13, 1 x 1, with the copies before it 15.5 -> 18.6).  The line, 3000
+// clocks of 75 multiply-adds a clock and SM, was drawn against those kernels (conv_simt, conv_fma); below it small_f32.cu is the faster one, the first
+// of these in 4.8.  From there to twice the line multiply-adds in its tiles would still be faster, but with two to three times the error.
 static bool plan_conv_f32(const xconv_desc* d, bool dgrad, ConvSplitPlan* p) {
   const double macs = (double)d->B * depth(d) * d->H * d->W * d->Cin * d->Cout * kdepth(d) * d->KH * d->KW;
   if (d->dtype != XCONV_F32 || macs <= 3000.0 * 148 * 75) return false;

@@ -1,6 +1,6 @@
 // Direct convolution (and, with the weights read transposed and mirrored, the exact input gradient) on FP32 multiply-adds
-// for float layers that conv_split.cu does not take (small ones, and calls whose scratch is the header alone);
-// conv_simt (simt_kernels.cuh) serves the layers too small for its tiles, and the 16-bit layers of odd
+// for float layers that neither conv_split.cu nor small_f32.cu takes (channels off the multiples of 4, circular shifts, and calls whose
+// scratch is the header alone); conv_simt (simt_kernels.cuh) serves the layers too small for its tiles, and the 16-bit layers of odd
 // channel counts or circular shifts.
 //
 //   out[b,y,x,co] = sum over (offset, ci) of w(co,ci,offset) * in[b,y+dy-p,x+dx-p,ci]

@@ -1,5 +1,5 @@
-// FP32-FMA kernels for every step of the layer.  They serve float storage (where the 1e-5 parity
-// bar rules out TF32/BF16 tensor-core products) and any bfloat16 shape the tcgen05 kernels do not
+// FP32-FMA kernels for every step of the layer.  They serve the float layers that the kernels with split operands and those of
+// small_f32.cu do not take (the 1e-5 parity bar rules out plain TF32/BF16 products) and any 16-bit shape the tcgen05 kernels do not
 // cover.  All tensors are channels-last; all sums are accumulated in float.
 #pragma once
 
