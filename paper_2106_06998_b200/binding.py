@@ -200,6 +200,12 @@ def _geo(t: torch.Tensor):
     return (1, t.shape[2], t.shape[3]) if t.dim() == 4 else (t.shape[2], t.shape[3], t.shape[4])
 
 
+def _kernel_depth(t: torch.Tensor, kernel_depth: int):
+    """Refuses a kernel over planes for planar tensors: the result would be allocated without them."""
+    if t.dim() == 4 and kernel_depth > 1:
+        raise ValueError("kernel_depth must be 1 for 4-d (planar) tensors")
+
+
 def _like(shape_head, geo, dim, **kw):
     """An empty tensor (head..., [D,] H, W) in the channels-last format of a `dim`-d tensor."""
     D, H, W = geo
@@ -391,6 +397,7 @@ def xconv_wgrad_seeded(sketch: torch.Tensor, dY: torch.Tensor, seed: int, Cin: i
         if out is not None:
             return out
     _cl(dY, "dY")
+    _kernel_depth(dY, kernel_depth)
     B, Cout = dY.shape[:2]
     D, H, Wd = _geo(dY)
     r = sketch.shape[0]
@@ -437,8 +444,8 @@ def xconv_forward(X: torch.Tensor, W: torch.Tensor, Z: torch.Tensor, circular: b
     Cout, K = W.shape[0], W.shape[-1]
     KD = W.shape[2] if W.dim() == 5 else 1
     r = Z.shape[0]
-    if (W.shape[1] != Cin or W.dim() != X.dim() or tuple(Z.shape[1:]) != tuple(X.shape[1:]) or W.dtype != X.dtype
-            or Z.dtype != X.dtype):
+    if (W.shape[1] != Cin or W.dim() != X.dim() or W.shape[-2] != K or tuple(Z.shape[1:]) != tuple(X.shape[1:])
+            or W.dtype != X.dtype or Z.dtype != X.dtype):
         raise ValueError("shape or dtype mismatch between X, W and Z")
     desc = make_desc(B, Cin, Cout, H, Wd, r, X.dtype, K, D=D, KD=KD, circular=circular)
     Y = _like((B, Cout), (D, H, Wd), X.dim(), dtype=X.dtype, device=X.device)
@@ -457,6 +464,7 @@ def xconv_wgrad(sketch: torch.Tensor, dY: torch.Tensor, Z: torch.Tensor, kernel_
         if out is not None:
             return out
     _cl(dY, "dY"); _cl(Z, "Z")
+    _kernel_depth(dY, kernel_depth)
     B, Cout = dY.shape[:2]
     D, H, Wd = _geo(dY)
     r, Cin = Z.shape[0], Z.shape[1]
@@ -495,6 +503,7 @@ def xconv_wgrad_independent(sketch: torch.Tensor, dY: torch.Tensor, Z: torch.Ten
                             kernel_depth: int = 1, circular: bool = False) -> torch.Tensor:
     """dW estimate per channel pair from the per-channel sketch: float32 (Cout, Cin, [KD,] K, K), channels-last."""
     _cl(dY, "dY"); _cl(Z, "Z")
+    _kernel_depth(dY, kernel_depth)
     B, Cout = dY.shape[:2]
     D, H, Wd = _geo(dY)
     r, Cin = Z.shape[0], Z.shape[1]
@@ -538,6 +547,7 @@ def xconv_contract(L: torch.Tensor, Z: torch.Tensor, kernel_size: int = 3,
         if out is not None:
             return out
     _cl(L, "L"); _cl(Z, "Z")
+    _kernel_depth(L, kernel_depth)
     r, Cout = L.shape[:2]
     D, H, Wd = _geo(L)
     Cin = Z.shape[1]
@@ -562,7 +572,7 @@ def xconv_dgrad(dY: torch.Tensor, W: torch.Tensor, circular: bool = False) -> to
     D, H, Wd = _geo(dY)
     Cin, K = W.shape[1], W.shape[-1]
     KD = W.shape[2] if W.dim() == 5 else 1
-    if W.shape[0] != Cout or W.dtype != dY.dtype or W.dim() != dY.dim():
+    if W.shape[0] != Cout or W.dtype != dY.dtype or W.dim() != dY.dim() or W.shape[-2] != K:
         raise ValueError("shape or dtype mismatch between dY and W")
     desc = make_desc(B, Cin, Cout, H, Wd, 1, dY.dtype, K, D=D, KD=KD, circular=circular)
     dX = _like((B, Cin), (D, H, Wd), dY.dim(), dtype=dY.dtype, device=dY.device)

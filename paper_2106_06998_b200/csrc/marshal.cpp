@@ -99,6 +99,11 @@ bool small_int(PyObject* o, int32_t* v) {
   return true;
 }
 
+// A square kernel, as the descriptor has it (which is made from the last extent alone).
+bool square(const Image& W) { return W.H == W.W && W.W <= 64 && W.D <= 64; }
+// A kernel over planes, for tensors that have planes: the weights of a planar layer are allocated without them.
+bool planes_fit(const Image& g, int32_t KD) { return g.dim == 5 || KD == 1; }
+
 xconv_desc descriptor(int32_t B, int32_t Cin, int32_t Cout, const Image& g, int32_t r, int32_t K, int32_t KD, bool circular) {
   xconv_desc d;
   std::memset(&d, 0, sizeof d);
@@ -178,7 +183,7 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   XM_BEGIN(4)
   const Image X(a[0]), W(a[1]), Z(a[2]);
   if (!X || !W || !Z || !PyBool_Check(a[3])) Py_RETURN_NONE;
-  if (!Z.same_plane(X) || Z.c != X.c || W.c != X.c || W.dim != X.dim || W.dtype != X.dtype || W.W > 64 || W.D > 64) Py_RETURN_NONE;
+  if (!Z.same_plane(X) || Z.c != X.c || W.c != X.c || W.dim != X.dim || W.dtype != X.dtype || !square(W)) Py_RETURN_NONE;
   const xconv_desc d = descriptor(X.n, X.c, W.n, X, Z.n, W.W, W.D, a[3] == Py_True);
   const at::Tensor Y = image_like(X, X.n, W.n), S = matrix_like(X, Z.n, X.n);
   if (!run(X, d, XCONV_OP_FORWARD, "xconv_forward", [&](const xconv_desc* q, void* ws, size_t n, void* st) {
@@ -225,7 +230,7 @@ PyObject* wgrad(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   XM_BEGIN(6)
   const Image Y(a[1]), Z(a[2]);
   int32_t K, KD;
-  if (!Y || !Z || !Z.same_plane(Y) || !small_int(a[3], &K) || !small_int(a[4], &KD) || !PyBool_Check(a[5])) Py_RETURN_NONE;
+  if (!Y || !Z || !Z.same_plane(Y) || !small_int(a[3], &K) || !small_int(a[4], &KD) || !planes_fit(Y, KD) || !PyBool_Check(a[5])) Py_RETURN_NONE;
   const at::Tensor* S = sketch_of(a[0], Y.n);
   if (!S || S->size(0) != Z.n) Py_RETURN_NONE;
   const xconv_desc d = descriptor(Y.n, Z.c, Y.c, Y, Z.n, K, KD, a[5] == Py_True);
@@ -242,7 +247,8 @@ PyObject* wgrad_seeded(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   XM_BEGIN(7)
   const Image Y(a[1]);
   int32_t K, KD;
-  if (!Y || !PyLong_CheckExact(a[2]) || !PyLong_CheckExact(a[3]) || !small_int(a[4], &K) || !small_int(a[5], &KD) || !PyBool_Check(a[6])) Py_RETURN_NONE;
+  if (!Y || !PyLong_CheckExact(a[2]) || !PyLong_CheckExact(a[3]) || !small_int(a[4], &K) || !small_int(a[5], &KD) || !planes_fit(Y, KD) || !PyBool_Check(a[6]))
+    Py_RETURN_NONE;
   int over = 0;
   const long Cin = PyLong_AsLongAndOverflow(a[3], &over);
   if (over || Cin <= 0 || Cin > INT32_MAX) Py_RETURN_NONE;
@@ -262,7 +268,7 @@ PyObject* wgrad_seeded(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
 PyObject* dgrad(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   XM_BEGIN(3)
   const Image Y(a[0]), W(a[1]);
-  if (!Y || !W || !PyBool_Check(a[2]) || W.n != Y.c || W.dtype != Y.dtype || W.dim != Y.dim || W.W > 64 || W.D > 64) Py_RETURN_NONE;
+  if (!Y || !W || !PyBool_Check(a[2]) || W.n != Y.c || W.dtype != Y.dtype || W.dim != Y.dim || !square(W)) Py_RETURN_NONE;
   const xconv_desc d = descriptor(Y.n, W.c, Y.c, Y, 1, W.W, W.D, a[2] == Py_True);
   const at::Tensor dX = image_like(Y, Y.n, W.c);
   if (!run(Y, d, XCONV_OP_DGRAD, "xconv_dgrad", [&](const xconv_desc* q, void* ws, size_t n, void* st) {
@@ -293,7 +299,7 @@ PyObject* contract(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   XM_BEGIN(5)
   const Image L(a[0]), Z(a[1]);
   int32_t K, KD;
-  if (!L || !Z || !Z.same_plane(L) || Z.n != L.n || !small_int(a[2], &K) || !small_int(a[3], &KD) || !PyBool_Check(a[4])) Py_RETURN_NONE;
+  if (!L || !Z || !Z.same_plane(L) || Z.n != L.n || !small_int(a[2], &K) || !small_int(a[3], &KD) || !planes_fit(L, KD) || !PyBool_Check(a[4])) Py_RETURN_NONE;
   const xconv_desc d = descriptor(1, Z.c, L.c, L, L.n, K, KD, a[4] == Py_True);
   const at::Tensor dW = weights_like(L, L.c, Z.c, K, KD);
   if (!run(L, d, XCONV_OP_WGRAD, "xconv_contract", [&](const xconv_desc* q, void* ws, size_t n, void* st) {

@@ -121,6 +121,18 @@ def test_what_was_refused_is_refused_with_the_same_error(monkeypatch):
     torch.cuda.synchronize()
 
 
+def test_kernels_that_the_descriptor_cannot_state_are_refused_on_both_paths(monkeypatch):
+    d = _layer(4, 8, 16, (6, 7), 3, torch.bfloat16)
+    flat = [dict(d, W=torch.zeros(16, 8, *k, device="cuda", dtype=torch.bfloat16).contiguous(memory_format=torch.channels_last)) for k in ((1, 3), (5, 3))]
+    for native in (xb._load_native(), _PythonPath()):
+        monkeypatch.setattr(xb, "_native", native)
+        for case, calls in [(c, (0, 5)) for c in flat] + [(dict(d, KD=3), (3, 4, 7))]:
+            for i in calls:
+                with pytest.raises(ValueError):
+                    _calls(case)[i]()
+    torch.cuda.synchronize()
+
+
 def test_scratch_buffers_are_bounded_and_given_back():
     d = _layer(16, 32, 64, (40, 40), 32, torch.bfloat16)
     nbytes = xb.workspace_bytes(xb.make_desc(16, 32, 64, 40, 40, 32, torch.bfloat16), xb.OP_WGRAD)

@@ -31,3 +31,40 @@ def test_the_python_path_raises_as_before(native):
             call()
     with pytest.raises(TypeError):
         native.use_library(1, 2)
+
+
+@pytest.fixture
+def python_path(monkeypatch):
+    """The Python path on host tensors, up to where it would call the library."""
+    class Reached(Exception):
+        pass
+
+    def reached():
+        raise Reached
+    monkeypatch.setattr(xb, "_native", type("Declines", (), {"__getattr__": lambda self, name: lambda *a: None})())
+    monkeypatch.setattr(xb, "_cl", lambda t, name: t)
+    monkeypatch.setattr(xb, "lib", reached)
+    return Reached
+
+
+def test_a_kernel_that_the_descriptor_cannot_state_is_refused(python_path):
+    """The descriptor has one kernel extent, and a planar layer's weights have no planes: with anything else the kernels would read or write past a tensor."""
+    x, s = torch.zeros(2, 8, 6, 6), torch.zeros(3, 2)
+    z, l = torch.zeros(3, 8, 6, 6), torch.zeros(3, 8, 6, 6)
+    for shape in ((1, 3), (5, 3), (3, 1)):
+        w = torch.zeros(8, 8, *shape)
+        for call in (lambda: xb.xconv_forward(x, w, z), lambda: xb.xconv_dgrad(x, w)):
+            with pytest.raises(ValueError, match="mismatch"):
+                call()
+    v, vz = torch.zeros(2, 8, 4, 6, 6), torch.zeros(3, 8, 4, 6, 6)
+    with pytest.raises(ValueError, match="mismatch"):
+        xb.xconv_forward(v, torch.zeros(8, 8, 3, 1, 3), vz)
+    for depth in (2, 3):
+        for call in (lambda **k: xb.xconv_wgrad(s, x, z, **k), lambda **k: xb.xconv_wgrad_seeded(s, x, 1, 8, **k), lambda **k: xb.xconv_contract(l, z, **k),
+                     lambda **k: xb.xconv_wgrad_independent(torch.zeros(3, 8, 2), x, z, **k)):
+            with pytest.raises(ValueError, match="kernel_depth"):
+                call(kernel_depth=depth)
+    for ok in (lambda: xb.xconv_forward(x, torch.zeros(8, 8, 3, 3), z), lambda: xb.xconv_forward(v, torch.zeros(8, 8, 1, 3, 3), vz),
+               lambda: xb.xconv_wgrad(s, v, vz, kernel_depth=3), lambda: xb.xconv_wgrad(s, v, vz), lambda: xb.xconv_contract(l, z)):
+        with pytest.raises(python_path):
+            ok()
