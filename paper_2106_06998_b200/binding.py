@@ -206,6 +206,15 @@ def _kernel_depth(t: torch.Tensor, kernel_depth: int):
         raise ValueError("kernel_depth must be 1 for 4-d (planar) tensors")
 
 
+def _scale(chan_scale, Cin: int):
+    """The channels' scale as the library reads it: Cin floats in a row in device memory."""
+    if chan_scale is None:
+        return None
+    if chan_scale.dtype != torch.float32 or chan_scale.numel() != Cin or not chan_scale.is_cuda:
+        raise ValueError("chan_scale must hold Cin float32 values in device memory")
+    return chan_scale.contiguous()
+
+
 def _like(shape_head, geo, dim, **kw):
     """An empty tensor (head..., [D,] H, W) in the channels-last format of a `dim`-d tensor."""
     D, H, W = geo
@@ -401,8 +410,8 @@ def xconv_wgrad_seeded(sketch: torch.Tensor, dY: torch.Tensor, seed: int, Cin: i
     B, Cout = dY.shape[:2]
     D, H, Wd = _geo(dY)
     r = sketch.shape[0]
-    if tuple(sketch.shape) != (r, B) or sketch.dtype != torch.float32 or not sketch.is_contiguous():
-        raise ValueError("sketch must be a contiguous float32 [r, B] tensor")
+    if tuple(sketch.shape) != (r, B) or sketch.dtype != torch.float32 or not sketch.is_contiguous() or not sketch.is_cuda:
+        raise ValueError("sketch must be a contiguous float32 [r, B] CUDA tensor")
     K = kernel_size
     desc = make_desc(B, Cin, Cout, H, Wd, r, dY.dtype, K, D=D, KD=kernel_depth, circular=circular)
     dW = _like((Cout, Cin), (kernel_depth, K, K), dY.dim(), dtype=torch.float32, device=dY.device)
@@ -468,12 +477,11 @@ def xconv_wgrad(sketch: torch.Tensor, dY: torch.Tensor, Z: torch.Tensor, kernel_
     B, Cout = dY.shape[:2]
     D, H, Wd = _geo(dY)
     r, Cin = Z.shape[0], Z.shape[1]
-    if tuple(sketch.shape) != (r, B) or sketch.dtype != torch.float32 or not sketch.is_contiguous():
-        raise ValueError("sketch must be a contiguous float32 [r, B] tensor")
+    if tuple(sketch.shape) != (r, B) or sketch.dtype != torch.float32 or not sketch.is_contiguous() or not sketch.is_cuda:
+        raise ValueError("sketch must be a contiguous float32 [r, B] CUDA tensor")
     if tuple(Z.shape[2:]) != tuple(dY.shape[2:]) or Z.dtype != dY.dtype:
         raise ValueError("shape or dtype mismatch between dY and Z")
-    if chan_scale is not None and (chan_scale.dtype != torch.float32 or chan_scale.numel() != Cin):
-        raise ValueError("chan_scale must hold Cin float32 values")
+    chan_scale = _scale(chan_scale, Cin)
     K = kernel_size
     desc = make_desc(B, Cin, Cout, H, Wd, r, dY.dtype, K, chan_scale, D=D, KD=kernel_depth, zero_blocks=zero_blocks,
                      circular=circular)
@@ -507,8 +515,8 @@ def xconv_wgrad_independent(sketch: torch.Tensor, dY: torch.Tensor, Z: torch.Ten
     B, Cout = dY.shape[:2]
     D, H, Wd = _geo(dY)
     r, Cin = Z.shape[0], Z.shape[1]
-    if tuple(sketch.shape) != (r, Cin, B) or sketch.dtype != torch.float32 or not sketch.is_contiguous():
-        raise ValueError("sketch must be a contiguous float32 [r, Cin, B] tensor")
+    if tuple(sketch.shape) != (r, Cin, B) or sketch.dtype != torch.float32 or not sketch.is_contiguous() or not sketch.is_cuda:
+        raise ValueError("sketch must be a contiguous float32 [r, Cin, B] CUDA tensor")
     if tuple(Z.shape[2:]) != tuple(dY.shape[2:]) or Z.dtype != dY.dtype:
         raise ValueError("shape or dtype mismatch between dY and Z")
     K = kernel_size
@@ -529,8 +537,8 @@ def xconv_backprobe(sketch: torch.Tensor, dY: torch.Tensor) -> torch.Tensor:
     B, Cout = dY.shape[:2]
     D, H, Wd = _geo(dY)
     r = sketch.shape[0]
-    if tuple(sketch.shape) != (r, B) or sketch.dtype != torch.float32 or not sketch.is_contiguous():
-        raise ValueError("sketch must be a contiguous float32 [r, B] tensor")
+    if tuple(sketch.shape) != (r, B) or sketch.dtype != torch.float32 or not sketch.is_contiguous() or not sketch.is_cuda:
+        raise ValueError("sketch must be a contiguous float32 [r, B] CUDA tensor")
     desc = make_desc(B, 1, Cout, H, Wd, r, dY.dtype, D=D)
     L = _like((r, Cout), (D, H, Wd), dY.dim(), dtype=dY.dtype, device=dY.device)
     ws = workspace(workspace_bytes(desc, OP_WGRAD), dY.device)
@@ -553,6 +561,7 @@ def xconv_contract(L: torch.Tensor, Z: torch.Tensor, kernel_size: int = 3,
     Cin = Z.shape[1]
     if Z.shape[0] != r or tuple(Z.shape[2:]) != tuple(L.shape[2:]) or Z.dtype != L.dtype:
         raise ValueError("shape or dtype mismatch between L and Z")
+    chan_scale = _scale(chan_scale, Cin)
     K = kernel_size
     desc = make_desc(1, Cin, Cout, H, Wd, r, L.dtype, K, chan_scale, D=D, KD=kernel_depth, zero_blocks=zero_blocks,
                      circular=circular)

@@ -133,6 +133,14 @@ def test_kernels_that_the_descriptor_cannot_state_are_refused_on_both_paths(monk
     torch.cuda.synchronize()
 
 
+def test_a_scale_whose_values_lie_apart():
+    d = _layer(4, 8, 16, (6, 7), 3, torch.bfloat16)
+    scale = torch.arange(1.0, 17.0, device="cuda")[::2]
+    for call in (lambda c: xb.xconv_wgrad(d["S"], d["dY"], d["Z"], chan_scale=c), lambda c: xb.xconv_contract(d["L"], d["Z"], chan_scale=c)):
+        assert torch.equal(call(scale), call(scale.contiguous()))
+        assert torch.equal(call(torch.ones(1, device="cuda").expand(8)), call(torch.ones(8, device="cuda")))
+
+
 def test_scratch_buffers_are_bounded_and_given_back():
     d = _layer(16, 32, 64, (40, 40), 32, torch.bfloat16)
     nbytes = xb.workspace_bytes(xb.make_desc(16, 32, 64, 40, 40, 32, torch.bfloat16), xb.OP_WGRAD)

@@ -33,6 +33,11 @@ def test_the_python_path_raises_as_before(native):
         native.use_library(1, 2)
 
 
+class _OnDevice(torch.Tensor):
+    """A host tensor that passes for one in device memory."""
+    is_cuda = True
+
+
 @pytest.fixture
 def python_path(monkeypatch):
     """The Python path on host tensors, up to where it would call the library."""
@@ -49,7 +54,7 @@ def python_path(monkeypatch):
 
 def test_a_kernel_that_the_descriptor_cannot_state_is_refused(python_path):
     """The descriptor has one kernel extent, and a planar layer's weights have no planes: with anything else the kernels would read or write past a tensor."""
-    x, s = torch.zeros(2, 8, 6, 6), torch.zeros(3, 2)
+    x, s = torch.zeros(2, 8, 6, 6), torch.zeros(3, 2).as_subclass(_OnDevice)
     z, l = torch.zeros(3, 8, 6, 6), torch.zeros(3, 8, 6, 6)
     for shape in ((1, 3), (5, 3), (3, 1)):
         w = torch.zeros(8, 8, *shape)
@@ -68,3 +73,18 @@ def test_a_kernel_that_the_descriptor_cannot_state_is_refused(python_path):
                lambda: xb.xconv_wgrad(s, v, vz, kernel_depth=3), lambda: xb.xconv_wgrad(s, v, vz), lambda: xb.xconv_contract(l, z)):
         with pytest.raises(python_path):
             ok()
+
+
+def test_what_lies_in_host_memory_is_refused_beside_the_images_too(python_path):
+    x, z, s = torch.zeros(2, 8, 6, 6), torch.zeros(3, 8, 6, 6), torch.zeros(3, 2)
+    for call in (lambda: xb.xconv_wgrad(s, x, z), lambda: xb.xconv_wgrad_seeded(s, x, 1, 8), lambda: xb.xconv_backprobe(s, x),
+                 lambda: xb.xconv_wgrad_independent(torch.zeros(3, 8, 2), x, z)):
+        with pytest.raises(ValueError, match="sketch"):
+            call()
+    device = s.as_subclass(_OnDevice)
+    for scale in (torch.ones(8), torch.ones(7).as_subclass(_OnDevice), torch.ones(8, dtype=torch.float16).as_subclass(_OnDevice)):
+        for call in (lambda: xb.xconv_wgrad(device, x, z, chan_scale=scale), lambda: xb.xconv_contract(z, z, chan_scale=scale)):
+            with pytest.raises(ValueError, match="chan_scale"):
+                call()
+    with pytest.raises(python_path):
+        xb.xconv_wgrad(device, x, z, chan_scale=torch.ones(8).as_subclass(_OnDevice))
