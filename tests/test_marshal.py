@@ -1,7 +1,11 @@
 """The binding's native calls (csrc/marshal.cpp) leave everything but ordinary CUDA tensors to the Python path, which raises the errors.  (No GPU.)"""
+import sys
+import warnings
+
 import pytest
 import torch
 
+import paper_2106_06998_b200 as package
 from paper_2106_06998_b200 import binding as xb
 
 
@@ -88,3 +92,23 @@ def test_what_lies_in_host_memory_is_refused_beside_the_images_too(python_path):
                 call()
     with pytest.raises(python_path):
         xb.xconv_wgrad(device, x, z, chan_scale=torch.ones(8).as_subclass(_OnDevice))
+
+
+def test_without_the_native_module_every_call_takes_the_python_path(monkeypatch):
+    """One warning, and the errors of the Python path; a library that is missing is still an error."""
+    x = torch.zeros(2, 8, 4, 4).contiguous(memory_format=torch.channels_last)
+    monkeypatch.setitem(sys.modules, package.__name__ + "._marshal", None)
+    monkeypatch.delattr(package, "_marshal", raising=False)
+    monkeypatch.setattr(xb, "_native", None)
+    with pytest.warns(RuntimeWarning, match="_marshal.so cannot be loaded"), pytest.raises(ValueError, match="must be a CUDA tensor"):
+        xb.xconv_sketch(x, x)
+    with warnings.catch_warnings():
+        warnings.simplefilter("error")
+        for call in (lambda: xb.xconv_forward(x, x, x), lambda: xb.xconv_dgrad(x, x), lambda: xb.xconv_sketch_seeded(x, 1, 4)):
+            with pytest.raises(ValueError, match="must be a CUDA tensor"):
+                call()
+    monkeypatch.setattr(xb, "_native", None)
+    monkeypatch.setattr(xb, "_lib", None)
+    monkeypatch.setattr(xb, "LIB_PATH", "/nowhere/libxconv.so")
+    with pytest.raises(RuntimeError, match="is missing"):
+        xb.xconv_sketch(x, x)
