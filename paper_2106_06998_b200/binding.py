@@ -17,6 +17,8 @@ from ctypes import POINTER, Structure, c_char_p, c_float, c_int, c_int32, c_size
 
 import torch
 
+from .build import marshal_key
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libxconv.so")
 
@@ -138,6 +140,8 @@ def _load_native():
     L = lib()                                   # (before `_native` is set)
     try:
         from . import _marshal
+        if getattr(_marshal, "key", None) != marshal_key():
+            raise ImportError(f"it was not compiled as {marshal_key()}")
     except ImportError as e:
         warnings.warn(f"{os.path.join(_HERE, '_marshal.so')} cannot be loaded ({e}): calls go through ctypes, which takes some 10 us more of the host each; "
                       "build it with `python -m paper_2106_06998_b200.build`", RuntimeWarning, stacklevel=3)

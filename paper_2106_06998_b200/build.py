@@ -4,6 +4,7 @@ from __future__ import annotations
 import os
 import shutil
 import subprocess
+import warnings
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
@@ -30,27 +31,53 @@ def _stale() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def marshal_key() -> str:
+    """What the binding's native part is compiled against, beside its sources: it uses torch's C++ classes and the interpreter's ABI."""
+    import sysconfig
+    import torch
+    return f"xconv marshal for torch {torch.__version__}, {sysconfig.get_config_var('SOABI')}"
+
+
+def _marshal_current() -> bool:
+    if not os.path.exists(MARSHAL):
+        return False
+    header = os.path.join(HERE, "..", "include", "xconv.h")
+    with open(MARSHAL, "rb") as f:
+        return os.path.getmtime(MARSHAL) >= max(map(os.path.getmtime, (MARSHAL_SOURCE, header))) and marshal_key().encode() + b"\0" in f.read()
+
+
 def build_marshal(force: bool = False) -> str:
     """Compiles the binding's calls on ordinary tensors (csrc/marshal.cpp) against the installed torch; returns the module's path."""
-    header = os.path.join(HERE, "..", "include", "xconv.h")
-    if not force and os.path.exists(MARSHAL) and os.path.getmtime(MARSHAL) >= max(map(os.path.getmtime, (MARSHAL_SOURCE, header))):
+    if not force and _marshal_current():
         return MARSHAL
     import sysconfig
     import torch
     top = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
+    fresh = os.path.join(HERE, "_marshal_fresh.so")
+    # (the CUDA runtime that it calls is the one that libc10_cuda brings with it)
     subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
-                    "-isystem", os.path.join(top, "include"), "-isystem", os.path.join(top, "include", "torch", "csrc", "api", "include"),
-                    "-isystem", sysconfig.get_paths()["include"], "-isystem", os.path.join(cuda, "include"), MARSHAL_SOURCE, "-o", MARSHAL,
-                    "-L" + os.path.join(top, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-L" + os.path.join(cuda, "lib64"), "-lcudart"], check=True)
+                    f'-DXM_KEY="{marshal_key()}"', "-isystem", os.path.join(top, "include"), "-isystem", os.path.join(top, "include", "torch", "csrc", "api", "include"),
+                    "-isystem", sysconfig.get_paths()["include"], "-isystem", os.path.join(cuda, "include"), MARSHAL_SOURCE, "-o", fresh,
+                    "-L" + os.path.join(top, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"], check=True)
+    os.replace(fresh, MARSHAL)
     return MARSHAL
+
+
+def _try_build_marshal(force: bool) -> None:
+    """The library alone is enough (the binding then calls it through ctypes): a machine without torch's or Python's headers, or without a
+    host compiler, gets a warning."""
+    try:
+        build_marshal(force)
+    except (OSError, subprocess.CalledProcessError, ImportError) as e:
+        warnings.warn(f"{MARSHAL} was not built ({e}): calls will go through ctypes", RuntimeWarning, stacklevel=3)
 
 
 def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     """Compile every CUDA source into one shared library; returns its path.
     ``extra_flags`` go to nvcc."""
     if not force and not _stale():
-        build_marshal()
+        _try_build_marshal(False)
         return LIB
     objs, jobs = [], []
     for src in SOURCES:
@@ -66,7 +93,7 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
         if code != 0:
             raise subprocess.CalledProcessError(code, cmd)
     subprocess.run([_nvcc(), "-shared", "-cudart", "static", "-o", LIB, *objs, "-ldl"], check=True)
-    build_marshal(force)
+    _try_build_marshal(force)
     return LIB
 
 

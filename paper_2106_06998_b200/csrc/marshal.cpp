@@ -338,4 +338,9 @@ PyModuleDef module_def = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, method
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__marshal() { return PyModule_Create(&module_def); }
+// (`key`: what the module was compiled against; binding.py and build.py compare it with what is installed)
+PyMODINIT_FUNC PyInit__marshal() {
+  PyObject* m = PyModule_Create(&module_def);
+  if (m && PyModule_AddStringConstant(m, "key", XM_KEY) != 0) { Py_DECREF(m); return nullptr; }
+  return m;
+}

@@ -7,6 +7,7 @@ import torch
 
 import paper_2106_06998_b200 as package
 from paper_2106_06998_b200 import binding as xb
+from paper_2106_06998_b200 import build
 
 
 @pytest.fixture(scope="module")
@@ -112,3 +113,23 @@ def test_without_the_native_module_every_call_takes_the_python_path(monkeypatch)
     monkeypatch.setattr(xb, "LIB_PATH", "/nowhere/libxconv.so")
     with pytest.raises(RuntimeError, match="is missing"):
         xb.xconv_sketch(x, x)
+
+
+def test_a_module_for_another_torch_is_neither_used_nor_kept(monkeypatch):
+    build.build()
+    x = torch.zeros(2, 8, 4, 4).contiguous(memory_format=torch.channels_last)
+    assert build._marshal_current() and xb._load_native().key == build.marshal_key()
+    monkeypatch.setattr(xb, "marshal_key", lambda: "another")
+    monkeypatch.setattr(xb, "_native", None)
+    with pytest.warns(RuntimeWarning, match="not compiled as another"), pytest.raises(ValueError, match="must be a CUDA tensor"):
+        xb.xconv_sketch(x, x)
+    monkeypatch.setattr(build, "marshal_key", lambda: "another")
+    assert not build._marshal_current()
+
+
+def test_the_library_is_built_where_the_native_module_cannot_be(monkeypatch):
+    build.build()
+    monkeypatch.setenv("CXX", "/nowhere/g++")
+    monkeypatch.setattr(build, "_marshal_current", lambda: False)
+    with pytest.warns(RuntimeWarning, match="was not built"):
+        assert build.build() == build.LIB
