@@ -8,7 +8,6 @@ library is missing or a layer has no kernel, a RuntimeError is raised.
 """
 from __future__ import annotations
 
-import atexit
 import ctypes
 import os
 import threading
@@ -147,8 +146,7 @@ def _load_native():
                       "build it with `python -m paper_2106_06998_b200.build`", RuntimeWarning, stacklevel=3)
         _native = _Declines()
         return _native
-    _marshal.use_library(*(ctypes.cast(getattr(L, name), c_void_p).value for name in _NATIVE_CALLS), _check)
-    atexit.register(_marshal.release)
+    _marshal.use_library(*(ctypes.cast(getattr(L, name), c_void_p).value for name in _NATIVE_CALLS), _check, workspace)
     _native = _marshal
     return _marshal
 
@@ -246,7 +244,7 @@ def _capturing() -> bool:
 
 
 # Calls on different streams or from different host threads may overlap, so each of them has a scratch buffer of its own: per
-# host thread (which gives them back when it ends), those of the streams it came to last.
+# host thread (which gives them back when it ends), those of the streams that it first came to last.  The native calls take theirs here too.
 _ws_cache = threading.local()
 _WS_STREAMS = 8
 

@@ -4,8 +4,10 @@
 //
 // A function returns None for whatever is not the ordinary case (tensors that are not dense CUDA tensors, subclasses, modes that want to see every call, a
 // layout or shape that does not fit, an option that is rarely given): binding.py then goes its own way, which is where every error is raised.
+#include <torch/csrc/Device.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
+#include <torch/csrc/utils/object_ptr.h>
 
 #include <ATen/ATen.h>
 #include <ATen/PythonTorchFunctionTLS.h>
@@ -20,7 +22,7 @@
 
 namespace {
 
-// Entry points of the library that binding.py has loaded, and its function that raises for a status.
+// Entry points of the library that binding.py has loaded, and its functions that raise for a status and hand out scratch buffers.
 struct Library {
   decltype(&xconv_workspace_bytes) workspace_bytes;
   decltype(&xconv_forward) forward;
@@ -32,7 +34,7 @@ struct Library {
   decltype(&xconv_backprobe) backprobe;
   decltype(&xconv_contract) contract;
 } lib{};
-PyObject* raise_for_status = nullptr;
+PyObject *raise_for_status = nullptr, *workspace = nullptr;
 
 bool watched() {      // modes that are to see the tensor functions of the Python path
   return at::impl::PythonTorchFunctionTLS::stack_len() > 0 || c10::impl::TorchDispatchModeTLS::any_modes_set();
@@ -126,25 +128,29 @@ size_t scratch_bytes(const xconv_desc& d, int op) {
   return e.bytes;
 }
 
-// A scratch buffer per host thread and stream, the eight streams used last, as binding.workspace keeps them; none is kept from a capture.
-struct Scratch { c10::DeviceIndex device; cudaStream_t stream; at::Tensor buffer; };
-struct ScratchPool { std::vector<Scratch> kept; };
-thread_local ScratchPool pool;
+// binding.workspace's buffer for this thread and stream.  That pool owns it; what is kept here only finds it again without the interpreter, and holds nothing alive.
+struct Found { c10::DeviceIndex device; cudaStream_t stream; c10::weak_intrusive_ptr<c10::TensorImpl> buffer; };
+thread_local std::vector<Found> found;
 
 at::Tensor scratch(size_t bytes, const at::Tensor& like, cudaStream_t stream) {
-  const auto fresh = [&] { return at::empty({(int64_t)std::max<size_t>(bytes, 256)}, like.options().dtype(at::kByte).requires_grad(false)); };
-  if (stream && c10::cuda::currentStreamCaptureStatusMayInitCtx() != c10::cuda::CaptureStatus::None) return fresh();
-  auto& kept = pool.kept;
+  if (stream && c10::cuda::currentStreamCaptureStatusMayInitCtx() != c10::cuda::CaptureStatus::None)      // (the graph's own, as binding.workspace does)
+    return at::empty({(int64_t)std::max<size_t>(bytes, 256)}, like.options().dtype(at::kByte).requires_grad(false));
   const c10::DeviceIndex device = like.device().index();
-  for (size_t i = 0; i < kept.size(); ++i)
-    if (kept[i].device == device && kept[i].stream == stream) {
-      if ((size_t)kept[i].buffer.numel() >= bytes) return kept[i].buffer;
-      kept.erase(kept.begin() + (long)i);
+  for (size_t i = 0; i < found.size(); ++i)
+    if (found[i].device == device && found[i].stream == stream) {
+      auto impl = found[i].buffer.lock();
+      if (impl && (size_t)impl->numel() >= bytes) return at::Tensor(std::move(impl));
+      found.erase(found.begin() + (long)i);
       break;
     }
-  if (kept.size() >= 8) kept.erase(kept.begin());
-  kept.push_back({device, stream, fresh()});
-  return kept.back().buffer;
+  THPObjectPtr where(THPDevice_New(like.device()));
+  THPObjectPtr buffer(where ? PyObject_CallFunction(workspace, "nO", (Py_ssize_t)bytes, where.get()) : nullptr);
+  if (!buffer) throw python_error();
+  TORCH_CHECK(THPVariable_Check(buffer.get()), "workspace() returns a tensor");
+  at::Tensor t = THPVariable_Unpack(buffer.get());
+  if (found.size() >= 8) found.erase(found.begin());
+  found.push_back({device, stream, c10::weak_intrusive_ptr<c10::TensorImpl>(t.getIntrusivePtr())});
+  return t;
 }
 
 at::Tensor image_like(const Image& g, int64_t n, int64_t c) {
@@ -309,10 +315,10 @@ PyObject* contract(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   XM_END
 }
 
-// use_library(address of each entry point in the order of Library, raise(status, name))
+// use_library(address of each entry point in the order of Library, raise(status, name), workspace(bytes, device))
 PyObject* use_library(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   constexpr Py_ssize_t N = sizeof(Library) / sizeof(void*);
-  if (nargs != N + 1) { PyErr_SetString(PyExc_TypeError, "use_library takes the entry points and a function"); return nullptr; }
+  if (nargs != N + 2) { PyErr_SetString(PyExc_TypeError, "use_library takes the entry points and two functions"); return nullptr; }
   void* at[N];
   for (Py_ssize_t i = 0; i < N; ++i) {
     at[i] = PyLong_AsVoidPtr(a[i]);
@@ -321,19 +327,15 @@ PyObject* use_library(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   std::memcpy(&lib, at, sizeof lib);
   Py_INCREF(a[N]);
   Py_XSETREF(raise_for_status, a[N]);
-  Py_RETURN_NONE;
-}
-
-// release(): gives back this thread's scratch buffers (at the interpreter's exit: before CUDA goes).
-PyObject* release(PyObject*, PyObject*) {
-  pool.kept.clear();
+  Py_INCREF(a[N + 1]);
+  Py_XSETREF(workspace, a[N + 1]);
   Py_RETURN_NONE;
 }
 
 PyMethodDef methods[] = {
 #define XM_FAST(F) {#F, (PyCFunction)(void (*)(void))F, METH_FASTCALL, nullptr}
     XM_FAST(forward), XM_FAST(sketch), XM_FAST(sketch_seeded), XM_FAST(wgrad), XM_FAST(wgrad_seeded), XM_FAST(dgrad), XM_FAST(backprobe), XM_FAST(contract),
-    XM_FAST(use_library), {"release", release, METH_NOARGS, nullptr}, {nullptr, nullptr, 0, nullptr}};
+    XM_FAST(use_library), {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module_def = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace

@@ -167,6 +167,35 @@ def test_scratch_buffers_are_bounded_and_given_back():
     assert torch.cuda.memory_allocated() < before + nbytes
 
 
+def test_both_paths_take_one_buffer():
+    """A thread that mixes calls of both paths on a stream holds one scratch buffer, the larger one; a smaller call finds it, and it is not held beyond the pool."""
+    small, large = _layer(8, 32, 64, (40, 40), 16, torch.bfloat16), _layer(16, 32, 64, (40, 40), 32, torch.bfloat16)
+    sizes = [xb.workspace_bytes(xb.make_desc(len(d["X"]), 32, 64, 40, 40, d["r"], torch.bfloat16), xb.OP_WGRAD) for d in (small, large)]
+    scale = torch.ones(32, device="cuda")
+    held = []
+
+    def job():
+        with torch.cuda.stream(torch.cuda.Stream()):
+            for d, kw in ((small, {}), (small, dict(chan_scale=scale)), (large, dict(chan_scale=scale)), (large, {}), (small, {})):
+                xb.xconv_wgrad(d["S"], d["dY"], d["Z"], **kw)
+                held.append(torch.cuda.memory_allocated() - before)
+            torch.cuda.current_stream().synchronize()
+            del xb._ws_cache.buffers
+            held.append(torch.cuda.memory_allocated() - before)
+            xb.xconv_wgrad(small["S"], small["dY"], small["Z"])
+            torch.cuda.current_stream().synchronize()
+
+    torch.cuda.synchronize()
+    before = torch.cuda.memory_allocated()
+    t = threading.Thread(target=job)
+    t.start()
+    t.join()
+    slack = 2 << 20                                                 # the allocator hands out whole blocks of 2 MB above 10 MB, and leaves a rest below 1 MB with its block
+    assert sizes[0] > 4 * slack and sizes[1] > sizes[0] + slack
+    for got, want in zip(held, (sizes[0], sizes[0], sizes[1], sizes[1], sizes[1], 0)):
+        assert want <= got <= want + slack
+
+
 def test_threads_and_streams_share_no_scratch():
     layers = [_layer(16, 3, 32, (40, 44), 32, torch.bfloat16, seed=1), _layer(8, 16, 24, (30, 33), 40, torch.float16, seed=2), _layer(4, 8, 8, (64, 64), 9, torch.float32, seed=3)]
     want = [[t for c in _calls(d) for t in (lambda o: o if isinstance(o, tuple) else (o,))(c())] for d in layers]
