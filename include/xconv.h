@@ -136,6 +136,19 @@ size_t xconv_workspace_bytes(const xconv_desc* desc, int op);
 /* Engine the dominant kernel of `op` runs on for this layer (XCONV_ENGINE_NONE if unsupported). */
 int xconv_engine_for(const xconv_desc* desc, int op);
 
+/* Forms of the kernels that `op` takes on this layer, given the scratch that xconv_workspace_bytes asks for: a sum of the values below, 0 for
+ * the general forms or an invalid descriptor.  XCONV_OP_FORWARD and XCONV_OP_DGRAD speak of the convolution alone.  The forms differ in time, not in what
+ * they compute; the rules that choose between them may change.  Host arithmetic only. */
+typedef enum {
+  XCONV_VARIANT_SMALL_TILES = 1, /* convolution, contraction: float layers of a few microseconds */
+  XCONV_VARIANT_WALK = 2,        /* convolution: along an axis of the image, one product for all kernel offsets along it */
+  XCONV_VARIANT_ROW_BOXES = 4,   /* sketch, back-probe: long rows, copied eight at a time */
+  XCONV_VARIANT_STREAM = 8,      /* sketch, back-probe: few samples or probes, through registers */
+  XCONV_VARIANT_SIGN_PAIRS = 16, /* seeded back-probe in a stream: 128 signs of a row drawn together */
+  XCONV_VARIANT_WIDE_SUMS = 32   /* sketch, contraction: 32 threads to a sum of many partial ones */
+} xconv_variant;
+int xconv_variants_for(const xconv_desc* desc, int op);
+
 /* Algorithm 1, forward pass: Y = conv(X, W) (step 1, Eq. 5) and S = Z^T X (step 3).
  * X [B,H,W,Cin], W [Cout,KH,KW,Cin], Z [r,H,W,Cin] in desc.dtype; Y [B,H,W,Cout] in desc.dtype;
  * sketch [r,B] float.  After this call the caller may drop X and keep only `sketch` and Z (or the

@@ -24,11 +24,12 @@ LIB_PATH = os.path.join(_HERE, "libxconv.so")
 XCONV_F32, XCONV_BF16, XCONV_F16 = 0, 1, 2
 OP_FORWARD, OP_WGRAD, OP_DGRAD, OP_SKETCH, OP_BACKPROBE, OP_CONTRACT, OP_SKETCH_SEEDED, OP_WGRAD_SEEDED, OP_WGRAD_INDEPENDENT = 0, 1, 2, 3, 4, 5, 6, 7, 8
 OP_SKETCH_SEEDED_GAUSSIAN, OP_WGRAD_SEEDED_GAUSSIAN = 9, 10
+VARIANT_NAMES = {1: "small_tiles", 2: "walk", 4: "row_boxes", 8: "stream", 16: "sign_pairs", 32: "wide_sums"}
 ENGINE_NAMES = {0: "none", 1: "simt_f32", 2: "tcgen05_bf16", 3: "tcgen05_f16", 4: "tcgen05_f32"}
 STATUS_OK = 0
 
 # every symbol include/xconv.h declares
-EXPORTS = ("xconv_workspace_bytes", "xconv_engine_for", "xconv_forward", "xconv_sketch", "xconv_wgrad",
+EXPORTS = ("xconv_workspace_bytes", "xconv_engine_for", "xconv_variants_for", "xconv_forward", "xconv_sketch", "xconv_wgrad",
            "xconv_dgrad", "xconv_probes_from_seed", "xconv_sketch_seeded", "xconv_wgrad_seeded", "xconv_backprobe_bytes", "xconv_backprobe", "xconv_contract", "xconv_host_arena_bytes", "xconv_sketch_wgrad_host", "xconv_sketch_static",
            "xconv_workspace_status", "xconv_selftest_wait_limit", "xconv_measure_fma_rate",
            "xconv_sketch_independent", "xconv_wgrad_independent", "xconv_zero_blocks", "xconv_zero_blocks_used",
@@ -68,6 +69,7 @@ def lib() -> ctypes.CDLL:
     P = POINTER(XConvDesc)
     L.xconv_workspace_bytes.argtypes = [P, c_int]; L.xconv_workspace_bytes.restype = c_size_t
     L.xconv_engine_for.argtypes = [P, c_int]; L.xconv_engine_for.restype = c_int
+    L.xconv_variants_for.argtypes = [P, c_int]; L.xconv_variants_for.restype = c_int
     L.xconv_forward.argtypes = [P, c_void_p, c_void_p, c_void_p, c_void_p, c_void_p, c_void_p, c_size_t, c_void_p]
     L.xconv_forward.restype = c_int
     L.xconv_sketch.argtypes = [P, c_void_p, c_void_p, c_void_p, c_void_p, c_size_t, c_void_p]
@@ -275,6 +277,12 @@ def workspace_bytes(desc: XConvDesc, op: int) -> int:
 
 def engine_for(desc: XConvDesc, op: int) -> str:
     return ENGINE_NAMES[lib().xconv_engine_for(ctypes.byref(desc), op)]
+
+
+def variants_for(desc: XConvDesc, op: int) -> set:
+    """Names of the forms of the kernels that a call takes (host arithmetic only; see include/xconv.h)."""
+    bits = lib().xconv_variants_for(ctypes.byref(desc), op)
+    return {name for bit, name in VARIANT_NAMES.items() if bits & bit}
 
 
 def _check(status: int, where: str):

@@ -455,11 +455,12 @@ static size_t probes_bytes(const xconv_desc* d) {
 // Every block of a dependent launch pays for its go-ahead and its wait: 51200 blocks (5 x 5, 128 -> 512 channels) 34 us without,
 // 54 with; 36000 blocks 26 and 38; 18000 14 and 20.  It saves 2 us of launch (1280 blocks 22.6 without, 20.3 with).
 static const unsigned REDUCE_PDL_BLOCKS = 6000;
+// Many splits of few outputs: four times the threads to an output, and twice the loads in flight (us a launch, 441 to 4096 outputs of 128 to 296 splits:
+// 5.9 -> 4.0; with the loads alone few splits of many outputs lose, 65536 of 7 3.8 -> 5.1).
+static bool wide_sums(long count, int splits) { return splits >= 64 && count <= 16384; }
 static xconv_status run_reduce(const float* part, float* out, long count, int splits, float alpha, const float* chan_scale,
                                int period, cudaStream_t st) {
-  // Many splits of few outputs: four times the threads to an output, and twice the loads in flight (us a launch, 441 to 4096 outputs of 128 to 296 splits:
-  // 5.9 -> 4.0; with the loads alone few splits of many outputs lose, 65536 of 7 3.8 -> 5.1).
-  const bool few = splits >= 64 && count <= 16384;
+  const bool few = wide_sums(count, splits);
   const dim3 grid((unsigned)cdiv(count, few ? 8 : 32)), block(256);
   cudaError_t e;
   if (few) {
@@ -876,6 +877,38 @@ static xconv_status run_rebuild_indep(const xconv_desc* d, const float* S, const
   return check_launch();
 }
 
+// Forms of the kernels (see xconv_variants_for), step by step as the plans and the launchers above choose them.
+static int sketch_variants(const xconv_desc* d, const SketchPlan& p) {
+  if (p.tc) return p.t.row_boxes ? XCONV_VARIANT_ROW_BOXES : 0;
+  const int splits = p.stream ? p.s.splits : p.split ? (int)p.g.splits : p.splits;
+  return (p.stream ? XCONV_VARIANT_STREAM : 0) | (wide_sums((long)d->r * d->B, splits) ? XCONV_VARIANT_WIDE_SUMS : 0);
+}
+static int backprobe_variants(const xconv_desc* d, const WgradPlan& p, bool redrawn) {
+  const xconv_desc f = flat(d);
+  if (p.split_bp) return 0;
+  if (p.stream_bp) return XCONV_VARIANT_STREAM | (redrawn && tc_stream_draws_pairs(&f) ? XCONV_VARIANT_SIGN_PAIRS : 0);
+  return p.tc_bp && tc_backprobe_row_boxes(&f, redrawn) ? XCONV_VARIANT_ROW_BOXES : 0;
+}
+static int contract_variants(const xconv_desc* d, const WgradPlan& p) {
+  if (p.halo || p.split || p.tc_ct) return 0;
+  return (small_contract_serves(d) ? XCONV_VARIANT_SMALL_TILES : 0) |
+         (wide_sums((long)d->Cout * d->Cin * kdepth(d) * d->KH * d->KW, p.splits) ? XCONV_VARIANT_WIDE_SUMS : 0);
+}
+static int wgrad_variants(const xconv_desc* d, bool seeded) {
+  SwappedWgrad sw;
+  const WgradPlan p = plan_wgrad(d, &sw);
+  if (sw.on) return backprobe_variants(&sw.d1, sw.p1, seeded && wgrad_redraws(d)) | contract_variants(&sw.d2, sw.p2);
+  return backprobe_variants(d, p, false) | contract_variants(d, p);
+}
+static int conv_variants(const xconv_desc* d, bool dgrad) {
+  xconv_desc e;
+  TcConvPlan t;
+  ConvSplitPlan f;
+  if (plan_conv_f32(d, dgrad, &f)) return 0;
+  if (plan_conv(d, dgrad, &e, &t)) return t.slide ? XCONV_VARIANT_WALK : 0;
+  return d->dtype == XCONV_F32 && small_conv_serves(d) ? XCONV_VARIANT_SMALL_TILES : 0;
+}
+
 int launches() { return g_launches; }
 void count_launch() { ++g_launches; }
 void set_cuda_error(int e) { g_last_cuda_error = e; }
@@ -934,6 +967,27 @@ int xconv_engine_for(const xconv_desc* desc, int op) {
       return plan_conv(desc, op == XCONV_OP_DGRAD, &e, &t) ? tc : XCONV_ENGINE_SIMT_F32;
     }
     default: return XCONV_ENGINE_NONE;
+  }
+}
+
+int xconv_variants_for(const xconv_desc* desc, int op) {
+  if (validate(desc) != XCONV_OK) return 0;
+  switch (op) {
+    case XCONV_OP_FORWARD: return conv_variants(desc, false);
+    case XCONV_OP_DGRAD: return conv_variants(desc, true);
+    case XCONV_OP_SKETCH: {
+      const xconv_desc f = flat(desc);
+      return sketch_variants(&f, plan_sketch(desc));
+    }
+    case XCONV_OP_SKETCH_SEEDED: {
+      const xconv_desc f = flat(desc);
+      return sketch_variants(&f, plan_sketch(desc, true));
+    }
+    case XCONV_OP_BACKPROBE: return backprobe_variants(desc, plan_wgrad(desc), false);
+    case XCONV_OP_CONTRACT: return contract_variants(desc, plan_wgrad(desc));
+    case XCONV_OP_WGRAD: return wgrad_variants(desc, false);
+    case XCONV_OP_WGRAD_SEEDED: return wgrad_variants(desc, true);
+    default: return 0;
   }
 }
 

@@ -630,12 +630,13 @@ bool tc_backprobe_streams(const xconv_desc* d, bool other) {
   return !other || (d->r <= 16 && (d->B <= 64 || Q >= 2L * 64 * 16 * 148));
 }
 
+// Pairs of groups draw half the blocks, but only where every warp of the grid has a group of its own all the same (16 rows: 256 terms, 2.1 M
+// columns 91 -> 77 us, 498 terms, 4608 columns 28 -> 34).  Above 16 rows their accumulators would not fit the registers.
+bool tc_stream_draws_pairs(const xconv_desc* d) { return d->r <= 16 && cdiv_((long)d->H * d->W * d->Cout, 64) > 8L * 148 * 2; }
+
 template <bool F16, int MT>
-static cudaError_t launch_backprobe_seeded(const BackprobeStream& q, const SignKeys& signs, bool split, unsigned grid, size_t smem, cudaStream_t st) {
-  // Pairs of groups draw half the blocks, but only where every warp of the grid has a group of its own all the same (16 rows: 256 terms, 2.1 M
-  // columns 91 -> 77 us, 498 terms, 4608 columns 28 -> 34).
+static cudaError_t launch_backprobe_seeded(const BackprobeStream& q, const SignKeys& signs, bool pairs, bool split, unsigned grid, size_t smem, cudaStream_t st) {
   constexpr int PAIR = MT == 1 ? 2 : 1;
-  const bool pairs = q.groups > 8L * 148 * 2;
   void (*kernel)(BackprobeStream, SignKeys);
   if (split) kernel = pairs ? backprobe_seeded_kernel<F16, MT, PAIR, true> : backprobe_seeded_kernel<F16, MT, 1, true>;
   else if (MT > 1) return cudaErrorInvalidValue;
@@ -646,8 +647,8 @@ static cudaError_t launch_backprobe_seeded(const BackprobeStream& q, const SignK
 }
 
 template <bool F16, int MT>
-static cudaError_t launch_backprobe_stream(const BackprobeStream& q, const SignKeys* signs, bool split, unsigned grid, size_t smem, cudaStream_t st) {
-  if (signs) return launch_backprobe_seeded<F16, MT>(q, *signs, split, grid, smem, st);
+static cudaError_t launch_backprobe_stream(const BackprobeStream& q, const SignKeys* signs, bool pairs, bool split, unsigned grid, size_t smem, cudaStream_t st) {
+  if (signs) return launch_backprobe_seeded<F16, MT>(q, *signs, pairs, split, grid, smem, st);
   constexpr int KC = MT == 1 ? 2 : 1;
   void (*kernel)(BackprobeStream);
   if (split) kernel = backprobe_stream_kernel<F16, MT, KC, false, true>;
@@ -678,15 +679,16 @@ xconv_status tc_run_backprobe_stream(const xconv_desc* d, const float* S, long s
   const int mt = d->r > 32 ? 4 : d->r > 16 ? 2 : 1;
   const unsigned grid = (unsigned)std::min<long>(cdiv_(q.groups, 8), 148L * (mt == 4 ? 1 : 2));
   const size_t smem = stream_smem(mt, d->B, seed != nullptr, split);
+  const bool pairs = tc_stream_draws_pairs(d);
   cudaError_t e;
   if (d->dtype == XCONV_F16)
-    e = mt == 4 ? launch_backprobe_stream<true, 4>(q, signs, split, grid, smem, st)
-        : mt == 2 ? launch_backprobe_stream<true, 2>(q, signs, split, grid, smem, st)
-                  : launch_backprobe_stream<true, 1>(q, signs, split, grid, smem, st);
+    e = mt == 4 ? launch_backprobe_stream<true, 4>(q, signs, pairs, split, grid, smem, st)
+        : mt == 2 ? launch_backprobe_stream<true, 2>(q, signs, pairs, split, grid, smem, st)
+                  : launch_backprobe_stream<true, 1>(q, signs, pairs, split, grid, smem, st);
   else
-    e = mt == 4 ? launch_backprobe_stream<false, 4>(q, signs, split, grid, smem, st)
-        : mt == 2 ? launch_backprobe_stream<false, 2>(q, signs, split, grid, smem, st)
-                  : launch_backprobe_stream<false, 1>(q, signs, split, grid, smem, st);
+    e = mt == 4 ? launch_backprobe_stream<false, 4>(q, signs, pairs, split, grid, smem, st)
+        : mt == 2 ? launch_backprobe_stream<false, 2>(q, signs, pairs, split, grid, smem, st)
+                  : launch_backprobe_stream<false, 1>(q, signs, pairs, split, grid, smem, st);
   count_launch();
   if (e != cudaSuccess) { set_cuda_error((int)e); return XCONV_ERR_CUDA; }
   return XCONV_OK;

@@ -86,6 +86,7 @@ bool tc_sketch_can_redraw(const xconv_desc* d);
 // the kernel from the Philox stream of *seed -- the first step of the estimator when it sums over the probes first.
 xconv_status tc_run_backprobe(const xconv_desc* d, const TcWgradPlan& p, const void* S_bf16, const void* dY,
                               void* L, char* ws_head, cudaStream_t st, const unsigned long long* seed = nullptr);
+bool tc_backprobe_row_boxes(const xconv_desc* d, bool seeded);      // dY copied eight rows at a time
 xconv_status tc_run_contract(const xconv_desc* d, const TcWgradPlan& p, const void* L, const void* Z, float* dW,
                              float alpha, char* ws_head, char* part, cudaStream_t st);
 
@@ -101,6 +102,7 @@ bool tc_plan_sketch_stream(const xconv_desc* d, bool seeded, StreamSketchPlan* p
 xconv_status tc_run_sketch_stream(const xconv_desc* d, const StreamSketchPlan& p, const void* X, const void* Z, float* part,
                                   char* ws_head, cudaStream_t st, const unsigned long long* seed);
 bool tc_backprobe_streams(const xconv_desc* d, bool other);
+bool tc_stream_draws_pairs(const xconv_desc* d);                     // a warp of the seeded one takes two groups of 64 columns
 // (`split`: S with more than its 16-bit rounding, see the kernel.)
 xconv_status tc_run_backprobe_stream(const xconv_desc* d, const float* S, long s_row, long s_k, const void* dY, void* L,
                                      bool split, char* ws_head, cudaStream_t st, const unsigned long long* seed);

@@ -1483,6 +1483,10 @@ __global__ void __launch_bounds__(1024) list_nonzero_blocks(const unsigned char*
   if (threadIdx.x == 0) { row[0] = (uint32_t)base; row[1 + base] = 0u; }
 }
 
+// Rows of dY 2 MB apart or more: boxes of eight rows, as in the sketch (plan there).  64 channels of 160 x 160, 128 samples and probes 200 -> 155 us,
+// 200 samples, 80 probes 217 -> 159 (4.2 -> 5.8 TB/s), 64 and 128 152 -> 137; rows of 1.6 MB 78 -> 79 and 85 -> 88.
+bool tc_backprobe_row_boxes(const xconv_desc* d, bool seeded) { return !seeded && (long)d->H * d->W * d->Cout >= (1L << 20); }
+
 xconv_status tc_run_backprobe(const xconv_desc* d, const TcWgradPlan& pl, const void* S_bf16, const void* dY,
                               void* L, char* ws_head, cudaStream_t st, const unsigned long long* seed) {
   const long Q = (long)d->H * d->W * d->Cout;
@@ -1496,9 +1500,7 @@ xconv_status tc_run_backprobe(const xconv_desc* d, const TcWgradPlan& pl, const 
   const uint64_t db[3] = {64, (uint64_t)d->B, (uint64_t)(Q / 64)};
   const uint64_t sa[1] = {(uint64_t)d->B * 2}, sb[2] = {(uint64_t)Q * 2, 128};
   const uint32_t box_a[2] = {64, (uint32_t)pl.bp_rows_box};           // 128-byte rows whatever bk is (zero fill past B)
-  // Rows of dY 2 MB apart or more: boxes of eight rows, as in the sketch (plan there).  64 channels of 160 x 160, 128 samples and probes 200 -> 155 us,
-  // 200 samples, 80 probes 217 -> 159 (4.2 -> 5.8 TB/s), 64 and 128 152 -> 137; rows of 1.6 MB 78 -> 79 and 85 -> 88.
-  const bool row_boxes = !seed && Q >= (1L << 20);
+  const bool row_boxes = tc_backprobe_row_boxes(d, seed != nullptr);
   const uint32_t box_b[3] = {64, row_boxes ? 8u : (uint32_t)bk, row_boxes ? (uint32_t)pl.bp_tile_n / 64 : 1};
   // (seeded: the streamed operand is never read, and its map stands in with the output's address)
   if (!make_map(&ma, S_bf16, 2, da, sa, box_a, f16) || !make_map(&mb, seed ? L : dY, 3, db, sb, box_b, f16)) return XCONV_ERR_CUDA;
