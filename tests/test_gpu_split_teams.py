@@ -1,5 +1,5 @@
 """Float sketches and back-probes whose stages are converted by teams of warps in turn (gemm_split.cu), with as many k-blocks a CTA as make the
-teams' last turns differ.  Whole numbers: every product and partial sum is exact, so the results are too."""
+teams' last turns differ; and sums of many splits with 32 threads to an output, of each kernel that leaves such.  Whole numbers: every product and partial sum is exact, so the results are too."""
 import pytest
 import torch
 
@@ -44,3 +44,20 @@ def test_float_backprobe_of_whole_numbers_is_exact(r, B, C, H, W):
     dY = torch.randint(-9, 10, (B, H, W, C), generator=g, device="cuda").float()
     L = xb.xconv_backprobe(S, dY.permute(0, 3, 1, 2))
     assert torch.equal(L.permute(0, 2, 3, 1).reshape(r, -1).double(), S.double() @ dY.reshape(B, -1).double())
+
+
+@pytest.mark.parametrize("dtype,r,B,C,H,W,wide", [
+    ("f32", 7, 3, 16, 32, 32, True),          # multiply-adds; a last block of five outputs
+    ("f32", 128, 128, 32, 64, 64, True),      # split operands, the most outputs that are summed so
+    ("f32", 129, 128, 32, 64, 64, False),     # ... and the first that are not
+    ("f32", 70, 33, 32, 128, 128, True),
+    ("bf16", 101, 5, 16, 64, 64, True),       # in a stream
+])
+def test_sums_of_many_splits_are_exact(dtype, r, B, C, H, W, wide):
+    storage = torch.float32 if dtype == "f32" else torch.bfloat16
+    assert ("wide_sums" in xb.variants_for(xb.make_desc(B, C, 1, H, W, r, storage), xb.OP_SKETCH)) == wide
+    g = torch.Generator(device="cuda").manual_seed(r * 1000 + B)
+    X = torch.randint(-9, 10, (B, H, W, C), generator=g, device="cuda").to(storage)
+    Z = (torch.randint(0, 2, (r, H, W, C), generator=g, device="cuda") * 2 - 1).to(storage)
+    S = xb.xconv_sketch(X.permute(0, 3, 1, 2), Z.permute(0, 3, 1, 2))
+    assert torch.equal(S.double(), Z.reshape(r, -1).double() @ X.reshape(B, -1).double().T)
