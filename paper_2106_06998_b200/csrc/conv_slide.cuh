@@ -1,7 +1,7 @@
 // The exact convolutions of layers with few channels out (conv_tc.cu), along one axis of the image.
 //
-// An MMA of 32 columns holds the tensor pipe as long as shared memory takes to hand it 128 rows of the input (32 clocks and a quarter of its
-// columns), and the issuing warp some 60 clocks whatever its width.  So one MMA here serves the KS kernel offsets along one axis, the image
+// An MMA needs shared memory for 32 clocks and a quarter of its columns to be handed 128 rows of the input (40 clocks for 32 columns, 56 for 96), and one follows
+// another no sooner than some 56 to 62 clocks in the kernels measured here, whatever its width up to 96.  So one MMA here serves the KS kernel offsets along one axis, the image
 // rows (planar layers) or the planes (3 x 3 x 3 kernels): the input plane s, moved by one of the other offsets, is multiplied with the weights of
 // all KS offsets side by side, and the sums go to the KS outputs s - pad .. s + pad, whose accumulators lie side by side in tensor memory:
 //
@@ -12,7 +12,7 @@
 // lies between the outputs an MMA is done in two, and so is the first one of a plane, which starts the newest output's sum instead of adding
 // to it.  A planar layer's tile has no halo along the axis and takes rows of several images where one is shorter than 128 pixels.
 //
-// What bounds it: 3 x 3 kernels of 32 channels the issuing warp (some 230 clocks a plane beside 45 an MMA), volumes and wider layers the pipe (62 clocks an MMA
+// What bounds it (tensor pipe active 0.25 on 256 x 256, 0.32 in volumes; memory at 0.4 and 0.1 of its rate): 3 x 3 kernels of 32 channels the issuing warp (some 230 clocks a plane beside 45 an MMA), volumes and wider layers the pipe (62 clocks an MMA
 // of 96 columns, 96 one of 192).  us a launch, one MMA per offset -> this: 16 images of 256 x 256, 32 -> 32 channels 42.2 -> 33.4; 4 volumes of 48^3,
 // 32 -> 32 46.2 -> 36.5; 208 images of 123 x 126, 16 -> 24 108 -> 82; 5 x 5, 375 of 97 x 97, 32 -> 16 328 -> 208; 5 volumes of 22 x 34 x 34, 96 -> 24 (weights kept
 // here, streamed there) 153 -> 60.

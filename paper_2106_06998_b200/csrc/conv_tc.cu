@@ -498,7 +498,8 @@ bool tc_plan_conv(const xconv_desc* d, bool dgrad, TcConvPlan* p) {
           if (room - w_all >= 2 * o_bytes + 2 * a_slot) p->o_per = 2;
           // Long runs of patches get as many boxes in flight as fit: four narrow ones leave the copies waiting for memory (1 x 1, 192 -> 24 channels,
           // 46 images of 129 x 129 75.9 -> 66.1 us, dX of 96 -> 16, 3 x 3, 16 of 188 x 256 46.9 -> 42.3; with runs of six 11.6 -> 12.0;
-          // 1 x 1 with more channels out than in is bound by its stores: 128 -> 192, 102 of 59 x 59 40.2 -> 41.3).
+          // 1 x 1 with more channels out than in is bound by its stores: 128 -> 192, 102 of 59 x 59 40.2 -> 41.3; with as many, 18 convolutions of
+          // 16 to 256, 1.006 of the time: dX of 96, 64 of 97 x 97 47.4 -> 42.2, but of 64, 300 of 90 x 90 101 -> 118).
           p->a_slots = (int)std::min<uint32_t>(per_cta >= 16 && (K > 1 || Ci > Co) ? CV_A_SLOTS : 4, 2 + (room - w_all - (p->o_per == 2 ? 2 * o_bytes : 0)) / a_slot);
         } else {
           p->a_slots = room >= a_slot + 4 * w_tile ? 3 : 2;
