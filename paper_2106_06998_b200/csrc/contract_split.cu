@@ -245,6 +245,7 @@ contract_split_kernel(const __grid_constant__ CUtensorMap map_l, const __grid_co
   const uint32_t n = (uint32_t)((unsigned long long)p.items * (split + 1) / p.splits) - i0;     // patches of this CTA (>= 1)
   const SplitUnit u = split_unit(p, ug);
   const int chains = (p.ksteps + p.chunk - 1) / p.chunk;
+  const int width = p.KS == 1 ? p.cols : min(p.j_per, p.KS - u.jg * p.j_per) * 32;      // columns of this unit's MMAs
   int again = 0;                                     // a sum is not finite
 
   if (!go) {
@@ -255,7 +256,6 @@ contract_split_kernel(const __grid_constant__ CUtensorMap map_l, const __grid_co
     const uint32_t s0 = (base & 0x3FFFFu) >> 4, stage16 = p.stage_bytes >> 4, ap = p.a_plane >> 4, bp = p.b_plane >> 4;
     const uint32_t a_add = p.a_lo0 + (p.rows_on_a ? (uint32_t)(u.mg % p.tiles) * p.a_tile16 : 0u);
     const uint32_t b_add = p.b_lo0 + (p.a_bytes >> 4) + (uint32_t)(u.jg * p.j_per) * 4u;             // (a pixel: 64 bytes)
-    const int shifts = min(p.j_per, p.KS - u.jg * p.j_per), width = p.KS == 1 ? p.cols : shifts * 32;
     const uint32_t idesc = p.idesc | ((uint32_t)(width >> 3) << 17);
     const uint32_t a_step = p.a_step16, b_step = p.b_step16, a_hi = p.a_hi, b_hi = p.b_hi;
     const uint32_t d = tmem_base + own * CT_COLS;
@@ -338,7 +338,9 @@ contract_split_kernel(const __grid_constant__ CUtensorMap map_l, const __grid_co
     }
   } else if (warp >= SP_EPILOGUE) {
     // ------------------------------------------------------------------ epilogue: chains to registers, registers to partial sums
-    const int quad = warp & 3, half = (warp - SP_EPILOGUE) >> 2, groups = p.cols >> 4;      // column groups half, half + 2, ... of 16
+    // Column groups half, half + 2, ... of 16, of the columns that the MMAs write: 5 x 5 kernels have units of two shifts, whose third lies in tensor memory
+    // as the kernel before left it.  (Read, and not finite by chance, it sent the block through split_again for nothing, 22 -> 32 us.)
+    const int quad = warp & 3, half = (warp - SP_EPILOGUE) >> 2, groups = width >> 4;
     const uint32_t tmem_q = tmem_base + ((uint32_t)(quad * 32) << 16);
     float sum[3][16];
 #pragma unroll
