@@ -478,13 +478,14 @@ static xconv_status run_reduce(const float* part, float* out, long count, int sp
 
 template <typename T>
 static xconv_status run_sketch_simt(const xconv_desc* d, const SketchPlan& p, const void* X, const void* Z,
-                                    float* S, char* ws, cudaStream_t st) {
+                                    float* S, char* ws, cudaStream_t st, bool held) {
   const long K = (long)d->H * d->W * d->Cin;
   float* part = reinterpret_cast<float*>(ws + p.part_off);
   dim3 grid((unsigned)cdiv(d->B, 64), (unsigned)cdiv(d->r, 64), (unsigned)p.splits);
   // (Started under the kernel before only if it is over at once: grids of a whole wave are dealt unevenly to SMs that that one still uses, 512 x 32 rows, 1176
-  // terms 10 -> 12.8 us, and the copies go through what L1 it leaves, 16 x 53 rows, 10816 terms in a training step 83 -> 86; 8 x 8 rows, 16384 terms 10.3 -> 8.0.)
-  const bool small = (long)grid.x * grid.y * grid.z <= 148 && (d->r + d->B) * K <= 1L << 19;
+  // terms 10 -> 12.8 us, and the copies go through what L1 it leaves, 16 x 53 rows, 10816 terms in a training step 83 -> 86; 8 x 8 rows, 16384 terms 10.3 -> 8.0.
+  // Behind a convolution that holds whole SMs that is next to nothing: the forward call of 16 -> 96 channels, 78 images of 4 x 34, r = 6, started under it 22.9 -> 28.5.)
+  const bool small = !held && (long)grid.x * grid.y * grid.z <= 148 && (d->r + d->B) * K <= 1L << 19;
   if (std::is_same<T, float>::value && K % 4 == 0 && p.k_per_split % GT_KS == 0) {
     const size_t smem = (size_t)GT_STAGES * 128 * GT_LD * sizeof(float);
     cudaError_t ea = cudaFuncSetAttribute(gemm_tn_simt_async, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -509,8 +510,9 @@ static bool sketch_redraws(const xconv_desc* d, const SketchPlan& p) {
   return p.stream || (p.tc && tc_sketch_can_redraw(&fl));
 }
 
+// `held`: the kernel before is one of the call's own that holds the SMs it runs on.
 static xconv_status run_sketch(const xconv_desc* d_, const void* X, const void* Z, float* S, void* ws,
-                               size_t ws_bytes, cudaStream_t st, const unsigned long long* seed = nullptr) {
+                               size_t ws_bytes, cudaStream_t st, const unsigned long long* seed = nullptr, bool held = false) {
   const xconv_desc fl = flat(d_);
   const xconv_desc* d = &fl;
   const SketchPlan p = plan_sketch(d, seed != nullptr);
@@ -535,9 +537,9 @@ static xconv_status run_sketch(const xconv_desc* d_, const void* X, const void* 
     xconv_status s = run_sketch_split(d, p.g, static_cast<const float*>(X), static_cast<const float*>(Z), part, w, st);
     return s == XCONV_OK ? run_reduce(part, S, (long)d->r * d->B, (int)p.g.splits, 1.0f, nullptr, 1, st) : s;
   }
-  return d->dtype == XCONV_F32 ? run_sketch_simt<float>(d, p, X, Z, S, w, st)
-         : d->dtype == XCONV_F16 ? run_sketch_simt<f16>(d, p, X, Z, S, w, st)
-                                 : run_sketch_simt<bf16>(d, p, X, Z, S, w, st);
+  return d->dtype == XCONV_F32 ? run_sketch_simt<float>(d, p, X, Z, S, w, st, held)
+         : d->dtype == XCONV_F16 ? run_sketch_simt<f16>(d, p, X, Z, S, w, st, held)
+                                 : run_sketch_simt<bf16>(d, p, X, Z, S, w, st, held);
 }
 
 template <typename T, typename TL>
@@ -674,9 +676,11 @@ static size_t conv_ws_bytes(const xconv_desc* d, bool dgrad) {
 }
 
 static xconv_status run_conv(const xconv_desc* d, bool dgrad, const void* in, const void* Wt, void* out,
-                             char* ws, size_t ws_bytes, cudaStream_t st) {
+                             char* ws, size_t ws_bytes, cudaStream_t st, bool* held = nullptr) {
   ConvSplitPlan f;
-  if (plan_conv_f32(d, dgrad, &f) && ws_bytes >= WS_HEADER + f.bytes)
+  const bool split = plan_conv_f32(d, dgrad, &f) && ws_bytes >= WS_HEADER + f.bytes;
+  if (held) *held = split;
+  if (split)
     return run_conv_split(d, f, dgrad, static_cast<const float*>(in), static_cast<const float*>(Wt), static_cast<float*>(out), ws,
                           ws + WS_HEADER, st);
   TcConvPlan t;
@@ -1155,9 +1159,10 @@ xconv_status xconv_forward(const xconv_desc* desc, const void* X, const void* W,
   if (!aligned16(ws)) return XCONV_ERR_ALIGNMENT;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   new_call();
-  s = run_conv(desc, false, X, W, Y, static_cast<char*>(ws), ws_bytes, st);
+  bool held;
+  s = run_conv(desc, false, X, W, Y, static_cast<char*>(ws), ws_bytes, st, &held);
   if (s != XCONV_OK) return s;
-  return run_sketch(desc, X, Z, sketch, ws, ws_bytes, st);
+  return run_sketch(desc, X, Z, sketch, ws, ws_bytes, st, nullptr, held);
 }
 
 xconv_status xconv_wgrad(const xconv_desc* desc, const float* sketch, const void* dY, const void* Z, float* dW,

@@ -53,3 +53,20 @@ def check(name, got, want, tol):
     assert worst <= MAX_C * tol * rms, (f"{name}: largest element error {worst:.3e} > {MAX_C:g} * {tol:.1e} * "
                                         f"rms(want) = {MAX_C * tol * rms:.3e}")
     return err
+
+
+def device_time(call, before=None, calls=1, repeats=21):
+    """Median device time of a call in us: alone behind `before`, or of `calls` in a row.  The host runs ahead of the device."""
+    times = []
+    for _ in range(repeats):
+        (before or call)()
+        torch.cuda.synchronize()
+        start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        torch.cuda._sleep(400_000 + 40_000 * calls)
+        start.record()
+        for _ in range(calls):
+            call()
+        end.record()
+        torch.cuda.synchronize()
+        times.append(start.elapsed_time(end) * 1e3 / calls)
+    return sorted(times)[len(times) // 2]

@@ -7,7 +7,7 @@ import torch
 import __graft_entry__ as entry
 from paper_2106_06998_b200 import binding as xb
 from paper_2106_06998_b200 import inputs
-from tests._util import host
+from tests._util import device_time, host
 
 pytestmark = pytest.mark.gpu
 INF, NAN, BIG = np.inf, np.nan, float(np.float32(3.4e38))
@@ -248,22 +248,6 @@ def test_time_and_status(call):
     assert all(t <= (2 if what == "one" else 3 if value != 3e38 else 4) * base + 20 for (_, what, value), t in seen.items()), (base, seen)
 
 
-def _device_time(before, call):
-    """Median time of a call behind another one, in us."""
-    times = []
-    for _ in range(21):
-        before()
-        torch.cuda.synchronize()
-        start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        torch.cuda._sleep(400000)                             # the host is ahead of the device
-        start.record()
-        call()
-        end.record()
-        torch.cuda.synchronize()
-        times.append(start.elapsed_time(end) * 1e3)
-    return sorted(times)[len(times) // 2]
-
-
 def test_what_another_kernel_left_in_tensor_memory_is_not_read():
     """5 x 5 kernels have units whose last columns no MMA writes.  Read as sums, an old NaN there sent the whole block through the sums that are not
     finite, for nothing: the same bits, 1.3 times the time."""
@@ -280,5 +264,5 @@ def test_what_another_kernel_left_in_tensor_memory_is_not_read():
         leave = lambda: xb.xconv_contract(left, Z3, 3)
         leave()
         assert torch.equal(call(), want)
-        times.append(_device_time(leave, call))
+        times.append(device_time(call, before=leave))
     assert times[1] < 1.12 * times[0], times
