@@ -62,18 +62,19 @@ __device__ __forceinline__ float4 sum_splits4(const float* src, size_t stride, i
   }
   return s;
 }
-template <int LANES, int DEEP>
-__device__ __forceinline__ float sum_splits(const float* src, size_t stride, int g, int splits) {
-  float s = 0.f;
+template <int LANES, int DEEP, int OWN>      // ... in OWN sums, which take them in turn
+__device__ __forceinline__ void sum_splits(const float* src, size_t stride, int g, int splits, float (&own)[OWN]) {
+  static_assert(DEEP % OWN == 0, "a load has the same sum in every round");
+#pragma unroll
+  for (int i = 0; i < OWN; ++i) own[i] = 0.f;
   for (int k = g; k < splits; k += DEEP * LANES) {
     float v[DEEP];
 #pragma unroll
     for (int i = 0; i < DEEP; ++i) v[i] = k + i * LANES < splits ? __ldcg(src + (size_t)(k + i * LANES) * stride) : 0.f;
 #pragma unroll
     for (int i = 0; i < DEEP; ++i)
-      if (k + i * LANES < splits) s += v[i];
+      if (k + i * LANES < splits) own[i % OWN] += v[i];
   }
-  return s;
 }
 
 __device__ __forceinline__ float to_f(float v) { return v; }

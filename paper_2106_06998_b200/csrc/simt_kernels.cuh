@@ -171,9 +171,10 @@ static __global__ void __launch_bounds__(256) gemm_tn_simt_async(const float* A,
 }
 
 // out[i] = scale(i) * sum_s part[s][i].  LANES threads share an output and take the splits in turn; their sums are added in a
-// fixed order, so results are reproducible.  scale(i) = chan_scale[i % period] if chan_scale else alpha.
-// Launch with 256 threads: 256 / LANES outputs per block.
-template <bool PDL, int LANES>
+// fixed order, so results are reproducible.  scale(i) = chan_scale[i % period] if chan_scale else alpha.  Launch with 256 threads: 256 / LANES outputs per block.
+// PAIRS: every 32nd split is added in turn and the 32 sums in pairs, the same bits with 32 lanes and with 8 (one after the other, 32 sums would be rounded at the
+// size of the whole more often than the eight of the other form, 1.13 times its error in the float sketch); eight loads of a thread are in flight.
+template <bool PDL, int LANES, bool PAIRS>
 static __global__ void __launch_bounds__(256)
 reduce_partials(const float* part, float* out, long count, int splits, float alpha, const float* chan_scale, int period) {
   constexpr int OUT = 256 / LANES;
@@ -183,8 +184,15 @@ reduce_partials(const float* part, float* out, long count, int splits, float alp
   const long i = (long)blockIdx.x * OUT + o;
   float s = 0.f;
   if (i < count) {
-    if (LANES == 32) {
-      s = sum_splits<LANES, 8>(part + i, (size_t)count, g, splits);
+    if (PAIRS) {
+      constexpr int OWN = 32 / LANES;                // sums of a thread: of the splits g, g + LANES, .. modulo 32
+      float own[OWN];
+      sum_splits<LANES, 8>(part + i, (size_t)count, g, splits, own);
+#pragma unroll
+      for (int h = OWN / 2; h > 0; h /= 2)
+#pragma unroll
+        for (int l = 0; l < h; ++l) own[l] += own[l + h];
+      s = own[0];
     } else {
 #pragma unroll 4
       for (int k = g; k < splits; k += LANES) s += __ldcg(part + (size_t)k * count + i);
@@ -194,24 +202,19 @@ reduce_partials(const float* part, float* out, long count, int splits, float alp
   acc[g][o] = s;
   __syncthreads();
   if (g != 0 || i >= count) return;
-  float t;
-  if (LANES == 32) {
-    // (in pairs: one after the other, 32 sums would be rounded at the size of the whole more often than the eight of the other form, 1.13 times its error
-    // in the float sketch)
-    float v[LANES];
+  float v[LANES];
 #pragma unroll
-    for (int l = 0; l < LANES; ++l) v[l] = acc[l][o];
+  for (int l = 0; l < LANES; ++l) v[l] = acc[l][o];
+  if (PAIRS) {
 #pragma unroll
     for (int h = LANES / 2; h > 0; h /= 2)
 #pragma unroll
       for (int l = 0; l < h; ++l) v[l] += v[l + h];
-    t = v[0];
   } else {
-    t = acc[0][o];
 #pragma unroll
-    for (int l = 1; l < LANES; ++l) t += acc[l][o];
+    for (int l = 1; l < LANES; ++l) v[0] += v[l];
   }
-  out[i] = t * (chan_scale ? chan_scale[i % period] : alpha);
+  out[i] = v[0] * (chan_scale ? chan_scale[i % period] : alpha);
 }
 
 // ---------------------------------------------------------------------------------------------
