@@ -455,11 +455,12 @@ static size_t probes_bytes(const xconv_desc* d) {
 // Every block of a dependent launch pays for its go-ahead and its wait: 51200 blocks (5 x 5, 128 -> 512 channels) 34 us without,
 // 54 with; 36000 blocks 26 and 38; 18000 14 and 20.  It saves 2 us of launch (1280 blocks 22.6 without, 20.3 with).
 static const unsigned REDUCE_PDL_BLOCKS = 6000;
-// Many splits of up to 16384 outputs are added in pairs, with eight loads of a thread in flight.  Up to 2304 outputs 32 threads share one: us a launch behind
-// a kernel that writes the partial sums, 8 threads -> 32: 64 outputs of 200 splits 6.3 -> 5.2, of 2048 21 -> 16.5, 1152 of 2048 26.7 -> 24.7, up to 140 splits
-// the same; but 4096 of 64 4.4 -> 6.3, 12960 of 140 8.2 -> 10.3.  Few splits, or more outputs, lose with that many loads: 65536 of 7 3.8 -> 5.1, of 200 18.6 -> 24.6.
+// Many splits of up to 16384 outputs are added in pairs, with eight loads of a thread in flight (few splits, or more outputs, lose with that many: us a launch,
+// 65536 of 7 3.8 -> 5.1, of 200 18.6 -> 24.6).  32 threads share an output while their blocks are one wave, eight to an SM: 9472 outputs.  Steps of 32 layers
+// with 440 to 16384 outputs of 64 to 296 splits take 0.996 of what they take with that line at 2304; behind a kernel that ends first, 8 threads -> 32, us: 64 outputs
+// of 200 splits 6.3 -> 5.2, of 2048 21 -> 16.5, 8192 of 64 to 200 the same or 1.9 more, but 12960 of 140 8.2 -> 10.3, of 512 14.5 -> 18.6.
 static bool paired_sums(long count, int splits) { return splits >= 64 && count <= 16384; }
-static bool wide_sums(long count, int splits) { return paired_sums(count, splits) && count <= 2304; }
+static bool wide_sums(long count, int splits) { return paired_sums(count, splits) && count <= 148L * 8 * 8; }
 static xconv_status run_reduce(const float* part, float* out, long count, int splits, float alpha, const float* chan_scale,
                                int period, cudaStream_t st) {
   const bool wide = wide_sums(count, splits);

@@ -48,13 +48,13 @@ def test_float_backprobe_of_whole_numbers_is_exact(r, B, C, H, W):
 
 @pytest.mark.parametrize("dtype,r,B,C,H,W,wide", [
     ("f32", 7, 3, 16, 32, 32, True),          # multiply-adds; a last block of five outputs
-    ("f32", 48, 48, 32, 128, 128, True),      # split operands, the most outputs that 32 threads share
-    ("f32", 49, 48, 32, 128, 128, False),     # ... and the first that eight share; a last block of sixteen
-    ("f32", 70, 33, 32, 128, 128, False),
+    ("f32", 96, 98, 32, 64, 64, True),        # split operands, nearly the most outputs that 32 threads share
+    ("f32", 97, 98, 32, 64, 64, False),       # ... and some of the first that eight share; a last block of two
+    ("f32", 70, 33, 32, 128, 128, True),
     ("f32", 128, 128, 32, 64, 64, False),     # ... the most that are added in pairs
     ("f32", 129, 128, 32, 64, 64, False),     # ... and the first that are not
     ("bf16", 101, 5, 16, 64, 64, True),       # in a stream
-    ("bf16", 601, 5, 16, 64, 64, False),
+    ("bf16", 2001, 5, 16, 64, 64, False),
 ])
 def test_sums_of_many_splits_are_exact(dtype, r, B, C, H, W, wide):
     storage = torch.float32 if dtype == "f32" else torch.bfloat16
